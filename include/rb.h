@@ -112,7 +112,8 @@ typedef struct rb_stats_t {
     double  ms_stage[12];
     int64_t corrections;      /* learned walk: band cells corrected by the network in the last walk */
     int64_t warp_iterations;  /* FP32 walk: warp iterations of the last walk (union walk: entries
-                                 processed, 32 targets each; group walk: frontier rounds, list
+                                 processed, 32 targets each, or with few particles rounds of up
+                                 to 32 entries of one target; group walk: frontier rounds, list
                                  entries and mixed-subtree iterations) */
     int64_t walk_group;       /* FP32 walk shape: 0 union walk, 4 group walk (4-lane subgroups
                                  for the mixed subtrees) */

@@ -245,9 +245,10 @@ void build_topology(const Tree& T, const PSet& P, Ctl* ctl, const BoxP* boxes, c
 // 10-level 2D Hilbert key of (x, y) (thin sheets), kTileHilbertXYZ by a
 // 7-level 3D Hilbert key, the box id above either; ties keep Morton order.
 void build_tile_order(Tree& T, const PSet& P, Ctl* ctl, int mode, int box_bits, cudaStream_t s);
-// Moments and walk records.  fp64: FP64 records only (FP64 walk, potential);
-// otherwise FP64 and FP32 records, and with f32q the quadrupole is summed in
-// FP32 (the FP64 quadrupole records then hold its FP32 values).
+// Moments and walk records.  fp64 (FP64 walk, potential): FP64 records and
+// the FP32 records of the opening test; otherwise all FP64 and FP32 records,
+// and with f32q the quadrupole is summed in FP32 (the FP64 quadrupole records
+// then hold its FP32 values).
 void build_gravity_records(const Tree& T, const PSet& P, Ctl* ctl, const BoxP* boxes,
                            const SimC& C, bool fp64, cudaStream_t s, bool f32q = false);
 // Collision records on the tree of the last gravity build at the current

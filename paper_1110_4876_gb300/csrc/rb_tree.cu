@@ -224,7 +224,7 @@ struct GravRecArgs {
     const Ctl* ctl;
     int ncap;
     double crit_scale;  // 1 / theta^2
-    bool fp32, inside;
+    bool q32, inside;   // q32: FP32 quadrupole records are read too (not by the FP64 walk)
 };
 
 // Leaf records (FP64 and FP32) of every particle.
@@ -236,14 +236,12 @@ __global__ void __launch_bounds__(256) k_leaf_records(GravRecArgs A) {
     const double x = A.x[p], y = A.y[p], z = A.z[p];
     const double m = A.has_test ? source_mass(A.boxes[A.box[p]], A.id[p], A.m[p]) : A.m[p];
     A.d_a[e] = make_double4_32a(x, y, z, -m);
-    if (A.fp32) {
-        float hx, lx, hy, ly, hz, lz;
-        split_hilo(x, hx, lx);
-        split_hilo(y, hy, ly);
-        split_hilo(z, hz, lz);
-        A.ra[e] = make_float4(hx, hy, hz, lz);
-        A.rb[e] = make_float4(lx, ly, -(float)m, __int_as_float(e + 1));
-    }
+    float hx, lx, hy, ly, hz, lz;
+    split_hilo(x, hx, lx);
+    split_hilo(y, hy, ly);
+    split_hilo(z, hz, lz);
+    A.ra[e] = make_float4(hx, hy, hz, lz);
+    A.rb[e] = make_float4(lx, ly, -(float)m, __int_as_float(e + 1));
 }
 
 // Cells per depth: counts (block histograms, one atomic per depth and
@@ -452,14 +450,14 @@ __device__ __forceinline__ void mom_finish(const GravRecArgs& A, int k, int dept
         c0z = __dadd_rn(lo, __dmul_rn(iz, w));
         A.d_c[k] = make_double4_32a(c0x, c0y, c0z, w);
     }
-    if (A.fp32) {
-        float hx, lx, hy, ly, hz, lz;
-        split_hilo(cx, hx, lx);
-        split_hilo(cy, hy, ly);
-        split_hilo(cz, hz, lz);
-        const float crit = never ? __int_as_float(0x7f800000) : (float)(ww * A.crit_scale);
-        A.ra[k] = make_float4(hx, hy, hz, lz);
-        A.rb[k] = make_float4(lx, ly, crit, __int_as_float(end));
+    float hx, lx, hy, ly, hz, lz;
+    split_hilo(cx, hx, lx);
+    split_hilo(cy, hy, ly);
+    split_hilo(cz, hz, lz);
+    const float crit = never ? __int_as_float(0x7f800000) : (float)(ww * A.crit_scale);
+    A.ra[k] = make_float4(hx, hy, hz, lz);
+    A.rb[k] = make_float4(lx, ly, crit, __int_as_float(end));
+    if (A.q32) {
         if (kF32Q) {
             A.rq0[k] = make_float4((float)S.M, S.qf[0], S.qf[1], S.qf[2]);
             A.rq1[k] = make_float4(S.qf[3], S.qf[4], S.qf[5], 0.f);
@@ -467,13 +465,13 @@ __device__ __forceinline__ void mom_finish(const GravRecArgs& A, int k, int dept
             A.rq0[k] = make_float4((float)S.M, (float)S.q[0], (float)S.q[1], (float)S.q[2]);
             A.rq1[k] = make_float4((float)S.q[3], (float)S.q[4], (float)S.q[5], 0.f);
         }
-        if (A.inside) {
-            split_hilo(c0x, hx, lx);
-            split_hilo(c0y, hy, ly);
-            split_hilo(c0z, hz, lz);
-            A.rc_hi[k] = make_float4(hx, hy, hz, (float)w);
-            A.rc_lo[k] = make_float4(lx, ly, lz, 0.f);
-        }
+    }
+    if (A.inside) {
+        split_hilo(c0x, hx, lx);
+        split_hilo(c0y, hy, ly);
+        split_hilo(c0z, hz, lz);
+        A.rc_hi[k] = make_float4(hx, hy, hz, (float)w);
+        A.rc_lo[k] = make_float4(lx, ly, lz, 0.f);
     }
 }
 
@@ -950,7 +948,7 @@ void build_gravity_records(const Tree& T, const PSet& P, Ctl* ctl, const BoxP* b
     A.ctl = ctl;
     A.ncap = n;
     A.crit_scale = C.crit_scale;
-    A.fp32 = !fp64;
+    A.q32 = !fp64;
     A.inside = C.theta2 > (1.0 / 3.0);
     k_leaf_records<<<ceil_div(n, 256), 256, 0, s>>>(A);
     cudaMemsetAsync(T.lvl, 0, sizeof(int32_t) * 96, s);

@@ -20,142 +20,12 @@
 #include <mutex>
 #include <vector>
 
-#include "rb_internal.cuh"
-#include "rb_mlp.cuh"
+#include <algorithm>
+
+#include "rb_walk.cuh"
 
 namespace rb {
 namespace {
-
-constexpr unsigned kFull = 0xffffffffu;
-
-struct GravArgs {
-    const double *x, *y, *z;
-    const int32_t* box;
-    Rec4 ra, rb, rq0, rq1, rc_hi, rc_lo;
-    const double4_32a *d_a, *d_q0, *d_q1, *d_c;
-    const int32_t *e_skip, *leaf_of, *box_root;
-    const uint32_t* order;      // tile order of the targets (nullptr: Morton order of the slots)
-    const int32_t* e_child;     // per cell entry: child entry of each octant (group walk)
-    const uint32_t* e_cmask;    // per cell entry: octants holding a child (0: depth-21 group)
-    const BoxP* boxes;
-    Ctl* ctl;
-    WalkOut out;
-    int ncap;
-    int ngx, ngy, ngz;
-    int half_step_offset;
-    double G, theta2, soft2, t0, half_dt;
-    float soft2f;
-    // recording of accepted cells in the band w/R > theta_lo (learned mode)
-    uint64_t* req;
-    int* req_count;
-    int req_cap;
-    float band_scale;   // (theta_lo / theta)^2: band iff (w/theta)^2 > band_scale R^2
-    uint32_t thresh;    // keep a request when its hash < thresh (0xffffffff: all)
-    uint32_t seed;
-    // learned walk: cell particle counts (an input of the network) and weights
-    const int32_t* e_count;
-    const mlp::Packed* wpk;
-    int ecap;   // entry capacity (every entry index below it is readable)
-    const ImgTab* img;   // [box][image] offsets at the time of this walk
-    int nimg;
-    int32_t* tq;         // tile queues (emptied by the image-table launch)
-    int nq;
-};
-
-__device__ __forceinline__ double4_32a ld_d4(const double4_32a* p) { return *p; }
-
-// Counter-based hash of a (target, cell, image) request for subsampling.
-__device__ __forceinline__ uint32_t req_hash(uint32_t slot, uint32_t entry, uint32_t code,
-                                             uint32_t seed) {
-    uint32_t h = slot * 0x9E3779B1u ^ (entry + 0x7F4A7C15u) * 0x85EBCA77u ^ code * 0xC2B2AE3Du ^ seed;
-    h ^= h >> 16;
-    h *= 0x7FEB352Du;
-    h ^= h >> 15;
-    h *= 0x846CA68Bu;
-    h ^= h >> 16;
-    return h;
-}
-
-// Opening test in FP64, operation for operation as the oracle evaluates it.
-__device__ __forceinline__ bool mac64(const double4_32a& a, double theta2, double tx, double ty,
-                                      double tz) {
-    const double dx = __dsub_rn(a.x, tx), dy = __dsub_rn(a.y, ty), dz = __dsub_rn(a.z, tz);
-    const double r2 = __dadd_rn(__dadd_rn(__dmul_rn(dx, dx), __dmul_rn(dy, dy)), __dmul_rn(dz, dz));
-    return a.w < __dmul_rn(theta2, r2);
-}
-
-// 1/sqrt(x) from the hardware estimate plus one Newton step
-// y' = y (3/2 - x y^2 / 2), which roughly halves its relative error.
-__device__ __forceinline__ float rsqrt_nr(float x) {
-    const float y = rsqrtf(x);
-    return y * fmaf((-0.5f * x) * y, y, 1.5f);
-}
-
-// Compensated (Kahan) accumulation: in a sheet the net force is often a
-// small remainder of much larger cancelling terms, and a plain FP32 running
-// sum loses ~1e-5 of it.  The walk sums terms plainly over at most 16 warp
-// iterations and adds those short partial sums into Kahan sums, whose
-// running compensation c keeps the lost low-order bits.
-__device__ __forceinline__ void kadd(float& s, float& c, float t) {
-    const float y = t - c;
-    const float u = s + y;
-    c = (u - s) - y;
-    s = u;
-}
-
-// Tile scheduling of the walks: queue q owns tiles [b_q, b_{q+1}) with
-// b_q = floor(q T / nq) of the T tiles of 32 consecutive targets.
-__device__ __forceinline__ int tile_begin(int q, int ntile, int nq) {
-    return (int)(((long long)q * ntile) / nq);
-}
-
-__device__ __forceinline__ int sm_queue(int nq) {
-    unsigned sm;
-    asm volatile("mov.u32 %0, %%smid;" : "=r"(sm));
-    return (int)(sm % (unsigned)nq);
-}
-
-// Slot of the k-th target in tile order.
-__device__ __forceinline__ int tile_slot(const uint32_t* order, int k) {
-    return order ? (int)__ldg(&order[k]) : k;
-}
-
-// The warp's next tile, or -1 when every queue is empty: its own SM's queue
-// first, then the following queues (32 probed per vote).  Warp-uniform.
-__device__ __noinline__ int next_tile(int32_t* tq, int nq, int q, int ntile) {
-    const int lane = threadIdx.x & 31;
-    int t = -1;
-    if (lane == 0) {
-        const int b = tile_begin(q, ntile, nq);
-        const int k = atomicAdd(&tq[q * kTileQStride], 1);
-        if (k < tile_begin(q + 1, ntile, nq) - b) t = b + k;
-    }
-    t = __shfl_sync(kFull, t, 0);
-    if (t >= 0) return t;
-    for (int k0 = 1; k0 < nq; k0 += 32) {
-        const int off = k0 + lane;
-        int qq = q + off;
-        if (qq >= nq) qq -= nq;
-        int b = 0, len = 0;
-        bool avail = false;
-        if (off < nq) {
-            b = tile_begin(qq, ntile, nq);
-            len = tile_begin(qq + 1, ntile, nq) - b;
-            avail = __ldcg(&tq[qq * kTileQStride]) < len;
-        }
-        for (unsigned m = __ballot_sync(kFull, avail); m; m &= m - 1) {
-            const int src = __ffs(m) - 1;
-            int got = -1;
-            if (lane == src) {
-                const int k = atomicAdd(&tq[qq * kTileQStride], 1);
-                if (k < len) got = b + k;
-            }
-            got = __shfl_sync(kFull, got, src);
-            if (got >= 0) return got;
-        }
-    }
-    return -1;
-}
 
 // Ghost-image table of the walk or search time: one thread per (box, image),
 // images in the kernels' loop order (gx outermost, gz innermost), for boxes
@@ -182,63 +52,6 @@ __global__ void k_img_table(const BoxP* __restrict__ boxes, const Ctl* __restric
     T.lo = make_float4(__double2float_rn(T.ox - (double)hx), __double2float_rn(T.oy - (double)hy),
                        __double2float_rn(T.oz - (double)hz), 0.f);
     tab[k] = T;
-}
-
-// t = p - o for hi/lo float pairs: the rounding error of ph - oh is kept
-// (Knuth's two-sum) and the low parts are subtracted, so t is good to about
-// 2^-45 of |p| without any FP64 arithmetic.
-__device__ __forceinline__ void sub_hilo(float ph, float pl, float oh, float ol, float& th, float& tl) {
-    const float s = ph - oh;
-    const float bb = s - ph;
-    const float e = (ph - (s - bb)) + (-oh - bb);
-    th = s;
-    tl = e + (pl - ol);
-}
-
-__device__ __forceinline__ void split_d(double v, float& hi, float& lo) {
-    hi = __double2float_rn(v);
-    lo = __double2float_rn(v - (double)hi);
-}
-
-// Is the target point inside the closed cube of a cell (FP64, exact sequence)?
-__device__ __forceinline__ bool inside64(const double4_32a& c, double tx, double ty, double tz) {
-    return c.x <= tx && tx <= __dadd_rn(c.x, c.w) && c.y <= ty && ty <= __dadd_rn(c.y, c.w) &&
-           c.z <= tz && tz <= __dadd_rn(c.z, c.w);
-}
-
-// Per-warp queue of the learned walk: accepted band cells waiting for the
-// network, which runs on 16 of them at a time (one m16 tile).
-struct LearnQ {
-    __nv_bfloat16 X[48][16];   // network inputs (columns 12..15 zero)
-    float unit[48];            // M / R^2 (G is applied with the walk's sums)
-    int own[48];               // lane whose sums receive the output
-    float Y[16][4];            // outputs of the tile being applied
-};
-
-// Rows r0 .. r0 + 15 of the queue through the network; unit * output is
-// added to the owning lanes' partial sums.  Warp-synchronous.
-__device__ __forceinline__ void learn_flush(LearnQ& Q, const mlp::Packed& w, int r0, int lane,
-                                            float& fx, float& fy, float& fz) {
-    __syncwarp();
-    float out[4];
-    mlp::forward_packed(w, &Q.X[r0][0], out);
-    const int g = lane >> 2, q = lane & 3;
-    if (q < 2) {
-        Q.Y[g][2 * q] = out[0];
-        Q.Y[g][2 * q + 1] = out[1];
-        Q.Y[g + 8][2 * q] = out[2];
-        Q.Y[g + 8][2 * q + 1] = out[3];
-    }
-    __syncwarp();
-#pragma unroll 4
-    for (int k = 0; k < 16; k++)
-        if (Q.own[r0 + k] == lane) {
-            const float u = Q.unit[r0 + k];
-            fx += u * Q.Y[k][0];
-            fy += u * Q.Y[k][1];
-            fz += u * Q.Y[k][2];
-        }
-    __syncwarp();
 }
 
 // kOne: a single box, so every lane's walk ends at the same entry and no
@@ -598,45 +411,6 @@ __device__ __forceinline__ void glane_count(GLane& L) {
         glane_flush(L);
         L.fcount = 0;
     }
-}
-
-// Monopole + quadrupole term of an accepted cell (reading R3), the same
-// arithmetic as the union walk's; a particle leaf is the cell with Q = 0.
-template <bool kQuad, bool kSoft>
-__device__ __forceinline__ void cell_term(float dx, float dy, float dz, float r2, const float4& q0,
-                                          const float4& q1, float soft2f, float& fx, float& fy,
-                                          float& fz) {
-    const float inv = rsqrt_nr(r2);
-    const float inv2 = inv * inv;
-    const float invs = kSoft ? rsqrt_nr(r2 + soft2f) : inv;
-    float fc = q0.x * (kSoft ? invs * invs * invs : inv2 * inv);
-    if (kQuad) {
-        const float qx = fmaf(q1.y, dz, fmaf(q1.x, dy, q0.y * dx));
-        const float qy = fmaf(q1.z, dz, fmaf(q0.z, dy, q1.x * dx));
-        const float qz = fmaf(q0.w, dz, fmaf(q1.z, dy, q1.y * dx));
-        const float dqd = fmaf(dz, qz, fmaf(dy, qy, dx * qx));
-        const float inv5 = inv2 * inv2 * inv;
-        fc = fmaf(2.5f, dqd * (inv5 * inv2), fc);
-        fx = fmaf(-inv5, qx, fx);
-        fy = fmaf(-inv5, qy, fy);
-        fz = fmaf(-inv5, qz, fz);
-    }
-    fx = fmaf(fc, dx, fx);
-    fy = fmaf(fc, dy, fy);
-    fz = fmaf(fc, dz, fz);
-}
-
-// Record minus target for the negated target point (nxy: x, y hi; lxy: x, y
-// lo; nz: z hi, lo).
-__device__ __forceinline__ void rec_diff(const float4& ra, const float4& rb, float2 nxy, float2 lxy,
-                                         float2 nz, float& dx, float& dy, float& dz, float& r2) {
-    const float2 dxy = __fadd2_rn(__fadd2_rn(make_float2(ra.x, ra.y), nxy),
-                                  __fadd2_rn(make_float2(rb.x, rb.y), lxy));
-    dx = dxy.x;
-    dy = dxy.y;
-    const float2 zz = __fadd2_rn(make_float2(ra.z, ra.w), nz);
-    dz = zz.x + zz.y;
-    r2 = fmaf(dz, dz, fmaf(dy, dy, dx * dx));
 }
 
 // The negated target point x - o of image img as hi/lo floats, formed from
@@ -1034,121 +808,6 @@ __global__ void __launch_bounds__(kMaxWalkBlock, 2) k_walk32_learn(GravArgs A) {
         walk32<true, kInside, false, kSoft, false, true>(A, &q[threadIdx.x >> 5], &w, t << 5, n);
 }
 
-// FP64 walk: the same traversal on FP64 records, every opening test in the
-// oracle's operation sequence.
-template <bool kQuad, bool kInside, bool kPot>
-__device__ __forceinline__ void walk64(const GravArgs& A, int wbase, int n) {
-    const int lane = threadIdx.x & 31;
-    const bool valid = wbase + lane < n;
-    const int ii = tile_slot(A.order, valid ? wbase + lane : n - 1);
-    const int i = ii;   // the target's slot
-    const double px = A.x[ii], py = A.y[ii], pz = A.z[ii];
-    const int root = A.box_root[A.box[ii]];
-    const int wend = root >= 0 ? A.e_skip[root] : 0;   // end of this box's tree
-    const int self_leaf = A.leaf_of[ii];
-    const ImgTab* itab = A.img + (size_t)A.box[ii] * A.nimg;
-    int gi = 0;
-    const double soft2 = A.soft2;
-    double ax = 0.0, ay = 0.0, az = 0.0, pot = 0.0;
-    int ncell = 0, nleaf = 0, nmac = 0;
-    for (int gx = -A.ngx; gx <= A.ngx; gx++)
-        for (int gy = -A.ngy; gy <= A.ngy; gy++)
-            for (int gz = -A.ngz; gz <= A.ngz; gz++, gi++) {
-                const double ox = itab[gi].ox, oy = itab[gi].oy, oz = itab[gi].oz;
-                const double tx = __dsub_rn(px, ox), ty = __dsub_rn(py, oy), tz = __dsub_rn(pz, oz);
-                const int self = (gx == 0 && gy == 0 && gz == 0) ? self_leaf : -1;
-                int next = (valid && root >= 0) ? root : kEnd;
-                for (;;) {
-                    if (next >= wend) next = kEnd;
-                    const int e = (int)__reduce_min_sync(kFull, (unsigned)next);
-                    if (e == kEnd) break;
-                    const double4_32a a = ld_d4(&A.d_a[e]);
-                    const bool act = next == e;
-                    if (__double_as_longlong(a.w) < 0) {
-                        if (act) {
-                            if (e != self) {
-                                const double dx = a.x - tx, dy = a.y - ty, dz = a.z - tz;
-                                const double r2 = fma(dz, dz, fma(dy, dy, dx * dx)) + soft2;
-                                const double inv = rsqrt(r2);
-                                const double f = -a.w * (inv * inv * inv);
-                                ax = fma(f, dx, ax);
-                                ay = fma(f, dy, ay);
-                                az = fma(f, dz, az);
-                                if (kPot) pot = fma(a.w, inv, pot);
-                                nleaf++;
-                            }
-                            next = e + 1;
-                        }
-                    } else if (act) {
-                        nmac++;
-                        bool acc = mac64(a, A.theta2, tx, ty, tz);
-                        if (kInside && acc) acc = !inside64(ld_d4(&A.d_c[e]), tx, ty, tz);
-                        if (acc) {
-                            const double4_32a q0 = ld_d4(&A.d_q0[e]);
-                            const double dx = a.x - tx, dy = a.y - ty, dz = a.z - tz;
-                            const double r2 = fma(dz, dz, fma(dy, dy, dx * dx));
-                            const double invs = rsqrt(r2 + soft2);
-                            const double f = q0.x * (invs * invs * invs);
-                            ax = fma(f, dx, ax);
-                            ay = fma(f, dy, ay);
-                            az = fma(f, dz, az);
-                            if (kPot) pot = fma(-q0.x, invs, pot);
-                            if (kQuad) {
-                                const double4_32a q1 = ld_d4(&A.d_q1[e]);
-                                const double inv = rsqrt(r2);
-                                const double inv2 = inv * inv;
-                                const double qx = fma(q1.y, dz, fma(q1.x, dy, q0.y * dx));
-                                const double qy = fma(q1.z, dz, fma(q0.z, dy, q1.x * dx));
-                                const double qz = fma(q0.w, dz, fma(q1.z, dy, q1.y * dx));
-                                const double dqd = fma(dz, qz, fma(dy, qy, dx * qx));
-                                const double inv5 = inv2 * inv2 * inv;
-                                const double c = 2.5 * dqd * (inv5 * inv2);
-                                ax = fma(c, dx, fma(-inv5, qx, ax));
-                                ay = fma(c, dy, fma(-inv5, qy, ay));
-                                az = fma(c, dz, fma(-inv5, qz, az));
-                                if (kPot) pot = fma(-0.5 * dqd, inv5, pot);
-                            }
-                            ncell++;
-                            next = A.e_skip[e];
-                        } else {
-                            next = e + 1;
-                        }
-                    }
-                }
-            }
-    if (valid) {
-        A.out.ax[i] = A.G * ax;
-        A.out.ay[i] = A.G * ay;
-        A.out.az[i] = A.G * az;
-        if (kPot) A.out.phi[i] = A.G * pot;
-        if (A.out.ncell) {
-            A.out.ncell[i] = ncell;
-            A.out.nleaf[i] = nleaf;
-            A.out.nmac[i] = nmac;
-        }
-    }
-    unsigned long long c0 = valid ? ncell : 0, c1 = valid ? nleaf : 0, c2 = valid ? nmac : 0;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        c0 += __shfl_down_sync(kFull, c0, o);
-        c1 += __shfl_down_sync(kFull, c1, o);
-        c2 += __shfl_down_sync(kFull, c2, o);
-    }
-    if (lane == 0) {
-        atomicAdd(&A.ctl->n_cell, c0);
-        atomicAdd(&A.ctl->n_leaf, c1);
-        atomicAdd(&A.ctl->n_mac, c2);
-    }
-}
-
-template <bool kQuad, bool kInside, bool kPot>
-__global__ void __launch_bounds__(kMaxWalkBlock) k_walk64(GravArgs A) {
-    const int n = min(A.ctl->n_live, A.ncap);
-    const int ntile = (n + 31) >> 5, q = sm_queue(A.nq);
-    for (int t = next_tile(A.tq, A.nq, q, ntile); t >= 0; t = next_tile(A.tq, A.nq, q, ntile))
-        walk64<kQuad, kInside, kPot>(A, t << 5, n);
-}
-
 struct CollArgs {
     const double *x, *y, *z, *r;
     const int32_t *id, *box;
@@ -1400,10 +1059,20 @@ int persistent_grid(F fn, int block, int cap_n) {
 
 template <typename F>
 void prepare_one(F fn) {
-    for (int b : {64, 128, 256}) residency(reinterpret_cast<const void*>(fn), b);
+    walk_prepare_kernel(reinterpret_cast<const void*>(fn));
 }
 
 }  // namespace
+
+void walk_prepare_kernel(const void* fn) {
+    for (int b : {64, 128, 256}) residency(fn, b);
+}
+
+int walk_grid(const void* fn, int block, long long warps) {
+    const long long need = (warps * 32 + block - 1) / block;
+    const long long fit = (long long)max(g_nsm, 1) * residency(fn, block);
+    return (int)std::max<long long>(1, std::min(need, fit));
+}
 
 int walk_prepare() {
     {
@@ -1433,10 +1102,7 @@ int walk_prepare() {
     prepare_one(k_walk32<true, false, false, true, true>); prepare_one(k_walk32<true, false, false, false, true>);
     prepare_one(k_walk32_learn<true, true>); prepare_one(k_walk32_learn<true, false>);
     prepare_one(k_walk32_learn<false, true>); prepare_one(k_walk32_learn<false, false>);
-    prepare_one(k_walk64<true, true, true>); prepare_one(k_walk64<true, true, false>);
-    prepare_one(k_walk64<true, false, true>); prepare_one(k_walk64<true, false, false>);
-    prepare_one(k_walk64<false, true, true>); prepare_one(k_walk64<false, true, false>);
-    prepare_one(k_walk64<false, false, true>); prepare_one(k_walk64<false, false, false>);
+    target_walk_prepare();
 #define RB_PREP_G(Q, I, S) \
     prepare_one(k_gwalk32<Q, I, S, true, 4>); prepare_one(k_gwalk32<Q, I, S, false, 4>)
     RB_PREP_G(true, true, true); RB_PREP_G(true, true, false);
@@ -1506,11 +1172,12 @@ void gravity_walk(const Tree& T, const PSet& P, Ctl* ctl, const BoxP* boxes, con
             RB_W32G(Q, I, S, false);                                       \
         }                                                                  \
     } while (0)
-#define RB_W64(Q, I, PO) RB_LAUNCH(k_walk64<Q, I, PO>)
     if (learn && !potential) {
         // FP32 walk with the learned correction of band cells (quadrupole on)
         A.band_scale = learn->band_scale;
-        if (inside) {
+        if (T.cap_n <= kTargetWalkMax) {
+            target_walk(A, TargetWalk::kLearned, true, inside, soft, false, block, T.cap_n, s);
+        } else if (inside) {
             if (soft) RB_LAUNCH(k_walk32_learn<true, true>);
             else RB_LAUNCH(k_walk32_learn<true, false>);
         } else {
@@ -1527,13 +1194,9 @@ void gravity_walk(const Tree& T, const PSet& P, Ctl* ctl, const BoxP* boxes, con
             else RB_LAUNCH(k_walk32<true, false, false, false, true>);
         }
     } else if (walk_mode == 0 || potential) {
-        if (quad) {
-            if (inside) { if (potential) RB_W64(true, true, true); else RB_W64(true, true, false); }
-            else { if (potential) RB_W64(true, false, true); else RB_W64(true, false, false); }
-        } else {
-            if (inside) { if (potential) RB_W64(false, true, true); else RB_W64(false, true, false); }
-            else { if (potential) RB_W64(false, false, true); else RB_W64(false, false, false); }
-        }
+        target_walk(A, TargetWalk::kFp64, quad, inside, soft, potential, block, T.cap_n, s);
+    } else if (group == 0 && T.cap_n <= kTargetWalkMax) {
+        target_walk(A, TargetWalk::kFp32, quad, inside, soft, false, block, T.cap_n, s);
     } else {
         if (quad) {
             if (inside) { if (soft) RB_W32(true, true, false, true); else RB_W32(true, true, false, false); }
@@ -1545,7 +1208,6 @@ void gravity_walk(const Tree& T, const PSet& P, Ctl* ctl, const BoxP* boxes, con
     }
 #undef RB_W32
 #undef RB_W32G
-#undef RB_W64
 }
 
 void collision_search(const Tree& T, const PSet& P, Ctl* ctl, const BoxP* boxes, const SimC& C,
