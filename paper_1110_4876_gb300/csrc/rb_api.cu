@@ -220,19 +220,13 @@ int alloc_pairs(rb_sim* s, int cap) {
     rc |= dalloc(s, &R.key_alt, cap, L);
     rc |= dalloc(s, &R.val, cap, L);
     rc |= dalloc(s, &R.val_alt, cap, L);
-    rc |= dalloc(s, &R.ekey, 2 * (size_t)cap, L);
-    rc |= dalloc(s, &R.ekey_alt, 2 * (size_t)cap, L);
-    rc |= dalloc(s, &R.eval, 2 * (size_t)cap, L);
-    rc |= dalloc(s, &R.eval_alt, 2 * (size_t)cap, L);
-    rc |= dalloc(s, &R.prev_a, cap, L);
-    rc |= dalloc(s, &R.prev_b, cap, L);
-    rc |= dalloc(s, &R.next_a, cap, L);
-    rc |= dalloc(s, &R.next_b, cap, L);
-    rc |= dalloc(s, &R.wait, cap, L);
-    rc |= dalloc(s, &R.queue, cap, L);
-    rc |= dalloc(s, &R.rcnt, 64, L);
+    R.ncap = s->ncap;
+    rc |= dalloc(s, &R.head, s->ncap, L);
+    rc |= dalloc(s, &R.link, cap, L);
+    rc |= dalloc(s, &R.done, cap, L);
+    rc |= dalloc(s, &R.rec, cap, L);
+    rc |= dalloc(s, &R.claim, 1, L);
     rc |= dalloc(s, &R.hist, radix_hist_words(cap), L);
-    rc |= dalloc(s, &R.ehist, radix_hist_words(2 * cap), L);
     R.slot_of_id = keep_slot;
     return rc ? RB_ERR_CUDA : RB_OK;
 }

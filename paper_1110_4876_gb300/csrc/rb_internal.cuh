@@ -66,8 +66,6 @@ struct Ctl {
     int n_entries;             // tree entries (cells + leaves) of the last build
     int pair_count;            // pairs found by the last search (may exceed capacity)
     int pair_n;                // pairs to resolve (0 when the search overflowed)
-    int pair_ends;             // 2 * pair_n
-    int pending;               // pairs not yet resolved
     int resolved;              // pairs that were approaching and were resolved
     int err;                   // error bits (kErr*)
     int req_count;             // learned-correction requests recorded by the last walk
@@ -153,20 +151,27 @@ struct Tree {
 // Target orders of the walk and search tiles (the values of RB_TILE_*).
 enum { kTileMorton = 0, kTileHilbertXY = 1, kTileHilbertXYZ = 2 };
 
+// A collision pair as the resolution reads it: separation (image of b) - a,
+// the image's y velocity offset, the factors of u.r that v_a gains and v_b
+// loses along it, the particles' slots, and the pairs that must come before.
+struct __align__(64) PairRec {
+    double rx, ry, rz, dvy, ka, kb;
+    int a, b;
+    int pa, pb;   // previous pair of particle a / b in resolution order, or -1
+};
+
 // Pairs and their resolution.
 struct Pairs {
     uint64_t *key, *key_alt;
     uint32_t *val, *val_alt;   // unused payload for the sort
-    uint64_t *ekey, *ekey_alt; // pair ends: particle slot (sort key)
-    uint32_t *eval, *eval_alt; // pair ends: 2 * pair + side
-    int32_t *prev_a, *prev_b;  // previous pair (queue order) of particle a / b, or -1
-    int32_t *next_a, *next_b;  // next pair of particle a / b, or -1
-    int32_t* wait;             // unresolved predecessors of each pair
-    int32_t* queue;            // pairs in the order they became ready (resolution)
-    int32_t* rcnt;             // queue counters: [0] slots written, [1] slots claimed
+    int32_t *head, *link;      // pairs of each particle as the higher id (lists; head: one per id)
+    int32_t* done;             // per pair: resolved
+    PairRec* rec;              // per pair: geometry, impulse factors, predecessors
+    int32_t* claim;            // pairs claimed so far by the resolving warps
     int32_t* slot_of_id;       // global id -> slot in the current set
-    uint32_t *hist, *ehist;
+    uint32_t* hist;
     int cap;
+    int ncap;                  // particle ids (entries of head)
     bool sorted_alt = false;   // the last pair sort left the sorted keys in key_alt
     const uint64_t* sorted() const { return sorted_alt ? key_alt : key; }
 };

@@ -11,11 +11,7 @@
 #include <algorithm>
 #include <climits>
 
-#include <cooperative_groups.h>
-
 #include "rb_internal.cuh"
-
-namespace cg = cooperative_groups;
 
 namespace rb {
 namespace {
@@ -218,170 +214,98 @@ __global__ void k_pairs_prep(Ctl* ctl, int cap) {
     const int c = ctl->pair_count;
     const int n = c <= cap ? c : 0;
     ctl->pair_n = n;
-    ctl->pair_ends = 2 * n;
-    ctl->pending = n;
     ctl->resolved = 0;
 }
 
 struct ResolveArgs {
     PSet P;
-    const uint64_t* key;
+    const uint64_t* key;          // sorted pairs (resolution order)
     const int32_t* slot_of_id;
-    const int32_t *prev_a, *prev_b;   // previous pair of particle a / b (queue order), or -1
-    const int32_t *next_a, *next_b;   // next pair of particle a / b, or -1
-    int32_t* wait;                    // predecessors of a pair not yet resolved
+    int32_t *head, *link;         // per particle: its pairs as the higher id, a list in any order
+    int32_t* done;                // per pair: 1 once resolved
+    PairRec* rec;
+    int32_t* claim;               // pairs claimed by running warps
     Ctl* ctl;
-    const BoxP* boxes;
-    int hs;
-    const ImgTab* img;   // [box][image] offsets at the detection time
+    const ImgTab* img;            // [box][image] offsets at the detection time
     int nimg, ngx, ngy, ngz;
 };
 
-__device__ __forceinline__ void pair_slots(const ResolveArgs& A, uint64_t k, int& sa, int& sb) {
-    sa = A.slot_of_id[(int)(k >> 36)];
-    sb = A.slot_of_id[(int)((k >> 12) & 0xFFFFFFull)];
+__device__ __forceinline__ int key_a(uint64_t k) { return (int)(k >> 36); }
+__device__ __forceinline__ int key_b(uint64_t k) { return (int)((k >> 12) & 0xFFFFFFull); }
+
+// Every pair joins the list of its higher particle id; head is -1 for every
+// particle on entry.
+__global__ void __launch_bounds__(256) k_pair_link(ResolveArgs A) {
+    const int n = A.ctl->pair_n;
+    if (blockIdx.x == 0 && threadIdx.x == 0) *A.claim = 0;
+    for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < n; k += gridDim.x * blockDim.x) {
+        A.link[k] = atomicExch(&A.head[key_b(A.key[k])], k);
+        A.done[k] = 0;
+    }
 }
 
-// Eq. 2 for one pair, in the oracle's operation order.  kCG: velocities are
-// read from L2 (other SMs update them while the queue runs).
-template <bool kCG = false>
-__device__ __forceinline__ bool resolve_one(const ResolveArgs& A, const SimC& C, uint64_t k) {
-    int a, b;
-    pair_slots(A, k, a, b);
-    const int code = (int)(k & 0xFFFull);
-    const int gx = (code & 15) - 7, gy = ((code >> 4) & 15) - 7, gz = ((code >> 8) & 15) - 7;
-    // the image's offsets from the table (same formulas as the search used)
-    const int g = ((gx + A.ngx) * (2 * A.ngy + 1) + (gy + A.ngy)) * (2 * A.ngz + 1) + (gz + A.ngz);
-    const ImgTab& T = A.img[(size_t)A.P.box[a] * A.nimg + g];
-    const double ox = T.ox, oy = T.oy, oz = T.oz, dvg = T.dvy;
-    const double rx = __dsub_rn(__dadd_rn(A.P.x[b], ox), A.P.x[a]);
-    const double ry = __dsub_rn(__dadd_rn(A.P.y[b], oy), A.P.y[a]);
-    const double rz = __dsub_rn(__dadd_rn(A.P.z[b], oz), A.P.z[a]);
-    double vxa, vya, vza, vxb, vyb, vzb;
-    if (kCG) {
-        vxa = __ldcg(&A.P.vx[a]); vya = __ldcg(&A.P.vy[a]); vza = __ldcg(&A.P.vz[a]);
-        vxb = __ldcg(&A.P.vx[b]); vyb = __ldcg(&A.P.vy[b]); vzb = __ldcg(&A.P.vz[b]);
-    } else {
-        vxa = A.P.vx[a]; vya = A.P.vy[a]; vza = A.P.vz[a];
-        vxb = A.P.vx[b]; vyb = A.P.vy[b]; vzb = A.P.vz[b];
-    }
-    const double ux = __dsub_rn(vxb, vxa), uy = __dsub_rn(__dadd_rn(vyb, dvg), vya),
-                 uz = __dsub_rn(vzb, vza);
-    const double rv = __dadd_rn(__dadd_rn(__dmul_rn(rx, ux), __dmul_rn(ry, uy)), __dmul_rn(rz, uz));
-    if (rv >= 0.0) return false;
-    // the impulse along n = r/|r| without forming n: v_a gains
-    // (1 + eps) (m_b/M) (u.r)/|r|^2 r, v_b loses the same with m_a (one
-    // division, no square root: GB300's FP64 rate is 1/64 of FP32)
-    const double r2 = __dadd_rn(__dadd_rn(__dmul_rn(rx, rx), __dmul_rn(ry, ry)), __dmul_rn(rz, rz));
-    double e = C.eps;
-    if (C.eps_law == 1) {
-        // velocity-dependent restitution: min(1, (|v_n| / v_c)^(-p)), |v_n| = |u.r| / |r|
-        const double vn = __ddiv_rn(rv, __dsqrt_rn(r2));
-        const double q = pow(__ddiv_rn(fabs(vn), C.eps_vc), -C.eps_p);
-        e = q < 1.0 ? q : 1.0;
-    }
-    const double ma = A.P.m[a], mb = A.P.m[b];
-    const double mt = __dadd_rn(ma, mb);
-    const double gi = __ddiv_rn(__dmul_rn(__dadd_rn(1.0, e), rv), __dmul_rn(r2, mt));
-    const double ga = __dmul_rn(gi, mb), gb = __dmul_rn(gi, ma);
-    A.P.vx[a] = __dadd_rn(vxa, __dmul_rn(ga, rx));
-    A.P.vy[a] = __dadd_rn(vya, __dmul_rn(ga, ry));
-    A.P.vz[a] = __dadd_rn(vza, __dmul_rn(ga, rz));
-    A.P.vx[b] = __dsub_rn(vxb, __dmul_rn(gb, rx));
-    A.P.vy[b] = __dsub_rn(vyb, __dmul_rn(gb, ry));
-    A.P.vz[b] = __dsub_rn(vzb, __dmul_rn(gb, rz));
-    return true;
+// 1/x from the hardware's coarse FP64 estimate and one step of the cubically
+// convergent iteration y (1 + h + h^2), h = 1 - x y; x outside the range
+// where the estimate is safe takes the division.
+__device__ __forceinline__ double rcp64(double x) {
+    const int e = (int)((__double_as_longlong(x) >> 52) & 0x7ff);
+    if (e < 64 || e > 1982) return __ddiv_rn(1.0, x);
+    double y;
+    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+    const double h = fma(-x, y, 1.0);
+    return fma(y, fma(h, h, h), y);
 }
 
-// Pair ends for the predecessor links: (particle slot, 2 * pair + side).
-__global__ void __launch_bounds__(256) k_pair_ends(ResolveArgs A, uint64_t* __restrict__ ekey,
-                                                   uint32_t* __restrict__ eval) {
+// The last pair before k in particle p's list (pairs in which p is the higher
+// id), or -1.  A list holds as many pairs as the particle has contacts from
+// below; they are resolved one after the other in any case.
+__device__ __forceinline__ int last_before(const ResolveArgs& A, int p, int k) {
+    int best = -1;
+    for (int j = A.head[p]; j >= 0; j = A.link[j])
+        if (j < k) best = max(best, j);
+    return best;
+}
+
+// Everything about a pair that does not depend on velocities: the separation
+// vector, the impulse factors of Eq. 2, and the previous pair in resolution
+// order of either particle.  The queue is sorted by (a, b), a < b, so a
+// particle's pairs as the higher id come before its pairs as the lower one:
+// b's previous pair is one in its list, a's is the pair before this one if
+// that has the same a, else the last one in a's list.
+__global__ void __launch_bounds__(256) k_pair_rec(ResolveArgs A, SimC C) {
     const int n = A.ctl->pair_n;
     for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < n; k += gridDim.x * blockDim.x) {
-        int a, b;
-        pair_slots(A, A.key[k], a, b);
-        ekey[2 * k] = (uint64_t)a;
-        ekey[2 * k + 1] = (uint64_t)b;
-        eval[2 * k] = 2u * k;
-        eval[2 * k + 1] = 2u * k + 1u;
+        const uint64_t key = A.key[k];
+        const int ia = key_a(key), ib = key_b(key), code = (int)(key & 0xFFFull);
+        const int gx = (code & 15) - 7, gy = ((code >> 4) & 15) - 7, gz = ((code >> 8) & 15) - 7;
+        const int g = ((gx + A.ngx) * (2 * A.ngy + 1) + (gy + A.ngy)) * (2 * A.ngz + 1) + (gz + A.ngz);
+        PairRec R;
+        R.a = A.slot_of_id[ia];
+        R.b = A.slot_of_id[ib];
+        const ImgTab& T = A.img[(size_t)A.P.box[R.a] * A.nimg + g];
+        R.rx = __dsub_rn(__dadd_rn(A.P.x[R.b], T.ox), A.P.x[R.a]);
+        R.ry = __dsub_rn(__dadd_rn(A.P.y[R.b], T.oy), A.P.y[R.a]);
+        R.rz = __dsub_rn(__dadd_rn(A.P.z[R.b], T.oz), A.P.z[R.a]);
+        R.dvy = T.dvy;
+        // the impulse along n = r/|r| without forming n: v_a gains
+        // (1 + eps) (m_b/M) (u.r)/|r|^2 r, v_b loses the same with m_a; the
+        // factors of u.r here, but for 1 + eps under the power law
+        const double r2 = fma(R.rz, R.rz, fma(R.ry, R.ry, R.rx * R.rx));
+        const double ma = A.P.m[R.a], mb = A.P.m[R.b];
+        const double d = r2 * (ma + mb);
+        const double y = rcp64(d);
+        const double num = C.eps_law == 1 ? 1.0 : 1.0 + C.eps;
+        double q = num * y;
+        q = fma(fma(-d, q, num), y, q);   // num / d to the last bit or so
+        R.ka = q * mb;
+        R.kb = q * ma;
+        R.pb = last_before(A, ib, k);
+        R.pa = k > 0 && key_a(A.key[k - 1]) == ia ? k - 1 : last_before(A, ia, k);
+        if (C.hold_pair && k == 0) R.pa = 0;   // test hook: waits for itself
+        A.rec[k] = R;
     }
 }
 
-// After a stable sort of the ends by particle, consecutive ends of the same
-// particle are consecutive pairs of that particle in queue order.
-__global__ void __launch_bounds__(256) k_pair_prev(const uint64_t* __restrict__ ekey,
-                                                   const uint32_t* __restrict__ eval,
-                                                   const Ctl* __restrict__ ctl,
-                                                   int32_t* __restrict__ prev_a,
-                                                   int32_t* __restrict__ prev_b,
-                                                   int32_t* __restrict__ next_a,
-                                                   int32_t* __restrict__ next_b) {
-    const int m = ctl->pair_ends;
-    for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < m; e += gridDim.x * blockDim.x) {
-        const uint32_t v = eval[e];
-        const int k = (int)(v >> 1);
-        const int prev = (e > 0 && ekey[e - 1] == ekey[e]) ? (int)(eval[e - 1] >> 1) : -1;
-        const int next = (e + 1 < m && ekey[e + 1] == ekey[e]) ? (int)(eval[e + 1] >> 1) : -1;
-        if (v & 1u) {
-            prev_b[k] = prev;
-            next_b[k] = next;
-        } else {
-            prev_a[k] = prev;
-            next_a[k] = next;
-        }
-    }
-}
-
-// The queue's first slots: the pairs that are the first pair of both their
-// particles; every pair waits for as many predecessors as it has.
-// One atomic per block and pass: the block's ready pairs are ranked with a
-// block scan of warp ballots (their order in the queue does not matter).
-__global__ void __launch_bounds__(256) k_res_seed(ResolveArgs A, SimC C, int32_t* __restrict__ list,
-                                                  int32_t* __restrict__ rcnt) {
-    __shared__ int wcount[8], base;
-    const int n = A.ctl->pair_n;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    for (int k0 = blockIdx.x * blockDim.x; k0 < n; k0 += gridDim.x * blockDim.x) {
-        const int k = k0 + threadIdx.x;
-        bool ready = false;
-        if (k < n) {
-            const int w = (A.prev_a[k] >= 0 ? 1 : 0) + (A.prev_b[k] >= 0 ? 1 : 0) +
-                          (C.hold_pair && k == 0 ? 1 : 0);
-            A.wait[k] = w;
-            ready = w == 0;
-        }
-        const unsigned m = __ballot_sync(0xffffffffu, ready);
-        if (lane == 0) wcount[warp] = __popc(m);
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            int t = 0;
-            for (int q = 0; q < (int)(blockDim.x >> 5); q++) t += wcount[q];
-            base = t ? atomicAdd(&rcnt[0], t) : 0;
-        }
-        __syncthreads();
-        if (ready) {
-            int pos = base + __popc(m & ((1u << lane) - 1u));
-            for (int q = 0; q < warp; q++) pos += wcount[q];
-            list[pos] = k;
-        }
-        __syncthreads();   // wcount and base are reused
-    }
-}
-
-// The queue of ready pairs, worked by every resident thread in one launch.
-// A pair enters the queue (after the seed's pairs, in the order they become
-// ready) once every earlier pair of the sorted queue that shares a particle
-// with it is resolved; its wait count of unresolved predecessors reaches zero
-// at the release of the last one.  Threads claim queue slots in order (32
-// per warp vote) and wait for their slot to be written; a slot is written by
-// the thread that released its pair, after the velocities it wrote are made
-// visible (fence), and the velocities are read from L2.  Every pair sees all
-// earlier pairs that share a particle with it, so the outcome equals
-// resolving the sorted queue one pair at a time.  The claims are in queue
-// order and a thread resolves its pair as soon as the slot is written, so
-// the wait ends however many of the launch's blocks are resident (slots are
-// claimed only by running threads); it is bounded all the same (half a
-// second), and reports kErrResolveStall if it ever gives up.
 constexpr unsigned long long kWaitLimitNs = 500000000ull;   // half a second
 
 __device__ __forceinline__ unsigned long long global_ns() {
@@ -390,66 +314,115 @@ __device__ __forceinline__ unsigned long long global_ns() {
     return t;
 }
 
-__device__ __forceinline__ void queue_push(int32_t* list, int32_t* tail, int k) {
-    cg::coalesced_group g = cg::coalesced_threads();
-    int base = 0;
-    if (g.thread_rank() == 0) base = atomicAdd(tail, (int)g.size());
-    *(volatile int32_t*)&list[g.shfl(base, 0) + (int)g.thread_rank()] = k;
+__device__ __forceinline__ int ld_flag(const int32_t* p) {
+    int v;
+    asm volatile("ld.relaxed.gpu.global.b32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+    return v;
 }
 
-__global__ void __launch_bounds__(256) k_res_queue(ResolveArgs A, SimC C, int32_t* __restrict__ list,
-                                                   int32_t* __restrict__ q) {
-    // q[0]: slots written (the seed's pairs first), q[1]: slots claimed
-    const int np = A.ctl->pair_n;
+// Eq. 2 for every pair, as if one after the other in queue order.  Warps claim
+// 32 pairs at a time in that order, each lane holds one, with its record
+// already read, and resolves it as soon as the previous pair of either
+// particle is marked done: it reads the velocities from L2, where the other
+// SMs left them, writes the new ones and marks its own pair (release).  A
+// lane's predecessors come earlier in the queue, so they are held by running
+// warps or by lanes of its own warp, which the loop serves in turn, and every
+// wait ends however many blocks are resident; it is bounded all the same (half
+// a second in which no warp of the launch finishes its pairs, or at once when
+// another thread gave up) and reports kErrResolveStall.
+// What bounds it is the chain of dependent pairs, one link at a time: a flag
+// read, a velocity read, 15 FP64 operations, and a release after the
+// velocities have reached L2.  The whole resolution, links and records
+// included: 53 us for 2,233 pairs and 231 us for 944k, against 144 and 452 us
+// with a queue of ready pairs, wait counts and a sort of the pair ends (six
+// dependent round trips and 60 FP64 operations a link).
+template <bool kPower>
+__global__ void __launch_bounds__(256) k_resolve(ResolveArgs A, SimC C) {
+    const int n = A.ctl->pair_n;
     const int lane = threadIdx.x & 31;
-    int nres = 0, ndone = 0;
+    int nres = 0;
     for (;;) {
         int base = 0;
-        if (lane == 0) base = atomicAdd(&q[1], 32);
+        if (lane == 0) base = atomicAdd(A.claim, 32);
         base = __shfl_sync(0xffffffffu, base, 0);
-        if (base >= np) break;
-        const int idx = base + lane;
-        bool stalled = false;
-        if (idx < np) {
-            int k = *(volatile int32_t*)&list[idx];
-            const unsigned long long t0 = k < 0 ? global_ns() : 0ull;
-            while (k < 0) {
-                // bounded: half a second, or at once when another thread gave up
-                if ((*(volatile int*)&A.ctl->err & kErrResolveStall) || global_ns() - t0 > kWaitLimitNs) {
-                    atomicOr(&A.ctl->err, kErrResolveStall);
-                    stalled = true;
-                    break;
+        if (base >= n) break;
+        const int k = base + lane;
+        bool pending = k < n, stalled = false;
+        PairRec R;
+        if (pending) R = A.rec[k];
+        unsigned long long t0 = 0;
+        int seen = 0;
+        for (int spin = 0; __any_sync(0xffffffffu, pending); spin++) {
+            bool moved = false;
+            if (pending) {
+                if (R.pa >= 0 && ld_flag(&A.done[R.pa])) R.pa = -1;
+                if (R.pb >= 0 && ld_flag(&A.done[R.pb])) R.pb = -1;
+                if (R.pa < 0 && R.pb < 0) {
+                    __threadfence();   // the predecessors' velocities before the reads below
+                    double *xa = &A.P.vx[R.a], *ya = &A.P.vy[R.a], *za = &A.P.vz[R.a];
+                    double *xb = &A.P.vx[R.b], *yb = &A.P.vy[R.b], *zb = &A.P.vz[R.b];
+                    const double vxa = __ldcg(xa), vya = __ldcg(ya), vza = __ldcg(za);
+                    const double vxb = __ldcg(xb), vyb = __ldcg(yb), vzb = __ldcg(zb);
+                    const double ux = vxb - vxa, uy = (vyb + R.dvy) - vya, uz = vzb - vza;
+                    const double rv = fma(R.rz, uz, fma(R.ry, uy, R.rx * ux));
+                    if (rv < 0.0) {
+                        double g = rv;
+                        if (kPower) {
+                            // velocity-dependent restitution: min(1, (|v_n| / v_c)^(-p)),
+                            // |v_n| = |u.r| / |r|
+                            const double r2 = fma(R.rz, R.rz, fma(R.ry, R.ry, R.rx * R.rx));
+                            const double vn = __ddiv_rn(rv, __dsqrt_rn(r2));
+                            const double q = pow(__ddiv_rn(fabs(vn), C.eps_vc), -C.eps_p);
+                            g = (1.0 + (q < 1.0 ? q : 1.0)) * rv;
+                        }
+                        const double ga = g * R.ka, gb = g * R.kb;
+                        __stcg(xa, fma(ga, R.rx, vxa));
+                        __stcg(ya, fma(ga, R.ry, vya));
+                        __stcg(za, fma(ga, R.rz, vza));
+                        __stcg(xb, fma(-gb, R.rx, vxb));
+                        __stcg(yb, fma(-gb, R.ry, vyb));
+                        __stcg(zb, fma(-gb, R.rz, vzb));
+                        nres++;
+                    }
+                    asm volatile("st.release.gpu.global.b32 [%0], %1;" ::"l"(&A.done[k]), "r"(1) : "memory");
+                    pending = false;
+                    moved = true;
                 }
-                __nanosleep(200);
-                k = *(volatile int32_t*)&list[idx];
             }
-            if (!stalled) {
-                __threadfence();   // the releasing thread's velocities before ours
-                nres += resolve_one<true>(A, C, A.key[k]) ? 1 : 0;
-                ndone++;
-                __threadfence();   // our velocities before the successors are released
-                const int na = A.next_a[k], nb = A.next_b[k];
-                if (na >= 0 && atomicSub(&A.wait[na], 1) == 1) queue_push(list, &q[0], na);
-                if (nb >= 0 && atomicSub(&A.wait[nb], 1) == 1) queue_push(list, &q[0], nb);
+            if (!__any_sync(0xffffffffu, moved) && (spin & 63) == 63) {
+                // no lane's turn came: look at the clock now and then, and
+                // whether any warp has gone on to its next pairs meanwhile
+                const unsigned long long t = global_ns();
+                const int c = ld_flag(A.claim);
+                if (t0 == 0 || c != seen) {
+                    t0 = t;
+                    seen = c;
+                }
+                stalled = (*(volatile int*)&A.ctl->err & kErrResolveStall) || t - t0 > kWaitLimitNs;
+                if (stalled) atomicOr(&A.ctl->err, kErrResolveStall);
+                if (__any_sync(0xffffffffu, stalled)) break;
             }
         }
         if (__any_sync(0xffffffffu, stalled)) break;
     }
-    if (ndone) atomicSub(&A.ctl->pending, ndone);
-    if (nres) atomicAdd(&A.ctl->resolved, nres);
+    nres = __reduce_add_sync(0xffffffffu, nres);
+    if (lane == 0 && nres) atomicAdd(&A.ctl->resolved, nres);
 }
 
-int g_queue_blocks = 0;   // resident blocks of k_res_queue on the whole GPU
+int g_resolve_blocks[2] = {0, 0};   // resident blocks of k_resolve<false / true> on the whole GPU
 
 }  // namespace
 
 void resolve_prepare(int nsm) {
-    int per_sm = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_res_queue, 256, 0) != cudaSuccess) {
-        cudaGetLastError();
-        per_sm = 1;
+    const void* fn[2] = {(const void*)k_resolve<false>, (const void*)k_resolve<true>};
+    for (int p = 0; p < 2; p++) {
+        int per_sm = 0;
+        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn[p], 256, 0) != cudaSuccess) {
+            cudaGetLastError();
+            per_sm = 1;
+        }
+        g_resolve_blocks[p] = std::max(nsm, 1) * std::max(per_sm, 1);
     }
-    g_queue_blocks = std::max(nsm, 1) * std::max(per_sm, 1);
 }
 
 namespace {
@@ -612,26 +585,18 @@ void resolve_pairs(const PSet& P, Ctl* ctl, const BoxP* boxes, const SimC& C, Pa
                    int half_step_offset, ImgTab* img, cudaStream_t s) {
     ResolveArgs A;
     A.P = P; A.key = PR.sorted(); A.slot_of_id = PR.slot_of_id;
-    A.prev_a = PR.prev_a; A.prev_b = PR.prev_b;
-    A.next_a = PR.next_a; A.next_b = PR.next_b; A.wait = PR.wait;
+    A.head = PR.head; A.link = PR.link; A.done = PR.done; A.rec = PR.rec; A.claim = PR.claim;
     A.img = img;
     A.ngx = C.ngx; A.ngy = C.ngy; A.ngz = C.ngz;
     A.nimg = build_image_table(boxes, ctl, C, half_step_offset, img, s);
-    A.ctl = ctl; A.boxes = boxes; A.hs = half_step_offset;
-    const int grid = std::min(ceil_div(PR.cap, 256), 4 * 152);
-    k_pair_ends<<<grid, 256, 0, s>>>(A, PR.ekey, PR.eval);
-    // particle slots are < 2^24: three 8-bit passes, stable in queue order
-    const int which = radix_sort(PR.ekey, PR.eval, PR.ekey_alt, PR.eval_alt, 2 * PR.cap,
-                                 &ctl->pair_ends, 24, nullptr, 0, PR.ehist, &ctl->err, s);
-    k_pair_prev<<<2 * grid, 256, 0, s>>>(which ? PR.ekey_alt : PR.ekey,
-                                         which ? PR.eval_alt : PR.eval, ctl, PR.prev_a, PR.prev_b,
-                                         PR.next_a, PR.next_b);
-    cudaMemsetAsync(PR.rcnt, 0, sizeof(int32_t) * 64, s);
-    cudaMemsetAsync(PR.queue, 0xff, sizeof(int32_t) * (size_t)PR.cap, s);   // every slot unwritten
-    k_res_seed<<<grid, 256, 0, s>>>(A, C, PR.queue, PR.rcnt);
-    // resident blocks only: a thread may wait for a slot that another writes
-    const int qgrid = std::max(1, std::min(ceil_div(PR.cap, 256), g_queue_blocks));
-    k_res_queue<<<qgrid, 256, 0, s>>>(A, C, PR.queue, PR.rcnt);
+    A.ctl = ctl;
+    cudaMemsetAsync(PR.head, 0xff, sizeof(int32_t) * (size_t)PR.ncap, s);   // empty lists
+    const int grid = std::min(ceil_div(PR.cap, 256), 8 * 152);
+    k_pair_link<<<grid, 256, 0, s>>>(A);
+    k_pair_rec<<<grid, 256, 0, s>>>(A, C);
+    const int rgrid = std::max(1, std::min(ceil_div(PR.cap, 256), g_resolve_blocks[C.eps_law == 1]));
+    if (C.eps_law == 1) k_resolve<true><<<rgrid, 256, 0, s>>>(A, C);
+    else k_resolve<false><<<rgrid, 256, 0, s>>>(A, C);
 }
 
 void energy_terms(const PSet& P, Ctl* ctl, const SimC& C, const double* phi, int box,
