@@ -59,9 +59,9 @@ enum { RB_COLL_NONE = 0, RB_COLL_TREE = 1, RB_COLL_SWEEP = 2 };
  * or a velocity-dependent one): cfg.eps_restitution, or the power law
  * eps(v_n) = min(1, (|v_n| / v_c)^(-p)) of the normal approach speed. */
 enum { RB_EPS_CONSTANT = 0, RB_EPS_POWER = 1 };
-/* Order in which the walks and the collision search take their targets, 32
- * per warp (a launch shape: results per target do not depend on it, except
- * for the FP32 summation order of the walk): the Morton order of the tree;
+/* Order in which the gravity walks take their targets, 32 per warp (a launch
+ * shape: results per target do not depend on it, except for the FP32
+ * summation order of the walk): the Morton order of the tree;
  * a 2D Hilbert order of (x, y) on a 1024 x 1024 grid of the root cube (thin
  * sheets: a warp's targets then span a compact patch of the sheet); a 3D
  * Hilbert order on a 128^3 grid.  The box comes first in every order. */
@@ -117,11 +117,13 @@ typedef struct rb_stats_t {
                                  entries and mixed-subtree iterations) */
     int64_t walk_group;       /* FP32 walk shape: 0 union walk, 4 group walk (4-lane subgroups
                                  for the mixed subtrees) */
-    int64_t tile_order;       /* order in which walks and search take their targets (RB_TILE_*) */
-    int64_t search_visits;    /* tree search: entries (cells and leaves) tested by the targets of
-                                 the last collision search, all images; counted only at
+    int64_t tile_order;       /* order in which the gravity walks take their targets (RB_TILE_*) */
+    int64_t search_visits;    /* tree search: entries (cells and leaves) tested for the targets of
+                                 the last collision search, all images, each counted once per
+                                 target it was tested for; counted only at
                                  rb_set_profiling level 2 (else 0; 0 for the plane sweep) */
-    int64_t search_iterations;/* tree search: warp iterations of that search (32 targets each) */
+    int64_t search_iterations;/* tree search: entries tested by that search (each for up to 32
+                                 targets) */
 } rb_stats_t;
 
 typedef struct rb_sim rb_sim; /* opaque, owned by the library */
@@ -231,8 +233,8 @@ int rb_stats(rb_sim* sim, rb_stats_t* out);
 /* on = 1: record CUDA events between the stages of every step (event nodes
  * inside the step graph) so rb_stats reports per-stage device times.
  * on = 2: also run the tree collision search in its counting variant, so
- * rb_stats reports search_visits and search_iterations (that variant is
- * about 9% slower; at 0 and 1 both counters read 0).  on = 0 turns both off.
+ * rb_stats reports search_visits and search_iterations (at 0 and 1 both
+ * counters read 0).  on = 0 turns both off.
  * Errors: RB_ERR_ARG (on outside 0..2). */
 int rb_set_profiling(rb_sim* sim, int on);
 /* Time the gravity walk and the tree collision search on the current

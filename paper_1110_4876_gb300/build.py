@@ -20,12 +20,13 @@ CSRC = os.path.join(PKG, "csrc")
 INCLUDE = os.path.join(ROOT, "include")
 OUT = os.path.join(PKG, "librb.so")
 BUILD = os.path.join(PKG, "_build")
-SOURCES = ["rb_sort.cu", "rb_tree.cu", "rb_walk.cu", "rb_twalk.cu", "rb_step.cu", "rb_api.cu", "rb_noalloc.cu",
+SOURCES = ["rb_sort.cu", "rb_tree.cu", "rb_walk.cu", "rb_twalk.cu", "rb_collide.cu", "rb_step.cu", "rb_api.cu", "rb_noalloc.cu",
            "rb_mlp.cu", "rb_sweep.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 # The FP32 walks spell out every fused multiply-add, so that all their
 # variants (block sizes, prefetching, learned) round identically.
-PER_FILE = {"rb_walk.cu": ["-fmad=false"], "rb_twalk.cu": ["-fmad=false"]}
+PER_FILE = {"rb_walk.cu": ["-fmad=false"], "rb_twalk.cu": ["-fmad=false"],
+            "rb_collide.cu": ["-fmad=false"]}
 
 
 def nvcc() -> str:

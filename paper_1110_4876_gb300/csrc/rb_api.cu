@@ -274,7 +274,6 @@ int upload(rb_sim* s) {
         rc |= dalloc(s, &T.e_first, ecap, L); rc |= dalloc(s, &T.e_count, ecap, L);
         rc |= dalloc(s, &T.e_skip, ecap, L); rc |= dalloc(s, &T.e_child, 8 * (size_t)ecap, L);
         rc |= dalloc(s, &T.e_cmask, ecap, L); rc |= dalloc(s, &T.e_arrive, ecap, L);
-        rc |= dalloc(s, &T.e_top, ecap, L);
         rc |= dalloc(s, &T.e_level, ecap, L);
         rc |= dalloc(s, &T.leaf_of, cap, L);
         {
@@ -475,10 +474,10 @@ int record_step(rb_sim* s, int p) {
         discard_live_count(s->ctl, st);
         mark(s, 7);
         mark(s, 8);
-        build_collision_aabb(s->T, s->P[c], s->ctl, s->d_boxes, s->C, s->rmax, st);
+        build_collision_aabb(s->T, s->P[c], s->ctl, s->C, st);
         mark(s, 9);
-        collision_search(s->T, s->P[c], s->ctl, s->d_boxes, s->C, s->PR, 2, st, s->search_block, true,
-                         s->rmax, s->profiling == 2);
+        collision_search(s->T, s->P[c], s->ctl, s->d_boxes, s->C, s->PR, 2, st, s->search_block, s->rmax,
+                         s->profiling == 2);
         mark(s, 10);
         sort_pairs(s->PR, s->ctl, st, pair_key_bits(s));
         mark(s, 11);
@@ -488,12 +487,11 @@ int record_step(rb_sim* s, int p) {
         c = 1 - c;
         mark(s, 7);
         build_topology(s->T, s->P[c], s->ctl, s->d_boxes, s->C, st);
-        build_tile_order(s->T, s->P[c], s->ctl, s->tile_order, s->box_bits, st);
         mark(s, 8);
-        build_collision_records(s->T, s->P[c], s->ctl, s->d_boxes, s->C, s->rmax, st);
+        build_collision_aabb(s->T, s->P[c], s->ctl, s->C, st);
         mark(s, 9);
-        collision_search(s->T, s->P[c], s->ctl, s->d_boxes, s->C, s->PR, 2, st, s->search_block, false,
-                         0.0, s->profiling == 2);
+        collision_search(s->T, s->P[c], s->ctl, s->d_boxes, s->C, s->PR, 2, st, s->search_block, s->rmax,
+                         s->profiling == 2);
         mark(s, 10);
         sort_pairs(s->PR, s->ctl, st, pair_key_bits(s));
         mark(s, 11);
@@ -556,7 +554,7 @@ int clear_err(rb_sim* s) {
 
 // Collision search + pair sort on set c at half-step offset hs; grows the
 // pair buffer and searches again if it overflowed.  Resolves when asked.
-int collide_with_retry(rb_sim* s, int c, int hs, bool resolve, bool aabb) {
+int collide_with_retry(rb_sim* s, int c, int hs, bool resolve) {
     for (int attempt = 0; attempt < 2; attempt++) {
         RB_CUDA(s, cudaMemsetAsync(&s->ctl->pair_count, 0, sizeof(int), s->stream));
         clear_search_stats(s->ctl, s->stream);
@@ -565,7 +563,7 @@ int collide_with_retry(rb_sim* s, int c, int hs, bool resolve, bool aabb) {
             sweep_search(s->P[c], s->ctl, s->d_boxes, s->C, s->SW, s->PR, hs, s->ncap, s->stream);
         else
             collision_search(s->T, s->P[c], s->ctl, s->d_boxes, s->C, s->PR, hs, s->stream,
-                             s->search_block, aabb, s->rmax, s->profiling == 2);
+                             s->search_block, s->rmax, s->profiling == 2);
         sort_pairs(s->PR, s->ctl, s->stream, pair_key_bits(s));
         if (read_ctl(s)) return RB_ERR_CUDA;
         if (s->hctl.err & kErrSweepLong)
@@ -928,8 +926,7 @@ int rb_step(rb_sim* s, int64_t nsteps) {
             return fail(s, RB_ERR_TIMEOUT, "radix sort: a bounded look-back wait gave up");
         if (s->cfg.collisions && s->hctl.pair_count > s->PR.cap) {
             // the step ended before resolution: search again with a larger buffer
-            const bool aabb = s->cfg.gravity && s->cfg.collisions == RB_COLL_TREE;
-            if ((rc = collide_with_retry(s, s->cur, 0, true, aabb))) return rc;
+            if ((rc = collide_with_retry(s, s->cur, 0, true))) return rc;
         }
     }
     return RB_OK;
@@ -1034,8 +1031,8 @@ int rb_detect_collisions(rb_sim* s) {
     if (s->ntot == 0) return RB_OK;
     rebuild_now(s);
     if (s->cfg.collisions != RB_COLL_SWEEP)
-        build_collision_records(s->T, s->P[s->cur], s->ctl, s->d_boxes, s->C, s->rmax, s->stream);
-    return collide_with_retry(s, s->cur, 0, false, false);
+        build_collision_aabb(s->T, s->P[s->cur], s->ctl, s->C, s->stream);
+    return collide_with_retry(s, s->cur, 0, false);
 }
 
 int rb_get_pairs(rb_sim* s, int box, int64_t cap, int64_t* n, int64_t* id_a, int64_t* id_b,
@@ -1270,26 +1267,14 @@ int rb_autotune(rb_sim* s, int use_cache) {
             s->acc_set = -1;   // the tuning walks left no consistent acceleration record
         }
         if (s->cfg.collisions == RB_COLL_TREE) {
-            // the records the step uses: boxes on the gravity tree, or Eq. 3's
-            // spheres on a collision tree when gravity is off
-            const bool aabb = s->cfg.gravity != 0;
             rebuild_now(s);
-            if (!s->cfg.gravity && t != kTileMorton)
-                total += time_best(s, [&] {
-                    build_tile_order(s->T, s->P[s->cur], s->ctl, t, s->box_bits, s->stream);
-                });
-            if (aabb) {
-                build_gravity_records(s->T, s->P[s->cur], s->ctl, s->d_boxes, s->C, false, s->stream);
-                build_collision_aabb(s->T, s->P[s->cur], s->ctl, s->d_boxes, s->C, s->rmax, s->stream);
-            } else {
-                build_collision_records(s->T, s->P[s->cur], s->ctl, s->d_boxes, s->C, s->rmax, s->stream);
-            }
+            build_collision_aabb(s->T, s->P[s->cur], s->ctl, s->C, s->stream);
             float best = 1e30f;
             for (int b : cand) {
                 const float ms = time_best(s, [&] {
                     cudaMemsetAsync(&s->ctl->pair_count, 0, sizeof(int), s->stream);
                     collision_search(s->T, s->P[s->cur], s->ctl, s->d_boxes, s->C, s->PR, 0, s->stream, b,
-                                     aabb, s->rmax);
+                                     s->rmax);
                 });
                 if (ms < best) { best = ms; sb_t = b; }
             }

@@ -121,7 +121,6 @@ struct Tree {
     int32_t *e_first, *e_count, *e_skip, *e_arrive;
     int32_t* e_child;           // per cell entry: the child entry of each octant (8 slots)
     uint32_t* e_cmask;          // per cell entry: octants that hold a child
-    int32_t* e_top;             // collision records on spheres: largest particle slot below
     int8_t* e_level;            // depth of a cell; 22 marks a particle leaf
     int32_t* leaf_of;           // per particle: its leaf entry
     double *M, *cx, *cy, *cz, *Q;   // FP64 moments per entry (Q: 6 x cap, xx yy zz xy xz yz)
@@ -256,13 +255,9 @@ void build_tile_order(Tree& T, const PSet& P, Ctl* ctl, int mode, int box_bits, 
 // then hold its FP32 values).
 void build_gravity_records(const Tree& T, const PSet& P, Ctl* ctl, const BoxP* boxes,
                            const SimC& C, bool fp64, cudaStream_t s, bool f32q = false);
-// Collision records on the tree of the last gravity build at the current
-// positions (cells as FP32 boxes of their particles); for collision_search
-// with aabb = true.
-void build_collision_aabb(const Tree& T, const PSet& P, Ctl* ctl, const BoxP* boxes, const SimC& C,
-                          double rmax, cudaStream_t s);
-void build_collision_records(const Tree& T, const PSet& P, Ctl* ctl, const BoxP* boxes,
-                             const SimC& C, double rmax, cudaStream_t s);
+// Collision records on the tree of the last build at the current positions
+// (cells as FP32 boxes of their particles).
+void build_collision_aabb(const Tree& T, const PSet& P, Ctl* ctl, const SimC& C, cudaStream_t s);
 
 // rb_walk.cu
 struct WalkOut {
@@ -313,12 +308,13 @@ void gravity_walk(const Tree& T, const PSet& P, Ctl* ctl, const BoxP* boxes, con
                   int walk_mode, int half_step_offset, const WalkOut& out, bool potential,
                   bool counts, cudaStream_t s, const WalkRecord* rec = nullptr, int block = 128,
                   const WalkLearn* learn = nullptr, int group = 0);
-// aabb: the records of build_collision_aabb, with rmax the largest radius.
-// count: the variant that adds the entries its targets test and its warp
-// iterations to ctl->n_visit and ctl->n_siter.
+// rb_collide.cu: on the records of build_collision_aabb, with rmax the
+// largest radius.  count: the variant that adds the entries it tests, once per
+// target they are tested for, to ctl->n_visit, and once per warp to
+// ctl->n_siter.
 void collision_search(const Tree& T, const PSet& P, Ctl* ctl, const BoxP* boxes, const SimC& C,
-                      const Pairs& PR, int half_step_offset, cudaStream_t s, int block = 128,
-                      bool aabb = false, double rmax = 0.0, bool count = false);
+                      const Pairs& PR, int half_step_offset, cudaStream_t s, int block, double rmax,
+                      bool count = false);
 
 // rb_sweep.cu: plane-sweep search on set P at half-step offset hs; the
 // canonical pair keys are appended to PR like the tree search's.

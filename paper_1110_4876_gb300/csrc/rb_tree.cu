@@ -554,52 +554,13 @@ __global__ void __launch_bounds__(256) k_moments_level(GravRecArgs A, const int3
 struct CollRecArgs {
     const double *x, *y, *z, *r;
     const int32_t* box;
-    const uint64_t* key;
-    const BoxP* boxes;
-    const int32_t *e_first, *e_skip, *leaf_of, *e_count, *e_child;
-    const uint32_t* e_cmask;
-    int32_t* e_top;
+    const int32_t *e_first, *e_skip, *leaf_of, *e_count;
     const int8_t* e_level;
     Rec4 ra, rb;
     const Ctl* ctl;
     int ecap, ncap, nbox;
-    double rmax;
     float4* pbox = nullptr;   // box items (pairs lo, hi): slots, then runs of 32, then runs of 256
 };
-
-// Collision-search records (Sect. 5.2): per cell its geometric centre
-// (hi/lo) and the opening radius (sqrt(3)/2) w + R_max of Eq. 3, rounded up;
-// per leaf the particle's position (hi/lo), slot and radius (the search
-// leaves skip implicitly to the next entry).
-__global__ void __launch_bounds__(256) k_coll_records(CollRecArgs A) {
-    const int E = min(A.ctl->n_entries, A.ecap);
-    const int k = blockIdx.x * blockDim.x + threadIdx.x;
-    if (k >= E) return;
-    const int v = A.e_level[k];
-    const int first = A.e_first[k];
-    if (v == 22) {
-        float hx, lx, hy, ly, hz, lz;
-        split_hilo(A.x[first], hx, lx);
-        split_hilo(A.y[first], hy, ly);
-        split_hilo(A.z[first], hz, lz);
-        A.ra[k] = make_float4(hx, hy, hz, __int_as_float(~first));
-        A.rb[k] = make_float4(lx, ly, lz, (float)A.r[first]);
-        return;
-    }
-    const BoxP bp = A.boxes[A.box[first]];
-    const double w = ldexp(bp.L, -v);
-    const double lo = -0.5 * bp.L;
-    double ix, iy, iz;
-    cell_index(A.key[first], v, ix, iy, iz);
-    float hx, lx, hy, ly, hz, lz;
-    split_hilo(lo + (ix + 0.5) * w, hx, lx);
-    split_hilo(lo + (iy + 0.5) * w, hy, ly);
-    split_hilo(lo + (iz + 0.5) * w, hz, lz);
-    const float h = __double2float_ru(0.8660254037844387 * w + A.rmax);
-    A.ra[k] = make_float4(hx, hy, hz, h);
-    A.rb[k] = make_float4(lx, ly, lz, __int_as_float(A.e_skip[k]));
-    A.e_top[k] = first + A.e_count[k] - 1;   // particles below sit at slots first ..
-}
 
 // Collision records on the gravity tree, at the positions after the second
 // drift (Sect. 5.2, with a tighter pruning volume than Eq. 3's sphere): the
@@ -964,26 +925,14 @@ void build_gravity_records(const Tree& T, const PSet& P, Ctl* ctl, const BoxP* b
     }
 }
 
-void build_collision_records(const Tree& T, const PSet& P, Ctl* ctl, const BoxP* boxes,
-                             const SimC& C, double rmax, cudaStream_t s) {
+void build_collision_aabb(const Tree& T, const PSet& P, Ctl* ctl, const SimC& C, cudaStream_t s) {
+    if (T.cap_n <= 0) return;
     CollRecArgs A;
     A.x = P.x; A.y = P.y; A.z = P.z; A.r = P.r;
-    A.box = P.box; A.key = T.key; A.boxes = boxes;
+    A.box = P.box;
     A.e_first = T.e_first; A.e_skip = T.e_skip; A.e_level = T.e_level; A.leaf_of = T.leaf_of;
-    A.e_count = T.e_count; A.e_top = T.e_top; A.e_child = T.e_child; A.e_cmask = T.e_cmask;
-    A.ra = T.ra; A.rb = T.rb; A.ctl = ctl; A.ecap = T.cap_e; A.rmax = rmax;
-    A.ncap = T.cap_n; A.nbox = C.nbox;
-    k_coll_records<<<ceil_div(T.cap_e, 256), 256, 0, s>>>(A);
-}
-
-void build_collision_aabb(const Tree& T, const PSet& P, Ctl* ctl, const BoxP* boxes, const SimC& C,
-                          double rmax, cudaStream_t s) {
-    CollRecArgs A;
-    A.x = P.x; A.y = P.y; A.z = P.z; A.r = P.r;
-    A.box = P.box; A.key = T.key; A.boxes = boxes;
-    A.e_first = T.e_first; A.e_skip = T.e_skip; A.e_level = T.e_level; A.leaf_of = T.leaf_of;
-    A.e_count = T.e_count; A.e_top = T.e_top; A.e_child = T.e_child; A.e_cmask = T.e_cmask;
-    A.ra = T.ra; A.rb = T.rb; A.ctl = ctl; A.ecap = T.cap_e; A.rmax = rmax;
+    A.e_count = T.e_count;
+    A.ra = T.ra; A.rb = T.rb; A.ctl = ctl; A.ecap = T.cap_e;
     A.ncap = T.cap_n; A.nbox = C.nbox;
     A.pbox = T.pbox;
     k_aabb_leaves<<<ceil_div(T.cap_n, kRunB), kRunB, 0, s>>>(A);

@@ -1,5 +1,5 @@
-// rb_walk.cu -- Barnes-Hut gravity walk (Sect. 4.2, Eq. 1) and tree
-// collision search (Sect. 5.2, Eq. 3) over the ghost images of Sect. 2.3.
+// rb_walk.cu -- Barnes-Hut gravity walk (Sect. 4.2, Eq. 1) over the ghost
+// images of Sect. 2.3.
 //
 // Warp-cooperative stackless walk.  Each warp owns 32 consecutive targets in
 // Morton order (spatially close); each lane keeps its own "next entry" in the
@@ -811,204 +811,6 @@ __global__ void __launch_bounds__(kMaxWalkBlock, 2) k_walk32_learn(GravArgs A) {
         walk32<true, kInside, false, kSoft, false, true>(A, &q[threadIdx.x >> 5], &w, t << 5, n);
 }
 
-struct CollArgs {
-    const double *x, *y, *z, *r;
-    const int32_t *id, *box;
-    Rec4 ra, rb;
-    const int32_t *box_root, *e_skip;
-    const BoxP* boxes;
-    Ctl* ctl;
-    uint64_t* pair_key;
-    int pair_cap;
-    int ncap;
-    int ngx, ngy, ngz;
-    int half_step_offset;
-    double t0, half_dt;
-    const ImgTab* img;   // [box][image] offsets at the time of this search
-    int nimg;
-    int32_t* tq;         // tile queues (emptied by the image-table launch)
-    int nq;
-    float rmaxf;         // largest radius, rounded up (box records)
-    const int32_t* e_top;   // sphere records: largest particle slot below each cell
-    const uint32_t* order;  // tile order of the targets (nullptr: Morton order of the slots)
-};
-
-// Overlap test of Sect. 5.1 on the canonical orientation (a = lower id, b
-// seen through image offset o), operation for operation as the oracle.
-// kNeg: the offset is -o (b + (-o) and b - o round identically in IEEE
-// arithmetic, so no negated copy of o is formed).
-template <bool kNeg = false>
-__device__ __forceinline__ bool overlap64(double xa, double ya, double za, double ra, double xb,
-                                          double yb, double zb, double rb, double ox, double oy,
-                                          double oz) {
-    const double rx = __dsub_rn(kNeg ? __dsub_rn(xb, ox) : __dadd_rn(xb, ox), xa);
-    const double ry = __dsub_rn(kNeg ? __dsub_rn(yb, oy) : __dadd_rn(yb, oy), ya);
-    const double rz = __dsub_rn(kNeg ? __dsub_rn(zb, oz) : __dadd_rn(zb, oz), za);
-    const double r2 = __dadd_rn(__dadd_rn(__dmul_rn(rx, rx), __dmul_rn(ry, ry)), __dmul_rn(rz, rz));
-    const double sr = __dadd_rn(ra, rb);
-    return r2 < __dmul_rn(sr, sr);
-}
-
-// Tree collision search (Sect. 5.2): descend while the distance from the
-// target point to a cell's centre is below R_i + R_max + (sqrt(3)/2) w (Eq. 3,
-// tested in FP32 with a 2e-5 relative margin so that no overlap is pruned);
-// kAABB: while the distance to the box of the cell's particles is below
-// R_i + R_max (records of build_collision_aabb; a subset of Eq. 3's volume
-// that still holds every overlap).
-// Each unordered pair is examined once, from its lower slot (the other
-// particle reaches it through the opposite image), so a subtree whose
-// particles all sit at slots <= i is skipped as well.  A leaf's overlap is
-// decided in FP32 on hi/lo positions (distance good to ~1e-7 relative) unless
-// d^2 lies within 1e-4 of (R_a + R_b)^2; only those pairs get the exact FP64
-// test in the oracle's operation order on the canonical orientation (lower
-// id a, image of b as seen from a).  On GB300 an FP64 instruction occupies
-// the SM's FP64 pipe 16 cycles per warp, so the exact test on every overlap
-// kept that pipe busy for most of the search.
-// kCount: also count the entries the targets test (nodes visited) and the
-// warp iterations; a separate variant, since the counters cost the
-// 32-register search about 9% of its time in spilled registers.
-template <bool kAABB, bool kCount>
-__device__ __forceinline__ void collide(const CollArgs& A, int wbase, int n) {
-    const int lane = threadIdx.x & 31;
-    const bool valid = wbase + lane < n;
-    const int ii = tile_slot(A.order, valid ? wbase + lane : n - 1);
-    const int i = ii;   // the target's slot
-    const double px = A.x[ii], py = A.y[ii], pz = A.z[ii], pr = A.r[ii];
-    const int pid = A.id[ii];
-    const int root = A.box_root[A.box[ii]];
-    const int wend = root >= 0 ? A.e_skip[root] : 0;   // end of this box's tree
-    const float prf = (float)pr;
-    float phx, plx, phy, ply, phz, plz;
-    split_d(px, phx, plx);
-    split_d(py, phy, ply);
-    split_d(pz, phz, plz);
-    const ImgTab* itab = A.img + (size_t)A.box[ii] * A.nimg;
-    int gi = 0;
-    // kCount: entries the warp's targets tested and warp iterations
-    // (both warp-uniform)
-    unsigned nvis = 0, siter = 0;
-    for (int gx = -A.ngx; gx <= A.ngx; gx++)
-        for (int gy = -A.ngy; gy <= A.ngy; gy++)
-            for (int gz = -A.ngz; gz <= A.ngz; gz++, gi++) {
-                const int code = (gx + 7) | ((gy + 7) << 4) | ((gz + 7) << 8);
-                float thx, thy, thz, tlx, tly, tlz;
-                {
-                    const float4 oh = itab[gi].hi, ol = itab[gi].lo;
-                    sub_hilo(phx, plx, oh.x, ol.x, thx, tlx);
-                    sub_hilo(phy, ply, oh.y, ol.y, thy, tly);
-                    sub_hilo(phz, plz, oh.z, ol.z, thz, tlz);
-                }
-                const float2 nth = make_float2(-thx, -thy), ntl = make_float2(-tlx, -tly);
-                int next = (valid && root >= 0) ? root : kEnd;
-                for (;;) {
-                    if (next >= wend) next = kEnd;
-                    const int e = (int)__reduce_min_sync(kFull, (unsigned)next);
-                    if (e == kEnd) break;
-                    const float4 ra = __ldg(&A.ra[e]);
-                    const bool act = next == e;
-                    if (kCount) {
-                        nvis += __popc(__ballot_sync(kFull, act));
-                        siter++;
-                    }
-                    bool hit = false;
-                    uint64_t key = 0;
-                    if (__float_as_int(ra.w) < 0) {
-                        if (act) {
-                            const int j = ~__float_as_int(ra.w);
-                            if (j > i) {
-                                const float4 rb = __ldg(&A.rb[e]);
-                                const float2 dxy = __fadd2_rn(__fadd2_rn(make_float2(ra.x, ra.y), nth),
-                                                              __fadd2_rn(make_float2(rb.x, rb.y), ntl));
-                                const float dx = dxy.x, dy = dxy.y;
-                                const float dz = (ra.z - thz) + (rb.z - tlz);
-                                const float d2 = fmaf(dz, dz, fmaf(dy, dy, dx * dx));
-                                const float sr = prf + rb.w;
-                                const float s2 = sr * sr;
-                                if (d2 < s2 * 1.0001f) {
-                                    const int jid = A.id[j];
-                                    const bool low = pid < jid;
-                                    if (d2 < s2 * 0.9999f) {
-                                        // clear of the threshold (the FP32 distance is good to
-                                        // ~1e-7): an overlap without FP64 work
-                                        hit = true;
-                                    } else {
-                                        const double ox = itab[gi].ox, oy = itab[gi].oy, oz = itab[gi].oz;
-                                        // j the lower id: this particle is its image -g, whose
-                                        // offset is exactly -o (the table is symmetric)
-                                        hit = low ? overlap64(px, py, pz, pr, A.x[j], A.y[j], A.z[j],
-                                                              A.r[j], ox, oy, oz)
-                                                  : overlap64<true>(A.x[j], A.y[j], A.z[j], A.r[j], px,
-                                                                    py, pz, pr, ox, oy, oz);
-                                    }
-                                    const int ncode = (-gx + 7) | ((-gy + 7) << 4) | ((-gz + 7) << 8);
-                                    key = low ? ((uint64_t)pid << 36) | ((uint64_t)jid << 12) | (uint64_t)code
-                                              : ((uint64_t)jid << 36) | ((uint64_t)pid << 12) | (uint64_t)ncode;
-                                }
-                            }
-                            next = e + 1;
-                        }
-                    } else if (act) {
-                        const float4 rb = __ldg(&A.rb[e]);
-                        if (kAABB) {
-                            // distance to the cell's box [ra.xyz, rb.xyz] of particle
-                            // positions; opened unless farther than R_i + R_max, or
-                            // unless every particle below sits at a slot <= i (those
-                            // pairs are examined from the other particle)
-                            // (t - b) + l = -((b - t) - l) exactly, so the upper side
-                            // comes negated out of the same packed adds
-                            const float2 u = __fadd2_rn(__fadd2_rn(make_float2(ra.x, ra.y), nth), ntl);
-                            const float2 v = __fadd2_rn(__fadd2_rn(make_float2(rb.x, rb.y), nth), ntl);
-                            const float ex = fmaxf(fmaxf(u.x, -v.x), 0.f);
-                            const float ey = fmaxf(fmaxf(u.y, -v.y), 0.f);
-                            const float ez = fmaxf(fmaxf((ra.z - thz) - tlz, (thz - rb.z) + tlz), 0.f);
-                            const float d2 = fmaf(ez, ez, fmaf(ey, ey, ex * ex));
-                            const float lim = (prf + A.rmaxf) * 1.0001f +
-                                              4e-7f * (fabsf(thx) + fabsf(thy) + fabsf(thz));
-                            next = (__float_as_int(ra.w) > i && d2 < lim * lim) ? e + 1
-                                                                                : __float_as_int(rb.w);
-                        } else {
-                            const float2 dxy = __fadd2_rn(__fadd2_rn(make_float2(ra.x, ra.y), nth),
-                                                          __fadd2_rn(make_float2(rb.x, rb.y), ntl));
-                            const float dx = dxy.x, dy = dxy.y;
-                            const float dz = (ra.z - thz) + (rb.z - tlz);
-                            const float d2 = fmaf(dz, dz, fmaf(dy, dy, dx * dx));
-                            const float lim = (prf + ra.w) * 1.00002f;
-                            next = (__ldg(&A.e_top[e]) > i && d2 < lim * lim) ? e + 1
-                                                                              : __float_as_int(rb.w);
-                        }
-                    }
-                    const unsigned hits = __ballot_sync(kFull, hit);
-                    if (hits) {
-                        int base = 0;
-                        const int leader = __ffs(hits) - 1;
-                        if (lane == leader) base = atomicAdd(&A.ctl->pair_count, __popc(hits));
-                        base = __shfl_sync(kFull, base, leader);
-                        if (hit) {
-                            const int slot = base + __popc(hits & ((1u << lane) - 1u));
-                            if (slot < A.pair_cap) A.pair_key[slot] = key;
-                            else atomicOr(&A.ctl->err, kErrPairOverflow);
-                        }
-                    }
-                }
-            }
-    if (kCount && lane == 0) {
-        atomicAdd(&A.ctl->n_visit, (unsigned long long)nvis);
-        atomicAdd(&A.ctl->n_siter, (unsigned long long)siter);
-    }
-}
-
-// At most 32 registers (8 blocks of 256 threads per SM, every warp slot
-// resident): the search is latency-bound, and going from 40 resident warps
-// per SM (48 registers) to 48 (40) and 64 (32, with a few spilled values)
-// took 4% and another 2% off it.
-template <bool kAABB, bool kCount = false>
-__global__ void __launch_bounds__(kMaxWalkBlock, 8) k_collide(CollArgs A) {
-    const int n = min(A.ctl->n_live, A.ncap);
-    const int ntile = (n + 31) >> 5, q = sm_queue(A.nq);
-    for (int t = next_tile(A.tq, A.nq, q, ntile); t >= 0; t = next_tile(A.tq, A.nq, q, ntile))
-        collide<kAABB, kCount>(A, t << 5, n);
-}
-
 }  // namespace
 
 int build_image_table(const BoxP* boxes, const Ctl* ctl, const SimC& C, int half_step_offset, ImgTab* tab,
@@ -1113,10 +915,7 @@ int walk_prepare() {
     RB_PREP_G(false, true, true); RB_PREP_G(false, true, false);
     RB_PREP_G(false, false, true); RB_PREP_G(false, false, false);
 #undef RB_PREP_G
-    prepare_one(k_collide<true>);
-    prepare_one(k_collide<false>);
-    prepare_one(k_collide<true, true>);
-    prepare_one(k_collide<false, true>);
+    collision_search_prepare();
     return g_nsm;
 }
 
@@ -1211,36 +1010,6 @@ void gravity_walk(const Tree& T, const PSet& P, Ctl* ctl, const BoxP* boxes, con
     }
 #undef RB_W32
 #undef RB_W32G
-}
-
-void collision_search(const Tree& T, const PSet& P, Ctl* ctl, const BoxP* boxes, const SimC& C,
-                      const Pairs& PR, int half_step_offset, cudaStream_t s, int block, bool aabb,
-                      double rmax, bool count) {
-    if (T.cap_n <= 0) return;
-    block = (block == 64 || block == 256) ? block : 128;
-    CollArgs A;
-    A.rmaxf = (float)rmax;
-    if ((double)A.rmaxf < rmax) A.rmaxf = nextafterf(A.rmaxf, FLT_MAX);
-    A.x = P.x; A.y = P.y; A.z = P.z; A.r = P.r; A.id = P.id; A.box = P.box;
-    A.ra = T.ra; A.rb = T.rb; A.box_root = T.box_root; A.e_skip = T.e_skip; A.boxes = boxes;
-    A.e_top = T.e_top;
-    A.order = T.order;
-    A.ctl = ctl;
-    A.pair_key = PR.key; A.pair_cap = PR.cap; A.ncap = T.cap_n;
-    A.ngx = C.ngx; A.ngy = C.ngy; A.ngz = C.ngz;
-    A.half_step_offset = half_step_offset; A.t0 = C.t0; A.half_dt = C.half_dt;
-    A.img = T.img;
-    A.tq = T.tq;
-    A.nq = T.nq;
-    A.nimg = build_image_table(boxes, ctl, C, half_step_offset, T.img, s, T.tq, T.nq);
-    if (count) {
-        if (aabb) RB_LAUNCH(k_collide<true, true>);
-        else RB_LAUNCH(k_collide<false, true>);
-    } else if (aabb) {
-        RB_LAUNCH(k_collide<true>);
-    } else {
-        RB_LAUNCH(k_collide<false>);
-    }
 #undef RB_LAUNCH
 }
 

@@ -61,6 +61,7 @@ enum class TargetWalk { kFp32, kFp64, kLearned };
 void target_walk(const GravArgs& A, TargetWalk mode, bool quad, bool inside, bool soft, bool pot, int block,
                  int cap_n, cudaStream_t s);
 void target_walk_prepare();
+void collision_search_prepare();   // rb_collide.cu
 
 namespace {
 
