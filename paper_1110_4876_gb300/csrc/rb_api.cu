@@ -61,6 +61,7 @@ struct rb_sim {
     double *acc_x = nullptr, *acc_y = nullptr, *acc_z = nullptr, *phi = nullptr;
     int32_t *cnt_cell = nullptr, *cnt_leaf = nullptr, *cnt_mac = nullptr;
     int acc_set = -1;     // particle set the last gravity walk ran on
+    bool q32 = false;     // the quadrupoles of that walk's tree are in its FP32 records only
     double* e_part = nullptr;
     double* e_out = nullptr;
     int ncap = 0, ntot = 0, box_bits = 0;
@@ -247,6 +248,7 @@ int upload(rb_sim* s) {
         free_list(s, s->pair_allocs);
         const int cap = std::max(n, 1);
         const int ecap = 2 * cap;
+        const size_t erec = (size_t)ecap + moment_pieces(cap);   // moment records
         auto& L = s->allocs;
         int rc = RB_OK;
         for (int k = 0; k < 2; k++) {
@@ -273,25 +275,25 @@ int upload(rb_sim* s) {
         rc |= dalloc(s, &T.node_v, cap, L);
         rc |= dalloc(s, &T.e_first, ecap, L); rc |= dalloc(s, &T.e_count, ecap, L);
         rc |= dalloc(s, &T.e_skip, ecap, L); rc |= dalloc(s, &T.e_child, 8 * (size_t)ecap, L);
-        rc |= dalloc(s, &T.e_cmask, ecap, L); rc |= dalloc(s, &T.e_arrive, ecap, L);
+        rc |= dalloc(s, &T.e_cmask, ecap, L);
         rc |= dalloc(s, &T.e_level, ecap, L);
         rc |= dalloc(s, &T.leaf_of, cap, L);
         {
             // FP32 record pairs, each pair interleaved (Rec4)
             float4 *rab = nullptr, *rq = nullptr, *rcc = nullptr;
-            rc |= dalloc(s, &rab, 2 * (size_t)ecap, L);
-            rc |= dalloc(s, &rq, 2 * (size_t)ecap, L);
+            rc |= dalloc(s, &rab, 2 * erec, L);
+            rc |= dalloc(s, &rq, 2 * erec, L);
             rc |= dalloc(s, &rcc, 2 * (size_t)ecap, L);
             rc |= dalloc(s, &T.pbox, 2 * (size_t)box_items(cap), L);
             T.ra.p = rab; T.rb.p = rab ? rab + 1 : nullptr;
             T.rq0.p = rq; T.rq1.p = rq ? rq + 1 : nullptr;
             T.rc_hi.p = rcc; T.rc_lo.p = rcc ? rcc + 1 : nullptr;
         }
-        rc |= dalloc(s, &T.d_a, ecap, L); rc |= dalloc(s, &T.d_q0, ecap, L);
-        rc |= dalloc(s, &T.d_q1, ecap, L); rc |= dalloc(s, &T.d_c, ecap, L);
+        rc |= dalloc(s, &T.d_a, erec, L); rc |= dalloc(s, &T.d_q0, erec, L);
+        rc |= dalloc(s, &T.d_q1, erec, L); rc |= dalloc(s, &T.d_c, ecap, L);
         rc |= dalloc(s, &T.box_first, s->nbox + 1, L);
         rc |= dalloc(s, &T.box_root, s->nbox + 1, L);
-        rc |= dalloc(s, &T.lvl, 96, L);
+        rc |= dalloc(s, &T.span, moment_span_words(cap), L);
         rc |= dalloc(s, &T.tq, kMaxTileQueues * kTileQStride, L);
         T.nq = s->nsm > 0 ? min(s->nsm, kMaxTileQueues) : 1;
         rc |= dalloc(s, &T.img, (size_t)(s->nbox + 1) * (2 * s->cfg.nghost[0] + 1) * (2 * s->cfg.nghost[1] + 1) *
@@ -627,6 +629,7 @@ int gravity_now(rb_sim* s, bool potential) {
                      s->walk_group);
     }
     s->acc_set = s->cur;
+    s->q32 = !fp64;
     RB_CUDA(s, cudaGetLastError());
     if (int rc = read_ctl(s)) return rc;
     if (s->hctl.err & kErrWalk)
@@ -912,6 +915,7 @@ int rb_step(rb_sim* s, int64_t nsteps) {
                 cudaEventElapsedTime(&s->stage_ms[q], s->ev_stage[q], s->ev_stage[q + 1]);
         s->cur = s->gafter[p];
         s->acc_set = s->cfg.gravity ? s->cur : -1;   // the walk's particle set (no second sort)
+        s->q32 = s->cfg.walk != RB_WALK_FP64;
         if (s->hctl.err & kErrNonFinite)
             return fail(s, RB_ERR_NONFINITE, "a position became non-finite (or left the box by more than "
                                              "4096 box lengths in one drift half)");
@@ -999,6 +1003,16 @@ int rb_get_tree(rb_sim* s, int box, int64_t cap, int64_t* ncell, int32_t* depth,
         d2h(s, roots, s->T.box_root, s->nbox) || d2h(s, da, s->T.d_a, E) || d2h(s, q0, s->T.d_q0, E) ||
         d2h(s, q1, s->T.d_q1, E))
         return RB_ERR_CUDA;
+    if (s->q32) {
+        // summed in FP32: the quadrupole is in the records of the FP32 walk
+        std::vector<float4> rq;
+        if (d2h(s, rq, s->T.rq0.p, 2 * (size_t)E)) return RB_ERR_CUDA;
+        for (int e = 0; e < E; e++) {
+            const float4 a = rq[2 * e], b = rq[2 * e + 1];
+            q0[e] = make_double4_32a(q0[e].x, a.y, a.z, a.w);
+            q1[e] = make_double4_32a(b.x, b.y, b.z, 0.0);
+        }
+    }
     int64_t k = 0, mk = 0;
     const int r0 = roots[box];
     if (r0 >= 0) {
@@ -1439,6 +1453,7 @@ int rb_mlp_samples(rb_sim* s, double theta_hi, double theta_lo, double prob, uin
     gravity_walk(s->T, s->P[s->cur], s->ctl, s->d_boxes, C2, RB_WALK_FP32, 0, walk_out(s), false, true,
                  s->stream, &rec);
     s->acc_set = s->cur;
+    s->q32 = false;
     mlp::label_async(req_args(s, s->cur, 0, req, (int)cap), dX, dY, dmeta, (int)cap, s->stream);
     rc = read_ctl(s);
     const int64_t n = std::min<int64_t>(s->hctl.req_count, cap);

@@ -118,7 +118,7 @@ struct Tree {
     int32_t* start;             // per particle: first entry starting there (n + 1)
     int32_t *node_a, *node_b;   // per split: first particle of its cell (last: reps only)
     int8_t* node_v;             // per split: cell depth (+32 unless representative), -1 none
-    int32_t *e_first, *e_count, *e_skip, *e_arrive;
+    int32_t *e_first, *e_count, *e_skip;
     int32_t* e_child;           // per cell entry: the child entry of each octant (8 slots)
     uint32_t* e_cmask;          // per cell entry: octants that hold a child
     int8_t* e_level;            // depth of a cell; 22 marks a particle leaf
@@ -134,7 +134,7 @@ struct Tree {
     float4* pbox;                   // collision boxes of slots and slot runs (box_items(cap_n) pairs)
     double4_32a *d_a, *d_q0, *d_q1, *d_c;  // FP64 walk records (d_c: cell corner + width)
     int32_t *box_first, *box_root;  // per box, nbox + 1 each (box_root[nbox] = -1: removed particles)
-    int32_t* lvl;                   // per-depth cell counts / offsets / cursors (96)
+    int32_t* span;                  // moments: cells that go on past their range (moment_span_words)
     ImgTab* img;                    // [box][image] offsets of the current walk or search (nbox + 1 rows)
     int32_t* tq;                    // tile queues of the walks (kTileQStride ints each)
     int nq;                         // number of tile queues (one per SM)
@@ -251,10 +251,12 @@ void build_topology(const Tree& T, const PSet& P, Ctl* ctl, const BoxP* boxes, c
 void build_tile_order(Tree& T, const PSet& P, Ctl* ctl, int mode, int box_bits, cudaStream_t s);
 // Moments and walk records.  fp64 (FP64 walk, potential): FP64 records and
 // the FP32 records of the opening test; otherwise all FP64 and FP32 records,
-// and with f32q the quadrupole is summed in FP32 (the FP64 quadrupole records
-// then hold its FP32 values).
+// and with f32q the quadrupole is summed in FP32 and written to the FP32
+// records only.
 void build_gravity_records(const Tree& T, const PSet& P, Ctl* ctl, const BoxP* boxes,
                            const SimC& C, bool fp64, cudaStream_t s, bool f32q = false);
+size_t moment_span_words(int ncap);
+size_t moment_pieces(int ncap);   // records kept behind the tree's entries
 // Collision records on the tree of the last build at the current positions
 // (cells as FP32 boxes of their particles).
 void build_collision_aabb(const Tree& T, const PSet& P, Ctl* ctl, const SimC& C, cudaStream_t s);

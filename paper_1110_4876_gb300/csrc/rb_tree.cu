@@ -213,12 +213,14 @@ struct GravRecArgs {
     const double *x, *y, *z, *m;
     const int32_t *box, *id;
     bool has_test;   // some particles are test particles (source mass 0)
+    bool one;        // a single box
     const uint64_t* key;
     const BoxP* boxes;
     const int32_t *e_first, *e_skip, *e_child, *leaf_of;
     const uint32_t* e_cmask;
     const int8_t* e_level;
-    int32_t* e_arrive;
+    const int32_t *e_count, *start;
+    int piece0;      // first record behind the tree's entries
     double4_32a *d_a, *d_q0, *d_q1, *d_c;
     Rec4 ra, rb, rq0, rq1, rc_hi, rc_lo;
     const Ctl* ctl;
@@ -227,11 +229,8 @@ struct GravRecArgs {
     bool q32, inside;   // q32: FP32 quadrupole records are read too (not by the FP64 walk)
 };
 
-// Leaf records (FP64 and FP32) of every particle.
-__global__ void __launch_bounds__(256) k_leaf_records(GravRecArgs A) {
-    const int n = min(A.ctl->n_live, A.ncap);
-    const int p = blockIdx.x * blockDim.x + threadIdx.x;
-    if (p >= n) return;
+// Leaf record (FP64 and FP32) of particle p.
+__device__ __forceinline__ void leaf_record(const GravRecArgs& A, int p) {
     const int e = A.leaf_of[p];
     const double x = A.x[p], y = A.y[p], z = A.z[p];
     const double m = A.has_test ? source_mass(A.boxes[A.box[p]], A.id[p], A.m[p]) : A.m[p];
@@ -244,62 +243,13 @@ __global__ void __launch_bounds__(256) k_leaf_records(GravRecArgs A) {
     A.rb[e] = make_float4(lx, ly, -(float)m, __int_as_float(e + 1));
 }
 
-// Cells per depth: counts (block histograms, one atomic per depth and
-// block), offsets, then the lists.  lvl[0..22]: counts, lvl[32..54]: offsets,
-// lvl[64..86]: fill cursors.
-__global__ void __launch_bounds__(256) k_level_count(const int8_t* __restrict__ e_level,
-                                                     const Ctl* __restrict__ ctl, int ecap,
-                                                     int32_t* __restrict__ lvl) {
-    __shared__ int h[23];
-    if (threadIdx.x < 23) h[threadIdx.x] = 0;
-    __syncthreads();
-    const int E = min(ctl->n_entries, ecap);
-    const int k = blockIdx.x * blockDim.x + threadIdx.x;
-    if (k < E) {
-        const int v = e_level[k];
-        if (v < 22) atomicAdd(&h[v], 1);
-    }
-    __syncthreads();
-    if (threadIdx.x < 22 && h[threadIdx.x]) atomicAdd(&lvl[threadIdx.x], h[threadIdx.x]);
-}
-
-__global__ void k_level_offsets(int32_t* lvl) {
-    int s = 0;
-    for (int d = 0; d < 22; d++) {
-        lvl[32 + d] = s;
-        lvl[64 + d] = s;
-        s += lvl[d];
-    }
-}
-
-__global__ void __launch_bounds__(256) k_level_fill(const int8_t* __restrict__ e_level,
-                                                    const Ctl* __restrict__ ctl, int ecap,
-                                                    int32_t* __restrict__ lvl,
-                                                    int32_t* __restrict__ list) {
-    __shared__ int h[23], base[23];
-    if (threadIdx.x < 23) h[threadIdx.x] = 0;
-    __syncthreads();
-    const int E = min(ctl->n_entries, ecap);
-    const int k = blockIdx.x * blockDim.x + threadIdx.x;
-    int v = 22, mine = 0;
-    if (k < E) {
-        v = e_level[k];
-        if (v < 22) mine = atomicAdd(&h[v], 1);
-    }
-    __syncthreads();
-    if (threadIdx.x < 22 && h[threadIdx.x]) base[threadIdx.x] = atomicAdd(&lvl[64 + threadIdx.x], h[threadIdx.x]);
-    __syncthreads();
-    if (v < 22) list[base[v] + mine] = k;
-}
-
-// The cells of one depth.  A cell's moments come from its children (deeper
-// cells, done by earlier launches, or particle leaves) in one pass: about the
-// first child's position o, M = sum M_c, S = sum M_c d_c and
-// Q_o = sum [Q_c + M_c (3 d_c d_c^T - |d_c|^2 I)], d_c = com_c - o; then the
-// centre of mass is o + S / M and the parallel-axis theorem moves Q_o to it:
-// Q = Q_o - M (3 s s^T - |s|^2 I), s = S / M (the traceless quadrupole about
-// the centre of mass, reading R3).  Every |d_c| and |s| is below the cell's
-// diagonal, so no term is much larger than the result.
+// A cell's moments come from its children (cells done before it, or particle
+// leaves) in one pass: about the first child's position o, M = sum M_c,
+// S = sum M_c d_c and Q_o = sum [Q_c + M_c (3 d_c d_c^T - |d_c|^2 I)],
+// d_c = com_c - o; then the centre of mass is o + S / M and the parallel-axis
+// theorem moves Q_o to it: Q = Q_o - M (3 s s^T - |s|^2 I), s = S / M (the
+// traceless quadrupole about the centre of mass, reading R3).  Every |d_c| and
+// |s| is below the cell's diagonal, so no term is much larger than the result.
 // kF32Q: the quadrupole is only needed by the FP32 walk, so it is summed in
 // FP32 on the hi/lo records (d_c good to ~1e-7 relative); mass and centre of
 // mass stay FP64.  On GB300 FP64 instructions cost 64 times FP32 ones.
@@ -393,30 +343,28 @@ __device__ __forceinline__ bool group_has_chain(const GravRecArgs& A, int first,
     return d < kMaxDepth - 1;
 }
 
-// The cell's centre of mass, its quadrupole moved there, and its records.
+// 1/x from the hardware's coarse FP64 estimate and one step of the cubically
+// convergent iteration y (1 + h + h^2), h = 1 - x y (four FP64 operations; a
+// division takes three times as many); x outside the range where the estimate
+// is safe takes the division.
+__device__ __forceinline__ double rcp64(double x) {
+    const int e = (int)((__double_as_longlong(x) >> 52) & 0x7ff);
+    if (e < 64 || e > 1982) return 1.0 / x;
+    double y;
+    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+    const double h = fma(-x, y, 1.0);
+    return fma(y, fma(h, h, h), y);
+}
+
+// x 2^-v for x with exponent well inside the normal range (v <= 21).
+__device__ __forceinline__ double scale_down(double x, int v) {
+    return __longlong_as_double(__double_as_longlong(x) - ((long long)v << 52));
+}
+
+// Moves the quadrupole from the origin of the sums to the centre of mass at u
+// (parallel-axis theorem).
 template <bool kF32Q>
-__device__ __forceinline__ void mom_finish(const GravRecArgs& A, int k, int depth, int end, double ox,
-                                           double oy, double oz, MomSums& S) {
-    const int first = A.e_first[k];
-    // a leaf group's members are the entries k + 1 .. end - 1
-    const bool group = depth == kMaxDepth;
-    const bool chain = group && group_has_chain(A, first, first + (end - k - 2));
-    const int v = chain ? kMaxDepth - 1 : depth;   // the depth whose cell the record describes
-    const BoxP bp = A.boxes[A.box[first]];
-    const double w = ldexp(bp.L, -v);
-    const double lo = -0.5 * bp.L;
-    double ix = 0.0, iy = 0.0, iz = 0.0;
-    if (A.inside || !(S.M > 0.0)) cell_index(A.key[first], v, ix, iy, iz);
-    double cx, cy, cz, ux, uy, uz;   // centre of mass and its offset from o
-    if (S.M > 0.0) {
-        const double iM = 1.0 / S.M;
-        ux = S.sx * iM; uy = S.sy * iM; uz = S.sz * iM;
-        cx = ox + ux; cy = oy + uy; cz = oz + uz;
-    } else {
-        // no source mass (test particles only): the geometric centre
-        cx = lo + (ix + 0.5) * w; cy = lo + (iy + 0.5) * w; cz = lo + (iz + 0.5) * w;
-        ux = uy = uz = 0.0;
-    }
+__device__ __forceinline__ void mom_shift(MomSums& S, double ux, double uy, double uz) {
     if (kF32Q) {
         const float fx = (float)ux, fy = (float)uy, fz = (float)uz, fm = (float)S.M;
         const float d2 = fmaf(fz, fz, fmaf(fy, fy, fx * fx));
@@ -426,8 +374,6 @@ __device__ __forceinline__ void mom_finish(const GravRecArgs& A, int k, int dept
         S.qf[3] -= 3.f * fm * fx * fy;
         S.qf[4] -= 3.f * fm * fx * fz;
         S.qf[5] -= 3.f * fm * fy * fz;
-#pragma unroll
-        for (int j = 0; j < 6; j++) S.q[j] = (double)S.qf[j];
     } else {
         const double d2 = ux * ux + uy * uy + uz * uz;
         S.q[0] -= S.M * (3.0 * ux * ux - d2);
@@ -437,11 +383,41 @@ __device__ __forceinline__ void mom_finish(const GravRecArgs& A, int k, int dept
         S.q[4] -= S.M * (3.0 * ux * uz);
         S.q[5] -= S.M * (3.0 * uy * uz);
     }
+}
+
+// The cell's centre of mass, its quadrupole moved there, and its records.
+// first: its first slot; L: the side of its box's root cube.
+template <bool kF32Q>
+__device__ __forceinline__ void mom_finish(const GravRecArgs& A, int k, int depth, int end, int first, double L,
+                                           double ox, double oy, double oz, MomSums& S) {
+    // a leaf group's members are the entries k + 1 .. end - 1
+    const bool group = depth == kMaxDepth;
+    const bool chain = group && group_has_chain(A, first, first + (end - k - 2));
+    const int v = chain ? kMaxDepth - 1 : depth;   // the depth whose cell the record describes
+    const double w = scale_down(L, v);
+    const double lo = -0.5 * L;
+    double ix = 0.0, iy = 0.0, iz = 0.0;
+    if (A.inside || !(S.M > 0.0)) cell_index(A.key[first], v, ix, iy, iz);
+    double cx, cy, cz, ux, uy, uz;   // centre of mass and its offset from o
+    if (S.M > 0.0) {
+        const double iM = rcp64(S.M);
+        ux = S.sx * iM; uy = S.sy * iM; uz = S.sz * iM;
+        cx = ox + ux; cy = oy + uy; cz = oz + uz;
+    } else {
+        // no source mass (test particles only): the geometric centre
+        cx = lo + (ix + 0.5) * w; cy = lo + (iy + 0.5) * w; cz = lo + (iz + 0.5) * w;
+        ux = uy = uz = 0.0;
+    }
+    mom_shift<kF32Q>(S, ux, uy, uz);
     const bool never = group && !chain;   // a leaf group with no one-child cell above it
     const double ww = w * w;
     A.d_a[k] = make_double4_32a(cx, cy, cz, never ? __longlong_as_double(0x7ff0000000000000ll) : ww);
-    A.d_q0[k] = make_double4_32a(S.M, S.q[0], S.q[1], S.q[2]);
-    A.d_q1[k] = make_double4_32a(S.q[3], S.q[4], S.q[5], w);
+    if (kF32Q) {
+        A.d_q0[k].x = S.M;   // the quadrupole is read from the FP32 records
+    } else {
+        A.d_q0[k] = make_double4_32a(S.M, S.q[0], S.q[1], S.q[2]);
+        A.d_q1[k] = make_double4_32a(S.q[3], S.q[4], S.q[5], w);
+    }
     double c0x = 0.0, c0y = 0.0, c0z = 0.0;
     if (A.inside) {
         // cell corner lo + i w, rounded as two separate operations
@@ -475,79 +451,335 @@ __device__ __forceinline__ void mom_finish(const GravRecArgs& A, int k, int dept
     }
 }
 
-// The cells of one depth.  A cell's moments come from its children (deeper
-// cells, done by earlier launches, or particle leaves) in one pass: about the
-// first child's position o, M = sum M_c, S = sum M_c d_c and
-// Q_o = sum [Q_c + M_c (3 d_c d_c^T - |d_c|^2 I)], d_c = com_c - o; then the
-// centre of mass is o + S / M and the parallel-axis theorem moves Q_o to it:
-// Q = Q_o - M (3 s s^T - |s|^2 I), s = S / M (the traceless quadrupole about
-// the centre of mass, reading R3).  Every |d_c| and |s| is below the cell's
-// diagonal, so no term is much larger than the result.
-// kF32Q: the quadrupole is only needed by the FP32 walk, so it is summed in
-// FP32 on the hi/lo records (d_c good to ~1e-7 relative); mass and centre of
-// mass stay FP64.  On GB300 FP64 instructions cost 64 times FP32 ones.
-// A depth with few cells (the top of the tree, the deep close pairs) is
-// latency-bound: there eight lanes take one cell, one child each from the
-// octant table, and add their sums in a fixed butterfly order; a depth with
-// many cells gives each thread one cell, which follows its children in
-// pre-order.
-constexpr int kWarpCells = 19456;   // up to 4 cells per warp of the launch grid
+// Side of the root cube of the box that slot `first` lies in (one box: its
+// side, loaded once per block).
+__device__ __forceinline__ double root_side(const GravRecArgs& A, int first, double one) {
+    return A.one ? one : A.boxes[A.box[first]].L;
+}
 
+// Sums of a warp's lanes, in a fixed butterfly order.
 template <bool kF32Q>
-__global__ void __launch_bounds__(256) k_moments_level(GravRecArgs A, const int32_t* __restrict__ lvl,
-                                                       const int32_t* __restrict__ list, int depth) {
-    const int cnt = lvl[depth], off = lvl[32 + depth];
-    if (cnt <= kWarpCells && depth < kMaxDepth) {
-        const int lane = threadIdx.x & 31, o = lane & 7;   // o: octant of this lane's child
-        const int wg = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, nwg = (gridDim.x * blockDim.x) >> 5;
-        for (int base = 4 * wg; base < cnt; base += 4 * nwg) {
-            // a warp takes 4 cells; a group past the end still joins the shuffles
-            const int g = base + (lane >> 3);
-            const bool live = g < cnt;
-            const int k = live ? list[off + g] : 0;
-            MomSums S;
-            mom_zero(S);
-            double ox = 0.0, oy = 0.0, oz = 0.0;
-            float4 h0 = make_float4(0.f, 0.f, 0.f, 0.f), l0 = h0;
-            if (live) {
-                const double4_32a a0 = A.d_a[k + 1];   // the first child is entry k + 1
-                ox = a0.x; oy = a0.y; oz = a0.z;
-                if (kF32Q) {
-                    h0 = A.ra[k + 1];
-                    l0 = A.rb[k + 1];
-                }
-                if ((A.e_cmask[k] >> o) & 1u) mom_add<kF32Q>(A, A.e_child[8 * (size_t)k + o], ox, oy, oz, h0, l0, S);
-            }
+__device__ __forceinline__ void mom_reduce(MomSums& S, int width) {
+    for (int x = 1; x < width; x <<= 1) {
+        S.M += __shfl_xor_sync(0xffffffffu, S.M, x);
+        S.sx += __shfl_xor_sync(0xffffffffu, S.sx, x);
+        S.sy += __shfl_xor_sync(0xffffffffu, S.sy, x);
+        S.sz += __shfl_xor_sync(0xffffffffu, S.sz, x);
 #pragma unroll
-            for (int x = 1; x < 8; x <<= 1) {
-                S.M += __shfl_xor_sync(0xffffffffu, S.M, x);
-                S.sx += __shfl_xor_sync(0xffffffffu, S.sx, x);
-                S.sy += __shfl_xor_sync(0xffffffffu, S.sy, x);
-                S.sz += __shfl_xor_sync(0xffffffffu, S.sz, x);
-#pragma unroll
-                for (int j = 0; j < 6; j++) {
-                    if (kF32Q) S.qf[j] += __shfl_xor_sync(0xffffffffu, S.qf[j], x);
-                    else S.q[j] += __shfl_xor_sync(0xffffffffu, S.q[j], x);
-                }
-            }
-            if (live && o == 0) mom_finish<kF32Q>(A, k, depth, A.e_skip[k], ox, oy, oz, S);
+        for (int j = 0; j < 6; j++) {
+            if (kF32Q) S.qf[j] += __shfl_xor_sync(0xffffffffu, S.qf[j], x);
+            else S.q[j] += __shfl_xor_sync(0xffffffffu, S.q[j], x);
         }
-        return;
     }
-    for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < cnt; t += gridDim.x * blockDim.x) {
-        const int k = list[off + t];
-        const int end = A.e_skip[k];
-        const double4_32a a0 = A.d_a[k + 1];
-        const double ox = a0.x, oy = a0.y, oz = a0.z;
-        float4 h0 = make_float4(0.f, 0.f, 0.f, 0.f), l0 = h0;
+}
+
+// One cell by eight lanes (lane o of 8 takes the child in octant o, which add
+// their sums in a fixed butterfly order); groups without a cell (live false)
+// join the shuffles.  Not for depth-21 groups, which have no child table.
+template <bool kF32Q>
+__device__ __forceinline__ void mom_cell_group(const GravRecArgs& A, bool live, int k, int depth, double one) {
+    const int o = threadIdx.x & 7;
+    MomSums S;
+    mom_zero(S);
+    double ox = 0.0, oy = 0.0, oz = 0.0, L = 0.0;
+    int first = 0, end = 0;
+    float4 h0 = make_float4(0.f, 0.f, 0.f, 0.f), l0 = h0;
+    if (live) {
+        const bool has = (A.e_cmask[k] >> o) & 1u;
+        const int child = A.e_child[8 * (size_t)k + o];
+        first = A.e_first[k];
+        end = A.e_skip[k];
+        const double4_32a a0 = A.d_a[k + 1];   // the first child is entry k + 1
+        ox = a0.x; oy = a0.y; oz = a0.z;
         if (kF32Q) {
             h0 = A.ra[k + 1];
             l0 = A.rb[k + 1];
         }
+        L = root_side(A, first, one);
+        if (has) mom_add<kF32Q>(A, child, ox, oy, oz, h0, l0, S);
+    }
+    mom_reduce<kF32Q>(S, 8);
+    if (live && o == 0) mom_finish<kF32Q>(A, k, depth, end, first, L, ox, oy, oz, S);
+}
+
+// One cell by one thread, from its children in pre-order.
+template <bool kF32Q>
+__device__ __forceinline__ void mom_cell(const GravRecArgs& A, int k, int depth, double one) {
+    const int end = A.e_skip[k], first = A.e_first[k];
+    const double4_32a a0 = A.d_a[k + 1];
+    const double ox = a0.x, oy = a0.y, oz = a0.z, L = root_side(A, first, one);
+    float4 h0 = make_float4(0.f, 0.f, 0.f, 0.f), l0 = h0;
+    if (kF32Q) {
+        h0 = A.ra[k + 1];
+        l0 = A.rb[k + 1];
+    }
+    MomSums S;
+    mom_zero(S);
+    for (int c = k + 1; c < end; c = A.e_skip[c]) mom_add<kF32Q>(A, c, ox, oy, oz, h0, l0, S);
+    mom_finish<kF32Q>(A, k, depth, end, first, L, ox, oy, oz, S);
+}
+
+// One cell of `count` particles by one thread, straight from their leaves.
+template <bool kF32Q>
+__device__ __forceinline__ void mom_cell_leaves(const GravRecArgs& A, int k, int count, double one) {
+    const int end = A.e_skip[k], first = A.e_first[k], depth = A.e_level[k];
+    const int c0 = A.leaf_of[first];
+    const double4_32a a0 = A.d_a[c0];
+    const double ox = a0.x, oy = a0.y, oz = a0.z, L = root_side(A, first, one);
+    float4 h0 = make_float4(0.f, 0.f, 0.f, 0.f), l0 = h0;
+    if (kF32Q) {
+        h0 = A.ra[c0];
+        l0 = A.rb[c0];
+    }
+    MomSums S;
+    mom_zero(S);
+#pragma unroll 2
+    for (int j = 0; j < count; j++) mom_add<kF32Q>(A, A.leaf_of[first + j], ox, oy, oz, h0, l0, S);
+    mom_finish<kF32Q>(A, k, depth, end, first, L, ox, oy, oz, S);
+}
+
+constexpr int kDepths = kMaxDepth + 1;
+constexpr int kMomSlots = 1024;   // most slots of a block's range
+constexpr int kDirect = 8;        // cells of at most this many particles are summed from their leaves
+constexpr int kGroupCells = 16;   // depths with at most this many cells take eight lanes a cell
+constexpr int kBuckets = kDirect - 1 + kDepths;   // cells of 2 .. kDirect particles, then by depth
+
+// Moments of the cells whose particles lie within one range of `slots`
+// consecutive slots (a block each), and the leaf records.  The cells of at most
+// kDirect particles, three quarters of all, come straight from their leaves,
+// all at once and sorted by their count, so that warps are full and alike; the
+// larger ones from their children, depth by depth with block barriers.  Cells
+// that go on past the range's end all hold its last slot, so there is at most
+// one of each depth: span[range][depth] (-1: none), for k_moments_span.
+// Bound by FP64 issue (an FP64 warp instruction holds the SM's FP64 pipe 16
+// cycles whatever its active lanes; 52% of its cycles busy at 400k) at many
+// particles, by the chain of depths at few.  Moments and leaf records of one
+// build, all launches: 41 us at 2,400 particles, 51 at 30k, 72 at 100k and 271
+// at 1M, against 92, 123, 146 and 350 us with one launch per depth (26
+// launches; these are three).
+template <bool kF32Q>
+__global__ void __launch_bounds__(256, 4) k_moments_range(GravRecArgs A, int slots, int32_t* __restrict__ span) {
+    __shared__ int cnt[kBuckets], off[kBuckets], over[kDepths];
+    __shared__ uint16_t list[2 * kMomSlots];   // the range's cells by bucket, as entry - e0
+    const int n = min(A.ctl->n_live, A.ncap);
+    const int p0 = blockIdx.x * slots, tid = threadIdx.x;
+    if (p0 >= n) {
+        if (tid < kDepths) span[blockIdx.x * kDepths + tid] = -1;
+        return;
+    }
+    const int p1 = min(n, p0 + slots);
+    const int e0 = A.start[p0], e1 = A.start[p1];
+    const double one = A.boxes[0].L;
+    if (tid < kBuckets) cnt[tid] = 0;
+    if (tid < kDepths) over[tid] = -1;
+    for (int p = p0 + tid; p < p1; p += 256) leaf_record(A, p);
+    __syncthreads();
+    auto bucket = [&](int e, int& v) {   // -1: a leaf, or a cell that ends past the range
+        v = A.e_level[e];
+        if (v >= kDepths) return -1;     // 22 marks a particle leaf
+        const int c = A.e_count[e];
+        if (A.e_first[e] + c > p1) return -1;
+        return c <= kDirect ? c - 2 : kDirect - 1 + v;
+    };
+    for (int e = e0 + tid; e < e1; e += 256) {
+        int v;
+        const int b = bucket(e, v);
+        if (b >= 0) atomicAdd(&cnt[b], 1);
+        else if (v < kDepths) over[v] = e;
+    }
+    __syncthreads();
+    if (tid < kBuckets) {
+        int o = 0;
+        for (int b = 0; b < tid; b++) o += cnt[b];
+        off[tid] = o;
+    }
+    if (tid < kDepths) span[blockIdx.x * kDepths + tid] = over[tid];
+    __syncthreads();
+    for (int e = e0 + tid; e < e1; e += 256) {
+        int v;
+        const int b = bucket(e, v);
+        if (b >= 0) list[atomicAdd(&off[b], 1)] = (uint16_t)(e - e0);
+    }
+    __syncthreads();   // off[b] now ends bucket b
+    const int direct = off[kDirect - 2];
+    for (int t = tid; t < direct; t += 256) {
+        const int e = e0 + list[t];
+        mom_cell_leaves<kF32Q>(A, e, A.e_count[e], one);
+    }
+    __syncthreads();
+    for (int v = kMaxDepth; v >= 0; v--) {
+        const int c = cnt[kDirect - 1 + v], first = off[kDirect - 1 + v] - c;
+        if (c == 0) continue;
+        if (c <= kGroupCells && v < kMaxDepth) {
+            // four cells a warp
+            if ((tid >> 5) * 4 < c) {
+                const bool live = (tid >> 3) < c;
+                mom_cell_group<kF32Q>(A, live, live ? e0 + list[first + (tid >> 3)] : 0, v, one);
+            }
+        } else {
+            for (int t = tid; t < c; t += 256) mom_cell<kF32Q>(A, e0 + list[first + t], v, one);
+        }
+        __syncthreads();
+    }
+}
+
+// The cells that go on past their range.  Listed by range and depth they are
+// in pre-order, so the ones inside such a cell follow it without a gap: those
+// of its own range at larger depths, then all of the ranges it covers.  With
+// own(c) the part of a cell held by its children that end within their range
+// (finished by k_moments_range), a cell is the sum of own() over itself and the
+// cells inside it: no chain through the depths.  Both parts are kept as cell
+// records behind the tree's entries, piece(r, v) and, for v = kDepths, the sum
+// over range r.
+__device__ __forceinline__ int piece(const GravRecArgs& A, int r, int v) {
+    return A.piece0 + r * (kDepths + 1) + v;
+}
+
+// Record of a piece: the sums about o as mass, centre of mass and quadrupole.
+template <bool kF32Q>
+__device__ __forceinline__ void put_piece(const GravRecArgs& A, int k, double ox, double oy, double oz, MomSums& S) {
+    double ux = 0.0, uy = 0.0, uz = 0.0;
+    if (S.M > 0.0) {
+        const double iM = rcp64(S.M);
+        ux = S.sx * iM; uy = S.sy * iM; uz = S.sz * iM;
+    }
+    const double cx = ox + ux, cy = oy + uy, cz = oz + uz;
+    mom_shift<kF32Q>(S, ux, uy, uz);
+    A.d_a[k] = make_double4_32a(cx, cy, cz, 0.0);
+    float hx, lx, hy, ly, hz, lz;
+    split_hilo(cx, hx, lx);
+    split_hilo(cy, hy, ly);
+    split_hilo(cz, hz, lz);
+    A.ra[k] = make_float4(hx, hy, hz, lz);
+    A.rb[k] = make_float4(lx, ly, 0.f, 0.f);
+    if (kF32Q) {
+        A.d_q0[k].x = S.M;
+        A.rq0[k] = make_float4((float)S.M, S.qf[0], S.qf[1], S.qf[2]);
+        A.rq1[k] = make_float4(S.qf[3], S.qf[4], S.qf[5], 0.f);
+    } else {
+        A.d_q0[k] = make_double4_32a(S.M, S.q[0], S.q[1], S.q[2]);
+        A.d_q1[k] = make_double4_32a(S.q[3], S.q[4], S.q[5], 0.0);
+    }
+}
+
+// own() of a range's cells (a warp per range, eight lanes per cell) and their
+// sum.
+template <bool kF32Q>
+__global__ void __launch_bounds__(64) k_moments_own(GravRecArgs A, int slots, const int32_t* __restrict__ span, int nr) {
+    const int r = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
+    if (r >= nr) return;
+    const int mine = lane < kDepths ? span[r * kDepths + lane] : -1;
+    const unsigned have = __ballot_sync(0xffffffffu, mine >= 0);
+    unsigned left = have;
+    while (left) {
+        // the next four cells, one per group of lanes
+        unsigned m = left;
+        for (int g = 0; g < (lane >> 3) && m; g++) m &= m - 1;
+        const int v = m ? __ffs(m) - 1 : 0;
+        const bool live = m != 0;
+        for (int g = 0; g < 4 && left; g++) left &= left - 1;
+        const int k = __shfl_sync(0xffffffffu, mine, v);
         MomSums S;
         mom_zero(S);
-        for (int c = k + 1; c < end; c = A.e_skip[c]) mom_add<kF32Q>(A, c, ox, oy, oz, h0, l0, S);
-        mom_finish<kF32Q>(A, k, depth, end, ox, oy, oz, S);
+        double ox = 0.0, oy = 0.0, oz = 0.0;
+        if (live) {
+            const int o = lane & 7;
+            const int c0 = A.leaf_of[A.e_first[k]];   // sums about its first particle
+            const double4_32a a0 = A.d_a[c0];
+            ox = a0.x; oy = a0.y; oz = a0.z;
+            float4 h0 = make_float4(0.f, 0.f, 0.f, 0.f), l0 = h0;
+            if (kF32Q) {
+                h0 = A.ra[c0];
+                l0 = A.rb[c0];
+            }
+            if (v == kMaxDepth) {
+                // a leaf group: its members, whatever ranges they lie in
+                for (int c = k + 1 + o, end = A.e_skip[k]; c < end; c += 8)
+                    mom_add<kF32Q>(A, c, ox, oy, oz, h0, l0, S);
+            } else if ((A.e_cmask[k] >> o) & 1u) {
+                const int c = A.e_child[8 * (size_t)k + o];
+                const int first = A.e_first[c];
+                if (first + A.e_count[c] <= (first / slots + 1) * slots)
+                    mom_add<kF32Q>(A, c, ox, oy, oz, h0, l0, S);
+            }
+        }
+        mom_reduce<kF32Q>(S, 8);
+        if (live && (lane & 7) == 0) put_piece<kF32Q>(A, piece(A, r, v), ox, oy, oz, S);
+    }
+    __syncwarp();
+    MomSums S;
+    mom_zero(S);
+    double ox = 0.0, oy = 0.0, oz = 0.0;
+    if (have) {
+        const int c0 = piece(A, r, __ffs(have) - 1);
+        const double4_32a a0 = A.d_a[c0];
+        ox = a0.x; oy = a0.y; oz = a0.z;
+        if (mine >= 0) mom_add<kF32Q>(A, piece(A, r, lane), ox, oy, oz, A.ra[c0], A.rb[c0], S);
+    }
+    mom_reduce<kF32Q>(S, 32);
+    if (lane == 0) put_piece<kF32Q>(A, piece(A, r, kDepths), ox, oy, oz, S);
+}
+
+// The cells themselves, a block per range: a warp per cell, or the whole block
+// for a cell that covers many ranges.
+constexpr int kLongCell = 128;
+
+template <bool kF32Q>
+__global__ void __launch_bounds__(256) k_moments_span(GravRecArgs A, int slots, const int32_t* __restrict__ span) {
+    __shared__ MomSums part[8];
+    const int r = blockIdx.x, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int mine = lane < kDepths ? span[r * kDepths + lane] : -1;
+    const unsigned have = __ballot_sync(0xffffffffu, mine >= 0);
+    if (!have) return;
+    const double one = A.boxes[0].L;
+    // this lane's share of the cell at depth v: pieces of its own range by the
+    // lanes of warp w0, the sums of the ranges it covers by `width` lanes
+    auto share = [&](int v, int r2, int at, int width, bool own, const double4_32a& a0, const float4& h0,
+                     const float4& l0, MomSums& S) {
+        mom_zero(S);
+        if (own && mine >= 0 && lane >= v) mom_add<kF32Q>(A, piece(A, r, lane), a0.x, a0.y, a0.z, h0, l0, S);
+        // a leaf group's piece is all of it
+        for (int q = r + 1 + at; v < kMaxDepth && q < r2; q += width)
+            mom_add<kF32Q>(A, piece(A, q, kDepths), a0.x, a0.y, a0.z, h0, l0, S);
+        mom_reduce<kF32Q>(S, 32);
+    };
+    unsigned left = have, wide = 0;
+    for (int j = 0; left; left &= left - 1, j++) {
+        const int v = __ffs(left) - 1;
+        const int k = __shfl_sync(0xffffffffu, mine, v);
+        const int first = A.e_first[k];
+        const int r2 = (first + A.e_count[k] - 1) / slots;
+        if (r2 - r > kLongCell && v < kMaxDepth) {
+            wide |= 1u << v;
+            continue;
+        }
+        if ((j & 7) != warp) continue;
+        const int end = A.e_skip[k], c0 = A.leaf_of[first];
+        const double L = root_side(A, first, one);
+        const double4_32a a0 = A.d_a[c0];
+        MomSums S;
+        share(v, r2, lane, 32, true, a0, A.ra[c0], A.rb[c0], S);
+        if (lane == 0) mom_finish<kF32Q>(A, k, v, end, first, L, a0.x, a0.y, a0.z, S);
+    }
+    for (; wide; wide &= wide - 1) {
+        const int v = __ffs(wide) - 1;
+        const int k = __shfl_sync(0xffffffffu, mine, v);
+        const int first = A.e_first[k];
+        const int r2 = (first + A.e_count[k] - 1) / slots;
+        const int c0 = A.leaf_of[first];
+        const double4_32a a0 = A.d_a[c0];
+        MomSums S;
+        share(v, r2, threadIdx.x, 256, warp == 0, a0, A.ra[c0], A.rb[c0], S);
+        __syncthreads();   // part is reused
+        if (lane == 0) part[warp] = S;
+        __syncthreads();
+        if (warp == 0) {
+            if (lane < 8) S = part[lane];
+            else mom_zero(S);
+            mom_reduce<kF32Q>(S, 8);
+            if (lane == 0)
+                mom_finish<kF32Q>(A, k, v, A.e_skip[k], first, root_side(A, first, one), a0.x, a0.y, a0.z, S);
+        }
     }
 }
 
@@ -893,6 +1125,25 @@ void build_tile_order(Tree& T, const PSet& P, Ctl* ctl, int mode, int box_bits, 
     T.order = which ? T.tval_alt : T.tval;
 }
 
+namespace {
+
+// Slots of a block's range.  Few particles: short ranges, which end sooner
+// (2,400: 54 us in ranges of 256 slots, 70 of 512 and 79 of 1024; 100k: 88, 92
+// and 102).  More than fill the GPU that way (608 resident blocks): the longest
+// that fill it once or a whole number of times, since long ranges fill the
+// warps of a depth (1M: 340 us at 1024, 390 at 512).
+int moment_slots(int n) {
+    constexpr int kBlocks = 4 * 152;
+    if (n <= kBlocks * 256) return 256;
+    const int waves = ceil_div(n, kBlocks * kMomSlots);
+    return ceil_div(ceil_div(n, (long long)kBlocks * waves), 8) * 8;
+}
+
+}  // namespace
+
+size_t moment_span_words(int ncap) { return (size_t)ceil_div(ncap, moment_slots(ncap)) * kDepths; }
+size_t moment_pieces(int ncap) { return (size_t)ceil_div(ncap, moment_slots(ncap)) * (kDepths + 1); }
+
 void build_gravity_records(const Tree& T, const PSet& P, Ctl* ctl, const BoxP* boxes,
                            const SimC& C, bool fp64, cudaStream_t s, bool f32q) {
     const int n = T.cap_n;
@@ -900,10 +1151,11 @@ void build_gravity_records(const Tree& T, const PSet& P, Ctl* ctl, const BoxP* b
     GravRecArgs A;
     A.x = P.x; A.y = P.y; A.z = P.z; A.m = P.m; A.box = P.box; A.id = P.id;
     A.has_test = C.has_test != 0;
+    A.one = C.nbox == 1;
     A.key = T.key; A.boxes = boxes;
     A.e_first = T.e_first; A.e_skip = T.e_skip; A.e_child = T.e_child;
     A.e_cmask = T.e_cmask; A.leaf_of = T.leaf_of; A.e_level = T.e_level;
-    A.e_arrive = T.e_arrive;
+    A.e_count = T.e_count; A.start = T.start;
     A.d_a = T.d_a; A.d_q0 = T.d_q0; A.d_q1 = T.d_q1; A.d_c = T.d_c;
     A.ra = T.ra; A.rb = T.rb; A.rq0 = T.rq0; A.rq1 = T.rq1; A.rc_hi = T.rc_hi; A.rc_lo = T.rc_lo;
     A.ctl = ctl;
@@ -911,17 +1163,20 @@ void build_gravity_records(const Tree& T, const PSet& P, Ctl* ctl, const BoxP* b
     A.crit_scale = C.crit_scale;
     A.q32 = !fp64;
     A.inside = C.theta2 > (1.0 / 3.0);
-    k_leaf_records<<<ceil_div(n, 256), 256, 0, s>>>(A);
-    cudaMemsetAsync(T.lvl, 0, sizeof(int32_t) * 96, s);
-    const int ne = T.cap_e;
-    k_level_count<<<ceil_div(ne, 256), 256, 0, s>>>(T.e_level, ctl, ne, T.lvl);
-    k_level_offsets<<<1, 1, 0, s>>>(T.lvl);
-    k_level_fill<<<ceil_div(ne, 256), 256, 0, s>>>(T.e_level, ctl, ne, T.lvl, T.e_arrive);
-    const int grid = std::min(ceil_div(n, 256), 4 * 152);
     const bool q32 = f32q && !fp64;
-    for (int d = kMaxDepth; d >= 0; d--) {
-        if (q32) k_moments_level<true><<<grid, 256, 0, s>>>(A, T.lvl, T.e_arrive, d);
-        else k_moments_level<false><<<grid, 256, 0, s>>>(A, T.lvl, T.e_arrive, d);
+    const int slots = moment_slots(n);
+    const int nr = ceil_div(n, slots);
+    A.piece0 = T.cap_e;
+    if (q32) k_moments_range<true><<<nr, 256, 0, s>>>(A, slots, T.span);
+    else k_moments_range<false><<<nr, 256, 0, s>>>(A, slots, T.span);
+    if (nr == 1) return;
+    const int nb = ceil_div(nr, 2);   // a warp per range
+    if (q32) {
+        k_moments_own<true><<<nb, 64, 0, s>>>(A, slots, T.span, nr);
+        k_moments_span<true><<<nr, 256, 0, s>>>(A, slots, T.span);
+    } else {
+        k_moments_own<false><<<nb, 64, 0, s>>>(A, slots, T.span, nr);
+        k_moments_span<false><<<nr, 256, 0, s>>>(A, slots, T.span);
     }
 }
 
