@@ -233,9 +233,12 @@ int radix_sort_passes(int key_bits, bool box_pass, int box_bits);
 // (k0, v0) and 1 if it is in (k1, v1).  hist holds radix_hist_words(ncap)
 // words; ncap < 2^30.  A look-back wait that gives up sets kErrSortStall in
 // *err (device memory).
+// low_bit > 0: key bits [low_bit, key_bits) by passes, the bits below it
+// within each run of keys that agree above, once the runs are together; for
+// keys whose runs are short (any length gives the same order).
 int radix_sort(uint64_t* k0, uint32_t* v0, uint64_t* k1, uint32_t* v1, int ncap, const int* d_n,
                int key_bits, const int32_t* box_digits, int box_bits, uint32_t* hist, int* err,
-               cudaStream_t s);
+               cudaStream_t s, int low_bit = 0);
 size_t radix_hist_words(int ncap);
 void exclusive_scan_i32(int32_t* data, int n_cap, const int* d_n, int32_t* part, int32_t* total,
                         cudaStream_t s);

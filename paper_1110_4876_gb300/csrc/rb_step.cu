@@ -488,11 +488,16 @@ void drift_keys(const PSet& P, const Tree& T, Ctl* ctl, const BoxP* boxes, const
     k_drift_keys<<<ceil_div(ncap, 256), 256, 0, s>>>(A, C);
 }
 
+// Morton bits below those that the passes sort.
+constexpr int kMortonLowBits = 24;
+
 void sort_and_permute(const PSet& src, const PSet& dst, Tree& T, Pairs& PR, Ctl* ctl,
                       const SimC& C, int ncap, int box_bits, cudaStream_t s) {
     if (ncap <= 0) return;
+    // five passes over the top 40 bits (depth 13), the rest within the short
+    // runs that agree there
     const int which = radix_sort(T.key, T.idx, T.key_alt, T.idx_alt, ncap, nullptr, 64,
-                                 C.nbox > 1 ? T.sbox : nullptr, box_bits, T.hist, &ctl->err, s);
+                                 C.nbox > 1 ? T.sbox : nullptr, box_bits, T.hist, &ctl->err, s, kMortonLowBits);
     if (which == 1) {
         // keep the sorted keys in T.key for the topology kernels
         uint64_t* k = T.key; T.key = T.key_alt; T.key_alt = k;
@@ -575,10 +580,11 @@ void reset_slots(const PSet& P, int32_t* slot_of_id, int n, int ncap, int nbox, 
 
 void sort_pairs(Pairs& PR, Ctl* ctl, cudaStream_t s, int key_bits) {
     k_pairs_prep<<<1, 1, 0, s>>>(ctl, PR.cap);
+    // passes over the lower id's bits, then each id's pairs among themselves;
     // an odd number of passes leaves the keys in key_alt; the buffers are
     // not swapped, so every captured graph finds them in the same place
     PR.sorted_alt = radix_sort(PR.key, PR.val, PR.key_alt, PR.val_alt, PR.cap, &ctl->pair_n,
-                               key_bits, nullptr, 0, PR.hist, &ctl->err, s) == 1;
+                               key_bits, nullptr, 0, PR.hist, &ctl->err, s, 36) == 1;
 }
 
 void resolve_pairs(const PSet& P, Ctl* ctl, const BoxP* boxes, const SimC& C, Pairs& PR,
