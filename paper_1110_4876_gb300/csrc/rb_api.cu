@@ -313,8 +313,8 @@ int upload(rb_sim* s) {
             rc |= dalloc(s, &s->SW.key, ic, L); rc |= dalloc(s, &s->SW.key_alt, ic, L);
             rc |= dalloc(s, &s->SW.val, ic, L); rc |= dalloc(s, &s->SW.val_alt, ic, L);
             rc |= dalloc(s, &s->SW.hist, radix_hist_words(ic), L);
-            double4_32a* recs = nullptr;   // 64-byte records: two double4 each
-            rc |= dalloc(s, &recs, 2 * (size_t)ic, L);
+            float4* recs = nullptr;   // 48-byte records
+            rc |= dalloc(s, &recs, 3 * (size_t)ic, L);
             s->SW.rec = recs;
             s->SW.cap = ic;
         }

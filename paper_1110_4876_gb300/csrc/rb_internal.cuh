@@ -180,7 +180,7 @@ struct Sweep {
     uint64_t *key, *key_alt;   // (box << 32) | quantised lower end
     uint32_t *val, *val_alt;   // (particle slot << 3) | copy
     uint32_t* hist;
-    void* rec;                 // per sorted item: the particle's state (64 B)
+    void* rec;                 // per sorted item: the particle's state (48 B)
     int cap, box_bits;         // cap = particles x (1 + nghost_x)
 };
 

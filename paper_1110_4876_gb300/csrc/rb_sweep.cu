@@ -14,16 +14,12 @@
 //      extents overlap P's and start after it, the trajectories already in the
 //      paper's list when P enters it.  Each candidate (at least one original
 //      particle, two different particles) is tested with the straight-line
-//      criterion over every y/z image, in FP64 with the oracle's operation
-//      sequence, on the canonical orientation (lower id a, image of b).
+//      criterion for every y/z image within reach, in FP32 clear of the
+//      threshold, else in FP64 with the oracle's operation sequence on the
+//      canonical orientation (lower id a, image of b).
 // The quantisation is a monotone map of the FP64 extents, so the scan never
-// stops before an overlapping item; the exact FP64 comparison of the extents
-// and a conservative y test only prune candidates the criterion rejects.
-#include <cooperative_groups.h>
-
+// stops before an overlapping item.
 #include "rb_internal.cuh"
-
-namespace cg = cooperative_groups;
 
 namespace rb {
 namespace {
@@ -125,12 +121,20 @@ __global__ void __launch_bounds__(256) k_sweep_items(SweepArgs A) {
 }
 
 // Particle data of the sorted items, gathered once so that the scans read
-// neighbouring records instead of scattered particle slots.
+// neighbouring records instead of scattered particle slots: positions as hi/lo
+// floats, velocities and radius as floats (the particle's own, unshifted).
 struct __align__(16) SweepRec {
-    double x, y, z, vx, vy, vz, r;   // the particle's own (unshifted) state
-    int id;                          // global id
-    uint32_t sc;                     // (slot << 3) | copy
+    float xh, yh, zh, r;
+    float xl, yl, zl, vx;
+    float vy, vz;
+    uint32_t sc;     // (slot << 3) | copy
+    float vsum;      // |vx| + |vy| + |vz|
 };
+
+__device__ __forceinline__ void split_hl(double v, float& hi, float& lo) {
+    hi = __double2float_rn(v);
+    lo = __double2float_rn(v - (double)hi);
+}
 
 __global__ void __launch_bounds__(256) k_sweep_gather(SweepArgs A, const uint32_t* __restrict__ val,
                                                       SweepRec* __restrict__ rec) {
@@ -140,10 +144,14 @@ __global__ void __launch_bounds__(256) k_sweep_gather(SweepArgs A, const uint32_
     const uint32_t v = val[k];
     const int i = (int)(v >> 3);
     SweepRec q;
-    q.x = A.P.x[i]; q.y = A.P.y[i]; q.z = A.P.z[i];
-    q.vx = A.P.vx[i]; q.vy = A.P.vy[i]; q.vz = A.P.vz[i];
-    q.r = A.P.r[i];
-    q.id = A.P.id[i];
+    split_hl(A.P.x[i], q.xh, q.xl);
+    split_hl(A.P.y[i], q.yh, q.yl);
+    split_hl(A.P.z[i], q.zh, q.zl);
+    q.vx = (float)A.P.vx[i];
+    q.vy = (float)A.P.vy[i];
+    q.vz = (float)A.P.vz[i];
+    q.r = (float)A.P.r[i];
+    q.vsum = fabsf(q.vx) + fabsf(q.vy) + fabsf(q.vz);
     q.sc = v;
     rec[k] = q;
 }
@@ -151,14 +159,14 @@ __global__ void __launch_bounds__(256) k_sweep_gather(SweepArgs A, const uint32_
 // Straight-line criterion (Sect. 5.3, readings S1/S2) for particle a and the
 // image of b (offset o, y velocity offset dvy), in the oracle's operation
 // sequence.
-__device__ __forceinline__ bool line_hit(const SweepRec& a, const SweepRec& b, double h, double ox,
-                                         double oy, double oz, double dvy) {
-    const double rx = __dsub_rn(__dadd_rn(b.x, ox), a.x);
-    const double ry = __dsub_rn(__dadd_rn(b.y, oy), a.y);
-    const double rz = __dsub_rn(__dadd_rn(b.z, oz), a.z);
-    const double ux = __dsub_rn(b.vx, a.vx);
-    const double uy = __dsub_rn(__dadd_rn(b.vy, dvy), a.vy);
-    const double uz = __dsub_rn(b.vz, a.vz);
+__device__ __forceinline__ bool line_hit(const PSet& P, int a, int b, double h, double ox, double oy, double oz,
+                                         double dvy) {
+    const double rx = __dsub_rn(__dadd_rn(P.x[b], ox), P.x[a]);
+    const double ry = __dsub_rn(__dadd_rn(P.y[b], oy), P.y[a]);
+    const double rz = __dsub_rn(__dadd_rn(P.z[b], oz), P.z[a]);
+    const double ux = __dsub_rn(P.vx[b], P.vx[a]);
+    const double uy = __dsub_rn(__dadd_rn(P.vy[b], dvy), P.vy[a]);
+    const double uz = __dsub_rn(P.vz[b], P.vz[a]);
     const double uu = __dadd_rn(__dadd_rn(__dmul_rn(ux, ux), __dmul_rn(uy, uy)), __dmul_rn(uz, uz));
     const double ru = __dadd_rn(__dadd_rn(__dmul_rn(rx, ux), __dmul_rn(ry, uy)), __dmul_rn(rz, uz));
     double tau = 0.0;
@@ -171,69 +179,177 @@ __device__ __forceinline__ bool line_hit(const SweepRec& a, const SweepRec& b, d
     const double dy = __dadd_rn(ry, __dmul_rn(uy, tau));
     const double dz = __dadd_rn(rz, __dmul_rn(uz, tau));
     const double d2 = __dadd_rn(__dadd_rn(__dmul_rn(dx, dx), __dmul_rn(dy, dy)), __dmul_rn(dz, dz));
-    const double s = __dadd_rn(a.r, b.r);
+    const double s = __dadd_rn(P.r[a], P.r[b]);
     return d2 < __dmul_rn(s, s);
 }
 
+// Pairs found by a warp and not yet recorded.
+struct SweepQueue {
+    int si[64], sj[64];   // slots of the scanning item's particle and of the other one
+    int img[64];          // image of the other as seen from the first: code, bit 12: clear of the threshold
+};
+
+// Records n (<= 32) queued pairs, a lane each, on the canonical orientation
+// (lower id a, image of b); those not clear of the threshold take the exact
+// criterion.
+__device__ __forceinline__ void sweep_record(const SweepArgs& A, const SweepQueue& Q, int from, int n) {
+    const int lane = threadIdx.x & 31;
+    bool hit = false;
+    uint64_t key = 0;
+    if (lane < n) {
+        const int i = Q.si[from + lane], j = Q.sj[from + lane], c = Q.img[from + lane];
+        int gx = (c & 15) - 7, gy = ((c >> 4) & 15) - 7, gz = ((c >> 8) & 15) - 7;
+        const int ii = A.P.id[i], ij = A.P.id[j];
+        const bool flip = ij < ii;
+        if (flip) {
+            gx = -gx;
+            gy = -gy;
+            gz = -gz;
+        }
+        hit = (c >> 12) & 1;
+        if (!hit) {
+            const BoxP bp = A.boxes[A.P.box[i]];
+            const double s = shear_offset(bp, time_of(A.ctl, A.t0, A.half_dt, A.hs));
+            double ox, oy, oz;
+            image_offset(bp, s, gx, gy, gz, ox, oy, oz);
+            hit = line_hit(A.P, flip ? j : i, flip ? i : j, A.h, ox, oy, oz, __dmul_rn(-(double)gx, bp.shear_speed));
+        }
+        key = ((uint64_t)min(ii, ij) << 36) | ((uint64_t)max(ii, ij) << 12) |
+              (uint64_t)((gx + 7) | ((gy + 7) << 4) | ((gz + 7) << 8));
+    }
+    const unsigned hits = __ballot_sync(0xffffffffu, hit);
+    if (!hits) return;
+    int base = 0;
+    if (lane == 0) base = atomicAdd(&A.ctl->pair_count, __popc(hits));
+    base = __shfl_sync(0xffffffffu, base, 0);
+    if (hit) {
+        const int at = base + __popc(hits & ((1u << lane) - 1u));
+        if (at < A.pair_cap) A.pair_key[at] = key;
+        else atomicOr(&A.ctl->err, kErrPairOverflow);
+    }
+}
+
+// One thread per sorted item scans the items that start before its own ends,
+// the lanes of a warp in step.  A candidate's y images within reach are found
+// by division instead of a loop over all, and the criterion is decided in FP32
+// (positions as hi/lo differences) unless the distance lies within the error
+// bound of the threshold; only those few take the FP64 criterion, when the
+// queued pairs are recorded (an FP64 instruction holds the SM's FP64 pipe 16
+// cycles per warp: with every candidate's y extent and criterion in FP64,
+// %%
 __global__ void __launch_bounds__(128) k_sweep_pairs(SweepArgs A, const SweepRec* __restrict__ rec) {
-    const int k = blockIdx.x * blockDim.x + threadIdx.x;
+    __shared__ SweepQueue queue[4];
+    SweepQueue& Q = queue[threadIdx.x >> 5];
+    const int k = blockIdx.x * blockDim.x + threadIdx.x, lane = threadIdx.x & 31;
+    const unsigned lt = (1u << lane) - 1u;
     const int nitem = min(A.ctl->sweep_items, A.item_cap);
-    if (k >= nitem) return;
-    const SweepRec Pk = rec[k];
-    const int ci = (int)(Pk.sc & 7u);
-    const int si = (int)(Pk.sc >> 3);
-    const int b = (int)(A.key[k] >> 32);
+    if (k - lane >= nitem) return;   // the whole warp
+    bool scan = k < nitem;
+    const SweepRec P = rec[scan ? k : nitem - 1];
+    const int ci = (int)(P.sc & 7u);
+    const int si = (int)(P.sc >> 3);
+    const int b = (int)(A.key[scan ? k : nitem - 1] >> 32);
     const BoxP bp = A.boxes[b];
-    const Range g = range_of(A, bp);
-    const double hi = __dadd_rn(__dadd_rn(Pk.x, __dmul_rn((double)ci, g.lx)),
-                                __dadd_rn(__dadd_rn(__dmul_rn(fabs(Pk.vx), A.h), Pk.r), g.m));
-    const uint64_t khi = ((uint64_t)b << 32) | quant(hi, g.base, g.scale);
+    uint64_t khi;
+    {
+        const Range g = range_of(A, bp);
+        const double hi = __dadd_rn(__dadd_rn(A.P.x[si], __dmul_rn((double)ci, g.lx)), __dadd_rn(ext_of(A, si), g.m));
+        khi = ((uint64_t)b << 32) | quant(hi, g.base, g.scale);
+    }
     // more trajectories cut by the plane than the sweep is meant for (the
     // O(N N_SWEEPL) cost of Sect. 5.3 turning quadratic): report, do not scan
     const int lim = k + 1 + kMaxSweepScan;
-    if (lim < nitem && A.key[lim] <= khi) {
+    if (scan && lim < nitem && A.key[lim] <= khi) {
         atomicOr(&A.ctl->err, kErrSweepLong);
-        return;
+        scan = false;
     }
-    const double s = shear_offset(bp, time_of(A.ctl, A.t0, A.half_dt, A.hs));
-    for (int j = k + 1; j < nitem; j++) {
-        if (A.key[j] > khi) break;   // at the latest at lim (keys are sorted)
-        if (((j - k) & 1023) == 0 && (*(volatile const int*)&A.ctl->err & kErrSweepLong)) break;
-        const SweepRec Q = rec[j];
-        const int cj = (int)(Q.sc & 7u);
-        if ((ci != 0 && cj != 0) || (int)(Q.sc >> 3) == si) continue;
-        // image of Q's particle as seen from Pk's, then the canonical orientation
-        int gx = cj - ci;
-        const bool flip = Q.id < Pk.id;
-        if (flip) gx = -gx;
-        const SweepRec ra = flip ? Q : Pk;
-        const SweepRec rbb = flip ? Pk : Q;
-        const double dvy = __dmul_rn(-(double)gx, bp.shear_speed);
-        // y extent of the relative motion: |dy(tau)| <= |dy(0)| + |u_y| h for every image
-        const double uy = fabs(__dsub_rn(__dadd_rn(rbb.vy, dvy), ra.vy));
-        const double ylim = (uy * A.h + (ra.r + rbb.r)) * (1.0 + 1e-12) + g.m;
-        const double dyab = rbb.y - ra.y;
-        const double gxs = __dmul_rn((double)gx, s);
-        for (int gy = -A.ngy; gy <= A.ngy; gy++) {
-            const double dy0 = dyab + (__dmul_rn((double)gy, bp.Ly) - gxs);
-            if (fabs(dy0) > ylim) continue;
-            for (int gz = -A.ngz; gz <= A.ngz; gz++) {
-                double ox, oy, oz;
-                image_offset(bp, s, gx, gy, gz, ox, oy, oz);
-                if (!line_hit(ra, rbb, A.h, ox, oy, oz, dvy)) continue;
-                const int code = (gx + 7) | ((gy + 7) << 4) | ((gz + 7) << 8);
-                // one atomic per group of lanes that hit together
-                cg::coalesced_group grp = cg::coalesced_threads();
-                int slot = 0;
-                if (grp.thread_rank() == 0) slot = atomicAdd(&A.ctl->pair_count, (int)grp.size());
-                slot = grp.shfl(slot, 0) + (int)grp.thread_rank();
-                if (slot < A.pair_cap)
-                    A.pair_key[slot] = ((uint64_t)ra.id << 36) | ((uint64_t)rbb.id << 12) | (uint64_t)code;
-                else
-                    atomicOr(&A.ctl->err, kErrPairOverflow);
+    const double s64 = shear_offset(bp, time_of(A.ctl, A.t0, A.half_dt, A.hs));
+    const float h = (float)A.h, Ly = (float)bp.Ly, iLy = 1.f / Ly, Lz = (float)bp.Lz, iLz = 1.f / Lz;
+    const float speed = (float)bp.shear_speed;
+    // hi/lo positions and offsets are good to 2^-47 of their size
+    const float far = 1e-13f * (fabsf(P.xh) + fabsf(P.yh) + fabsf(P.zh) +
+                                (float)(A.ngx + 1) * (float)bp.Lx + (float)(A.ngy + 1) * Ly + (float)(A.ngz + 1) * Lz);
+    int nq = 0;   // queued pairs (warp-uniform)
+    for (int j = k + 1; ; j++) {
+        scan = scan && j < nitem && A.key[j] <= khi;   // at the latest at lim (keys are sorted)
+        if (((j - k) & 1023) == 0 && (*(volatile const int*)&A.ctl->err & kErrSweepLong)) scan = false;
+        if (!__any_sync(0xffffffffu, scan)) break;
+        SweepRec R;
+        int gx = 0, sj = 0, gy = 1, gy1 = 0, gz0 = 0, gz1 = -1, gz = 0;
+        float rx = 0.f, ry = 0.f, rz = 0.f, ux = 0.f, uy = 0.f, uz = 0.f, sr = 0.f, err = 0.f;
+        if (scan) {
+            R = rec[j];
+            const int cj = (int)(R.sc & 7u);
+            sj = (int)(R.sc >> 3);
+            if ((ci == 0 || cj == 0) && sj != si) {
+                // image of R's particle as seen from P's
+                gx = cj - ci;
+                float oxh = 0.f, oxl = 0.f, oyh = 0.f, oyl = 0.f;
+                if (gx != 0) {
+                    split_hl((double)gx * bp.Lx, oxh, oxl);
+                    split_hl(-((double)gx * s64), oyh, oyl);
+                }
+                rx = ((R.xh - P.xh) + oxh) + ((R.xl - P.xl) + oxl);
+                ry = ((R.yh - P.yh) + oyh) + ((R.yl - P.yl) + oyl);
+                rz = (R.zh - P.zh) + (R.zl - P.zl);
+                ux = R.vx - P.vx;
+                uy = (R.vy - (float)gx * speed) - P.vy;
+                uz = R.vz - P.vz;
+                sr = P.r + R.r;
+                // bound of the FP32 distance's error: differences rounded to
+                // 2^-24, velocities and tau to a few times that
+                const float vel = h * (P.vsum + R.vsum + fabsf((float)gx * speed));
+                err = 1e-6f * (fabsf(rx) + fabsf(oxh) + fabsf(ry) + fabsf(oyh) + fabsf(rz) + vel + sr) + far;
+                // |d| <= sr needs |r_y| <= sr + |u_y| h for an image, and the same in z
+                const float ly = sr + fabsf(uy) * h + 2.f * err, lz = sr + fabsf(uz) * h + 2.f * err;
+                gy = max(-A.ngy, (int)ceilf((-ly - ry) * iLy - 4e-6f));
+                gy1 = min(A.ngy, (int)floorf((ly - ry) * iLy + 4e-6f));
+                gz0 = max(-A.ngz, (int)ceilf((-lz - rz) * iLz - 4e-6f));
+                gz1 = min(A.ngz, (int)floorf((lz - rz) * iLz + 4e-6f));
+                gz = gz0;
+                if (gz0 > gz1) gy = gy1 + 1;
+            }
+        }
+        while (__any_sync(0xffffffffu, gy <= gy1)) {
+            bool near = false, sure = false;
+            int code = 0;
+            if (gy <= gy1) {
+                const float oy = (float)gy * Ly, oz = (float)gz * Lz;
+                const float e = err + 1e-6f * (fabsf(oy) + fabsf(oz));
+                const float y = ry + oy, z = rz + oz;
+                const float uu = fmaf(uz, uz, fmaf(uy, uy, ux * ux));
+                const float ru = fmaf(z, uz, fmaf(y, uy, rx * ux));
+                const float tau = uu > 0.f ? fminf(fmaxf(-ru / uu, -h), h) : 0.f;
+                const float dx = fmaf(ux, tau, rx), dy = fmaf(uy, tau, y), dz = fmaf(uz, tau, z);
+                const float d2 = fmaf(dz, dz, fmaf(dy, dy, dx * dx));
+                const float out = sr + e, in = sr - e;
+                near = !(d2 > out * out);
+                sure = in > 0.f && d2 < in * in;
+                code = (gx + 7) | ((gy + 7) << 4) | ((gz + 7) << 8) | (sure ? 1 << 12 : 0);
+                if (++gz > gz1) {
+                    gz = gz0;
+                    gy++;
+                }
+            }
+            const unsigned m = __ballot_sync(0xffffffffu, near);
+            if (!m) continue;
+            if (near) {
+                const int at = nq + __popc(m & lt);
+                Q.si[at] = si;
+                Q.sj[at] = sj;
+                Q.img[at] = code;
+            }
+            nq += __popc(m);
+            if (nq >= 32) {
+                nq -= 32;
+                __syncwarp();
+                sweep_record(A, Q, nq, 32);
+                __syncwarp();
             }
         }
     }
+    __syncwarp();
+    sweep_record(A, Q, 0, nq);
 }
 
 __global__ void k_sweep_reset(Ctl* ctl) {
