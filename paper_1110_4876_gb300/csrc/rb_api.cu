@@ -647,53 +647,26 @@ int d2h(rb_sim* s, std::vector<T>& v, const T* src, size_t n) {
     return RB_OK;
 }
 
-// (local id, slot) of the live particles of box b in set c, by id.
-int live_slots(rb_sim* s, int c, int b, std::vector<std::pair<int64_t, int>>& out) {
-    std::vector<int32_t> id, bx;
-    if (d2h(s, id, s->P[c].id, s->ncap) || d2h(s, bx, s->P[c].box, s->ncap)) return RB_ERR_CUDA;
-    out.clear();
-    for (int i = 0; i < s->ncap; i++)
-        if (bx[i] == b) out.emplace_back((int64_t)id[i] - s->base[b], i);
-    std::sort(out.begin(), out.end());
-    return RB_OK;
-}
+// An open face (an open box, or the open z of a periodic or shearing box) may
+// have removed ids; otherwise every id of a box is live.
+bool may_lose_ids(const rb_sim* s) { return s->cfg.boundary == RB_BC_OPEN || !s->cfg.z_periodic; }
 
 bool bad_box(rb_sim* s, int box) { return !s || box < 0 || box >= s->nbox; }
 
-// The live particles of a box in id order: the device writes them in id
-// order into the idle particle set, then each requested field is copied
-// straight into the caller's array.  Ids removed by an open boundary leave
-// gaps that are closed on the host.
-int read_box(rb_sim* s, int box, int64_t cap, int64_t* n_out, double* const dst[8], int64_t* id) {
-    const int nb = (int)s->hb[box].n;
-    const PSet& out = s->P[1 - s->cur];
-    int32_t* flags = s->T.start;   // scratch: ncap + 1 ints, free between steps
-    particles_by_id(s->P[s->cur], out, box, (int)s->base[box], s->ncap, flags, nb, &s->ctl->out_live,
-                    s->stream);
-    // an open face (an open box, or the open z of a periodic or shearing box)
-    // may have removed ids; otherwise every id of the box is live
-    const bool may_remove = s->cfg.boundary == RB_BC_OPEN || !s->cfg.z_periodic;
-    bool want = id != nullptr;
-    for (int f = 0; f < 8; f++) want = want || dst[f] != nullptr;
-    int live = nb;
-    if (!want || (may_remove && cap < nb)) {
-        if (may_remove) {
-            if (read_ctl(s)) return RB_ERR_CUDA;
-            live = s->hctl.out_live;
-        }
-        if (n_out) *n_out = live;
-        if (!want) return RB_OK;   // a count query
-    }
-    if (live > cap) return fail(s, RB_ERR_ARG, "capacity too small");
-    const double* src[8] = {out.x, out.y, out.z, out.vx, out.vy, out.vz, out.m, out.r};
+// Copies `nf` fields written per id on the device (8-byte values, flags set
+// for live ids, ctl->out_live the live count) into the caller's arrays of `cap`
+// places, live entries only, in id order.  may_remove: ids may be missing;
+// `live` is the count where it is known already.
+template <typename T>
+int copy_by_id(rb_sim* s, int nb, bool may_remove, int64_t cap, int live, int64_t* n_out, const T* const* src,
+               T* const* dst, int nf, const int32_t* flags, int64_t* id) {
     std::vector<int32_t> fl;
     if (cap >= nb) {
         // every id's entry straight into the caller's arrays; with removals
         // possible, the count read waits for these copies as well
-        for (int f = 0; f < 8; f++)
+        for (int f = 0; f < nf; f++)
             if (dst[f])
-                RB_CUDA(s, cudaMemcpyAsync(dst[f], src[f], sizeof(double) * nb, cudaMemcpyDeviceToHost,
-                                           s->stream));
+                RB_CUDA(s, cudaMemcpyAsync(dst[f], src[f], sizeof(T) * nb, cudaMemcpyDeviceToHost, s->stream));
         if (may_remove) {
             if (read_ctl(s)) return RB_ERR_CUDA;
             live = s->hctl.out_live;
@@ -708,7 +681,7 @@ int read_box(rb_sim* s, int box, int64_t cap, int64_t* n_out, double* const dst[
         }
         // removed ids leave gaps: keep the live entries, in id order
         if (d2h(s, fl, flags, nb)) return RB_ERR_CUDA;
-        for (int f = 0; f < 8; f++) {
+        for (int f = 0; f < nf; f++) {
             if (!dst[f]) continue;
             int64_t k = 0;
             for (int j = 0; j < nb; j++)
@@ -717,8 +690,8 @@ int read_box(rb_sim* s, int box, int64_t cap, int64_t* n_out, double* const dst[
     } else {
         // fewer places than ids: through host buffers
         if (d2h(s, fl, flags, nb)) return RB_ERR_CUDA;
-        std::vector<double> buf;
-        for (int f = 0; f < 8; f++) {
+        std::vector<T> buf;
+        for (int f = 0; f < nf; f++) {
             if (!dst[f]) continue;
             if (d2h(s, buf, src[f], nb)) return RB_ERR_CUDA;
             int64_t k = 0;
@@ -732,6 +705,57 @@ int read_box(rb_sim* s, int box, int64_t cap, int64_t* n_out, double* const dst[
             if (fl[j]) id[k++] = j;
     }
     return RB_OK;
+}
+
+// The live particles of a box in id order: the device writes them in id
+// order into the idle particle set, then each requested field is copied
+// straight into the caller's array.  Ids removed by an open boundary leave
+// gaps that are closed on the host.
+int read_box(rb_sim* s, int box, int64_t cap, int64_t* n_out, double* const dst[8], int64_t* id) {
+    const int nb = (int)s->hb[box].n;
+    const PSet& out = s->P[1 - s->cur];
+    int32_t* flags = s->T.start;   // scratch: ncap + 1 ints, free between steps
+    particles_by_id(s->P[s->cur], out, box, (int)s->base[box], s->ncap, flags, nb, &s->ctl->out_live,
+                    s->stream);
+    const bool may_remove = may_lose_ids(s);
+    bool want = id != nullptr;
+    for (int f = 0; f < 8; f++) want = want || dst[f] != nullptr;
+    int live = nb;
+    if (!want || (may_remove && cap < nb)) {
+        if (may_remove) {
+            if (read_ctl(s)) return RB_ERR_CUDA;
+            live = s->hctl.out_live;
+        }
+        if (n_out) *n_out = live;
+        if (!want) return RB_OK;   // a count query
+    }
+    if (live > cap) return fail(s, RB_ERR_ARG, "capacity too small");
+    const double* src[8] = {out.x, out.y, out.z, out.vx, out.vy, out.vz, out.m, out.r};
+    return copy_by_id(s, nb, may_remove, cap, live, n_out, src, dst, 8, flags, id);
+}
+
+// Results of the last walk, per sorted slot, in id order: written by id on the
+// device into the scratch of the collision boxes, then copied like particles.
+template <typename T, typename V>
+int walk_results(rb_sim* s, int box, int64_t cap, const V* const src[3], T* const dst[3]) {
+    if (bad_box(s, box)) return fail(s, RB_ERR_ARG, "bad box");
+    if (s->acc_set < 0) return fail(s, RB_ERR_STATE, "no gravity walk yet");
+    // the box as it was uploaded (new particles may be staged already)
+    const int nb = (int)((box + 1 < s->nbox ? s->base[box + 1] : s->ntot) - s->base[box]);
+    T* out = reinterpret_cast<T*>(s->T.pbox);   // room for four 8-byte values per slot
+    const T* const by_id[3] = {out, out + s->ncap, out + 2 * (size_t)s->ncap};
+    int32_t* flags = s->T.start;   // scratch: ncap + 1 ints, free between steps
+    results_by_id(s->P[s->acc_set], src, out, box, (int)s->base[box], s->ncap, flags, nb, &s->ctl->out_live, s->stream);
+    const bool may_remove = may_lose_ids(s);
+    int live = nb;
+    if (cap < nb) {
+        if (may_remove) {
+            if (read_ctl(s)) return RB_ERR_CUDA;
+            live = s->hctl.out_live;
+        }
+        if (live > cap) return fail(s, RB_ERR_ARG, "capacity too small");
+    }
+    return copy_by_id(s, nb, may_remove, cap, live, (int64_t*)nullptr, by_id, dst, 3, flags, (int64_t*)nullptr);
 }
 
 // The current particles of every box back into the host copies, before
@@ -956,37 +980,17 @@ int rb_compute_gravity(rb_sim* s) {
 }
 
 int rb_get_accelerations(rb_sim* s, int box, int64_t cap, double* ax, double* ay, double* az) {
-    if (bad_box(s, box)) return fail(s, RB_ERR_ARG, "bad box");
-    if (s->acc_set < 0) return fail(s, RB_ERR_STATE, "no gravity walk yet");
-    std::vector<std::pair<int64_t, int>> sl;
-    if (live_slots(s, s->acc_set, box, sl)) return RB_ERR_CUDA;
-    if ((int64_t)sl.size() > cap) return fail(s, RB_ERR_ARG, "capacity too small");
-    const double* src[3] = {s->acc_x, s->acc_y, s->acc_z};
-    double* dst[3] = {ax, ay, az};
-    std::vector<double> buf;
-    for (int f = 0; f < 3; f++) {
-        if (!dst[f]) continue;
-        if (d2h(s, buf, src[f], s->ncap)) return RB_ERR_CUDA;
-        for (size_t k = 0; k < sl.size(); k++) dst[f][k] = buf[sl[k].second];
-    }
-    return RB_OK;
+    if (!s) return fail(s, RB_ERR_ARG, "bad box");
+    const double* const src[3] = {s->acc_x, s->acc_y, s->acc_z};
+    double* const dst[3] = {ax, ay, az};
+    return walk_results<double, double>(s, box, cap, src, dst);
 }
 
 int rb_get_counts(rb_sim* s, int box, int64_t cap, int64_t* ncell, int64_t* nleaf, int64_t* nmac) {
-    if (bad_box(s, box)) return fail(s, RB_ERR_ARG, "bad box");
-    if (s->acc_set < 0) return fail(s, RB_ERR_STATE, "no gravity walk yet");
-    std::vector<std::pair<int64_t, int>> sl;
-    if (live_slots(s, s->acc_set, box, sl)) return RB_ERR_CUDA;
-    if ((int64_t)sl.size() > cap) return fail(s, RB_ERR_ARG, "capacity too small");
-    const int32_t* src[3] = {s->cnt_cell, s->cnt_leaf, s->cnt_mac};
-    int64_t* dst[3] = {ncell, nleaf, nmac};
-    std::vector<int32_t> buf;
-    for (int f = 0; f < 3; f++) {
-        if (!dst[f]) continue;
-        if (d2h(s, buf, src[f], s->ncap)) return RB_ERR_CUDA;
-        for (size_t k = 0; k < sl.size(); k++) dst[f][k] = buf[sl[k].second];
-    }
-    return RB_OK;
+    if (!s) return fail(s, RB_ERR_ARG, "bad box");
+    const int32_t* const src[3] = {s->cnt_cell, s->cnt_leaf, s->cnt_mac};
+    int64_t* const dst[3] = {ncell, nleaf, nmac};
+    return walk_results<int64_t, int32_t>(s, box, cap, src, dst);
 }
 
 int rb_get_tree(rb_sim* s, int box, int64_t cap, int64_t* ncell, int32_t* depth, int64_t* count,

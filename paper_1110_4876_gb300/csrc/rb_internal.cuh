@@ -347,6 +347,11 @@ void step_advance(Ctl* ctl, cudaStream_t s);
 // the live count), and the slot layout of a freshly copied single box.
 void particles_by_id(const PSet& P, const PSet& out, int box, int base, int ncap, int32_t* flags,
                      int nflags, int* count, cudaStream_t s);
+// The same for three values per slot (accelerations; counts as 64-bit): value v
+// of id k at out[v * ncap + k].
+template <typename T, typename V>
+void results_by_id(const PSet& P, const V* const src[3], T* out, int box, int base, int ncap, int32_t* flags,
+                   int nflags, int* count, cudaStream_t s);
 void reset_slots(const PSet& P, int32_t* slot_of_id, int n, int ncap, int nbox, cudaStream_t s);
 // out2[0]: bit 0 non-finite state, bit 1 negative mass or radius; out2[1]:
 // the largest radius (double bits).  Particles [0, n) of P.

@@ -574,6 +574,38 @@ void particles_by_id(const PSet& P, const PSet& out, int box, int base, int ncap
     if (ncap > 0) k_by_id<<<ceil_div(ncap, 256), 256, 0, s>>>(P, out, box, base, ncap, flags, count);
 }
 
+// Three values per slot of one box's live particles, by id, as 8-byte values.
+template <typename T, typename V>
+__global__ void __launch_bounds__(256) k_results_by_id(PSet P, const V* __restrict__ a, const V* __restrict__ b,
+                                                       const V* __restrict__ c, T* __restrict__ out, int box, int base,
+                                                       int ncap, int32_t* __restrict__ flags, int* __restrict__ count) {
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    const bool mine = i < ncap && P.box[i] == box;
+    if (mine) {
+        const int k = P.id[i] - base;
+        out[k] = (T)a[i];
+        out[ncap + k] = (T)b[i];
+        out[2 * (size_t)ncap + k] = (T)c[i];
+        flags[k] = 1;
+    }
+    const unsigned m = __ballot_sync(0xffffffffu, mine);
+    if ((threadIdx.x & 31) == 0 && m) atomicAdd(count, __popc(m));
+}
+
+template <typename T, typename V>
+void results_by_id(const PSet& P, const V* const src[3], T* out, int box, int base, int ncap, int32_t* flags, int nflags,
+                   int* count, cudaStream_t s) {
+    cudaMemsetAsync(flags, 0, sizeof(int32_t) * (size_t)(nflags > 0 ? nflags : 1), s);
+    cudaMemsetAsync(count, 0, sizeof(int), s);
+    if (ncap > 0)
+        k_results_by_id<T, V><<<ceil_div(ncap, 256), 256, 0, s>>>(P, src[0], src[1], src[2], out, box, base, ncap, flags,
+                                                                  count);
+}
+template void results_by_id<double, double>(const PSet&, const double* const[3], double*, int, int, int, int32_t*, int,
+                                            int*, cudaStream_t);
+template void results_by_id<int64_t, int32_t>(const PSet&, const int32_t* const[3], int64_t*, int, int, int, int32_t*,
+                                              int, int*, cudaStream_t);
+
 void reset_slots(const PSet& P, int32_t* slot_of_id, int n, int ncap, int nbox, cudaStream_t s) {
     if (ncap > 0) k_reset_slots<<<ceil_div(ncap, 256), 256, 0, s>>>(P, slot_of_id, n, ncap, nbox);
 }
