@@ -229,7 +229,9 @@ int alloc_pairs(rb_sim* s, int cap) {
     rc |= dalloc(s, &R.claim, 1, L);
     rc |= dalloc(s, &R.hist, radix_hist_words(cap), L);
     R.slot_of_id = keep_slot;
-    return rc ? RB_ERR_CUDA : RB_OK;
+    if (rc) return RB_ERR_CUDA;
+    RB_CUDA(s, cudaMemsetAsync(R.hist, 0, sizeof(uint32_t) * radix_hist_words(cap), s->stream));
+    return RB_OK;
 }
 
 // Allocate for capacity n and upload the staged boxes.
@@ -268,7 +270,8 @@ int upload(rb_sim* s) {
         rc |= dalloc(s, &T.idx, cap, L); rc |= dalloc(s, &T.idx_alt, cap, L);
         rc |= dalloc(s, &T.sbox, cap, L);
         rc |= dalloc(s, &T.hist, radix_hist_words(cap), L);
-        rc |= dalloc(s, &T.scan_part, scan_part_words(cap), L);
+        rc |= dalloc(s, &T.thist, radix_hist_words(cap), L);
+        rc |= dalloc(s, &T.scan_stat, entry_scan_words(cap), L);
         rc |= dalloc(s, &T.mask, cap, L);
         rc |= dalloc(s, &T.start, cap + 1, L);
         rc |= dalloc(s, &T.node_a, cap, L); rc |= dalloc(s, &T.node_b, cap, L);
@@ -291,7 +294,6 @@ int upload(rb_sim* s) {
         }
         rc |= dalloc(s, &T.d_a, erec, L); rc |= dalloc(s, &T.d_q0, erec, L);
         rc |= dalloc(s, &T.d_q1, erec, L); rc |= dalloc(s, &T.d_c, ecap, L);
-        rc |= dalloc(s, &T.box_first, s->nbox + 1, L);
         rc |= dalloc(s, &T.box_root, s->nbox + 1, L);
         rc |= dalloc(s, &T.span, moment_span_words(cap), L);
         rc |= dalloc(s, &T.tq, kMaxTileQueues * kTileQStride, L);
@@ -319,6 +321,8 @@ int upload(rb_sim* s) {
             s->SW.cap = ic;
         }
         if (rc) return RB_ERR_CUDA;
+        RB_CUDA(s, cudaMemsetAsync(T.hist, 0, sizeof(uint32_t) * radix_hist_words(cap), s->stream));
+        RB_CUDA(s, cudaMemsetAsync(s->ctl, 0, sizeof(Ctl), s->stream));
         s->ncap = cap;
         // a freshly drawn dense sheet overlaps about one pair per particle
         if (alloc_pairs(s, 2 * cap + 4096) != RB_OK) return RB_ERR_CUDA;
@@ -418,14 +422,12 @@ void mark(rb_sim* s, int k) {
 // that holds the particles afterwards.
 int record_step(rb_sim* s, int p) {
     cudaStream_t st = s->stream;
-    cudaMemsetAsync(&s->ctl->pair_count, 0, sizeof(int), st);
-    cudaMemsetAsync(&s->ctl->err, 0, sizeof(int), st);
-    clear_walk_stats(s->ctl, st);
+    clear_step(s->ctl, st);
     int c = p;
     mark(s, 0);
     if (s->cfg.gravity) {
         drift_keys(s->P[c], s->T, s->ctl, s->d_boxes, s->C, s->ncap, 1, 1, nullptr, nullptr, nullptr,
-                   false, st);
+                   false, true, st);
         mark(s, 1);
         sort_and_permute(s->P[c], s->P[1 - c], s->T, s->PR, s->ctl, s->C, s->ncap, s->box_bits, st);
         c = 1 - c;
@@ -444,7 +446,6 @@ int record_step(rb_sim* s, int p) {
         if (s->cfg.walk == RB_WALK_FP32_LEARNED) {
             // walk at theta; accepted cells with w/R > theta_fb get the
             // network's residual inside the walk
-            cudaMemsetAsync(&s->ctl->req_count, 0, sizeof(int), st);
             const WalkLearn L = learn_args(s);
             gravity_walk(s->T, s->P[c], s->ctl, s->d_boxes, s->C, RB_WALK_FP32, 1, walk_out(s), false,
                          true, st, nullptr, s->walk_block, &L);
@@ -454,26 +455,24 @@ int record_step(rb_sim* s, int p) {
         }
         mark(s, 5);
         drift_keys(s->P[c], s->T, s->ctl, s->d_boxes, s->C, s->ncap, 1, 2, s->acc_x, s->acc_y,
-                   s->acc_z, true, st);
+                   s->acc_z, true, false, st);
     } else {
         drift_keys(s->P[c], s->T, s->ctl, s->d_boxes, s->C, s->ncap, 2, 1, nullptr, nullptr, nullptr,
-                   false, st);
+                   false, s->cfg.collisions == RB_COLL_TREE, st);
         for (int k = 1; k <= 5; k++) mark(s, k);
     }
     mark(s, 6);
     if (s->cfg.collisions == RB_COLL_SWEEP) {
         // plane sweep on the particles where they are: no collision tree
-        discard_live_count(s->ctl, st);
         for (int k = 7; k <= 9; k++) mark(s, k);
         sweep_search(s->P[c], s->ctl, s->d_boxes, s->C, s->SW, s->PR, 2, s->ncap, st);
         mark(s, 10);
         sort_pairs(s->PR, s->ctl, st, pair_key_bits(s));
         mark(s, 11);
-        resolve_pairs(s->P[c], s->ctl, s->d_boxes, s->C, s->PR, 2, s->T.img, st);
+        resolve_pairs(s->P[c], s->ctl, s->d_boxes, s->C, s->PR, 2, s->T.img, false, true, st);
     } else if (s->cfg.collisions && s->cfg.gravity) {
         // the gravity tree still holds the same particles: boxes of their
         // current positions replace a second sort and build
-        discard_live_count(s->ctl, st);
         mark(s, 7);
         mark(s, 8);
         build_collision_aabb(s->T, s->P[c], s->ctl, s->C, st);
@@ -483,7 +482,7 @@ int record_step(rb_sim* s, int p) {
         mark(s, 10);
         sort_pairs(s->PR, s->ctl, st, pair_key_bits(s));
         mark(s, 11);
-        resolve_pairs(s->P[c], s->ctl, s->d_boxes, s->C, s->PR, 2, s->T.img, st);
+        resolve_pairs(s->P[c], s->ctl, s->d_boxes, s->C, s->PR, 2, s->T.img, true, true, st);
     } else if (s->cfg.collisions) {
         sort_and_permute(s->P[c], s->P[1 - c], s->T, s->PR, s->ctl, s->C, s->ncap, s->box_bits, st);
         c = 1 - c;
@@ -497,13 +496,12 @@ int record_step(rb_sim* s, int p) {
         mark(s, 10);
         sort_pairs(s->PR, s->ctl, st, pair_key_bits(s));
         mark(s, 11);
-        resolve_pairs(s->P[c], s->ctl, s->d_boxes, s->C, s->PR, 2, s->T.img, st);
+        resolve_pairs(s->P[c], s->ctl, s->d_boxes, s->C, s->PR, 2, s->T.img, true, true, st);
     } else {
-        discard_live_count(s->ctl, st);   // no sort follows the last drift
         for (int k = 7; k <= 11; k++) mark(s, k);
     }
     mark(s, 12);
-    step_advance(s->ctl, st);
+    if (!s->cfg.collisions) step_advance(s->ctl, st);   // else with the resolution
     return c;
 }
 
@@ -575,7 +573,8 @@ int collide_with_retry(rb_sim* s, int c, int hs, bool resolve) {
             return fail(s, RB_ERR_TIMEOUT, "radix sort: a bounded look-back wait gave up");
         if (s->hctl.pair_count <= s->PR.cap) {
             if (resolve) {
-                resolve_pairs(s->P[c], s->ctl, s->d_boxes, s->C, s->PR, hs, s->T.img, s->stream);
+                resolve_pairs(s->P[c], s->ctl, s->d_boxes, s->C, s->PR, hs, s->T.img,
+                              s->cfg.collisions != RB_COLL_SWEEP, false, s->stream);
                 if (read_ctl(s)) return RB_ERR_CUDA;
                 if (s->hctl.err & kErrResolveStall)
                     return fail(s, RB_ERR_TIMEOUT,
@@ -603,7 +602,7 @@ int ensure_ready(rb_sim* s) {
 int rebuild_now(rb_sim* s) {
     const int c = s->cur;
     drift_keys(s->P[c], s->T, s->ctl, s->d_boxes, s->C, s->ncap, 0, 0, nullptr, nullptr, nullptr,
-               false, s->stream);
+               false, true, s->stream);
     sort_and_permute(s->P[c], s->P[1 - c], s->T, s->PR, s->ctl, s->C, s->ncap, s->box_bits, s->stream);
     s->cur = 1 - c;
     build_topology(s->T, s->P[s->cur], s->ctl, s->d_boxes, s->C, s->stream);

@@ -64,18 +64,21 @@ struct Ctl {
     int n_live;                // live particles after the last sort
     int n_live_next;           // live particles counted by the keys kernel
     int n_entries;             // tree entries (cells + leaves) of the last build
-    int pair_count;            // pairs found by the last search (may exceed capacity)
     int pair_n;                // pairs to resolve (0 when the search overflowed)
     int resolved;              // pairs that were approaching and were resolved
-    int err;                   // error bits (kErr*)
-    int req_count;             // learned-correction requests recorded by the last walk
     int sweep_items;           // plane sweep: trajectory extents of the last search
     int out_live;              // host exchange: live particles of the box read out
     int pad_;
+    // cleared at the start of every step (clear_step)
+    int pair_count;            // pairs found by the last search (may exceed capacity)
+    int err;                   // error bits (kErr*)
+    int req_count;             // learned walk: cells corrected by the last walk
+    int pad2_;
     unsigned long long n_cell, n_leaf, n_mac, n_recheck;
     unsigned long long n_iter;        // warp iterations of the last FP32 walk (entries visited)
     unsigned long long n_visit;       // tree entries tested by the targets of the last collision search
     unsigned long long n_siter;       // warp iterations of the last collision search
+    // (end of what clear_step clears)
     unsigned long long sweep_wbits;   // plane sweep: largest half extent (double bits)
 };
 constexpr int kErrNonFinite = 1;
@@ -113,7 +116,7 @@ struct Tree {
     uint32_t *idx, *idx_alt;    // sort values: slot in the unsorted set
     int32_t* sbox;              // box digit per unsorted slot (nbox for removed)
     uint32_t* hist;             // radix sort block histograms
-    int32_t* scan_part;         // block partials of the entry scan
+    uint32_t* scan_stat;        // status words of the entry scan, one per tile
     uint32_t* mask;             // per particle: levels of cells starting there
     int32_t* start;             // per particle: first entry starting there (n + 1)
     int32_t *node_a, *node_b;   // per split: first particle of its cell (last: reps only)
@@ -133,7 +136,7 @@ struct Tree {
     Rec4 rc_hi, rc_lo;              // FP32 cell corner (hi/lo) + width, inside test
     float4* pbox;                   // collision boxes of slots and slot runs (box_items(cap_n) pairs)
     double4_32a *d_a, *d_q0, *d_q1, *d_c;  // FP64 walk records (d_c: cell corner + width)
-    int32_t *box_first, *box_root;  // per box, nbox + 1 each (box_root[nbox] = -1: removed particles)
+    int32_t* box_root;              // per box: root entry, -1 if empty (box_root[nbox] = -1: removed particles)
     int32_t* span;                  // moments: cells that go on past their range (moment_span_words)
     ImgTab* img;                    // [box][image] offsets of the current walk or search (nbox + 1 rows)
     int32_t* tq;                    // tile queues of the walks (kTileQStride ints each)
@@ -144,6 +147,7 @@ struct Tree {
     // sorted by a Hilbert key (built by build_tile_order for each tree).
     uint64_t *tkey, *tkey_alt;
     uint32_t *tval, *tval_alt;
+    uint32_t* thist;
     const uint32_t* order = nullptr;
 };
 
@@ -235,16 +239,17 @@ int radix_sort_passes(int key_bits, bool box_pass, int box_bits);
 // *err (device memory).
 // low_bit > 0: key bits [low_bit, key_bits) by passes, the bits below it
 // within each run of keys that agree above, once the runs are together; for
-// keys whose runs are short (any length gives the same order).
+// keys whose runs are short (any length gives the same order).  hist has to be
+// zero before such a sort and is left so.
+// pairs: the sort of the collision pairs also sets their number, pair_n, from
+// pair_count (0 when the search overflowed: it resolves nothing, and the host
+// grows the buffer and searches again on the unchanged state).
 int radix_sort(uint64_t* k0, uint32_t* v0, uint64_t* k1, uint32_t* v1, int ncap, const int* d_n,
                int key_bits, const int32_t* box_digits, int box_bits, uint32_t* hist, int* err,
-               cudaStream_t s, int low_bit = 0);
+               cudaStream_t s, int low_bit = 0, Ctl* pairs = nullptr);
 size_t radix_hist_words(int ncap);
-void exclusive_scan_i32(int32_t* data, int n_cap, const int* d_n, int32_t* part, int32_t* total,
-                        cudaStream_t s);
-size_t scan_part_words(int ncap);
-
 // rb_tree.cu
+size_t entry_scan_words(int ncap);
 void build_topology(const Tree& T, const PSet& P, Ctl* ctl, const BoxP* boxes, const SimC& C,
                     cudaStream_t s);
 // Tile order of the current tree (T.key sorted, P its particles): mode
@@ -329,11 +334,11 @@ void sweep_search(const PSet& P, Ctl* ctl, const BoxP* boxes, const SimC& C, Swe
 // rb_step.cu
 void drift_keys(const PSet& P, const Tree& T, Ctl* ctl, const BoxP* boxes, const SimC& C,
                 int ncap, int ndrift, int half_step_offset, const double* ax, const double* ay,
-                const double* az, bool kick, cudaStream_t s);
+                const double* az, bool kick, bool keys, cudaStream_t s);
 void sort_and_permute(const PSet& src, const PSet& dst, Tree& T, Pairs& PR, Ctl* ctl,
                       const SimC& C, int ncap, int box_bits, cudaStream_t s);
 void resolve_pairs(const PSet& P, Ctl* ctl, const BoxP* boxes, const SimC& C, Pairs& PR,
-                   int half_step_offset, ImgTab* img, cudaStream_t s);
+                   int half_step_offset, ImgTab* img, bool have_img, bool advance, cudaStream_t s);
 // Queries the resident blocks of the resolution queue once (outside any
 // stream capture).
 void resolve_prepare(int nsm);
@@ -356,9 +361,6 @@ void reset_slots(const PSet& P, int32_t* slot_of_id, int n, int ncap, int nbox, 
 // out2[0]: bit 0 non-finite state, bit 1 negative mass or radius; out2[1]:
 // the largest radius (double bits).  Particles [0, n) of P.
 void check_particles(const PSet& P, int n, unsigned long long* out2, cudaStream_t s);
-// The live count the keys kernel accumulated, dropped when no sort follows
-// (the particles keep their slots; removed ones stay flagged).
-void discard_live_count(Ctl* ctl, cudaStream_t s);
 
 // rb_api.cu: message returned by rb_last_error(NULL) on this thread.
 void set_global_error(const std::string& msg);
@@ -395,6 +397,7 @@ cudaError_t grad_f32_async(const float* w, const float* X, const float* Y, int n
 void to_bf16_async(const float* w, void* wbf, cudaStream_t s);
 void label_async(const ReqArgs& A, float* X, float* Y, int64_t* meta, int max_req, cudaStream_t s);
 }  // namespace mlp
+void clear_step(Ctl* ctl, cudaStream_t s);
 void clear_walk_stats(Ctl* ctl, cudaStream_t s);
 void clear_search_stats(Ctl* ctl, cudaStream_t s);
 

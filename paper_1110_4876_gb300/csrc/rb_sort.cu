@@ -1,5 +1,5 @@
-// rb_sort.cu -- stable LSD radix sort of (64-bit key, 32-bit value) pairs and
-// an exclusive scan of int32 arrays, both sized on the device.
+// rb_sort.cu -- stable LSD radix sort of (64-bit key, 32-bit value) pairs,
+// sized on the device.
 //
 // The sort replaces the insertion/reconstruction of the paper's tree
 // (Sect. 4.2): particles are put in Morton order so that every cell is a
@@ -18,7 +18,6 @@ constexpr int kThreads = 256;
 constexpr int kItems = 8;
 constexpr int kTile = kThreads * kItems;   // 2048 keys per block
 constexpr int kBins = 256;
-constexpr int kScanThreads = 1024;
 
 __device__ __forceinline__ int read_n(const int* d_n, int ncap) {
     if (!d_n) return ncap;
@@ -34,6 +33,7 @@ constexpr uint32_t kFlagAgg = 1u << 30;
 constexpr uint32_t kFlagPre = 2u << 30;
 constexpr uint32_t kCountMask = (1u << 30) - 1u;
 constexpr int kMaxPasses = 12;   // 64-bit keys: 8 digits; 32-bit box digits: 4
+constexpr int kLongCount = (kMaxPasses - 1) * kBins;   // word of hist that counts long runs (no pass's total)
 constexpr int kLook = 16;   // predecessors read per look-back step
 constexpr unsigned long long kLookLimitNs = 500000000ull;   // half a second
 
@@ -71,12 +71,24 @@ __global__ void __launch_bounds__(kThreads) k_rs_hist(const uint64_t* __restrict
                                                       const int* d_n, int ncap, int low_bit,
                                                       int passes_key, int passes_box,
                                                       uint32_t* __restrict__ hist,
-                                                      uint32_t* __restrict__ status, int tiles_cap) {
+                                                      uint32_t* __restrict__ status, int tiles_cap,
+                                                      Ctl* pairs) {
     __shared__ uint32_t h[kMaxPasses][kBins];
     const int P = passes_key + passes_box;
     for (int i = threadIdx.x; i < P * kBins; i += kThreads) (&h[0][0])[i] = 0;
     __syncthreads();
-    const int n = read_n(d_n, ncap);
+    int n;
+    if (pairs) {
+        const int c = pairs->pair_count;
+        n = c <= ncap ? c : 0;
+        if (blockIdx.x == 0 && threadIdx.x == 0) {
+            pairs->pair_n = n;
+            pairs->resolved = 0;
+        }
+    } else {
+        n = read_n(d_n, ncap);
+    }
+    if (low_bit > 0 && blockIdx.x == 0 && threadIdx.x == 0) hist[kLongCount] = 0u;
     const int nt = (n + kTile - 1) / kTile;
     const size_t rows = (size_t)nt * kBins;
     const size_t stride = (size_t)gridDim.x * kThreads;
@@ -120,45 +132,6 @@ __global__ void __launch_bounds__(kThreads) k_rs_hist(const uint64_t* __restrict
         const uint32_t c = (&h[0][0])[i];
         if (c) atomicAdd(&hist[i], c);
     }
-}
-
-// Exclusive scan of `total` words in place by one block; the sum of all
-// words goes to *sum when sum is non-null.
-template <typename T>
-__global__ void __launch_bounds__(kScanThreads) k_scan_block(T* __restrict__ a, int total,
-                                                             T* __restrict__ sum) {
-    __shared__ T warp_sums[kScanThreads / 32];
-    const int per = (total + kScanThreads - 1) / kScanThreads;
-    const int b = threadIdx.x * per;
-    const int e = min(b + per, total);
-    T s = 0;
-    for (int i = b; i < e; i++) s += a[i];
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    T v = s;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        T t = __shfl_up_sync(0xffffffffu, v, o);
-        if (lane >= o) v += t;
-    }
-    if (lane == 31) warp_sums[w] = v;
-    __syncthreads();
-    if (w == 0) {
-        T x = warp_sums[lane];
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            T t = __shfl_up_sync(0xffffffffu, x, o);
-            if (lane >= o) x += t;
-        }
-        warp_sums[lane] = x;
-    }
-    __syncthreads();
-    T run = v - s + (w > 0 ? warp_sums[w - 1] : T(0));
-    for (int i = b; i < e; i++) {
-        T c = a[i];
-        a[i] = run;
-        run += c;
-    }
-    if (sum && threadIdx.x == kScanThreads - 1) *sum = run;
 }
 
 // One digit pass, one launch: block b takes tile b (2048 keys).  It ranks
@@ -366,10 +339,12 @@ __device__ __forceinline__ bool same_run(const uint64_t* key, const uint32_t* va
 // ones (removed particles) are equal and stay as they are.
 __global__ void __launch_bounds__(256) k_rs_runs(uint64_t* __restrict__ key, uint32_t* __restrict__ val,
                                                  const int32_t* __restrict__ box, const int* d_n, int ncap,
-                                                 int low_bit, uint32_t* __restrict__ nlong,
+                                                 int low_bit, uint32_t* __restrict__ hist,
                                                  uint32_t* __restrict__ list) {
     const int n = read_n(d_n, ncap);
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    // the digit totals are done with: zero for the next sort
+    for (int k = i; k < kLongCount; k += gridDim.x * blockDim.x) hist[k] = 0u;
     bool many = false;
     if (i + 1 < n && key[i] != ~0ull && same_run(key, val, box, low_bit, i, i + 1) &&
         (i == 0 || !same_run(key, val, box, low_bit, i - 1, i))) {
@@ -391,7 +366,7 @@ __global__ void __launch_bounds__(256) k_rs_runs(uint64_t* __restrict__ key, uin
             }
         }
     }
-    if (many) list[atomicAdd(nlong, 1u)] = (uint32_t)i;
+    if (many) list[atomicAdd(&hist[kLongCount], 1u)] = (uint32_t)i;
 }
 
 // The listed runs, a block each: nothing to do if in order already (equal
@@ -501,70 +476,6 @@ __global__ void __launch_bounds__(kThreads) k_rs_long(uint64_t* __restrict__ k0,
     }
 }
 
-// ---- int32 exclusive scan (3 phases) ----
-constexpr int kScanTile = 2048;   // 256 threads x 8
-
-__global__ void __launch_bounds__(256) k_scan_reduce(const int32_t* __restrict__ a, int ncap,
-                                                     const int* d_n, int32_t* __restrict__ part) {
-    const int n = d_n ? min(*d_n, ncap) : ncap;
-    const int base = blockIdx.x * kScanTile;
-    int s = 0;
-#pragma unroll
-    for (int r = 0; r < 8; r++) {
-        int i = base + r * 256 + threadIdx.x;
-        if (i < n) s += a[i];
-    }
-    __shared__ int ws[8];
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
-    if ((threadIdx.x & 31) == 0) ws[threadIdx.x >> 5] = s;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        int t = 0;
-        for (int w = 0; w < 8; w++) t += ws[w];
-        part[blockIdx.x] = t;
-    }
-}
-
-// Block scan of a 2048-element tile plus the tile's offset; a[n] = total.
-__global__ void __launch_bounds__(256) k_scan_down(int32_t* __restrict__ a, int ncap,
-                                                   const int* d_n,
-                                                   const int32_t* __restrict__ part,
-                                                   const int32_t* __restrict__ total) {
-    const int n = d_n ? min(*d_n, ncap) : ncap;
-    const int base = blockIdx.x * kScanTile;
-    if (base > n) return;
-    const int t0 = base + threadIdx.x * 8;
-    int v[8];
-    int s = 0;
-#pragma unroll
-    for (int r = 0; r < 8; r++) {
-        int i = t0 + r;
-        v[r] = i < n ? a[i] : 0;
-        s += v[r];
-    }
-    __shared__ int ws[8];
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    int x = s;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        int t = __shfl_up_sync(0xffffffffu, x, o);
-        if (lane >= o) x += t;
-    }
-    if (lane == 31) ws[w] = x;
-    __syncthreads();
-    int wo = 0;
-    for (int q = 0; q < w; q++) wo += ws[q];
-    int run = part[blockIdx.x] + wo + x - s;
-#pragma unroll
-    for (int r = 0; r < 8; r++) {
-        int i = t0 + r;
-        if (i < n) a[i] = run;
-        if (i == n) a[i] = *total;
-        run += v[r];
-    }
-}
-
 }  // namespace
 
 // Digit totals of every pass, then two banks of per-tile status words.
@@ -573,30 +484,28 @@ size_t radix_hist_words(int ncap) {
            2 * (size_t)kBins * (size_t)ceil_div(ncap > 0 ? ncap : 1, kTile);
 }
 
-size_t scan_part_words(int ncap) { return (size_t)ceil_div((long long)ncap + 1, kScanTile) + 1; }
-
 int radix_sort_passes(int key_bits, bool box_pass, int box_bits) {
     return ceil_div(key_bits, 8) + (box_pass ? ceil_div(box_bits, 8) : 0);
 }
 
 int radix_sort(uint64_t* k0, uint32_t* v0, uint64_t* k1, uint32_t* v1, int ncap, const int* d_n,
                int key_bits, const int32_t* box_digits, int box_bits, uint32_t* hist, int* err,
-               cudaStream_t s, int low_bit) {
+               cudaStream_t s, int low_bit, Ctl* pairs) {
     if (ncap <= 0) return 0;
     const int tiles_cap = ceil_div(ncap, kTile);
     uint32_t* status = hist + kMaxPasses * kBins;
     const int passes_key = ceil_div(key_bits - low_bit, 8);
     const int passes_box = box_digits ? ceil_div(box_bits, 8) : 0;
-    // digit totals start at zero; the status banks are cleared by the
-    // kernels, for the tiles in use only
-    cudaMemsetAsync(hist, 0, sizeof(uint32_t) * kMaxPasses * kBins, s);
+    // digit totals start at zero (k_rs_runs leaves them so); the status banks
+    // are cleared by the kernels, for the tiles in use only
+    if (low_bit == 0) cudaMemsetAsync(hist, 0, sizeof(uint32_t) * kMaxPasses * kBins, s);
     const int hgrid = std::max(1, std::min(ceil_div(ncap, 8 * kThreads), 1024));
     if (box_digits)
         k_rs_hist<true><<<hgrid, kThreads, 0, s>>>(k0, v0, box_digits, d_n, ncap, low_bit,
-                                                   passes_key, passes_box, hist, status, tiles_cap);
+                                                   passes_key, passes_box, hist, status, tiles_cap, pairs);
     else
         k_rs_hist<false><<<hgrid, kThreads, 0, s>>>(k0, v0, nullptr, d_n, ncap, low_bit, passes_key, 0, hist,
-                                                    status, tiles_cap);
+                                                    status, tiles_cap, pairs);
     int cur = 0;
     uint64_t* K[2] = {k0, k1};
     uint32_t* V[2] = {v0, v1};
@@ -615,22 +524,13 @@ int radix_sort(uint64_t* k0, uint32_t* v0, uint64_t* k1, uint32_t* v1, int ncap,
     }
     if (low_bit > 0) {
         // the list of long runs takes the status words, which the passes are
-        // done with (at most one run per kShortRun + 1 keys); its length, the
-        // first word of the digit totals behind the passes in use
-        uint32_t* nlong = hist + (kMaxPasses - 1) * kBins;
-        k_rs_runs<<<ceil_div(ncap, 256), 256, 0, s>>>(K[cur], V[cur], box_digits, d_n, ncap, low_bit, nlong, status);
+        // done with (at most one run per kShortRun + 1 keys)
+        const uint32_t* nlong = hist + kLongCount;
+        k_rs_runs<<<ceil_div(ncap, 256), 256, 0, s>>>(K[cur], V[cur], box_digits, d_n, ncap, low_bit, hist, status);
         k_rs_long<<<std::min(ceil_div(ncap, kShortRun), 152), kThreads, 0, s>>>(
             K[cur], V[cur], K[cur ^ 1], V[cur ^ 1], box_digits, d_n, ncap, low_bit, nlong, status);
     }
     return cur;
-}
-
-void exclusive_scan_i32(int32_t* data, int n_cap, const int* d_n, int32_t* part, int32_t* total,
-                        cudaStream_t s) {
-    const int nb = ceil_div((long long)n_cap + 1, kScanTile);
-    k_scan_reduce<<<nb, 256, 0, s>>>(data, n_cap, d_n, part);
-    k_scan_block<int32_t><<<1, kScanThreads, 0, s>>>(part, nb, total);
-    k_scan_down<<<nb, 256, 0, s>>>(data, n_cap, d_n, part, total);
 }
 
 }  // namespace rb

@@ -10,6 +10,7 @@
 // order without fused multiply-adds.
 #include <algorithm>
 #include <climits>
+#include <cstddef>
 
 #include "rb_internal.cuh"
 
@@ -145,11 +146,13 @@ struct DriftArgs {
 };
 
 // Optional kick (v += a dt), one or two drift halves each followed by the
-// boundaries, then the Morton key of the new position for the next sort.
+// boundaries, then, for the drifts that a sort follows (kKeys), the Morton key
+// of the new position.
+template <bool kKeys>
 __global__ void __launch_bounds__(256) k_drift_keys(DriftArgs A, SimC C) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= A.ncap) return;
-    A.idx[i] = (uint32_t)i;
+    if (kKeys) A.idx[i] = (uint32_t)i;
     bool live = A.P.box[i] < C.nbox;
     uint64_t key = kRemovedKey;
     if (live) {
@@ -172,25 +175,34 @@ __global__ void __launch_bounds__(256) k_drift_keys(DriftArgs A, SimC C) {
         }
         A.P.x[i] = x; A.P.y[i] = y; A.P.z[i] = z;
         A.P.vx[i] = vx; A.P.vy[i] = vy; A.P.vz[i] = vz;
-        if (live) {
+        if (kKeys && live) {
             const double lo = -bp.hx;   // the root cube's side L is Lx
             key = (spread3(icoord(x, lo, bp.L, bp.key_scale)) << 2) |
                   (spread3(icoord(y, lo, bp.L, bp.key_scale)) << 1) |
                   spread3(icoord(z, lo, bp.L, bp.key_scale));
         }
     }
+    if (!live) A.P.box[i] = C.nbox;
+    if (!kKeys) return;   // the particles keep their slots; removed ones stay flagged
     A.key[i] = key;
     A.sbox[i] = live ? A.P.box[i] : C.nbox;
-    if (!live) A.P.box[i] = C.nbox;
     const unsigned b = __ballot_sync(0xffffffffu, live);
     if ((threadIdx.x & 31) == 0 && b) atomicAdd(&A.ctl->n_live_next, __popc(b));
 }
 
+// The gather into sorted order.  Also commits the live count, and clears what
+// the topology kernels that follow fill in.
 __global__ void __launch_bounds__(256) k_permute(PSet S, PSet D, const uint32_t* __restrict__ idx,
-                                                 int32_t* __restrict__ slot_of_id, const Ctl* ctl,
-                                                 int ncap) {
+                                                 int32_t* __restrict__ slot_of_id, Ctl* ctl, int ncap,
+                                                 Tree T, int nstat, int nbox) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    const int nlive = ctl->n_live_next;   // cleared by k_nodes
+    if (i == 0) ctl->n_live = nlive;
+    for (int k = i; k < nstat; k += gridDim.x * blockDim.x) T.scan_stat[k] = 0u;
+    for (int k = i; k <= nbox; k += gridDim.x * blockDim.x) T.box_root[k] = -1;
     if (i >= ncap) return;
+    T.mask[i] = 0u;
+    reinterpret_cast<uint2*>(T.e_cmask)[i] = make_uint2(0u, 0u);   // two entries a slot
     const int j = (int)idx[i];
     D.x[i] = S.x[j]; D.y[i] = S.y[j]; D.z[i] = S.z[j];
     D.vx[i] = S.vx[j]; D.vy[i] = S.vy[j]; D.vz[i] = S.vz[j];
@@ -198,23 +210,7 @@ __global__ void __launch_bounds__(256) k_permute(PSet S, PSet D, const uint32_t*
     const int id = S.id[j];
     D.id[i] = id;
     D.box[i] = S.box[j];
-    if (i < ctl->n_live_next) slot_of_id[id] = i;
-}
-
-__global__ void k_commit_live(Ctl* ctl) {
-    ctl->n_live = ctl->n_live_next;
-    ctl->n_live_next = 0;
-}
-
-__global__ void k_discard_live(Ctl* ctl) { ctl->n_live_next = 0; }
-
-// An overflowing search resolves nothing: the host grows the buffer and runs
-// the search again on the unchanged state.
-__global__ void k_pairs_prep(Ctl* ctl, int cap) {
-    const int c = ctl->pair_count;
-    const int n = c <= cap ? c : 0;
-    ctl->pair_n = n;
-    ctl->resolved = 0;
+    if (i < nlive) slot_of_id[id] = i;
 }
 
 struct ResolveArgs {
@@ -228,6 +224,7 @@ struct ResolveArgs {
     Ctl* ctl;
     const ImgTab* img;            // [box][image] offsets at the detection time
     int nimg, ngx, ngy, ngz;
+    bool advance;                 // this resolution ends a step
 };
 
 __device__ __forceinline__ int key_a(uint64_t k) { return (int)(k >> 36); }
@@ -338,6 +335,7 @@ __device__ __forceinline__ int ld_flag(const int32_t* p) {
 // dependent round trips and 60 FP64 operations a link).
 template <bool kPower>
 __global__ void __launch_bounds__(256) k_resolve(ResolveArgs A, SimC C) {
+    if (A.advance && blockIdx.x == 0 && threadIdx.x == 0) A.ctl->step += 1;   // nothing here reads the time
     const int n = A.ctl->pair_n;
     const int lane = threadIdx.x & 31;
     int nres = 0;
@@ -479,13 +477,14 @@ __global__ void k_energy_final(const double* __restrict__ partials, int nparts,
 
 void drift_keys(const PSet& P, const Tree& T, Ctl* ctl, const BoxP* boxes, const SimC& C,
                 int ncap, int ndrift, int half_step_offset, const double* ax, const double* ay,
-                const double* az, bool kick, cudaStream_t s) {
+                const double* az, bool kick, bool keys, cudaStream_t s) {
     if (ncap <= 0) return;
     DriftArgs A;
     A.P = P; A.key = T.key; A.idx = T.idx; A.sbox = T.sbox; A.ctl = ctl; A.boxes = boxes;
     A.ax = ax; A.ay = ay; A.az = az;
     A.ncap = ncap; A.ndrift = ndrift; A.hs = half_step_offset; A.kick = kick;
-    k_drift_keys<<<ceil_div(ncap, 256), 256, 0, s>>>(A, C);
+    if (keys) k_drift_keys<true><<<ceil_div(ncap, 256), 256, 0, s>>>(A, C);
+    else k_drift_keys<false><<<ceil_div(ncap, 256), 256, 0, s>>>(A, C);
 }
 
 // Morton bits below those that the passes sort.
@@ -503,11 +502,9 @@ void sort_and_permute(const PSet& src, const PSet& dst, Tree& T, Pairs& PR, Ctl*
         uint64_t* k = T.key; T.key = T.key_alt; T.key_alt = k;
         uint32_t* v = T.idx; T.idx = T.idx_alt; T.idx_alt = v;
     }
-    k_permute<<<ceil_div(ncap, 256), 256, 0, s>>>(src, dst, T.idx, PR.slot_of_id, ctl, ncap);
-    k_commit_live<<<1, 1, 0, s>>>(ctl);
+    k_permute<<<ceil_div(ncap, 256), 256, 0, s>>>(src, dst, T.idx, PR.slot_of_id, ctl, ncap, T,
+                                                  (int)entry_scan_words(ncap), C.nbox);
 }
-
-void discard_live_count(Ctl* ctl, cudaStream_t s) { k_discard_live<<<1, 1, 0, s>>>(ctl); }
 
 // Live particles of one box written in id order (id - base) to out, with a
 // flag per id and a count.
@@ -611,23 +608,23 @@ void reset_slots(const PSet& P, int32_t* slot_of_id, int n, int ncap, int nbox, 
 }
 
 void sort_pairs(Pairs& PR, Ctl* ctl, cudaStream_t s, int key_bits) {
-    k_pairs_prep<<<1, 1, 0, s>>>(ctl, PR.cap);
     // passes over the lower id's bits, then each id's pairs among themselves;
     // an odd number of passes leaves the keys in key_alt; the buffers are
     // not swapped, so every captured graph finds them in the same place
     PR.sorted_alt = radix_sort(PR.key, PR.val, PR.key_alt, PR.val_alt, PR.cap, &ctl->pair_n,
-                               key_bits, nullptr, 0, PR.hist, &ctl->err, s, 36) == 1;
+                               key_bits, nullptr, 0, PR.hist, &ctl->err, s, 36, ctl) == 1;
 }
 
 void resolve_pairs(const PSet& P, Ctl* ctl, const BoxP* boxes, const SimC& C, Pairs& PR,
-                   int half_step_offset, ImgTab* img, cudaStream_t s) {
+                   int half_step_offset, ImgTab* img, bool have_img, bool advance, cudaStream_t s) {
     ResolveArgs A;
     A.P = P; A.key = PR.sorted(); A.slot_of_id = PR.slot_of_id;
     A.head = PR.head; A.link = PR.link; A.done = PR.done; A.rec = PR.rec; A.claim = PR.claim;
     A.img = img;
     A.ngx = C.ngx; A.ngy = C.ngy; A.ngz = C.ngz;
-    A.nimg = build_image_table(boxes, ctl, C, half_step_offset, img, s);
+    A.nimg = have_img ? C.nimg : build_image_table(boxes, ctl, C, half_step_offset, img, s);
     A.ctl = ctl;
+    A.advance = advance;
     cudaMemsetAsync(PR.head, 0xff, sizeof(int32_t) * (size_t)PR.ncap, s);   // empty lists
     const int grid = std::min(ceil_div(PR.cap, 256), 8 * 152);
     k_pair_link<<<grid, 256, 0, s>>>(A);
@@ -645,7 +642,12 @@ void energy_terms(const PSet& P, Ctl* ctl, const SimC& C, const double* phi, int
 
 void step_advance(Ctl* ctl, cudaStream_t s) { k_step_advance<<<1, 1, 0, s>>>(ctl); }
 
-// The walk's counters (n_cell .. n_iter) and the search's (n_visit, n_siter).
+// What a step starts from zero: the pair count, the error word, and the
+// counters of the walk (n_cell .. n_iter) and of the search (n_visit, n_siter).
+void clear_step(Ctl* ctl, cudaStream_t s) {
+    cudaMemsetAsync(&ctl->pair_count, 0, offsetof(Ctl, sweep_wbits) - offsetof(Ctl, pair_count), s);
+}
+
 void clear_walk_stats(Ctl* ctl, cudaStream_t s) {
     cudaMemsetAsync(&ctl->n_cell, 0, 7 * sizeof(unsigned long long), s);
 }

@@ -39,14 +39,14 @@ __device__ __forceinline__ int lcp_level(const uint64_t* __restrict__ key,
 // the cell's depth in mask[first].
 template <bool kMultiBox>
 __global__ void __launch_bounds__(256) k_nodes(const uint64_t* __restrict__ key,
-                                               const int32_t* __restrict__ box,
-                                               const Ctl* __restrict__ ctl, int ncap,
+                                               const int32_t* __restrict__ box, Ctl* ctl, int ncap,
                                                int32_t* __restrict__ node_a,
                                                int32_t* __restrict__ node_b,
                                                int8_t* __restrict__ node_v,
                                                uint32_t* __restrict__ mask) {
     const int n = min(ctl->n_live, ncap);
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i == 0) ctl->n_live_next = 0;   // committed by the gather
     if (i >= n - 1) return;
     const int v = lcp_level<kMultiBox>(key, box, i, i + 1);
     int8_t outv = -1;
@@ -90,12 +90,92 @@ __global__ void __launch_bounds__(256) k_nodes(const uint64_t* __restrict__ key,
     node_v[i] = outv;
 }
 
-__global__ void __launch_bounds__(256) k_entry_counts(const uint32_t* __restrict__ mask,
-                                                      const Ctl* __restrict__ ctl, int ncap,
-                                                      int32_t* __restrict__ start) {
+// First entry starting at each particle: the exclusive scan of 1 + (cells
+// starting there), start[n] and n_entries the total.  One launch: a block scans
+// a tile of 2048 particles and finds the total of the earlier tiles by a
+// decoupled look-back over one status word per tile (zero on entry; flag and
+// count in one word, as in the radix passes, whose argument that every wait
+// ends holds here too; bounded by half a second all the same).
+constexpr int kScanTile = 2048;
+constexpr uint32_t kScanAgg = 1u << 30, kScanPre = 2u << 30, kScanMask = (1u << 30) - 1u;
+
+__global__ void __launch_bounds__(256) k_entry_scan(const uint32_t* __restrict__ mask, Ctl* ctl, int ncap,
+                                                    int32_t* __restrict__ start, uint32_t* stat) {
+    __shared__ uint32_t ws[8], before_s;
     const int n = min(ctl->n_live, ncap);
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n) start[i] = 1 + __popc(mask[i]);
+    const int b = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int base = b * kScanTile;
+    if (base >= n) {
+        if (b == 0 && tid == 0) {
+            start[0] = 0;
+            ctl->n_entries = 0;
+        }
+        return;
+    }
+    const int t0 = base + tid * 8;
+    uint32_t v[8], s = 0;
+#pragma unroll
+    for (int r = 0; r < 8; r++) {
+        v[r] = t0 + r < n ? 1u + __popc(mask[t0 + r]) : 0u;
+        s += v[r];
+    }
+    uint32_t x = s;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t t = __shfl_up_sync(0xffffffffu, x, o);
+        if (lane >= o) x += t;
+    }
+    if (lane == 31) ws[warp] = x;
+    __syncthreads();
+    uint32_t in = x - s, total = 0;   // counts before this thread within the tile
+#pragma unroll
+    for (int w = 0; w < 8; w++) {
+        if (w < warp) in += ws[w];
+        total += ws[w];
+    }
+    volatile uint32_t* st = stat;
+    if (tid == 0) st[b] = (b == 0 ? kScanPre : kScanAgg) | total;
+    if (warp == 0) {
+        uint32_t excl = 0;
+        unsigned long long since = 0;
+        for (int j = b - 1; j >= 0;) {
+            // the 32 nearest tiles not yet counted, down to the first prefix
+            uint32_t w = kScanPre;
+            if (j - lane >= 0) w = st[j - lane];
+            const unsigned pre = __ballot_sync(0xffffffffu, w & kScanPre);
+            const unsigned none = __ballot_sync(0xffffffffu, (w & (kScanPre | kScanAgg)) == 0u);
+            const unsigned need = pre ? (2u << (__ffs(pre) - 1)) - 1u : 0xffffffffu;
+            if (none & need) {
+                unsigned long long now;
+                asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(now));
+                if (since == 0) since = now;
+                const bool give_up = (*(volatile int*)&ctl->err & kErrSortStall) || now - since > 500000000ull;
+                if (__any_sync(0xffffffffu, give_up)) {
+                    if (lane == 0) atomicOr(&ctl->err, kErrSortStall);
+                    break;
+                }
+                continue;
+            }
+            excl += __reduce_add_sync(0xffffffffu, (need >> lane) & 1u ? w & kScanMask : 0u);
+            if (pre) break;
+            j -= 32;
+        }
+        if (lane == 0) {
+            if (b > 0) st[b] = kScanPre | ((excl + total) & kScanMask);
+            before_s = excl;
+        }
+    }
+    __syncthreads();
+    uint32_t run = before_s + in;
+#pragma unroll
+    for (int r = 0; r < 8; r++) {
+        if (t0 + r < n) start[t0 + r] = (int32_t)run;
+        run += v[r];
+    }
+    if (tid == 0 && base + kScanTile >= n) {
+        start[n] = (int32_t)(before_s + total);
+        ctl->n_entries = (int32_t)(before_s + total);
+    }
 }
 
 // Entries in pre-order: cells (from their representative split) and leaves.
@@ -112,10 +192,17 @@ __global__ void __launch_bounds__(256) k_emit(const uint32_t* __restrict__ mask,
                                               int32_t* __restrict__ leaf_of,
                                               const uint64_t* __restrict__ key,
                                               int32_t* __restrict__ e_child,
-                                              uint32_t* __restrict__ e_cmask) {
+                                              uint32_t* __restrict__ e_cmask,
+                                              const int32_t* __restrict__ box,
+                                              int32_t* __restrict__ box_root) {
     const int n = min(ctl->n_live, ncap);
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
+    // the root of a box starts at its first particle; the others stay -1
+    // (empty boxes, and entry nbox, the box of particles that an open boundary
+    // removed: those still hold slots of the gravity tree when the step's
+    // collision search runs on it, and search nothing)
+    if (i == 0 || box[i] != box[i - 1]) box_root[box[i]] = start[i];
     const uint32_t mk = mask[i];
     const int li = start[i] + __popc(mk);
     e_first[li] = i;
@@ -154,37 +241,6 @@ __global__ void __launch_bounds__(256) k_emit(const uint32_t* __restrict__ mask,
         }
     }
 }
-
-// Box ranges in sorted order (empty boxes get empty ranges) and box roots.
-__global__ void __launch_bounds__(256) k_box_ranges(const int32_t* __restrict__ box,
-                                                    const Ctl* __restrict__ ctl, int ncap, int nbox,
-                                                    int32_t* __restrict__ box_first) {
-    const int n = min(ctl->n_live, ncap);
-    const int p = blockIdx.x * blockDim.x + threadIdx.x;
-    if (n == 0) {
-        if (p <= nbox) box_first[p] = 0;
-        return;
-    }
-    if (p >= n) return;
-    const int b = box[p];
-    const int prev = p == 0 ? -1 : box[p - 1];
-    for (int q = prev + 1; q <= b; q++) box_first[q] = p;
-    if (p == n - 1)
-        for (int q = b + 1; q <= nbox; q++) box_first[q] = n;
-}
-
-// Root entry of each box's tree, -1 for an empty box; entry nbox, -1, is the
-// root of the box that particles removed by an open boundary carry (nbox):
-// those still hold slots of the gravity tree when the step's collision
-// search runs on it, and search nothing.
-__global__ void k_box_roots(const int32_t* __restrict__ box_first,
-                            const int32_t* __restrict__ start, int nbox,
-                            int32_t* __restrict__ box_root) {
-    const int b = blockIdx.x * blockDim.x + threadIdx.x;
-    if (b > nbox) return;
-    box_root[b] = b < nbox && box_first[b] < box_first[b + 1] ? start[box_first[b]] : -1;
-}
-
 
 __device__ __forceinline__ uint32_t compact3(uint64_t x) {
     x &= 0x1249249249249249ull;
@@ -1019,25 +1075,23 @@ __global__ void __launch_bounds__(256) k_aabb_cells(CollRecArgs A) {
 
 }  // namespace
 
+size_t entry_scan_words(int ncap) { return (size_t)ceil_div(ncap > 0 ? ncap : 1, kScanTile); }
+
+// mask, e_cmask, box_root and scan_stat are cleared by the gather before.
 void build_topology(const Tree& T, const PSet& P, Ctl* ctl, const BoxP* boxes, const SimC& C,
                     cudaStream_t s) {
     const int n = T.cap_n;
     if (n <= 0) return;
     const int nb = ceil_div(n, 256);
-    cudaMemsetAsync(T.mask, 0, sizeof(uint32_t) * n, s);
     if (C.nbox > 1)
         k_nodes<true><<<nb, 256, 0, s>>>(T.key, P.box, ctl, n, T.node_a, T.node_b, T.node_v, T.mask);
     else
         k_nodes<false><<<nb, 256, 0, s>>>(T.key, P.box, ctl, n, T.node_a, T.node_b, T.node_v,
                                           T.mask);
-    k_entry_counts<<<nb, 256, 0, s>>>(T.mask, ctl, n, T.start);
-    exclusive_scan_i32(T.start, n, &ctl->n_live, T.scan_part, &ctl->n_entries, s);
-    cudaMemsetAsync(T.e_cmask, 0, sizeof(uint32_t) * T.cap_e, s);
+    k_entry_scan<<<ceil_div(n, kScanTile), 256, 0, s>>>(T.mask, ctl, n, T.start, T.scan_stat);
     k_emit<<<nb, 256, 0, s>>>(T.mask, T.start, T.node_a, T.node_b, T.node_v, ctl, n, T.e_first,
-                              T.e_count, T.e_skip, T.e_level, T.leaf_of, T.key, T.e_child, T.e_cmask);
-    k_box_ranges<<<ceil_div(n > C.nbox + 1 ? n : C.nbox + 1, 256), 256, 0, s>>>(
-        P.box, ctl, n, C.nbox, T.box_first);
-    k_box_roots<<<ceil_div(C.nbox + 1, 256), 256, 0, s>>>(T.box_first, T.start, C.nbox, T.box_root);
+                              T.e_count, T.e_skip, T.e_level, T.leaf_of, T.key, T.e_child, T.e_cmask, P.box,
+                              T.box_root);
 }
 
 namespace {
@@ -1121,7 +1175,7 @@ void build_tile_order(Tree& T, const PSet& P, Ctl* ctl, int mode, int box_bits, 
     }
     k_tile_keys<<<ceil_div(T.cap_n, 256), 256, 0, s>>>(T.key, P.box, ctl, T.cap_n, mode, T.tkey, T.tval);
     const int which = radix_sort(T.tkey, T.tval, T.tkey_alt, T.tval_alt, T.cap_n, &ctl->n_live,
-                                 21 + box_bits, nullptr, 0, T.hist, &ctl->err, s);
+                                 21 + box_bits, nullptr, 0, T.thist, &ctl->err, s);
     T.order = which ? T.tval_alt : T.tval;
 }
 

@@ -48,7 +48,8 @@ def _check(rb, P, L, walk, least):
 
 
 @pytest.mark.parametrize("walk", [0, 1])
-@pytest.mark.parametrize("n", [2, 255, 256, 257, 700, 5000])
+# edges of a range (256) and of a tile of the entry scan (2048)
+@pytest.mark.parametrize("n", [2, 255, 256, 257, 700, 2047, 2048, 2049, 5000])
 def test_every_cell_of_small_trees(rb, n, walk):
     assert _check(rb, I.random_cube(n, n), 1.0, walk, 2) >= 1
 
