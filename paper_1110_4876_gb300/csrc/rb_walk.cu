@@ -853,15 +853,6 @@ int residency(const void* fn, int block) {
     return per_sm;
 }
 
-// Persistent grid of kernel fn: the blocks that fit on the GPU at once, but
-// no more than the blocks that one target per thread would need.
-template <typename F>
-int persistent_grid(F fn, int block, int cap_n) {
-    const int need = ceil_div(cap_n, block);
-    const int fit = max(g_nsm, 1) * residency(reinterpret_cast<const void*>(fn), block);
-    return max(1, min(need, fit));
-}
-
 template <typename F>
 void prepare_one(F fn) {
     walk_prepare_kernel(reinterpret_cast<const void*>(fn));
@@ -874,9 +865,10 @@ void walk_prepare_kernel(const void* fn) {
 }
 
 int walk_grid(const void* fn, int block, long long warps) {
+    const int nsm = max(g_nsm, 1);
     const long long need = (warps * 32 + block - 1) / block;
-    const long long fit = (long long)max(g_nsm, 1) * residency(fn, block);
-    return (int)std::max<long long>(1, std::min(need, fit));
+    const long long per_sm = std::min<long long>((need + nsm - 1) / nsm, residency(fn, block));
+    return (int)(nsm * std::max<long long>(per_sm, 1));
 }
 
 int walk_prepare() {
@@ -961,7 +953,8 @@ void gravity_walk(const Tree& T, const PSet& P, Ctl* ctl, const BoxP* boxes, con
     A.nq = T.nq;
     A.nimg = build_image_table(boxes, ctl, C, half_step_offset, T.img, s, T.tq, T.nq);
     // every kernel below runs the persistent grid that fits on the GPU
-#define RB_LAUNCH(...) __VA_ARGS__<<<persistent_grid(__VA_ARGS__, block, T.cap_n), block, 0, s>>>(A)
+#define RB_LAUNCH(...)                                                                                     \
+    __VA_ARGS__<<<walk_grid((const void*)(__VA_ARGS__), block, ceil_div(T.cap_n, 32)), block, 0, s>>>(A)
 #define RB_W32G(Q, I, S, ONE) RB_LAUNCH(k_gwalk32<Q, I, S, ONE, 4>)
 #define RB_W32(Q, I, PO, S)                                                \
     do {                                                                   \

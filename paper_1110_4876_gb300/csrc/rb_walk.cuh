@@ -44,7 +44,12 @@ struct GravArgs {
 
 // Resident blocks of a walk kernel (queried once per kernel and block size,
 // outside any capture) and the persistent grid that runs `warps` warps of
-// work on them.
+// work on them: the same number of blocks on every SM, as many as the work
+// fills and as fit.  With a grid of just the blocks that the work fills, the
+// few SMs that get one block more end last: union walk of the sheet 425 -> 360
+// us at 60k targets, 501 -> 380 at 100k, 585 -> 468 at 150k (the same from 200k
+// on, where every SM is full either way), search 55 -> 47 us at 2400.  A block
+// without work finds the queues empty and ends.
 void walk_prepare_kernel(const void* fn);
 int walk_grid(const void* fn, int block, long long warps);
 
@@ -52,10 +57,11 @@ int walk_grid(const void* fn, int block, long long warps);
 // records and image table; block is 64, 128 or 256 threads (FP64).
 // FP32 walks take them up to kTargetWalkMax targets, where the chain of
 // entries that a warp of 32 targets steps through is longer than the work:
-// on the sheet (theta = 0.5, 9 images) 37 us against 262 at 2400 targets, 88
-// against 322 at 10k, 216 against 365 at 30k, 409 against 413 at 60k and 710
-// against 482 at 100k; learned walk (theta = 0.8) 101 against 597 at 5k, 361
-// against 760 at 20k, 1153 against 1117 at 60k.
+// on the sheet (theta = 0.5, 9 images) 147 us against 319 at 20k targets, 219
+// against 325 at 30k, 276 against 324 at 40k, 347 against 333 at 50k, 409
+// against 361 at 60k and 557 against 367 at 80k (theta = 0.8: 183 against 243
+// at 40k, 260 against 251 at 60k); learned walk (theta = 0.8) 182 against 608
+// at 10k, 752 against 871 at 40k, 1152 against 1070 at 60k.
 constexpr int kTargetWalkMax = 50000;
 enum class TargetWalk { kFp32, kFp64, kLearned };
 void target_walk(const GravArgs& A, TargetWalk mode, bool quad, bool inside, bool soft, bool pot, int block,
