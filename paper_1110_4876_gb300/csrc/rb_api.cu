@@ -90,7 +90,6 @@ struct rb_sim {
     Ctl hctl{};
     // learned far-field correction
     float* mlp_w = nullptr;      // padded FP32 weights
-    void* mlp_wbf = nullptr;     // padded BF16 weights
     mlp::Packed* mlp_pk = nullptr;  // inference layout read by the learned walk
     bool mlp_loaded = false;
     double theta_fb = 0.5;
@@ -1405,15 +1404,11 @@ int rb_load_mlp(rb_sim* s, const float* w, int64_t nw, double theta_fallback) {
     const int np = mlp::padded_size();
     if (!s->mlp_w) {
         if (dalloc(s, &s->mlp_w, np, s->mlp_allocs)) return RB_ERR_CUDA;
-        uint16_t* bf = nullptr;
-        if (dalloc(s, &bf, np, s->mlp_allocs)) return RB_ERR_CUDA;
-        s->mlp_wbf = bf;
         if (dalloc(s, &s->mlp_pk, 1, s->mlp_allocs)) return RB_ERR_CUDA;
     }
     std::vector<float> pad(np);
     mlp::to_padded(w, pad.data());
     RB_CUDA(s, cudaMemcpyAsync(s->mlp_w, pad.data(), sizeof(float) * np, cudaMemcpyHostToDevice, s->stream));
-    mlp::to_bf16_async(s->mlp_w, s->mlp_wbf, s->stream);
     mlp::pack_async(s->mlp_w, s->mlp_pk, s->stream);
     RB_CUDA(s, cudaStreamSynchronize(s->stream));
     s->mlp_loaded = true;
@@ -1513,13 +1508,14 @@ int rb_mlp_grad(const float* w, const float* X, const float* Y, int64_t n, float
     }
     const int np = mlp::padded_size();
     float* dw = B.alloc<float>(np);
-    uint16_t* dwb = B.alloc<uint16_t>(np);
+    uint8_t* dtw = B.alloc<uint8_t>(mlp::train_weights_bytes());
     float* dX = B.alloc<float>(12 * n);
     float* dY = B.alloc<float>(3 * n);
     int32_t* didx = B.alloc<int32_t>(n);
     float* dg = B.alloc<float>(np);
     float* dl = B.alloc<float>(1);
-    if (!dw || !dwb || !dX || !dY || !didx || !dg || !dl) {
+    float* dp = B.alloc<float>(mlp::grad_part_floats((int)n));
+    if (!dw || !dtw || !dX || !dY || !didx || !dg || !dl || !dp) {
         g_create_error = "rb_mlp_grad: device allocation failed";
         return RB_ERR_CUDA;
     }
@@ -1532,8 +1528,8 @@ int rb_mlp_grad(const float* w, const float* X, const float* Y, int64_t n, float
     cudaMemcpyAsync(dY, Y, sizeof(float) * 3 * n, cudaMemcpyHostToDevice, B.s);
     cudaMemcpyAsync(didx, idx.data(), sizeof(int32_t) * n, cudaMemcpyHostToDevice, B.s);
     cudaMemsetAsync(dl, 0, sizeof(float), B.s);
-    mlp::to_bf16_async(dw, dwb, B.s);
-    if (mlp::grad_async(dwb, dw, dX, dY, didx, (int)n, (int)n, dg, dl, B.s) != cudaSuccess) {
+    mlp::train_weights_async(dw, dtw, B.s);
+    if (mlp::grad_async(dtw, dw, dX, dY, didx, (int)n, (int)n, dp, dg, dl, B.s) != cudaSuccess) {
         g_create_error = "rb_mlp_grad: launch failed";
         return RB_ERR_CUDA;
     }
@@ -1608,13 +1604,13 @@ int rb_mlp_train(const float* X, const float* Y, int64_t n, int epochs, int batc
     float* dw = B.alloc<float>(np);
     float* dm = B.alloc<float>(np);
     float* dv = B.alloc<float>(np);
-    uint16_t* dwb = B.alloc<uint16_t>(np);
+    uint8_t* dtw = B.alloc<uint8_t>(mlp::train_weights_bytes());
     float* dX = B.alloc<float>(12 * n);
     float* dY = B.alloc<float>(3 * n);
     int32_t* didx = B.alloc<int32_t>(n);
-    float* dg = B.alloc<float>(np);
     float* dl = B.alloc<float>(epochs);
-    if (!dw || !dm || !dv || !dwb || !dX || !dY || !didx || !dg || !dl) {
+    float* dp = B.alloc<float>(mlp::grad_part_floats((int)std::min<int64_t>(batch, n)));
+    if (!dw || !dm || !dv || !dtw || !dX || !dY || !didx || !dl || !dp) {
         g_create_error = "rb_mlp_train: device allocation failed";
         return RB_ERR_CUDA;
     }
@@ -1645,7 +1641,7 @@ int rb_mlp_train(const float* X, const float* Y, int64_t n, int epochs, int batc
     cudaMemsetAsync(dl, 0, sizeof(float) * epochs, B.s);
     cudaMemcpyAsync(dX, Xn.data(), sizeof(float) * 12 * n, cudaMemcpyHostToDevice, B.s);
     cudaMemcpyAsync(dY, Yn.data(), sizeof(float) * 3 * n, cudaMemcpyHostToDevice, B.s);
-    mlp::to_bf16_async(dw, dwb, B.s);
+    mlp::train_weights_async(dw, dtw, B.s);
     std::vector<int32_t> idx(n);
     std::mt19937_64 rng(seed);
     int step = 0;
@@ -1655,11 +1651,11 @@ int rb_mlp_train(const float* X, const float* Y, int64_t n, int epochs, int batc
         cudaMemcpyAsync(didx, idx.data(), sizeof(int32_t) * n, cudaMemcpyHostToDevice, B.s);
         for (int64_t b0 = 0; b0 < n; b0 += batch) {
             const int nb = (int)std::min<int64_t>(batch, n - b0);
-            if (mlp::grad_async(dwb, dw, dX, dY, didx + b0, nb, nb, dg, dl + ep, B.s) != cudaSuccess) {
+            if (mlp::adam_step_async(dw, dm, dv, dtw, dX, dY, didx + b0, nb, (float)lr, ++step, dp, dl + ep, B.s) !=
+                cudaSuccess) {
                 g_create_error = "rb_mlp_train: launch failed";
                 return RB_ERR_CUDA;
             }
-            mlp::adam_async(dw, dm, dv, dg, dwb, (float)lr, ++step, B.s);
         }
         // the host permutation buffer is reused next epoch
         if (cudaStreamSynchronize(B.s) != cudaSuccess) {

@@ -385,16 +385,25 @@ struct ReqArgs {
 int padded_size();
 void to_padded(const float* canonical, float* padded);
 void from_padded(const float* padded, float* canonical);
-cudaError_t grad_async(const void* wbf, const float* wf, const float* X, const float* Y,
-                       const int32_t* idx, int n, int n_total, float* grad, float* loss,
-                       cudaStream_t s);
-void adam_async(float* w, float* m, float* v, const float* grad, void* wbf, float lr, int step,
-                cudaStream_t s);
+// Training weights (BF16 fragments, train_weights_bytes() bytes) of the padded
+// FP32 weights w.
+size_t train_weights_bytes();
+void train_weights_async(const float* w, void* tw, cudaStream_t s);
+// Scratch floats of a gradient over n rows (`part` below).
+size_t grad_part_floats(int n);
+// Gradient (padded) of the mean squared error of the rows idx[0..n) with
+// n_total as the mean's denominator; the summed squared error is added to
+// *loss.  Device pointers; async on s.
+cudaError_t grad_async(const void* tw, const float* wf, const float* X, const float* Y, const int32_t* idx, int n,
+                       int n_total, float* part, float* grad, float* loss, cudaStream_t s);
+// Adam step number `step` (from 1) on the rows idx[0..n): w, m, v and tw are
+// updated and the summed squared error before the step is added to *loss.
+cudaError_t adam_step_async(float* w, float* m, float* v, void* tw, const float* X, const float* Y,
+                            const int32_t* idx, int n, float lr, int step, float* part, float* loss, cudaStream_t s);
 // FP32 debug gradient on canonical (unpadded) weights: G holds n x 9347
 // per-row gradients, lrow n per-row squared errors.
 cudaError_t grad_f32_async(const float* w, const float* X, const float* Y, int n, float* G, float* lrow,
                            float* grad, float* loss, cudaStream_t s);
-void to_bf16_async(const float* w, void* wbf, cudaStream_t s);
 void label_async(const ReqArgs& A, float* X, float* Y, int64_t* meta, int max_req, cudaStream_t s);
 }  // namespace mlp
 void clear_step(Ctl* ctl, cudaStream_t s);

@@ -9,9 +9,10 @@
 // inference itself runs inside the gravity walk (rb_walk.cu).
 //
 // Tensor cores: every layer of the forward and backward pass is a BF16
-// mma.sync.m16n8k16 with FP32 accumulation on 16-row tiles per warp.  The
-// hidden activations stay in registers between forward layers (the FP32
-// accumulator fragment of one layer is the BF16 A fragment of the next).
+// mma.sync.m16n8k16 with FP32 accumulation.  Inference gives a warp 16 rows,
+// whose hidden activations stay in registers between layers (the FP32
+// accumulator fragment of one layer is the BF16 A fragment of the next);
+// training gives a block of 8 warps 32 rows.
 // Training keeps FP32 master weights (Adam) and hands BF16 copies to the
 // kernels.
 //
@@ -33,312 +34,410 @@ namespace rb {
 namespace mlp {
 namespace {
 
-constexpr int kWarps = 4;       // warps per block of the training kernel (16 rows each)
+constexpr int kRows = 32;         // rows of a block's tile in the gradient kernel
+constexpr int kMaxPartials = 152; // blocks of the gradient kernel, one per SM
+constexpr int kLdH = 72;          // row strides (BF16) of the staged activations and
+constexpr int kLdX = 24;          // inputs: ldmatrix reads 8 rows without bank conflicts
 
-__device__ __forceinline__ float gelu_grad(float z) {
-    const float t = tanhf(kGeluC * (z + 0.044715f * z * z * z));
-    return 0.5f * (1.f + t) + 0.5f * z * (1.f - t * t) * kGeluC * (1.f + 3.f * 0.044715f * z * z);
-}
-
-// Fragment loads from row-major BF16 matrices in shared memory (lane l:
-// g = l / 4, q = l % 4); ldA is shared with the inference path.
-// A tile of M^T: A[m][k] = M[k][m], m in [r0, r0+16), k in [c0, c0+16).
-__device__ __forceinline__ void ldAT(uint32_t (&a)[4], const __nv_bfloat16* M, int ld, int r0, int c0,
-                                     int g, int q) {
-    const int k0 = c0 + 2 * q, m0 = r0 + g;
-    a[0] = pack2h(M[k0 * ld + m0], M[(k0 + 1) * ld + m0]);
-    a[1] = pack2h(M[k0 * ld + m0 + 8], M[(k0 + 1) * ld + m0 + 8]);
-    a[2] = pack2h(M[(k0 + 8) * ld + m0], M[(k0 + 9) * ld + m0]);
-    a[3] = pack2h(M[(k0 + 8) * ld + m0 + 8], M[(k0 + 9) * ld + m0 + 8]);
-}
-// B tile (16 x 8) of M: B[k][n] = M[k][n], k in [k0, k0+16), n in [n0, n0+8).
-__device__ __forceinline__ void ldB(uint32_t& b0, uint32_t& b1, const __nv_bfloat16* M, int ld, int k0,
-                                    int n0, int g, int q) {
-    const int k = k0 + 2 * q, n = n0 + g;
-    b0 = pack2h(M[k * ld + n], M[(k + 1) * ld + n]);
-    b1 = pack2h(M[(k + 8) * ld + n], M[(k + 9) * ld + n]);
-}
-// B tile of M^T: B[k][n] = M[n][k].
-__device__ __forceinline__ void ldBT(uint32_t& b0, uint32_t& b1, const __nv_bfloat16* M, int ld, int k0,
-                                     int n0, int g, int q) {
-    b0 = *reinterpret_cast<const uint32_t*>(&M[(n0 + g) * ld + k0 + 2 * q]);
-    b1 = *reinterpret_cast<const uint32_t*>(&M[(n0 + g) * ld + k0 + 8 + 2 * q]);
-}
-
-// Shared-memory weights of one block: BF16 W (padded row-major) + FP32 biases.
-struct SW {
-    __nv_bfloat16 W1[16 * 64], W2[64 * 64], W3[64 * 64], W4[64 * 8];
-    float b1[64], b2[64], b3[64], b4[8];
+// BF16 weights of training as mma B fragments (as in Packed): F1..F4 those of
+// the forward pass, T4..T2 the tiles of W4^T, W3^T and W2^T that take an output
+// gradient back to the layer below (B[k][n] = W[n][k]).  One 8-byte load per
+// lane and MMA, straight into registers.
+struct TrainW {
+    uint2 F1[1][8][32], F2[4][8][32], F3[4][8][32], F4[4][1][32];
+    uint2 T4[1][8][32], T3[4][8][32], T2[4][8][32];
 };
 
-__device__ void load_weights(SW& s, const __nv_bfloat16* __restrict__ wbf, const float* __restrict__ wf) {
-    for (int i = threadIdx.x; i < 16 * 64; i += blockDim.x) s.W1[i] = wbf[kW1 + i];
-    for (int i = threadIdx.x; i < 64 * 64; i += blockDim.x) {
-        s.W2[i] = wbf[kW2 + i];
-        s.W3[i] = wbf[kW3 + i];
+// Writes padded parameter i (value v) into the fragments; biases are read in FP32.
+__device__ __forceinline__ void put_weight(TrainW& T, int i, float v) {
+    const __nv_bfloat16 h = __float2bfloat16_rn(v);
+    // element (k, n) of a B operand with nt column tiles
+    auto put = [&](uint2* F, int nt, int k, int n) {
+        const int lane = 4 * (n & 7) + ((k & 7) >> 1);
+        const int at = ((k >> 4) * nt + (n >> 3)) * 32 + lane;
+        reinterpret_cast<__nv_bfloat16*>(F + at)[((k >> 3) & 1) * 2 + (k & 1)] = h;
+    };
+    if (i < kB1) {
+        put(&T.F1[0][0][0], 8, i >> 6, i & 63);
+    } else if (i >= kW2 && i < kB2) {
+        put(&T.F2[0][0][0], 8, (i - kW2) >> 6, (i - kW2) & 63);
+        put(&T.T2[0][0][0], 8, (i - kW2) & 63, (i - kW2) >> 6);
+    } else if (i >= kW3 && i < kB3) {
+        put(&T.F3[0][0][0], 8, (i - kW3) >> 6, (i - kW3) & 63);
+        put(&T.T3[0][0][0], 8, (i - kW3) & 63, (i - kW3) >> 6);
+    } else if (i >= kW4 && i < kB4) {
+        put(&T.F4[0][0][0], 1, (i - kW4) >> 3, (i - kW4) & 7);
+        put(&T.T4[0][0][0], 8, (i - kW4) & 7, (i - kW4) >> 3);
     }
-    for (int i = threadIdx.x; i < 64 * 8; i += blockDim.x) s.W4[i] = wbf[kW4 + i];
-    for (int i = threadIdx.x; i < 64; i += blockDim.x) {
-        s.b1[i] = wf[kB1 + i];
-        s.b2[i] = wf[kB2 + i];
-        s.b3[i] = wf[kB3 + i];
-    }
-    if (threadIdx.x < 8) s.b4[threadIdx.x] = wf[kB4 + threadIdx.x];
 }
 
-// Forward pass of 16 rows held by one warp.  X: BF16 [16][16] (features in
-// columns 0..11).  If Z/H are given, the hidden pre-activations (FP32) and
-// activations (BF16) of layers 1..3 are stored as [3][16][64] for backward.
-// out: the output fragment (rows g and g+8, columns 2q and 2q+1).
-__device__ void forward(const SW& w, const __nv_bfloat16* X, float (&out)[4], float* Z,
-                        __nv_bfloat16* H) {
-    const int lane = threadIdx.x & 31, g = lane >> 2, q = lane & 3;
-    uint32_t a[4][4];
-    ldA(a[0], X, 16, 0, 0, g, q);
-    int kt = 1;
-    const __nv_bfloat16* Ws[3] = {w.W1, w.W2, w.W3};
-    const float* bs[3] = {w.b1, w.b2, w.b3};
-    for (int L = 0; L < 3; L++) {
-        float c[8][4];
+__device__ __forceinline__ uint32_t smem_u32(const void* p) {
+    return (uint32_t)__cvta_generic_to_shared(p);
+}
+__device__ __forceinline__ void ldsm4(uint32_t (&r)[4], const __nv_bfloat16* p) {
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(smem_u32(p)) : "memory");
+}
+__device__ __forceinline__ void ldsm4t(uint32_t (&r)[4], const __nv_bfloat16* p) {
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(smem_u32(p)) : "memory");
+}
+__device__ __forceinline__ void ldsm2t(uint32_t& r0, uint32_t& r1, const __nv_bfloat16* p) {
+    asm volatile("ldmatrix.sync.aligned.m8n8.x2.trans.shared.b16 {%0,%1}, [%2];"
+                 : "=r"(r0), "=r"(r1) : "r"(smem_u32(p)) : "memory");
+}
+
+// This lane's row address of each operand tile of a row-major matrix M (ld
+// columns): a 16 x 16 A tile at (r0, c0), ...
+__device__ __forceinline__ const __nv_bfloat16* at_a(const __nv_bfloat16* M, int ld, int r0, int c0, int lane) {
+    return M + (r0 + (lane & 15)) * ld + c0 + (lane >> 4) * 8;
+}
+// ... the A tile of M^T whose rows are columns c0 .. and whose k are rows r0 .., ...
+__device__ __forceinline__ const __nv_bfloat16* at_at(const __nv_bfloat16* M, int ld, int r0, int c0, int lane) {
+    return M + (r0 + (lane & 7) + (lane >> 4) * 8) * ld + c0 + ((lane >> 3) & 1) * 8;
+}
+// ... and two 16 x 8 B tiles at (r0, c0) and (r0, c0 + 8) (the lower 16 lanes: the first).
+__device__ __forceinline__ const __nv_bfloat16* at_b(const __nv_bfloat16* M, int ld, int r0, int c0, int lane) {
+    return M + (r0 + (lane & 15)) * ld + c0 + (lane >> 4) * 8;
+}
+
+// A hidden layer's forward pass for 16 rows and 16 columns of the tile:
+// activations to out, GELU's derivatives kept for the backward pass.
+template <int KT>
+__device__ __forceinline__ void train_hidden(const __nv_bfloat16* in, int ld, const uint2 (&F)[KT][2],
+                                             const float2 (&bias)[2], __nv_bfloat16* out, float (&gp)[2][4],
+                                             int r0, int c0, int lane) {
+    const int g = lane >> 2, q = lane & 3;
+    float c[2][4];
 #pragma unroll
-        for (int j = 0; j < 8; j++) {
-            c[j][0] = c[j][2] = bs[L][8 * j + 2 * q];
-            c[j][1] = c[j][3] = bs[L][8 * j + 2 * q + 1];
-        }
-        for (int t = 0; t < kt; t++)
-#pragma unroll
-            for (int j = 0; j < 8; j++) {
-                uint32_t b0, b1;
-                ldB(b0, b1, Ws[L], 64, 16 * t, 8 * j, g, q);
-                mma(c[j], a[t], b0, b1);
-            }
-#pragma unroll
-        for (int j = 0; j < 8; j++) {
-            float h[4];
-#pragma unroll
-            for (int e = 0; e < 4; e++) {
-                const int row = g + ((e >> 1) << 3), col = 8 * j + 2 * q + (e & 1);
-                if (Z) Z[(L * 16 + row) * 64 + col] = c[j][e];
-                h[e] = gelu(c[j][e]);
-                if (H) H[(L * 16 + row) * 64 + col] = __float2bfloat16_rn(h[e]);
-            }
-            const int t = j >> 1;
-            if ((j & 1) == 0) {
-                a[t][0] = pack2(h[0], h[1]);
-                a[t][1] = pack2(h[2], h[3]);
-            } else {
-                a[t][2] = pack2(h[0], h[1]);
-                a[t][3] = pack2(h[2], h[3]);
-            }
-        }
-        kt = 4;
+    for (int j = 0; j < 2; j++) {
+        c[j][0] = c[j][2] = bias[j].x;
+        c[j][1] = c[j][3] = bias[j].y;
     }
-    out[0] = out[2] = w.b4[2 * q];
-    out[1] = out[3] = w.b4[2 * q + 1];
+#pragma unroll
+    for (int t = 0; t < KT; t++) {
+        uint32_t a[4];
+        ldsm4(a, at_a(in, ld, r0, 16 * t, lane));
+#pragma unroll
+        for (int j = 0; j < 2; j++) mma(c[j], a, F[t][j].x, F[t][j].y);
+    }
+#pragma unroll
+    for (int j = 0; j < 2; j++) {
+        float h[4];
+#pragma unroll
+        for (int e = 0; e < 4; e++) {
+            const float z = c[j][e];
+            const float t = tanhf(kGeluC * (z + 0.044715f * z * z * z));
+            h[e] = 0.5f * z * (1.f + t);
+            gp[j][e] = 0.5f * (1.f + t) + 0.5f * z * (1.f - t * t) * kGeluC * (1.f + 3.f * 0.044715f * z * z);
+        }
+        __nv_bfloat16* o = out + (r0 + g) * kLdH + c0 + 8 * j + 2 * q;
+        *reinterpret_cast<uint32_t*>(o) = pack2(h[0], h[1]);
+        *reinterpret_cast<uint32_t*>(o + 8 * kLdH) = pack2(h[2], h[3]);
+    }
+}
+
+// dZ = dH gelu'(Z) of the warp's 16 rows and columns: FP32 column sums for the
+// bias, BF16 copy for the MMAs.
+__device__ __forceinline__ void train_dz(float (&dh)[2][4], const float (&gp)[2][4], float (&sb)[2][2],
+                                         __nv_bfloat16* D, int r0, int c0, int lane) {
+    const int g = lane >> 2, q = lane & 3;
+#pragma unroll
+    for (int j = 0; j < 2; j++) {
+#pragma unroll
+        for (int e = 0; e < 4; e++) dh[j][e] *= gp[j][e];
+        sb[j][0] += dh[j][0] + dh[j][2];
+        sb[j][1] += dh[j][1] + dh[j][3];
+        __nv_bfloat16* o = D + (r0 + g) * kLdH + c0 + 8 * j + 2 * q;
+        *reinterpret_cast<uint32_t*>(o) = pack2(dh[j][0], dh[j][1]);
+        *reinterpret_cast<uint32_t*>(o + 8 * kLdH) = pack2(dh[j][2], dh[j][3]);
+    }
+}
+
+// dH of the layer below: the warp's 16 rows and columns of dZ W^T.
+__device__ __forceinline__ void train_dh(float (&dh)[2][4], const __nv_bfloat16* D, const uint2 (&T)[4][2], int r0,
+                                         int lane) {
+#pragma unroll
+    for (int j = 0; j < 2; j++) dh[j][0] = dh[j][1] = dh[j][2] = dh[j][3] = 0.f;
 #pragma unroll
     for (int t = 0; t < 4; t++) {
-        uint32_t b0, b1;
-        ldB(b0, b1, w.W4, 8, 16 * t, 0, g, q);
-        mma(out, a[t], b0, b1);
+        uint32_t a[4];
+        ldsm4(a, at_a(D, kLdH, r0, 16 * t, lane));
+#pragma unroll
+        for (int j = 0; j < 2; j++) mma(dh[j], a, T[t][j].x, T[t][j].y);
     }
 }
 
-// Per-warp scratch of the training kernel.
-struct WarpScratch {
-    __nv_bfloat16 X[16 * 16];
-    float Z[3 * 16 * 64];
-    __nv_bfloat16 H[3 * 16 * 64];
-    __nv_bfloat16 D[16 * 64];    // current layer's output gradient (BF16)
-    __nv_bfloat16 D4[16 * 16];   // dY padded to 16 columns
-};
-
-struct TrainSmem {
-    SW w;
-    float grad[kPad];
-    WarpScratch ws[kWarps];
-    float loss[kWarps];
-};
-
-// Add a 16x8 fragment tile of a weight gradient (rows r0.., cols c0..) to
-// the block's gradient (row-major, ld columns).
-__device__ __forceinline__ void add_tile(float* G, int ld, int r0, int c0, const float (&c)[4], int g,
-                                         int q) {
-    atomicAdd(&G[(r0 + g) * ld + c0 + 2 * q], c[0]);
-    atomicAdd(&G[(r0 + g) * ld + c0 + 2 * q + 1], c[1]);
-    atomicAdd(&G[(r0 + g + 8) * ld + c0 + 2 * q], c[2]);
-    atomicAdd(&G[(r0 + g + 8) * ld + c0 + 2 * q + 1], c[3]);
+// acc += a 16-row product: each tile of 16 rows is an MMA of its own, so the
+// sum over rows runs in FP32 additions.
+__device__ __forceinline__ void add_mma(float (&acc)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
+    float c[4] = {0.f, 0.f, 0.f, 0.f};
+    mma(c, a, b0, b1);
+#pragma unroll
+    for (int e = 0; e < 4; e++) acc[e] += c[e];
 }
 
-// Sum over the 16 rows of a column pair (rows g and g+8 of every lane with
-// the same q): shuffle-reduce over g.
-__device__ __forceinline__ float rows_sum(float v) {
-    v += __shfl_xor_sync(0xffffffffu, v, 4);
-    v += __shfl_xor_sync(0xffffffffu, v, 8);
-    v += __shfl_xor_sync(0xffffffffu, v, 16);
-    return v;
+// Rows r0 .. r0 + 31 of In^T dZ: 16 rows (c0 ..) and 32 columns (n0 ..) of a
+// hidden layer's weight gradient.
+__device__ __forceinline__ void train_dw(float (&acc)[4][4], const __nv_bfloat16* in, const __nv_bfloat16* D, int c0,
+                                         int n0, int lane) {
+#pragma unroll
+    for (int k = 0; k < 2; k++) {
+        uint32_t a[4];
+        ldsm4t(a, at_at(in, kLdH, 16 * k, c0, lane));
+#pragma unroll
+        for (int j = 0; j < 2; j++) {
+            uint32_t b[4];
+            ldsm4t(b, at_b(D, kLdH, 16 * k, n0 + 16 * j, lane));
+            add_mma(acc[2 * j], a, b[0], b[1]);
+            add_mma(acc[2 * j + 1], a, b[2], b[3]);
+        }
+    }
 }
+
+struct GradSmem {
+    __nv_bfloat16 X[kRows * kLdX];       // inputs (columns 12..15 zero)
+    __nv_bfloat16 H[3][kRows * kLdH];    // activations of the hidden layers
+    __nv_bfloat16 D[3][kRows * kLdH];    // gradients of their pre-activations
+    __nv_bfloat16 D4[kRows * kLdX];      // output gradients (columns 0..7)
+    float b[2][200];                     // bias gradients of the two 16-row halves
+    float loss[2];
+};
 
 // Gradient of the mean squared error over the rows idx[0..n) (all rows of a
 // batch of size n_total): forward, then backward through the three hidden
-// layers; weight gradients are MMAs of activations^T x output gradients.
-__global__ void __launch_bounds__(kWarps * 32) k_mlp_grad(const __nv_bfloat16* __restrict__ wbf,
-                                                          const float* __restrict__ wf,
-                                                          const float* __restrict__ X,
-                                                          const float* __restrict__ Y,
-                                                          const int32_t* __restrict__ idx, int n,
-                                                          int n_total, float* __restrict__ grad,
-                                                          float* __restrict__ loss) {
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    TrainSmem& S = *reinterpret_cast<TrainSmem*>(smem_raw);
-    load_weights(S.w, wbf, wf);
-    for (int i = threadIdx.x; i < kPad; i += blockDim.x) S.grad[i] = 0.f;
-    if (threadIdx.x < kWarps) S.loss[threadIdx.x] = 0.f;
-    __syncthreads();
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, q = lane & 3;
-    WarpScratch& W = S.ws[warp];
-    const float scale = 2.f / (3.f * (float)n_total);
-    const int ntiles = (n + 15) / 16;
-    for (int tile = blockIdx.x * kWarps + warp; tile < ntiles; tile += gridDim.x * kWarps) {
-        // inputs
-        for (int e = lane; e < 16 * 16; e += 32) {
-            const int r = e >> 4, c = e & 15, row = tile * 16 + r;
-            const float v = (row < n && c < 12) ? X[(size_t)idx[row] * 12 + c] : 0.f;
-            W.X[e] = __float2bfloat16_rn(v);
-        }
-        __syncwarp();
-        float out[4];
-        forward(S.w, W.X, out, W.Z, W.H);
-        __syncwarp();
-        // output gradient dY = 2 (P - Y) / (3 n_total), zero outside
-        float dy[4], lsum = 0.f;
+// layers; weight gradients are MMAs of activations^T x output gradients.  A
+// block's 8 warps share tiles of 32 rows: each takes 16 rows and 16 columns of
+// every layer, and 16 x 32 of a weight gradient, which stays in registers until
+// the block's last tile and is then written as the block's part (summed by
+// k_mlp_update in a fixed order).
+// A batch has too few rows to fill the GPU (2048 rows: 64 blocks), so the time
+// is the chain of layers: the weights wait in registers and the layers hand on
+// through shared memory.  2048 rows: 7.5 us and 4.8 us for the update; a warp
+// per 16 rows with weights, operands and gradient sums (atomics) in shared
+// memory took 95 us (training 60,000 rows twice in such batches: 6.34 ms, now
+// 2.64 ms, of which 0.8 ms are kernels).
+__global__ void __launch_bounds__(256, 1) k_mlp_grad(const TrainW* __restrict__ tw, const float* __restrict__ wf,
+                                                     const float* __restrict__ X, const float* __restrict__ Y,
+                                                     const int32_t* __restrict__ idx, int n, int n_total,
+                                                     float* __restrict__ part, float* __restrict__ lpart) {
+    __shared__ __align__(16) GradSmem S;
+    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, q = lane & 3;
+    const int r0 = 16 * (w & 1), c0 = 16 * (w >> 1), j0 = c0 / 8;   // layers: rows and columns
+    const int m0 = 16 * (w & 3), n0 = 32 * (w >> 2);                // weight gradients
+    const bool outw = w < 2;                                        // the output layer's warps
+    uint2 f1[1][2], f2[4][2], f3[4][2], f4[4], t4[2], t3[4][2], t2[4][2];
+    float2 bias[3][2];
 #pragma unroll
-        for (int e = 0; e < 4; e++) {
-            const int r = g + ((e >> 1) << 3), c = 2 * q + (e & 1), row = tile * 16 + r;
-            float d = 0.f;
-            if (row < n && c < 3) {
-                const float diff = out[e] - Y[(size_t)idx[row] * 3 + c];
-                d = scale * diff;
+    for (int j = 0; j < 2; j++) {
+        f1[0][j] = tw->F1[0][j0 + j][lane];
+        t4[j] = tw->T4[0][j0 + j][lane];
+#pragma unroll
+        for (int t = 0; t < 4; t++) {
+            f2[t][j] = tw->F2[t][j0 + j][lane];
+            f3[t][j] = tw->F3[t][j0 + j][lane];
+            t3[t][j] = tw->T3[t][j0 + j][lane];
+            t2[t][j] = tw->T2[t][j0 + j][lane];
+        }
+        const int c = c0 + 8 * j + 2 * q;
+        bias[0][j] = *reinterpret_cast<const float2*>(wf + kB1 + c);
+        bias[1][j] = *reinterpret_cast<const float2*>(wf + kB2 + c);
+        bias[2][j] = *reinterpret_cast<const float2*>(wf + kB3 + c);
+    }
+#pragma unroll
+    for (int t = 0; t < 4; t++) f4[t] = tw->F4[t][0][lane];
+    const float2 bias4 = *reinterpret_cast<const float2*>(wf + kB4 + 2 * q);
+    float dw1[4] = {0.f}, dw2[4][4] = {{0.f}}, dw3[4][4] = {{0.f}}, dw4[4] = {0.f};
+    float sb1[2][2] = {{0.f}}, sb2[2][2] = {{0.f}}, sb3[2][2] = {{0.f}}, sb4[2] = {0.f, 0.f};
+    float lsum = 0.f;
+    const float scale = 2.f / (3.f * (float)n_total);
+    const int ntiles = (n - 1) / kRows + 1;
+    for (int tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
+        __syncthreads();   // the last tile's readers are done
+        if (threadIdx.x < 4 * kRows) {
+            // four values of a row; columns 12..15 are zero
+            const int r = threadIdx.x >> 2, c = threadIdx.x & 3;
+            const unsigned row = (unsigned)tile * kRows + r;
+            float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+            if (row < (unsigned)n && c < 3) v = *reinterpret_cast<const float4*>(X + (size_t)idx[row] * 12 + 4 * c);
+            *reinterpret_cast<uint2*>(&S.X[r * kLdX + 4 * c]) = make_uint2(pack2(v.x, v.y), pack2(v.z, v.w));
+        }
+        float y[4] = {0.f, 0.f, 0.f, 0.f};
+        if (outw) {
+#pragma unroll
+            for (int e = 0; e < 4; e++) {
+                const unsigned row = (unsigned)tile * kRows + r0 + g + ((e >> 1) << 3);
+                const int c = 2 * q + (e & 1);
+                if (row < (unsigned)n && c < 3) y[e] = Y[(size_t)idx[row] * 3 + c];
+            }
+        }
+        __syncthreads();
+        float gp1[2][4], gp2[2][4], gp3[2][4], dh[2][4];
+        train_hidden<1>(S.X, kLdX, f1, bias[0], S.H[0], gp1, r0, c0, lane);
+        __syncthreads();
+        train_hidden<4>(S.H[0], kLdH, f2, bias[1], S.H[1], gp2, r0, c0, lane);
+        __syncthreads();
+        train_hidden<4>(S.H[1], kLdH, f3, bias[2], S.H[2], gp3, r0, c0, lane);
+        __syncthreads();
+        if (outw) {
+            float out[4] = {bias4.x, bias4.y, bias4.x, bias4.y}, dy[4];
+#pragma unroll
+            for (int t = 0; t < 4; t++) {
+                uint32_t a[4];
+                ldsm4(a, at_a(S.H[2], kLdH, r0, 16 * t, lane));
+                mma(out, a, f4[t].x, f4[t].y);
+            }
+            // output gradient dY = 2 (P - Y) / (3 n_total), zero outside
+#pragma unroll
+            for (int e = 0; e < 4; e++) {
+                const unsigned row = (unsigned)tile * kRows + r0 + g + ((e >> 1) << 3);
+                const int c = 2 * q + (e & 1);
+                const float diff = row < (unsigned)n && c < 3 ? out[e] - y[e] : 0.f;
+                dy[e] = scale * diff;
                 lsum += diff * diff;
             }
-            dy[e] = d;
-            W.D4[r * 16 + c] = __float2bfloat16_rn(d);
-            W.D4[r * 16 + c + 8] = __float2bfloat16_rn(0.f);
+            sb4[0] += dy[0] + dy[2];
+            sb4[1] += dy[1] + dy[3];
+            __nv_bfloat16* o = S.D4 + (r0 + g) * kLdX + 2 * q;
+            *reinterpret_cast<uint32_t*>(o) = pack2(dy[0], dy[1]);
+            *reinterpret_cast<uint32_t*>(o + 8 * kLdX) = pack2(dy[2], dy[3]);
         }
-        for (int o = 16; o > 0; o >>= 1) lsum += __shfl_xor_sync(0xffffffffu, lsum, o);
-        if (lane == 0) S.loss[warp] += lsum;
-        __syncwarp();
-        // layer 4: b4, W4 (64 x 8) += H3^T dY
+        __syncthreads();
+        // dH3 = dY W4^T (k = the 8 outputs)
         {
-            const float s0 = rows_sum(dy[0] + dy[2]), s1 = rows_sum(dy[1] + dy[3]);
-            if (g == 0) {
-                atomicAdd(&S.grad[kB4 + 2 * q], s0);
-                atomicAdd(&S.grad[kB4 + 2 * q + 1], s1);
-            }
-            for (int mt = 0; mt < 4; mt++) {
-                float c[4] = {0.f, 0.f, 0.f, 0.f};
-                uint32_t a[4], b0, b1;
-                ldAT(a, W.H + 2 * 16 * 64, 64, 16 * mt, 0, g, q);
-                ldB(b0, b1, W.D4, 16, 0, 0, g, q);
-                mma(c, a, b0, b1);
-                add_tile(S.grad + kW4, 8, 16 * mt, 0, c, g, q);
-            }
-        }
-        // dH3 = dY W4^T; hidden layers 3, 2, 1
-        const __nv_bfloat16* Wl[3] = {S.w.W1, S.w.W2, S.w.W3};
-        const int offW[3] = {kW1, kW2, kW3}, offB[3] = {kB1, kB2, kB3};
-        for (int L = 2; L >= 0; L--) {
-            float dh[8][4];
-            // output gradient of layer L (16 x 64) from the layer above
+            const __nv_bfloat16* d = S.D4 + (r0 + g) * kLdX + 2 * q;
+            const uint32_t a[4] = {*reinterpret_cast<const uint32_t*>(d),
+                                   *reinterpret_cast<const uint32_t*>(d + 8 * kLdX), 0u, 0u};
 #pragma unroll
-            for (int j = 0; j < 8; j++) {
+            for (int j = 0; j < 2; j++) {
                 dh[j][0] = dh[j][1] = dh[j][2] = dh[j][3] = 0.f;
-                if (L == 2) {
-                    uint32_t a[4], b0, b1;
-                    ldA(a, W.D4, 16, 0, 0, g, q);
-                    // B[k = output o][n = hidden h] = W4[h][o]; rows o >= 8 are zero
-                    b0 = *reinterpret_cast<const uint32_t*>(&S.w.W4[(8 * j + g) * 8 + 2 * q]);
-                    b1 = 0u;
-                    mma(dh[j], a, b0, b1);
-                } else {
-                    for (int t = 0; t < 4; t++) {
-                        uint32_t a[4], b0, b1;
-                        ldA(a, W.D, 64, 0, 16 * t, g, q);
-                        ldBT(b0, b1, Wl[L + 1], 64, 16 * t, 8 * j, g, q);
-                        mma(dh[j], a, b0, b1);
-                    }
-                }
+                mma(dh[j], a, t4[j].x, 0u);
             }
-            __syncwarp();
-            // dZ = dH * gelu'(Z); bias gradient; keep dZ in BF16 for the MMAs
-#pragma unroll
-            for (int j = 0; j < 8; j++) {
-#pragma unroll
-                for (int e = 0; e < 4; e++) {
-                    const int r = g + ((e >> 1) << 3), c = 8 * j + 2 * q + (e & 1);
-                    dh[j][e] *= gelu_grad(W.Z[(L * 16 + r) * 64 + c]);
-                    W.D[r * 64 + c] = __float2bfloat16_rn(dh[j][e]);
-                }
-                const float s0 = rows_sum(dh[j][0] + dh[j][2]), s1 = rows_sum(dh[j][1] + dh[j][3]);
-                if (g == 0) {
-                    atomicAdd(&S.grad[offB[L] + 8 * j + 2 * q], s0);
-                    atomicAdd(&S.grad[offB[L] + 8 * j + 2 * q + 1], s1);
-                }
-            }
-            __syncwarp();
-            // W_L += (input of layer L)^T dZ
-            const __nv_bfloat16* in = L == 0 ? W.X : W.H + (L - 1) * 16 * 64;
-            const int ldin = L == 0 ? 16 : 64;
-            const int mts = L == 0 ? 1 : 4;
-            for (int mt = 0; mt < mts; mt++)
-#pragma unroll
-                for (int j = 0; j < 8; j++) {
-                    float c[4] = {0.f, 0.f, 0.f, 0.f};
-                    uint32_t a[4], b0, b1;
-                    ldAT(a, in, ldin, 16 * mt, 0, g, q);
-                    ldB(b0, b1, W.D, 64, 0, 8 * j, g, q);
-                    mma(c, a, b0, b1);
-                    add_tile(S.grad + offW[L], 64, 16 * mt, 8 * j, c, g, q);
-                }
-            __syncwarp();
         }
+        train_dz(dh, gp3, sb3, S.D[2], r0, c0, lane);
+        __syncthreads();
+        train_dh(dh, S.D[2], t3, r0, lane);
+        train_dz(dh, gp2, sb2, S.D[1], r0, c0, lane);
+        __syncthreads();
+        train_dh(dh, S.D[1], t2, r0, lane);
+        train_dz(dh, gp1, sb1, S.D[0], r0, c0, lane);
+        __syncthreads();
+        train_dw(dw3, S.H[1], S.D[2], m0, n0, lane);
+        train_dw(dw2, S.H[0], S.D[1], m0, n0, lane);
+#pragma unroll
+        for (int k = 0; k < 2; k++) {
+            uint32_t a[4], b0, b1;
+            ldsm4t(a, at_at(S.X, kLdX, 16 * k, 0, lane));
+            ldsm2t(b0, b1, at_b(S.D[0], kLdH, 16 * k, 8 * w, lane & 15));
+            add_mma(dw1, a, b0, b1);
+            if (w < 4) {
+                ldsm4t(a, at_at(S.H[2], kLdH, 16 * k, m0, lane));
+                ldsm2t(b0, b1, at_b(S.D4, kLdX, 16 * k, 0, lane & 15));
+                add_mma(dw4, a, b0, b1);
+            }
+        }
+    }
+    // the block's part of the gradient
+    float* P = part + (size_t)blockIdx.x * kPad;
+    auto put = [&](float* G, int ld, int r, int c, const float(&v)[4]) {
+        *reinterpret_cast<float2*>(&G[(r + g) * ld + c + 2 * q]) = make_float2(v[0], v[1]);
+        *reinterpret_cast<float2*>(&G[(r + g + 8) * ld + c + 2 * q]) = make_float2(v[2], v[3]);
+    };
+#pragma unroll
+    for (int j = 0; j < 4; j++) {
+        put(P + kW2, 64, m0, n0 + 8 * j, dw2[j]);
+        put(P + kW3, 64, m0, n0 + 8 * j, dw3[j]);
+    }
+    put(P + kW1, 64, 0, 8 * w, dw1);
+    if (w < 4) put(P + kW4, 8, m0, 0, dw4);
+    // bias gradients: over the rows of a warp, then over the two halves
+    auto rows = [&](float v) {
+        v += __shfl_xor_sync(0xffffffffu, v, 4);
+        v += __shfl_xor_sync(0xffffffffu, v, 8);
+        return v + __shfl_xor_sync(0xffffffffu, v, 16);
+    };
+#pragma unroll
+    for (int j = 0; j < 2; j++)
+#pragma unroll
+        for (int e = 0; e < 2; e++) {
+            const float v1 = rows(sb1[j][e]), v2 = rows(sb2[j][e]), v3 = rows(sb3[j][e]);
+            const int c = c0 + 8 * j + 2 * q + e;
+            if (g == 0) {
+                S.b[w & 1][c] = v1;
+                S.b[w & 1][64 + c] = v2;
+                S.b[w & 1][128 + c] = v3;
+            }
+        }
+    if (outw) {
+        const float v0 = rows(sb4[0]), v1 = rows(sb4[1]);
+        if (g == 0) {
+            S.b[w][192 + 2 * q] = v0;
+            S.b[w][192 + 2 * q + 1] = v1;
+        }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) lsum += __shfl_xor_sync(0xffffffffu, lsum, o);
+        if (lane == 0) S.loss[w] = lsum;
     }
     __syncthreads();
-    for (int i = threadIdx.x; i < kPad; i += blockDim.x)
-        if (S.grad[i] != 0.f) atomicAdd(&grad[i], S.grad[i]);
-    if (threadIdx.x == 0) {
-        float l = 0.f;
-        for (int w = 0; w < kWarps; w++) l += S.loss[w];
-        atomicAdd(loss, l);
+    if (threadIdx.x < 200) {
+        const int k = threadIdx.x;
+        const int at = k < 64 ? kB1 + k : k < 128 ? kB2 + k - 64 : k < 192 ? kB3 + k - 128 : kB4 + k - 192;
+        P[at] = S.b[0][k] + S.b[1][k];
     }
+    if (threadIdx.x == 0) lpart[blockIdx.x] = S.loss[0] + S.loss[1];
 }
 
-// Adam on the padded FP32 master weights (padding stays zero), then the
-// BF16 copies the kernels read.
-__global__ void k_mlp_adam(float* __restrict__ w, float* __restrict__ m, float* __restrict__ v,
-                           const float* __restrict__ grad, __nv_bfloat16* __restrict__ wbf, float lr,
-                           float c1, float c2) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= kPad) return;
-    const bool pad = (i < kB1 && (i - kW1) / 64 >= 12) || (i >= kW4 && i < kB4 && (i - kW4) % 8 >= 3) ||
-                     (i >= kB4 && i - kB4 >= 3);
-    if (pad) {
-        w[i] = 0.f;
-        wbf[i] = __float2bfloat16_rn(0.f);
+// Sum of the blocks' parts (8 warps per 32 parameters, in a fixed order), the
+// batch's squared error added to *loss; then the gradient (kAdam false), or
+// Adam on the padded FP32 master weights (padding stays zero) and the BF16
+// fragments that the next batch reads.
+template <bool kAdam>
+__global__ void __launch_bounds__(256) k_mlp_update(const float* __restrict__ part, const float* __restrict__ lpart,
+                                                    int np, float* __restrict__ loss, float* __restrict__ grad,
+                                                    float* __restrict__ w, float* __restrict__ m,
+                                                    float* __restrict__ v, TrainW* __restrict__ tw, float lr, float c1,
+                                                    float c2) {
+    __shared__ float red[8][32];
+    const int k = threadIdx.x >> 5, lane = threadIdx.x & 31, i = blockIdx.x * 32 + lane;
+    float sum = 0.f;
+    if (i < kPad) {
+#pragma unroll 8
+        for (int b = k; b < np; b += 8) sum += part[(size_t)b * kPad + i];
+    }
+    red[k][lane] = sum;
+    __syncthreads();
+    if (k == 1 && blockIdx.x == 0) {
+        float l = 0.f;
+        for (int b = lane; b < np; b += 32) l += lpart[b];
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) l += __shfl_xor_sync(0xffffffffu, l, o);
+        if (lane == 0) *loss += l;
+    }
+    if (k != 0 || i >= kPad) return;
+    float gi = 0.f;
+#pragma unroll
+    for (int j = 0; j < 8; j++) gi += red[j][lane];
+    if (!kAdam) {
+        grad[i] = gi;
         return;
     }
-    const float gi = grad[i];
-    const float mi = 0.9f * m[i] + 0.1f * gi;
-    const float vi = 0.999f * v[i] + 0.001f * gi * gi;
-    m[i] = mi;
-    v[i] = vi;
-    const float wi = w[i] - lr * (mi / c1) / (sqrtf(vi / c2) + 1e-8f);
+    const bool pad = (i < kB1 && (i - kW1) / 64 >= 12) || (i >= kW4 && i < kB4 && (i - kW4) % 8 >= 3) ||
+                     (i >= kB4 && i - kB4 >= 3);
+    float wi = 0.f;
+    if (!pad) {
+        const float mi = 0.9f * m[i] + 0.1f * gi;
+        const float vi = 0.999f * v[i] + 0.001f * gi * gi;
+        m[i] = mi;
+        v[i] = vi;
+        wi = w[i] - lr * (mi / c1) / (sqrtf(vi / c2) + 1e-8f);
+    }
     w[i] = wi;
-    wbf[i] = __float2bfloat16_rn(wi);
+    put_weight(*tw, i, wi);
 }
 
-__global__ void k_mlp_to_bf16(const float* __restrict__ w, __nv_bfloat16* __restrict__ wbf) {
+__global__ void k_mlp_train_weights(const float* __restrict__ w, TrainW* __restrict__ tw) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < kPad) wbf[i] = __float2bfloat16_rn(w[i]);
+    if (i < kPad) put_weight(*tw, i, w[i]);
 }
 
 // ---- FP32 debug gradient (canonical layout, no BF16 rounding) ----
@@ -631,26 +730,42 @@ void from_padded(const float* p, float* c) {
     }
 }
 
-size_t train_smem_bytes() { return sizeof(TrainSmem); }
+size_t train_weights_bytes() { return sizeof(TrainW); }
 
-// Gradient (padded; zeroed first) of the mean squared error of the rows
-// idx[0..n) with n_total as the mean's denominator; the summed squared
-// error is added to *loss.  Device pointers; async on s.
-cudaError_t grad_async(const void* wbf, const float* wf, const float* X, const float* Y,
-                       const int32_t* idx, int n, int n_total, float* grad, float* loss,
-                       cudaStream_t s) {
-    static bool attr = false;
-    if (!attr) {
-        cudaError_t e = cudaFuncSetAttribute(k_mlp_grad, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             (int)sizeof(TrainSmem));
-        if (e != cudaSuccess) return e;
-        attr = true;
-    }
-    cudaMemsetAsync(grad, 0, sizeof(float) * kPad, s);
-    const int tiles = (n + 15) / 16;
-    const int blocks = std::max(1, std::min((tiles + kWarps - 1) / kWarps, 2 * 152));
-    k_mlp_grad<<<blocks, kWarps * 32, sizeof(TrainSmem), s>>>(
-        static_cast<const __nv_bfloat16*>(wbf), wf, X, Y, idx, n, n_total, grad, loss);
+int grad_blocks(int n) { return std::max(1, std::min((n - 1) / kRows + 1, kMaxPartials)); }
+
+size_t grad_part_floats(int n) { return (size_t)grad_blocks(n) * (kPad + 1); }
+
+// The blocks' parts of the gradient of the mean squared error of the rows
+// idx[0..n), with n_total as the mean's denominator, and their squared errors
+// behind them.
+static cudaError_t grad_parts(const void* tw, const float* wf, const float* X, const float* Y, const int32_t* idx,
+                              int n, int n_total, float* part, cudaStream_t s) {
+    const int nb = grad_blocks(n);
+    k_mlp_grad<<<nb, 256, 0, s>>>(static_cast<const TrainW*>(tw), wf, X, Y, idx, n, n_total, part,
+                                  part + (size_t)nb * kPad);
+    return cudaGetLastError();
+}
+
+cudaError_t grad_async(const void* tw, const float* wf, const float* X, const float* Y, const int32_t* idx, int n,
+                       int n_total, float* part, float* grad, float* loss, cudaStream_t s) {
+    const cudaError_t e = grad_parts(tw, wf, X, Y, idx, n, n_total, part, s);
+    if (e != cudaSuccess) return e;
+    const int nb = grad_blocks(n);
+    k_mlp_update<false><<<(kPad + 31) / 32, 256, 0, s>>>(part, part + (size_t)nb * kPad, nb, loss, grad, nullptr,
+                                                         nullptr, nullptr, nullptr, 0.f, 1.f, 1.f);
+    return cudaGetLastError();
+}
+
+cudaError_t adam_step_async(float* w, float* m, float* v, void* tw, const float* X, const float* Y,
+                            const int32_t* idx, int n, float lr, int step, float* part, float* loss,
+                            cudaStream_t s) {
+    const cudaError_t e = grad_parts(tw, w, X, Y, idx, n, n, part, s);
+    if (e != cudaSuccess) return e;
+    const int nb = grad_blocks(n);
+    const float c1 = 1.f - powf(0.9f, (float)step), c2 = 1.f - powf(0.999f, (float)step);
+    k_mlp_update<true><<<(kPad + 31) / 32, 256, 0, s>>>(part, part + (size_t)nb * kPad, nb, loss, nullptr, w, m, v,
+                                                        static_cast<TrainW*>(tw), lr, c1, c2);
     return cudaGetLastError();
 }
 
@@ -661,15 +776,9 @@ cudaError_t grad_f32_async(const float* w, const float* X, const float* Y, int n
     return cudaGetLastError();
 }
 
-void adam_async(float* w, float* m, float* v, const float* grad, void* wbf, float lr, int step,
-                cudaStream_t s) {
-    const float c1 = 1.f - powf(0.9f, (float)step), c2 = 1.f - powf(0.999f, (float)step);
-    k_mlp_adam<<<(kPad + 255) / 256, 256, 0, s>>>(w, m, v, grad, static_cast<__nv_bfloat16*>(wbf),
-                                                  lr, c1, c2);
-}
-
-void to_bf16_async(const float* w, void* wbf, cudaStream_t s) {
-    k_mlp_to_bf16<<<(kPad + 255) / 256, 256, 0, s>>>(w, static_cast<__nv_bfloat16*>(wbf));
+void train_weights_async(const float* w, void* tw, cudaStream_t s) {
+    cudaMemsetAsync(tw, 0, sizeof(TrainW), s);   // the rows of W4^T's tiles beyond the 8 outputs
+    k_mlp_train_weights<<<(kPad + 255) / 256, 256, 0, s>>>(w, static_cast<TrainW*>(tw));
 }
 
 }  // namespace mlp
