@@ -11,6 +11,7 @@
 #include <algorithm>
 #include <climits>
 #include <cstddef>
+#include <type_traits>
 
 #include "rb_internal.cuh"
 
@@ -34,22 +35,31 @@ __device__ __forceinline__ uint64_t spread3(uint32_t v) {
 // both have the same floor.  For k in [1, 2^21) the floor and that distance
 // are read from k's bits with integer operations: on GB300 an FP64
 // instruction holds the SM's FP64 pipe 16 cycles per warp, and this kernel's
-// time is its FP64 instructions.  Other k and the few near a grid line take
-// the FP64 division.
-__device__ __forceinline__ uint32_t icoord(double x, double lo, double L, double scale) {
-    const double d = __dsub_rn(x, lo);
+// time is its FP64 instructions.  Other k and the few near a grid line (returns
+// false) take the FP64 division.
+__device__ __forceinline__ bool icoord_fast(double d, double scale, uint32_t& v) {
     const uint64_t b = (uint64_t)__double_as_longlong(__dmul_rn(d, scale));
     const int e = (int)(b >> 52) - 1023;   // unbiased exponent (sign set or NaN: e > 20)
-    if (e >= 0 && e <= 20) {
-        const int sh = 52 - e;             // fraction bits of k
-        const uint64_t m = (b & 0xfffffffffffffull) | (1ull << 52);
-        const uint64_t one = 1ull << sh, fr = m & (one - 1), tol = 1ull << (sh - 23);
-        if (fr >= tol && one - fr >= tol) return (uint32_t)(m >> sh);
-    }
+    const int sh = 52 - min(max(e, 0), 20);   // fraction bits of k
+    const uint64_t m = (b & 0xfffffffffffffull) | (1ull << 52);
+    const uint64_t one = 1ull << sh, fr = m & (one - 1), tol = 1ull << (sh - 23);
+    v = (uint32_t)(m >> sh);
+    return e >= 0 && e <= 20 && fr >= tol && one - fr >= tol;
+}
+
+__device__ __forceinline__ uint32_t icoord_div(double d, double L) {
     double k = floor(__dmul_rn(__ddiv_rn(d, L), 2097152.0));
     if (!(k >= 0.0)) k = 0.0;
     if (k > 2097151.0) k = 2097151.0;
     return (uint32_t)k;
+}
+
+__device__ __forceinline__ uint64_t morton(uint32_t x, uint32_t y, uint32_t z) {
+    return (spread3(x) << 2) | (spread3(y) << 1) | spread3(z);
+}
+
+__device__ __noinline__ uint64_t key_div(double dx, double dy, double dz, double L) {
+    return morton(icoord_div(dx, L), icoord_div(dy, L), icoord_div(dz, L));
 }
 
 // Order-preserving integer image of a double: for a, b not NaN (and -0 not
@@ -66,14 +76,15 @@ __device__ __forceinline__ bool finite_bits(double v) {
     return ((__double_as_longlong(v) >> 52) & 0x7ff) != 0x7ff;
 }
 
-__device__ __forceinline__ double time_at(const Ctl* ctl, const SimC& C, int hs) {
+__device__ __forceinline__ double time_at(const Ctl* ctl, int hs, double t0, double half_dt) {
     const double h = (double)(2 * ctl->step + hs);
-    return __dadd_rn(C.t0, __dmul_rn(h, C.half_dt));
+    return __dadd_rn(t0, __dmul_rn(h, half_dt));
 }
 
+template <bool kSei>
 __device__ __forceinline__ void drift_one(const SimC& C, double& x, double& y, double& z,
                                           double& vx, double& vy, double& vz) {
-    if (C.integrator == 0) {
+    if (!kSei) {
         x = __dadd_rn(x, __dmul_rn(vx, C.half_dt));
         y = __dadd_rn(y, __dmul_rn(vy, C.half_dt));
         z = __dadd_rn(z, __dmul_rn(vz, C.half_dt));
@@ -93,44 +104,62 @@ __device__ __forceinline__ void drift_one(const SimC& C, double& x, double& y, d
 // that would need more than this many is reported as a runaway.
 constexpr int kMaxWraps = 1 << 12;
 
-// Boundaries after a drift half; returns false if the particle left an open
-// boundary.  *runaway is set when the wraps did not bring it back.
-__device__ __forceinline__ bool wrap_one(const SimC& C, const BoxP& bp, const Ctl* ctl, int hs, double& x,
-                                         double& y, double& z, double& vy, bool* runaway) {
+// Boundaries of a particle outside its box.
+struct Wrapped {
+    double x, y, z, vy;
+    bool live, runaway;
+};
+__device__ __noinline__ Wrapped wrap_outside(const BoxP* box, bool z_periodic, const Ctl* ctl, int hs, double t0,
+                                             double half_dt, double x, double y, double z, double vy) {
+    const BoxP bp = *box;
     const int64_t ux = dord(bp.hx), uy = dord(bp.hy), uz = dord(bp.hz);   // ~u is -h
-    if (C.boundary == 0) {
-        const int64_t ox = dord(x), oy = dord(y), oz = dord(z);
-        return !(ox < ~ux || ox >= ux || oy < ~uy || oy >= uy || oz < ~uz || oz >= uz);
-    }
+    Wrapped w{x, y, z, vy, true, false};
     const double vs = bp.shear_speed;
     const int64_t ox = dord(x);
     const bool up = ox >= ux, down = ox < ~ux;
     // the shear offset only for the few particles that cross in x
-    const double s = (up || down) && (__double_as_longlong(vs) << 1) != 0
-                         ? fmod(__dmul_rn(vs, time_at(ctl, C, hs)), bp.Ly)
-                         : 0.0;
+    const double s = (up || down) && vs != 0.0 ? fmod(__dmul_rn(vs, time_at(ctl, hs, t0, half_dt)), bp.Ly) : 0.0;
     if (up) {
-        x = __dsub_rn(x, bp.Lx);
-        y = __dadd_rn(y, s);
-        vy = __dadd_rn(vy, vs);
+        w.x = __dsub_rn(x, bp.Lx);
+        w.y = __dadd_rn(y, s);
+        w.vy = __dadd_rn(vy, vs);
     } else if (down) {
-        x = __dadd_rn(x, bp.Lx);
-        y = __dsub_rn(y, s);
-        vy = __dsub_rn(vy, vs);
+        w.x = __dadd_rn(x, bp.Lx);
+        w.y = __dsub_rn(y, s);
+        w.vy = __dsub_rn(vy, vs);
     }
-    for (int k = 0; k < kMaxWraps && dord(y) >= uy; k++) y = __dsub_rn(y, bp.Ly);
-    for (int k = 0; k < kMaxWraps && dord(y) < ~uy; k++) y = __dadd_rn(y, bp.Ly);
-    const int64_t oy = dord(y);
-    if (oy >= uy || oy < ~uy) *runaway = true;
-    if (C.z_periodic) {
-        for (int k = 0; k < kMaxWraps && dord(z) >= uz; k++) z = __dsub_rn(z, bp.Lz);
-        for (int k = 0; k < kMaxWraps && dord(z) < ~uz; k++) z = __dadd_rn(z, bp.Lz);
-        const int64_t oz = dord(z);
-        if (oz >= uz || oz < ~uz) *runaway = true;
-        return true;
+    for (int k = 0; k < kMaxWraps && dord(w.y) >= uy; k++) w.y = __dsub_rn(w.y, bp.Ly);
+    for (int k = 0; k < kMaxWraps && dord(w.y) < ~uy; k++) w.y = __dadd_rn(w.y, bp.Ly);
+    const int64_t oy = dord(w.y);
+    if (oy >= uy || oy < ~uy) w.runaway = true;
+    if (z_periodic) {
+        for (int k = 0; k < kMaxWraps && dord(w.z) >= uz; k++) w.z = __dsub_rn(w.z, bp.Lz);
+        for (int k = 0; k < kMaxWraps && dord(w.z) < ~uz; k++) w.z = __dadd_rn(w.z, bp.Lz);
     }
-    const int64_t oz = dord(z);
-    return !(oz < ~uz || oz >= uz);
+    const int64_t oz = dord(w.z);
+    const bool out = oz < ~uz || oz >= uz;
+    if (z_periodic) w.runaway |= out;
+    else w.live = !out;
+    return w;
+}
+
+// Boundaries after a drift half; returns false if the particle left an open
+// boundary.  *runaway is set when the wraps did not bring it back.  Most
+// particles are inside and take no FP64 instruction here; with the wraps
+// inlined, 7 were issued (predicated off) for every particle.
+__device__ __forceinline__ bool wrap_one(const SimC& C, const BoxP& bp, const BoxP* box, const Ctl* ctl, int hs,
+                                         double& x, double& y, double& z, double& vy, bool* runaway) {
+    const int64_t ux = dord(bp.hx), uy = dord(bp.hy), uz = dord(bp.hz);   // ~u is -h
+    const int64_t ox = dord(x), oy = dord(y), oz = dord(z);
+    const bool in = ox >= ~ux && ox < ux && oy >= ~uy && oy < uy && oz >= ~uz && oz < uz;
+    if (in || C.boundary == 0) return in;
+    const Wrapped w = wrap_outside(box, C.z_periodic, ctl, hs, C.t0, C.half_dt, x, y, z, vy);
+    x = w.x;
+    y = w.y;
+    z = w.z;
+    vy = w.vy;
+    if (w.runaway) *runaway = true;
+    return w.live;
 }
 
 struct DriftArgs {
@@ -142,13 +171,15 @@ struct DriftArgs {
     const BoxP* boxes;
     const double *ax, *ay, *az;
     int ncap, ndrift, hs;
-    bool kick;
 };
 
-// Optional kick (v += a dt), one or two drift halves each followed by the
-// boundaries, then, for the drifts that a sort follows (kKeys), the Morton key
-// of the new position.
-template <bool kKeys>
+// Optional kick (v += a dt, kKick), one or two drift halves (kSei: Hill's
+// equations) each followed by the boundaries, then, for the drifts that a sort
+// follows (kKeys), the Morton key of the new position.  The time is the FP64
+// pipe's: a SEI half with its key issues 36 FP64 instructions per warp (63 with
+// the rare paths and the run-time options inlined).  1M particles of the sheet:
+// 103 -> 79 us with keys, 93 -> 76 us for the kick and drift.
+template <bool kKeys, bool kKick, bool kSei>
 __global__ void __launch_bounds__(256) k_drift_keys(DriftArgs A, SimC C) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= A.ncap) return;
@@ -159,15 +190,15 @@ __global__ void __launch_bounds__(256) k_drift_keys(DriftArgs A, SimC C) {
         double x = A.P.x[i], y = A.P.y[i], z = A.P.z[i];
         double vx = A.P.vx[i], vy = A.P.vy[i], vz = A.P.vz[i];
         const BoxP bp = A.boxes[A.P.box[i]];
-        if (A.kick) {
+        if (kKick) {
             vx = __dadd_rn(vx, __dmul_rn(A.ax[i], C.dt));
             vy = __dadd_rn(vy, __dmul_rn(A.ay[i], C.dt));
             vz = __dadd_rn(vz, __dmul_rn(A.az[i], C.dt));
         }
         bool runaway = false;
         for (int d = 0; d < A.ndrift && live; d++) {
-            drift_one(C, x, y, z, vx, vy, vz);
-            live = wrap_one(C, bp, A.ctl, A.hs + d, x, y, z, vy, &runaway);
+            drift_one<kSei>(C, x, y, z, vx, vy, vz);
+            live = wrap_one(C, bp, &A.boxes[A.P.box[i]], A.ctl, A.hs + d, x, y, z, vy, &runaway);
         }
         if (runaway || !(finite_bits(x) && finite_bits(y) && finite_bits(z))) {
             atomicOr(&A.ctl->err, kErrNonFinite);
@@ -177,9 +208,11 @@ __global__ void __launch_bounds__(256) k_drift_keys(DriftArgs A, SimC C) {
         A.P.vx[i] = vx; A.P.vy[i] = vy; A.P.vz[i] = vz;
         if (kKeys && live) {
             const double lo = -bp.hx;   // the root cube's side L is Lx
-            key = (spread3(icoord(x, lo, bp.L, bp.key_scale)) << 2) |
-                  (spread3(icoord(y, lo, bp.L, bp.key_scale)) << 1) |
-                  spread3(icoord(z, lo, bp.L, bp.key_scale));
+            const double dx = __dsub_rn(x, lo), dy = __dsub_rn(y, lo), dz = __dsub_rn(z, lo);
+            uint32_t kx, ky, kz;
+            const bool fx = icoord_fast(dx, bp.key_scale, kx), fy = icoord_fast(dy, bp.key_scale, ky);
+            const bool fz = icoord_fast(dz, bp.key_scale, kz);
+            key = fx && fy && fz ? morton(kx, ky, kz) : key_div(dx, dy, dz, bp.L);
         }
     }
     if (!live) A.P.box[i] = C.nbox;
@@ -482,9 +515,17 @@ void drift_keys(const PSet& P, const Tree& T, Ctl* ctl, const BoxP* boxes, const
     DriftArgs A;
     A.P = P; A.key = T.key; A.idx = T.idx; A.sbox = T.sbox; A.ctl = ctl; A.boxes = boxes;
     A.ax = ax; A.ay = ay; A.az = az;
-    A.ncap = ncap; A.ndrift = ndrift; A.hs = half_step_offset; A.kick = kick;
-    if (keys) k_drift_keys<true><<<ceil_div(ncap, 256), 256, 0, s>>>(A, C);
-    else k_drift_keys<false><<<ceil_div(ncap, 256), 256, 0, s>>>(A, C);
+    A.ncap = ncap; A.ndrift = ndrift; A.hs = half_step_offset;
+    const int grid = ceil_div(ncap, 256);
+    auto launch = [&](auto k, auto d) {
+        if (C.integrator == 0) k_drift_keys<k, d, false><<<grid, 256, 0, s>>>(A, C);
+        else k_drift_keys<k, d, true><<<grid, 256, 0, s>>>(A, C);
+    };
+    using std::bool_constant;
+    if (keys && kick) launch(bool_constant<true>{}, bool_constant<true>{});
+    else if (keys) launch(bool_constant<true>{}, bool_constant<false>{});
+    else if (kick) launch(bool_constant<false>{}, bool_constant<true>{});
+    else launch(bool_constant<false>{}, bool_constant<false>{});
 }
 
 // Morton bits below those that the passes sort.
