@@ -224,7 +224,6 @@ int alloc_pairs(rb_sim* s, int cap) {
     rc |= dalloc(s, &R.head, s->ncap, L);
     rc |= dalloc(s, &R.link, cap, L);
     rc |= dalloc(s, &R.done, cap, L);
-    rc |= dalloc(s, &R.rec, cap, L);
     rc |= dalloc(s, &R.claim, 1, L);
     rc |= dalloc(s, &R.hist, radix_hist_words(cap), L);
     R.slot_of_id = keep_slot;

@@ -154,22 +154,12 @@ struct Tree {
 // Target orders of the walk and search tiles (the values of RB_TILE_*).
 enum { kTileMorton = 0, kTileHilbertXY = 1, kTileHilbertXYZ = 2 };
 
-// A collision pair as the resolution reads it: separation (image of b) - a,
-// the image's y velocity offset, the factors of u.r that v_a gains and v_b
-// loses along it, the particles' slots, and the pairs that must come before.
-struct __align__(64) PairRec {
-    double rx, ry, rz, dvy, ka, kb;
-    int a, b;
-    int pa, pb;   // previous pair of particle a / b in resolution order, or -1
-};
-
 // Pairs and their resolution.
 struct Pairs {
     uint64_t *key, *key_alt;
     uint32_t *val, *val_alt;   // unused payload for the sort
     int32_t *head, *link;      // pairs of each particle as the higher id (lists; head: one per id)
     int32_t* done;             // per pair: resolved
-    PairRec* rec;              // per pair: geometry, impulse factors, predecessors
     int32_t* claim;            // pairs claimed so far by the resolving warps
     int32_t* slot_of_id;       // global id -> slot in the current set
     uint32_t* hist;

@@ -252,7 +252,6 @@ struct ResolveArgs {
     const int32_t* slot_of_id;
     int32_t *head, *link;         // per particle: its pairs as the higher id, a list in any order
     int32_t* done;                // per pair: 1 once resolved
-    PairRec* rec;
     int32_t* claim;               // pairs claimed by running warps
     Ctl* ctl;
     const ImgTab* img;            // [box][image] offsets at the detection time
@@ -298,42 +297,50 @@ __device__ __forceinline__ int last_before(const ResolveArgs& A, int p, int k) {
 
 // Everything about a pair that does not depend on velocities: the separation
 // vector, the impulse factors of Eq. 2, and the previous pair in resolution
-// order of either particle.  The queue is sorted by (a, b), a < b, so a
-// particle's pairs as the higher id come before its pairs as the lower one:
-// b's previous pair is one in its list, a's is the pair before this one if
-// that has the same a, else the last one in a's list.
-__global__ void __launch_bounds__(256) k_pair_rec(ResolveArgs A, SimC C) {
-    const int n = A.ctl->pair_n;
-    for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < n; k += gridDim.x * blockDim.x) {
-        const uint64_t key = A.key[k];
-        const int ia = key_a(key), ib = key_b(key), code = (int)(key & 0xFFFull);
-        const int gx = (code & 15) - 7, gy = ((code >> 4) & 15) - 7, gz = ((code >> 8) & 15) - 7;
-        const int g = ((gx + A.ngx) * (2 * A.ngy + 1) + (gy + A.ngy)) * (2 * A.ngz + 1) + (gz + A.ngz);
-        PairRec R;
-        R.a = A.slot_of_id[ia];
-        R.b = A.slot_of_id[ib];
-        const ImgTab& T = A.img[(size_t)A.P.box[R.a] * A.nimg + g];
-        R.rx = __dsub_rn(__dadd_rn(A.P.x[R.b], T.ox), A.P.x[R.a]);
-        R.ry = __dsub_rn(__dadd_rn(A.P.y[R.b], T.oy), A.P.y[R.a]);
-        R.rz = __dsub_rn(__dadd_rn(A.P.z[R.b], T.oz), A.P.z[R.a]);
-        R.dvy = T.dvy;
-        // the impulse along n = r/|r| without forming n: v_a gains
-        // (1 + eps) (m_b/M) (u.r)/|r|^2 r, v_b loses the same with m_a; the
-        // factors of u.r here, but for 1 + eps under the power law
-        const double r2 = fma(R.rz, R.rz, fma(R.ry, R.ry, R.rx * R.rx));
-        const double ma = A.P.m[R.a], mb = A.P.m[R.b];
-        const double d = r2 * (ma + mb);
-        const double y = rcp64(d);
-        const double num = C.eps_law == 1 ? 1.0 : 1.0 + C.eps;
-        double q = num * y;
-        q = fma(fma(-d, q, num), y, q);   // num / d to the last bit or so
-        R.ka = q * mb;
-        R.kb = q * ma;
-        R.pb = last_before(A, ib, k);
-        R.pa = k > 0 && key_a(A.key[k - 1]) == ia ? k - 1 : last_before(A, ia, k);
-        if (C.hold_pair && k == 0) R.pa = 0;   // test hook: waits for itself
-        A.rec[k] = R;
-    }
+// order of either particle.
+struct PairRec {
+    double rx, ry, rz, dvy;   // separation (with the image offset), velocity offset of the image
+    double ka, kb;            // impulse factors of u.r (of 1 + eps too, with a constant eps)
+    double rabs;              // power law: |r|
+    int32_t a, b;             // slots
+    int32_t pa, pb;           // previous pair of either particle, or -1
+};
+
+// The queue is sorted by (a, b), a < b, so a particle's pairs as the higher id
+// come before its pairs as the lower one: b's previous pair is one in its
+// list, a's is the pair before this one if that has the same a, else the last
+// one in a's list.
+template <bool kPower>
+__device__ __forceinline__ PairRec pair_rec(const ResolveArgs& A, const SimC& C, int k) {
+    const uint64_t key = A.key[k];
+    const int ia = key_a(key), ib = key_b(key), code = (int)(key & 0xFFFull);
+    const int gx = (code & 15) - 7, gy = ((code >> 4) & 15) - 7, gz = ((code >> 8) & 15) - 7;
+    const int g = ((gx + A.ngx) * (2 * A.ngy + 1) + (gy + A.ngy)) * (2 * A.ngz + 1) + (gz + A.ngz);
+    PairRec R;
+    R.a = A.slot_of_id[ia];
+    R.b = A.slot_of_id[ib];
+    const ImgTab& T = A.img[(size_t)A.P.box[R.a] * A.nimg + g];
+    R.rx = __dsub_rn(__dadd_rn(A.P.x[R.b], T.ox), A.P.x[R.a]);
+    R.ry = __dsub_rn(__dadd_rn(A.P.y[R.b], T.oy), A.P.y[R.a]);
+    R.rz = __dsub_rn(__dadd_rn(A.P.z[R.b], T.oz), A.P.z[R.a]);
+    R.dvy = T.dvy;
+    // the impulse along n = r/|r| without forming n: v_a gains
+    // (1 + eps) (m_b/M) (u.r)/|r|^2 r, v_b loses the same with m_a; the
+    // factors of u.r here, but for 1 + eps under the power law
+    const double r2 = fma(R.rz, R.rz, fma(R.ry, R.ry, R.rx * R.rx));
+    const double ma = A.P.m[R.a], mb = A.P.m[R.b];
+    const double d = r2 * (ma + mb);
+    const double y = rcp64(d);
+    const double num = kPower ? 1.0 : 1.0 + C.eps;
+    double q = num * y;
+    q = fma(fma(-d, q, num), y, q);   // num / d to the last bit or so
+    R.ka = q * mb;
+    R.kb = q * ma;
+    R.rabs = kPower ? __dsqrt_rn(r2) : 0.0;
+    R.pb = last_before(A, ib, k);
+    R.pa = k > 0 && key_a(A.key[k - 1]) == ia ? k - 1 : last_before(A, ia, k);
+    if (C.hold_pair && k == 0) R.pa = 0;   // test hook: waits for itself
+    return R;
 }
 
 constexpr unsigned long long kWaitLimitNs = 500000000ull;   // half a second
@@ -351,8 +358,8 @@ __device__ __forceinline__ int ld_flag(const int32_t* p) {
 }
 
 // Eq. 2 for every pair, as if one after the other in queue order.  Warps claim
-// 32 pairs at a time in that order, each lane holds one, with its record
-// already read, and resolves it as soon as the previous pair of either
+// 32 pairs at a time in that order, each lane forms the record of one (while
+// the pairs before it are being resolved) and resolves it as soon as the previous pair of either
 // particle is marked done: it reads the velocities from L2, where the other
 // SMs left them, writes the new ones and marks its own pair (release).  A
 // lane's predecessors come earlier in the queue, so they are held by running
@@ -362,10 +369,12 @@ __device__ __forceinline__ int ld_flag(const int32_t* p) {
 // another thread gave up) and reports kErrResolveStall.
 // What bounds it is the chain of dependent pairs, one link at a time: a flag
 // read, a velocity read, 15 FP64 operations, and a release after the
-// velocities have reached L2.  The whole resolution, links and records
-// included: 53 us for 2,233 pairs and 231 us for 944k, against 144 and 452 us
-// with a queue of ready pairs, wait counts and a sort of the pair ends (six
-// dependent round trips and 60 FP64 operations a link).
+// velocities have reached L2.  The whole resolution, links included: 47 us for
+// 2,233 pairs and 203 us for 944k (50 and 228 us with the records formed by a
+// kernel of their own and read back), against 144 and 452 us with a queue of
+// ready pairs, wait counts and a sort of the pair ends (six dependent round
+// trips and 60 FP64 operations a link).  With 944k pairs the FP64 pipe is busy
+// three quarters of the time: a warp evaluates its 32 pairs in about 4 rounds.
 template <bool kPower>
 __global__ void __launch_bounds__(256) k_resolve(ResolveArgs A, SimC C) {
     if (A.advance && blockIdx.x == 0 && threadIdx.x == 0) A.ctl->step += 1;   // nothing here reads the time
@@ -380,7 +389,7 @@ __global__ void __launch_bounds__(256) k_resolve(ResolveArgs A, SimC C) {
         const int k = base + lane;
         bool pending = k < n, stalled = false;
         PairRec R;
-        if (pending) R = A.rec[k];
+        if (pending) R = pair_rec<kPower>(A, C, k);
         unsigned long long t0 = 0;
         int seen = 0;
         for (int spin = 0; __any_sync(0xffffffffu, pending); spin++) {
@@ -400,10 +409,9 @@ __global__ void __launch_bounds__(256) k_resolve(ResolveArgs A, SimC C) {
                         double g = rv;
                         if (kPower) {
                             // velocity-dependent restitution: min(1, (|v_n| / v_c)^(-p)),
-                            // |v_n| = |u.r| / |r|
-                            const double r2 = fma(R.rz, R.rz, fma(R.ry, R.ry, R.rx * R.rx));
-                            const double vn = __ddiv_rn(rv, __dsqrt_rn(r2));
-                            const double q = pow(__ddiv_rn(fabs(vn), C.eps_vc), -C.eps_p);
+                            // |v_n| = |u.r| / |r|; 1 up to v_c (p is not negative)
+                            const double v = __ddiv_rn(__ddiv_rn(fabs(rv), R.rabs), C.eps_vc);
+                            const double q = v > 1.0 ? pow(v, -C.eps_p) : 1.0;
                             g = (1.0 + (q < 1.0 ? q : 1.0)) * rv;
                         }
                         const double ga = g * R.ka, gb = g * R.kb;
@@ -660,7 +668,7 @@ void resolve_pairs(const PSet& P, Ctl* ctl, const BoxP* boxes, const SimC& C, Pa
                    int half_step_offset, ImgTab* img, bool have_img, bool advance, cudaStream_t s) {
     ResolveArgs A;
     A.P = P; A.key = PR.sorted(); A.slot_of_id = PR.slot_of_id;
-    A.head = PR.head; A.link = PR.link; A.done = PR.done; A.rec = PR.rec; A.claim = PR.claim;
+    A.head = PR.head; A.link = PR.link; A.done = PR.done; A.claim = PR.claim;
     A.img = img;
     A.ngx = C.ngx; A.ngy = C.ngy; A.ngz = C.ngz;
     A.nimg = have_img ? C.nimg : build_image_table(boxes, ctl, C, half_step_offset, img, s);
@@ -669,7 +677,6 @@ void resolve_pairs(const PSet& P, Ctl* ctl, const BoxP* boxes, const SimC& C, Pa
     cudaMemsetAsync(PR.head, 0xff, sizeof(int32_t) * (size_t)PR.ncap, s);   // empty lists
     const int grid = std::min(ceil_div(PR.cap, 256), 8 * 152);
     k_pair_link<<<grid, 256, 0, s>>>(A);
-    k_pair_rec<<<grid, 256, 0, s>>>(A, C);
     const int rgrid = std::max(1, std::min(ceil_div(PR.cap, 256), g_resolve_blocks[C.eps_law == 1]));
     if (C.eps_law == 1) k_resolve<true><<<rgrid, 256, 0, s>>>(A, C);
     else k_resolve<false><<<rgrid, 256, 0, s>>>(A, C);
