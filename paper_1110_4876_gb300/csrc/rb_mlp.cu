@@ -39,10 +39,10 @@ constexpr int kMaxPartials = 152; // blocks of the gradient kernel, one per SM
 constexpr int kLdH = 72;          // row strides (BF16) of the staged activations and
 constexpr int kLdX = 24;          // inputs: ldmatrix reads 8 rows without bank conflicts
 
-// BF16 weights of training as mma B fragments (as in Packed): F1..F4 those of
-// the forward pass, T4..T2 the tiles of W4^T, W3^T and W2^T that take an output
-// gradient back to the layer below (B[k][n] = W[n][k]).  One 8-byte load per
-// lane and MMA, straight into registers.
+// BF16 weights of training as mma B fragments, an entry per MMA and lane: F1..F4
+// those of the forward pass, T4..T2 the tiles of W4^T, W3^T and W2^T that take
+// an output gradient back to the layer below (B[k][n] = W[n][k]).  One 8-byte
+// load per lane and MMA, straight into registers.
 struct TrainW {
     uint2 F1[1][8][32], F2[4][8][32], F3[4][8][32], F4[4][1][32];
     uint2 T4[1][8][32], T3[4][8][32], T2[4][8][32];
@@ -664,14 +664,14 @@ __global__ void k_mlp_pack(const float* __restrict__ w, Packed* __restrict__ P) 
         int k = i, off, ld, nt;
         uint2* dst;
         if (k < n1) {
-            off = kW1; ld = 64; nt = 8; dst = &P->B1[0][0][0];
+            off = kW1; ld = 64; nt = 8; dst = reinterpret_cast<uint2*>(P->B1);
         } else if ((k -= n1) < n2) {
-            off = kW2; ld = 64; nt = 8; dst = &P->B2[0][0][0];
+            off = kW2; ld = 64; nt = 8; dst = reinterpret_cast<uint2*>(P->B2);
         } else if ((k -= n2) < n2) {
-            off = kW3; ld = 64; nt = 8; dst = &P->B3[0][0][0];
+            off = kW3; ld = 64; nt = 8; dst = reinterpret_cast<uint2*>(P->B3);
         } else {
             k -= n2;
-            off = kW4; ld = 8; nt = 1; dst = &P->B4[0][0][0];
+            off = kW4; ld = 8; nt = 1; dst = reinterpret_cast<uint2*>(P->B4);
         }
         const int lane = k & 31, tile = k >> 5, t = tile / nt, j = tile % nt;
         const int g = lane >> 2, q = lane & 3, r = 16 * t + 2 * q, c = 8 * j + g;
@@ -679,7 +679,7 @@ __global__ void k_mlp_pack(const float* __restrict__ w, Packed* __restrict__ P) 
         uint2 b;
         b.x = pack2(W[r * ld + c], W[(r + 1) * ld + c]);
         b.y = pack2(W[(r + 8) * ld + c], W[(r + 9) * ld + c]);
-        dst[k] = b;
+        dst[nt == 1 ? k : ((t * 4 + (j >> 1)) * 32 + lane) * 2 + (j & 1)] = b;
     } else if ((i -= n1 + 2 * n2 + n4) < 200) {
         if (i < 64) P->b1[i] = w[kB1 + i];
         else if (i < 128) P->b2[i - 64] = w[kB2 + i - 64];
