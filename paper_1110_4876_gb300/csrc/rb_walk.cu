@@ -970,7 +970,7 @@ void gravity_walk(const Tree& T, const PSet& P, Ctl* ctl, const BoxP* boxes, con
     if (learn && !potential) {
         // FP32 walk with the learned correction of band cells (quadrupole on)
         A.band_scale = learn->band_scale;
-        if (T.cap_n <= kTargetWalkMax) {
+        if (T.cap_n <= kTargetWalkMaxLearned) {
             target_walk(A, TargetWalk::kLearned, true, inside, soft, false, block, T.cap_n, s);
         } else if (inside) {
             if (soft) RB_LAUNCH(k_walk32_learn<true, true>);
@@ -990,7 +990,7 @@ void gravity_walk(const Tree& T, const PSet& P, Ctl* ctl, const BoxP* boxes, con
         }
     } else if (walk_mode == 0 || potential) {
         target_walk(A, TargetWalk::kFp64, quad, inside, soft, potential, block, T.cap_n, s);
-    } else if (group == 0 && T.cap_n <= kTargetWalkMax) {
+    } else if (group == 0 && T.cap_n <= (T.order ? kTargetWalkMax : kTargetWalkMaxMorton)) {
         target_walk(A, TargetWalk::kFp32, quad, inside, soft, false, block, T.cap_n, s);
     } else {
         if (quad) {

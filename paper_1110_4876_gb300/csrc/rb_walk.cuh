@@ -55,14 +55,20 @@ int walk_grid(const void* fn, int block, long long warps);
 
 // rb_twalk.cu: the walks with a warp per target.  A holds the target order,
 // records and image table; block is 64, 128 or 256 threads (FP64).
-// FP32 walks take them up to kTargetWalkMax targets, where the chain of
-// entries that a warp of 32 targets steps through is longer than the work:
-// on the sheet (theta = 0.5, 9 images) 147 us against 319 at 20k targets, 219
-// against 325 at 30k, 276 against 324 at 40k, 347 against 333 at 50k, 409
-// against 361 at 60k and 557 against 367 at 80k (theta = 0.8: 183 against 243
-// at 40k, 260 against 251 at 60k); learned walk (theta = 0.8) 182 against 608
-// at 10k, 752 against 871 at 40k, 1152 against 1070 at 60k.
-constexpr int kTargetWalkMax = 50000;
+// FP32 walks take them up to a number of targets where the chain of entries that
+// a warp of 32 targets steps through is longer than the work.  Walk times on the
+// sheet (theta = 0.5, 9 images, targets in Hilbert order): 147 us against 319 at
+// 20k targets, 219 against 325 at 30k, 276 against 324 at 40k, 347 against 333 at
+// 50k and 409 against 361 at 60k.  In Morton order the 32 targets' walks have
+// less in common: a whole gravity evaluation takes 756 us against 818 at 80k and
+// 909 against 945 at 100k (sheet), 684 against 779 at 60k, 871 against 907 at 80k
+// and 1047 against 945 at 100k (Plummer sphere, theta = 0.8), 1033 against 1314 at
+// 80k (periodic cube).  With the network, whose rows a warp's one target fills
+// better than 32 lanes' band cells in turn: 573 us against 803 at 40k, 1516
+// against 1818 at 100k, 3171 against 2968 at 200k (theta = 0.8).
+constexpr int kTargetWalkMax = 50000;           // targets in a Hilbert order
+constexpr int kTargetWalkMaxMorton = 80000;
+constexpr int kTargetWalkMaxLearned = 130000;
 enum class TargetWalk { kFp32, kFp64, kLearned };
 void target_walk(const GravArgs& A, TargetWalk mode, bool quad, bool inside, bool soft, bool pot, int block,
                  int cap_n, cudaStream_t s);

@@ -10,7 +10,7 @@ from paper_1110_4876_gb300 import inputs as I
 
 pytestmark = pytest.mark.gpu
 
-LARGE = 50_001   # capacity from which the walk over 32 targets per warp runs
+LARGE = 130_001   # capacity from which every walk runs over 32 targets per warp
 
 
 @pytest.fixture(scope="module")
