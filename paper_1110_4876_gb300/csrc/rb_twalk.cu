@@ -1,5 +1,5 @@
-// rb_twalk.cu -- Barnes-Hut gravity walk with one warp per target (Sect. 4.2,
-// Eq. 1): the lanes take the target's cells, not its neighbours.
+// rb_twalk.cu -- Barnes-Hut gravity walk with one warp per target, or for two
+// (Sect. 4.2, Eq. 1): the lanes take the target's cells, not its neighbours.
 //
 // The walks of rb_walk.cu give each lane a target and step the warp through
 // the union of 32 walks, one tree entry after the other: about 700-1200
@@ -24,9 +24,18 @@
 // accepted terms alone are 1.2e9 FP64 lane operations, 1.9 ms at two lanes
 // per SM and clock.
 //
-// FP32, 30,011 targets: 216 us.  283 instructions a round at 64% of the issue
-// slots and 70% of the L1 wavefronts (every lane reads its own 32-byte records;
-// with 256-bit loads a record pair is one wavefront per lane instead of two).
+// FP32: a warp takes two neighbouring targets at once (k_twalk32x2) where there
+// are enough of them to fill the GPU.  An item carries the targets that visit it
+// in its two upper bits; its records are read once for both, whose terms are one
+// packed FP32 operation each, and its children are pushed for the targets that
+// opened it, so each target still tests exactly the entries of its own walk.
+// Neighbours' walks have most entries in common (the rounds of a pair are 1.06
+// times those of one).  One target per warp is bound by instruction issue (64%
+// of the slots) and the L1 wavefronts of its gathers (70%); pairs by the latency
+// of the gathers with 24 warps per SM.  30,011 targets of the sheet: 215 -> 160
+// us, 50,000: 345 -> 250, 5,000: 69 -> 49.  Loading the children before the
+// terms are formed is 5% of that; 16 warps per SM (no spills) take 20% longer,
+// 32 warps 8%.
 #include <algorithm>
 #include <type_traits>
 
@@ -42,6 +51,11 @@ constexpr int kStack = 512;
 constexpr int kReserve = 160;                       // depth-first room: 7 siblings on each of 22 levels
 
 constexpr int kUnit = 8;                            // targets a warp takes from a queue at once, at most
+
+// FP32 targets from which a warp takes two at a time: 39 us both ways at 2,400
+// in Morton order, 29 us for one against 37 for two at 1,000, 50 against 44 at
+// 4,000.
+constexpr int kPairMin = 3000;
 
 struct TSmem32 {
     int stack[kStack];           // (image of the batch << kEntBits) | entry
@@ -313,6 +327,7 @@ __device__ __forceinline__ void walk_target(const GravArgs& A, TSmem<k64>& S, Le
                 e = item & kEntMask;
                 const int g = item >> kEntBits;
                 ld_pair(A.ra, e, ra, rb);
+                if (!k64) ld_pair(A.rq0, e, q0, q1);   // of no meaning for a leaf
                 const float4 t = S.txy[g];
                 const float2 tz = S.tz[g];
                 rec_diff(ra, rb, make_float2(t.x, t.y), make_float2(t.z, t.w), tz, dx, dy, dz, r2);
@@ -355,8 +370,6 @@ __device__ __forceinline__ void walk_target(const GravArgs& A, TSmem<k64>& S, Le
                     if (leaf) {
                         q0 = make_float4(-crit, 0.f, 0.f, 0.f);
                         q1 = make_float4(0.f, 0.f, 0.f, 0.f);
-                    } else {
-                        ld_pair(A.rq0, e, q0, q1);
                     }
                     // a leaf is the cell with Q = 0; its distance may be zero when softened
                     inv = rsqrt_nr(kSoft && leaf ? r2 + A.soft2f : r2);
@@ -567,6 +580,328 @@ __device__ __forceinline__ void target_units(const GravArgs& A, int per, TSmem<k
     }
 }
 
+// ---- two targets per warp (FP32) ----
+
+// An item's upper bits: image of the batch, then the targets that visit it.
+constexpr int kImgBits = 5;
+constexpr unsigned kItemMask = (1u << (kEntBits + kImgBits)) - 1u;   // entry and image
+constexpr int kWhoShift = kEntBits + kImgBits;
+static_assert(kImgBatch <= 1 << kImgBits && kWhoShift == 30, "two bits are left for the targets");
+
+struct PSmem {
+    unsigned stack[kStack];
+    // negated targets of each image: x of both targets hi, then lo; y; z
+    float4 tx[kImgBatch], ty[kImgBatch], tz[kImgBatch];
+    float2 sum[kUnit][3];
+    int cnt[kUnit][4];
+};
+
+// Per-lane sums of a pair of targets (x: the first, y: the second).
+struct PSum {
+    float2 fx, fy, fz;             // plain sums of the last <= 16 rounds
+    float s[2][3], c[2][3];        // Kahan sums of the flushed partial sums
+    int ncell[2], nleaf[2], nmac[2];
+};
+
+__device__ __forceinline__ void psum_flush(PSum& L) {
+    kadd(L.s[0][0], L.c[0][0], L.fx.x);
+    kadd(L.s[0][1], L.c[0][1], L.fy.x);
+    kadd(L.s[0][2], L.c[0][2], L.fz.x);
+    kadd(L.s[1][0], L.c[1][0], L.fx.y);
+    kadd(L.s[1][1], L.c[1][1], L.fy.y);
+    kadd(L.s[1][2], L.c[1][2], L.fz.y);
+    L.fx = L.fy = L.fz = make_float2(0.f, 0.f);
+}
+
+__device__ __forceinline__ float2 two(float v) { return make_float2(v, v); }
+
+// rsqrt_nr of both.
+__device__ __forceinline__ float2 rsqrt2_nr(float2 x) {
+    const float2 y = make_float2(rsqrtf(x.x), rsqrtf(x.y));
+    return __fmul2_rn(y, __ffma2_rn(__fmul2_rn(__fmul2_rn(two(-0.5f), x), y), y, two(1.5f)));
+}
+
+// The records' differences to both targets, as rec_diff forms them.
+__device__ __forceinline__ void rec_diff2(const float4& ra, const float4& rb, const float4& tx, const float4& ty,
+                                          const float4& tz, float2& dx, float2& dy, float2& dz, float2& r2) {
+    dx = __fadd2_rn(__fadd2_rn(two(ra.x), make_float2(tx.x, tx.y)), __fadd2_rn(two(rb.x), make_float2(tx.z, tx.w)));
+    dy = __fadd2_rn(__fadd2_rn(two(ra.y), make_float2(ty.x, ty.y)), __fadd2_rn(two(rb.y), make_float2(ty.z, ty.w)));
+    dz = __fadd2_rn(__fadd2_rn(two(ra.z), make_float2(tz.x, tz.y)), __fadd2_rn(two(ra.w), make_float2(tz.z, tz.w)));
+    r2 = __ffma2_rn(dz, dz, __ffma2_rn(dy, dy, __fmul2_rn(dx, dx)));
+}
+
+// The walk of walk_target for the targets `who` (bit 0: i0, bit 1: i1) of one
+// box, adding to L.
+template <bool kQuad, bool kInside, bool kSoft>
+__device__ __forceinline__ void walk_pair(const GravArgs& A, PSmem& S, int i0, int i1, unsigned who, int box, PSum& L,
+                                          TTotal& N) {
+    const int lane = threadIdx.x & 31;
+    const unsigned lt = (1u << lane) - 1u;
+    const int root = A.box_root[box];
+    if (root < 0) return;
+    const int self0 = A.leaf_of[who & 1u ? i0 : i1], self1 = A.leaf_of[who & 2u ? i1 : i0];
+    const ImgTab* itab = A.img + (size_t)box * A.nimg;
+    const int centre = (A.ngx * (2 * A.ngy + 1) + A.ngy) * (2 * A.ngz + 1) + A.ngz;
+    int rounds = 0;   // warp-uniform
+    for (int g0 = 0; g0 < A.nimg; g0 += kImgBatch) {
+        const int nb = min(kImgBatch, A.nimg - g0);
+        __syncwarp();
+        if (lane < nb) {
+            const ImgTab& T = itab[g0 + lane];
+            const float4 oh = T.hi, ol = T.lo;
+            const float4 pa = A.ra[self0], pb = A.rb[self0], qa = A.ra[self1], qb = A.rb[self1];
+            float h, l, h1, l1;
+            sub_hilo(pa.x, pb.x, oh.x, ol.x, h, l);
+            sub_hilo(qa.x, qb.x, oh.x, ol.x, h1, l1);
+            S.tx[lane] = make_float4(-h, -h1, -l, -l1);
+            sub_hilo(pa.y, pb.y, oh.y, ol.y, h, l);
+            sub_hilo(qa.y, qb.y, oh.y, ol.y, h1, l1);
+            S.ty[lane] = make_float4(-h, -h1, -l, -l1);
+            sub_hilo(pa.z, pa.w, oh.z, ol.z, h, l);
+            sub_hilo(qa.z, qa.w, oh.z, ol.z, h1, l1);
+            S.tz[lane] = make_float4(-h, -h1, -l, -l1);
+            S.stack[lane] = (who << kWhoShift) | ((unsigned)lane << kEntBits) | (unsigned)root;
+        }
+        int fc = nb;   // items on the stack (warp-uniform)
+        // the targets' own leaves are no terms of the central image
+        const bool own = centre >= g0 && centre < g0 + nb;
+        const unsigned own0 = own ? ((unsigned)(centre - g0) << kEntBits) | (unsigned)self0 : ~0u;
+        const unsigned own1 = own ? ((unsigned)(centre - g0) << kEntBits) | (unsigned)self1 : ~0u;
+        while (fc > 0) {
+            const int k = min(min(32, fc), max(1, (kStack - kReserve - fc) / 7));
+            __syncwarp();
+            const unsigned item = lane < k ? S.stack[fc - k + lane] : 0u;
+            fc -= k;
+            __syncwarp();
+            unsigned opened = 0;   // targets that open the item's cell
+            uint32_t cm = 0;
+            int4 clo = make_int4(0, 0, 0, 0), chi = clo;
+            int e = 0;
+            if (item) {
+                e = (int)(item & kEntMask);
+                const int g = (int)((item & kItemMask) >> kEntBits);
+                const bool on0 = item & (1u << kWhoShift), on1 = item & (2u << kWhoShift);
+                float4 ra, rb;
+                ld_pair(A.ra, e, ra, rb);
+                const float4 tx = S.tx[g], ty = S.ty[g], tz = S.tz[g];
+                float2 dx, dy, dz, r2;
+                rec_diff2(ra, rb, tx, ty, tz, dx, dy, dz, r2);
+                const float crit = rb.z;   // leaf: -m; cell: (w / theta)^2
+                const bool leaf = __float_as_int(crit) < 0;
+                bool a0, a1;
+                if (leaf) {
+                    a0 = on0 && (item & kItemMask) != own0;
+                    a1 = on1 && (item & kItemMask) != own1;
+                    L.nleaf[0] += a0;
+                    L.nleaf[1] += a1;
+                } else {
+                    L.nmac[0] += on0;
+                    L.nmac[1] += on1;
+                    const ImgTab& T = itab[g0 + g];
+                    // the FP64 test near the threshold, also when r2 or crit leaves FP32's range
+                    auto accepted = [&](float d2, int i) {
+                        if (fabsf(crit - d2) > fmaf(1e-5f, d2, 1e-35f)) return crit < d2;
+                        N.nrecheck++;
+                        return mac64(ld_d4(&A.d_a[e]), A.theta2, __dsub_rn(A.x[i], T.ox), __dsub_rn(A.y[i], T.oy),
+                                     __dsub_rn(A.z[i], T.oz));
+                    };
+                    a0 = on0 && accepted(r2.x, i0);
+                    a1 = on1 && accepted(r2.y, i1);
+                    if (kInside && (a0 || a1)) {
+                        const float4 ch = __ldg(&A.rc_hi[e]);
+                        const float4 cl = __ldg(&A.rc_lo[e]);
+                        auto outside = [&](float hx, float lx, float hy, float ly, float hz, float lz, int i) {
+                            const float ux = (-hx - ch.x) + (-lx - cl.x);
+                            const float uy = (-hy - ch.y) + (-ly - cl.y);
+                            const float uz = (-hz - ch.z) + (-lz - cl.z);
+                            const float w = ch.w;
+                            const float mx =
+                                fminf(fminf(ux, w - ux), fminf(fminf(uy, w - uy), fminf(uz, w - uz)));
+                            if (fabsf(mx) > fmaf(1e-5f, w, 1e-35f)) return !(mx > 0.f);
+                            N.nrecheck++;
+                            return !inside64(ld_d4(&A.d_c[e]), __dsub_rn(A.x[i], T.ox), __dsub_rn(A.y[i], T.oy),
+                                             __dsub_rn(A.z[i], T.oz));
+                        };
+                        a0 = a0 && outside(tx.x, tx.z, ty.x, ty.z, tz.x, tz.z, i0);
+                        a1 = a1 && outside(tx.y, tx.w, ty.y, ty.w, tz.y, tz.w, i1);
+                    }
+                    L.ncell[0] += a0;
+                    L.ncell[1] += a1;
+                    opened = (on0 && !a0 ? 1u : 0u) | (on1 && !a1 ? 2u : 0u);
+                    // the children on their way while the terms are formed
+                    if (opened) {
+                        cm = __ldg(&A.e_cmask[e]);
+                        ld_children(A.e_child, e, clo, chi);
+                    }
+                }
+                if (a0 || a1) {
+                    // both targets' terms at once; a leaf is the cell with Q = 0, whose
+                    // distance may be zero when softened
+                    float4 q0, q1;
+                    if (leaf) {
+                        q0 = make_float4(-crit, 0.f, 0.f, 0.f);
+                        q1 = make_float4(0.f, 0.f, 0.f, 0.f);
+                    } else {
+                        ld_pair(A.rq0, e, q0, q1);
+                    }
+                    const float2 rs = kSoft ? __fadd2_rn(r2, two(A.soft2f)) : r2;
+                    const float2 inv = rsqrt2_nr(kSoft && leaf ? rs : r2);
+                    const float2 inv2 = __fmul2_rn(inv, inv);
+                    const float2 invs = kSoft ? rsqrt2_nr(rs) : inv;
+                    float2 f = __fmul2_rn(two(q0.x), __fmul2_rn(kSoft ? __fmul2_rn(invs, invs) : inv2, invs));
+                    if (kQuad) {
+                        const float2 qx =
+                            __ffma2_rn(two(q1.y), dz, __ffma2_rn(two(q1.x), dy, __fmul2_rn(two(q0.y), dx)));
+                        const float2 qy =
+                            __ffma2_rn(two(q1.z), dz, __ffma2_rn(two(q0.z), dy, __fmul2_rn(two(q1.x), dx)));
+                        const float2 qz =
+                            __ffma2_rn(two(q0.w), dz, __ffma2_rn(two(q1.z), dy, __fmul2_rn(two(q1.y), dx)));
+                        const float2 dqd = __ffma2_rn(dz, qz, __ffma2_rn(dy, qy, __fmul2_rn(dx, qx)));
+                        const float2 inv5 = __fmul2_rn(__fmul2_rn(inv2, inv2), inv);
+                        f = __ffma2_rn(two(2.5f), __fmul2_rn(dqd, __fmul2_rn(inv5, inv2)), f);
+                        const float2 n5 = make_float2(a0 ? -inv5.x : 0.f, a1 ? -inv5.y : 0.f);
+                        L.fx = __ffma2_rn(n5, qx, L.fx);
+                        L.fy = __ffma2_rn(n5, qy, L.fy);
+                        L.fz = __ffma2_rn(n5, qz, L.fz);
+                    }
+                    f = make_float2(a0 ? f.x : 0.f, a1 ? f.y : 0.f);
+                    L.fx = __ffma2_rn(f, dx, L.fx);
+                    L.fy = __ffma2_rn(f, dy, L.fy);
+                    L.fz = __ffma2_rn(f, dz, L.fz);
+                }
+            }
+            // members of an opened depth-21 group (no child table): exact terms, 32 at a time
+            for (unsigned m = __ballot_sync(kFull, opened && cm == 0); m; m &= m - 1) {
+                const int src = __ffs(m) - 1;
+                const unsigned gi = __shfl_sync(kFull, item, src), go = __shfl_sync(kFull, opened, src);
+                const int ge = (int)(gi & kEntMask), end = A.e_skip[ge];
+                const unsigned gimg = gi & kItemMask & ~(unsigned)kEntMask;
+                const float4 tx = S.tx[gimg >> kEntBits], ty = S.ty[gimg >> kEntBits], tz = S.tz[gimg >> kEntBits];
+                for (int c0 = ge + 1; c0 < end; c0 += 32) {
+                    const int c = c0 + lane;
+                    const bool a0 = c < end && (go & 1u) && (gimg | (unsigned)c) != own0;
+                    const bool a1 = c < end && (go & 2u) && (gimg | (unsigned)c) != own1;
+                    L.nleaf[0] += a0;
+                    L.nleaf[1] += a1;
+                    if (a0 || a1) {
+                        float4 pa, pb;
+                        ld_pair(A.ra, c, pa, pb);
+                        float2 dx, dy, dz, r2;
+                        rec_diff2(pa, pb, tx, ty, tz, dx, dy, dz, r2);
+                        const float2 iv = rsqrt2_nr(kSoft ? __fadd2_rn(r2, two(A.soft2f)) : r2);
+                        float2 f = __fmul2_rn(two(-pb.z), __fmul2_rn(__fmul2_rn(iv, iv), iv));
+                        f = make_float2(a0 ? f.x : 0.f, a1 ? f.y : 0.f);
+                        L.fx = __ffma2_rn(f, dx, L.fx);
+                        L.fy = __ffma2_rn(f, dy, L.fy);
+                        L.fz = __ffma2_rn(f, dz, L.fz);
+                    }
+                    psum_flush(L);
+                }
+            }
+            const uint32_t nch = opened ? (uint32_t)__popc(cm) : 0u;
+            const unsigned b0 = __ballot_sync(kFull, nch & 1u), b1 = __ballot_sync(kFull, nch & 2u);
+            const unsigned b2 = __ballot_sync(kFull, nch & 4u), b3 = __ballot_sync(kFull, nch & 8u);
+            if (nch) {
+                int pos = fc + __popc(b0 & lt) + 2 * __popc(b1 & lt) + 4 * __popc(b2 & lt) + 8 * __popc(b3 & lt);
+                const unsigned gb = (opened << kWhoShift) | (item & kItemMask & ~(unsigned)kEntMask);
+                if (cm & 1u) S.stack[pos++] = gb | (unsigned)clo.x;
+                if (cm & 2u) S.stack[pos++] = gb | (unsigned)clo.y;
+                if (cm & 4u) S.stack[pos++] = gb | (unsigned)clo.z;
+                if (cm & 8u) S.stack[pos++] = gb | (unsigned)clo.w;
+                if (cm & 16u) S.stack[pos++] = gb | (unsigned)chi.x;
+                if (cm & 32u) S.stack[pos++] = gb | (unsigned)chi.y;
+                if (cm & 64u) S.stack[pos++] = gb | (unsigned)chi.z;
+                if (cm & 128u) S.stack[pos++] = gb | (unsigned)chi.w;
+            }
+            fc += __popc(b0) + 2 * __popc(b1) + 4 * __popc(b2) + 8 * __popc(b3);
+            if ((++rounds & 15) == 0) psum_flush(L);
+        }
+    }
+    psum_flush(L);
+    N.rounds += rounds;
+}
+
+// Units of `per` (even, <= kUnit) targets as in target_units, two at a time.
+template <bool kQuad, bool kInside, bool kSoft>
+__device__ __forceinline__ void pair_units(const GravArgs& A, int per, PSmem& S) {
+    const int lane = threadIdx.x & 31;
+    const int n = min(A.ctl->n_live, A.ncap);
+    const int nunit = (n + per - 1) / per, q = sm_queue(A.nq);
+    TTotal N;
+    for (int u = next_tile(A.tq, A.nq, q, nunit); u >= 0; u = next_tile(A.tq, A.nq, q, nunit)) {
+        const int j0 = u * per, cnt = min(per, n - j0);
+        for (int j = 0; j < cnt; j += 2) {
+            const bool both = j + 1 < cnt;
+            const int i0 = tile_slot(A.order, j0 + j), i1 = both ? tile_slot(A.order, j0 + j + 1) : i0;
+            const int box0 = A.box[i0], box1 = A.box[i1];
+            PSum L;
+            L.fx = L.fy = L.fz = make_float2(0.f, 0.f);
+#pragma unroll
+            for (int t = 0; t < 2; t++) {
+#pragma unroll
+                for (int c = 0; c < 3; c++) L.s[t][c] = L.c[t][c] = 0.f;
+                L.ncell[t] = L.nleaf[t] = L.nmac[t] = 0;
+            }
+            // one walk for both, or one each when they lie in different boxes
+            for (unsigned who = both && box0 == box1 ? 3u : 1u; who; who = who == 1u && both ? 2u : 0u)
+                walk_pair<kQuad, kInside, kSoft>(A, S, i0, i1, who, who == 2u ? box1 : box0, L, N);
+#pragma unroll
+            for (int t = 0; t < 2; t++) {
+                N.ncell += L.ncell[t];
+                N.nleaf += L.nleaf[t];
+                N.nmac += L.nmac[t];
+#pragma unroll
+                for (int c = 0; c < 3; c++) {
+                    L.c[t][c] = -L.c[t][c];
+                    reduce_hilo(L.s[t][c], L.c[t][c]);
+                }
+                L.ncell[t] = __reduce_add_sync(kFull, L.ncell[t]);
+                L.nleaf[t] = __reduce_add_sync(kFull, L.nleaf[t]);
+                L.nmac[t] = __reduce_add_sync(kFull, L.nmac[t]);
+                if (lane == 0 && j + t < cnt) {
+#pragma unroll
+                    for (int c = 0; c < 3; c++) S.sum[j + t][c] = make_float2(L.s[t][c], L.c[t][c]);
+                    S.cnt[j + t][0] = L.ncell[t];
+                    S.cnt[j + t][1] = L.nleaf[t];
+                    S.cnt[j + t][2] = L.nmac[t];
+                    S.cnt[j + t][3] = t ? i1 : i0;
+                }
+            }
+        }
+        __syncwarp();
+        if (lane < cnt) {
+            const int i = S.cnt[lane][3];
+            double a[3];
+#pragma unroll
+            for (int c = 0; c < 3; c++) a[c] = (double)S.sum[lane][c].x + (double)S.sum[lane][c].y;
+            A.out.ax[i] = A.G * a[0];
+            A.out.ay[i] = A.G * a[1];
+            A.out.az[i] = A.G * a[2];
+            if (A.out.ncell) {
+                A.out.ncell[i] = S.cnt[lane][0];
+                A.out.nleaf[i] = S.cnt[lane][1];
+                A.out.nmac[i] = S.cnt[lane][2];
+            }
+        }
+        __syncwarp();
+    }
+    const unsigned long long c0 = warp_total(N.ncell), c1 = warp_total(N.nleaf), c2 = warp_total(N.nmac);
+    const unsigned long long c3 = warp_total(N.nrecheck);
+    if (lane == 0 && c1 + c2) {
+        atomicAdd(&A.ctl->n_cell, c0);
+        atomicAdd(&A.ctl->n_leaf, c1);
+        atomicAdd(&A.ctl->n_mac, c2);
+        atomicAdd(&A.ctl->n_recheck, c3);
+        atomicAdd(&A.ctl->n_iter, (unsigned long long)N.rounds);
+    }
+}
+
+template <bool kQuad, bool kInside, bool kSoft>
+__global__ void __launch_bounds__(kMaxWalkBlock, 3) k_twalk32x2(GravArgs A, int per) {
+    __shared__ PSmem s[kMaxWalkBlock / 32];
+    pair_units<kQuad, kInside, kSoft>(A, per, s[threadIdx.x >> 5]);
+}
+
 template <bool kQuad, bool kInside, bool kSoft>
 __global__ void __launch_bounds__(kMaxWalkBlock, 4) k_twalk32(GravArgs A, int per) {
     __shared__ TSmem<false> s[kMaxWalkBlock / 32];
@@ -596,12 +931,13 @@ __global__ void __launch_bounds__(128, 4) k_twalk32_learn(GravArgs A, int per) {
 }
 
 template <typename K>
-void launch(K kernel, const GravArgs& A, int block, int cap_n, cudaStream_t s) {
+void launch(K kernel, const GravArgs& A, int block, int cap_n, cudaStream_t s, bool pairs = false) {
     // several units per resident warp, so that the queues even out the
     // targets' different walks, and more targets per unit when there are many
     const void* fn = reinterpret_cast<const void*>(kernel);
     const long long fit = (long long)walk_grid(fn, block, 1ll << 40) * (block / 32);
-    const int per = (int)std::max<long long>(1, std::min<long long>(kUnit, cap_n / (8 * fit)));
+    int per = (int)std::max<long long>(1, std::min<long long>(kUnit, cap_n / (8 * fit)));
+    if (pairs) per = std::max(2, per & ~1);
     const int grid = walk_grid(fn, block, ceil_div(cap_n, per));
     kernel<<<grid, block, 0, s>>>(A, per);
 }
@@ -610,7 +946,8 @@ void launch(K kernel, const GravArgs& A, int block, int cap_n, cudaStream_t s) {
 
 void target_walk_prepare() {
 #define RB_P32(Q, I) \
-    walk_prepare_kernel((const void*)k_twalk32<Q, I, true>); walk_prepare_kernel((const void*)k_twalk32<Q, I, false>)
+    walk_prepare_kernel((const void*)k_twalk32<Q, I, true>); walk_prepare_kernel((const void*)k_twalk32<Q, I, false>); \
+    walk_prepare_kernel((const void*)k_twalk32x2<Q, I, true>); walk_prepare_kernel((const void*)k_twalk32x2<Q, I, false>)
 #define RB_P64(Q, I, S) \
     walk_prepare_kernel((const void*)k_twalk64<Q, I, S, true>); walk_prepare_kernel((const void*)k_twalk64<Q, I, S, false>)
     RB_P32(true, true); RB_P32(true, false); RB_P32(false, true); RB_P32(false, false);
@@ -633,6 +970,15 @@ void target_walk(const GravArgs& A, TargetWalk mode, bool quad, bool inside, boo
         if (soft) { if (pot) RB_L(k_twalk64<Q, I, true, true>); else RB_L(k_twalk64<Q, I, true, false>); } \
         else { if (pot) RB_L(k_twalk64<Q, I, false, true>); else RB_L(k_twalk64<Q, I, false, false>); }    \
     } while (0)
+#define RB_P(Q, I)                                                                       \
+    do {                                                                                 \
+        if (pairs) {                                                                     \
+            if (soft) launch(k_twalk32x2<Q, I, true>, A, block, cap_n, s, true);         \
+            else launch(k_twalk32x2<Q, I, false>, A, block, cap_n, s, true);             \
+        } else {                                                                         \
+            RB_SOFT(k_twalk32, Q, I);                                                    \
+        }                                                                                \
+    } while (0)
     if (mode == TargetWalk::kLearned) {
         block = 128;
         if (inside) RB_SOFT(k_twalk32_learn, true);
@@ -641,10 +987,12 @@ void target_walk(const GravArgs& A, TargetWalk mode, bool quad, bool inside, boo
         if (quad) { if (inside) RB_64(true, true); else RB_64(true, false); }
         else { if (inside) RB_64(false, true); else RB_64(false, false); }
     } else {
-        block = kMaxWalkBlock;   // at 30k: 216 us, 231 in blocks of 128 and 322 in blocks of 64
-        if (quad) { if (inside) RB_SOFT(k_twalk32, true, true); else RB_SOFT(k_twalk32, true, false); }
-        else { if (inside) RB_SOFT(k_twalk32, false, true); else RB_SOFT(k_twalk32, false, false); }
+        block = kMaxWalkBlock;   // pairs at 30k: 162 us; in blocks of 128: 166
+        const bool pairs = cap_n >= kPairMin;
+        if (quad) { if (inside) RB_P(true, true); else RB_P(true, false); }
+        else { if (inside) RB_P(false, true); else RB_P(false, false); }
     }
+#undef RB_P
 #undef RB_64
 #undef RB_SOFT
 #undef RB_L

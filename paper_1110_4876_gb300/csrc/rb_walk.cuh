@@ -1,6 +1,6 @@
 // rb_walk.cuh -- device pieces shared by the gravity walks (rb_walk.cu: the
-// walks over 32 targets per warp; rb_twalk.cu: the walks with a warp per
-// target) and the collision search: kernel arguments, tile scheduling, the
+// walks over 32 targets per warp; rb_twalk.cu: the walks with one or two
+// targets per warp) and the collision search: kernel arguments, tile scheduling, the
 // opening and inside tests, interaction terms and the learned walk's queue.
 #pragma once
 #include "rb_internal.cuh"
@@ -53,21 +53,22 @@ struct GravArgs {
 void walk_prepare_kernel(const void* fn);
 int walk_grid(const void* fn, int block, long long warps);
 
-// rb_twalk.cu: the walks with a warp per target.  A holds the target order,
-// records and image table; block is 64, 128 or 256 threads (FP64).
+// rb_twalk.cu: the walks with one or two targets per warp.  A holds the target
+// order, records and image table; block is 64, 128 or 256 threads (FP64).
 // FP32 walks take them up to a number of targets where the chain of entries that
 // a warp of 32 targets steps through is longer than the work.  Walk times on the
-// sheet (theta = 0.5, 9 images, targets in Hilbert order): 147 us against 319 at
-// 20k targets, 219 against 325 at 30k, 276 against 324 at 40k, 347 against 333 at
-// 50k and 409 against 361 at 60k.  In Morton order the 32 targets' walks have
-// less in common: a whole gravity evaluation takes 756 us against 818 at 80k and
-// 909 against 945 at 100k (sheet), 684 against 779 at 60k, 871 against 907 at 80k
-// and 1047 against 945 at 100k (Plummer sphere, theta = 0.8), 1033 against 1314 at
-// 80k (periodic cube).  With the network, whose rows a warp's one target fills
+// sheet (theta = 0.5, 9 images, targets in Hilbert order), two targets per warp
+// against 32: 117 us against 319 at 20k targets, 154 against 325 at 30k, 242
+// against 331 at 50k, 333 against 344 at 70k, 381 against 366 at 80k and 481
+// against 378 at 100k.  In Morton order the 32 targets' walks have less in
+// common: a whole gravity evaluation takes 579 us against 812 at 80k, 698 against
+// 948 at 100k and 884 against 973 at 130k (sheet), 1772 against 2002 at 100k and
+// 2491 against 2259 at 130k (Plummer sphere, theta = 0.5), 1344 against 1508 at
+// 130k (periodic cube).  With the network, whose rows a warp's one target fills
 // better than 32 lanes' band cells in turn: 573 us against 803 at 40k, 1516
 // against 1818 at 100k, 3171 against 2968 at 200k (theta = 0.8).
-constexpr int kTargetWalkMax = 50000;           // targets in a Hilbert order
-constexpr int kTargetWalkMaxMorton = 80000;
+constexpr int kTargetWalkMax = 75000;           // targets in a Hilbert order
+constexpr int kTargetWalkMaxMorton = 125000;
 constexpr int kTargetWalkMaxLearned = 130000;
 enum class TargetWalk { kFp32, kFp64, kLearned };
 void target_walk(const GravArgs& A, TargetWalk mode, bool quad, bool inside, bool soft, bool pot, int block,
