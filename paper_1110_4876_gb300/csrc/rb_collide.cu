@@ -1,8 +1,8 @@
 // rb_collide.cu -- tree collision search (Sect. 5.2) over the ghost images of
 // Sect. 2.3.
 //
-// A warp takes 32 consecutive targets and searches the tree once for all of
-// them.  The lanes hold a frontier of (ghost image, entry) items: each round
+// A warp takes up to 32 consecutive targets and searches the tree once for all
+// of them.  The lanes hold a frontier of (ghost image, entry) items: each round
 // they test up to 32 entries against the bounding box of the targets, push
 // the children of cells that come within R_max of it and put the leaves that
 // do into a list of candidates in shared memory; then every lane tests its
@@ -12,7 +12,7 @@
 // Against a walk of each target's own (lane per target, the warp stepping
 // through the union of 32 walks, about 260 dependent entries), a tile of the
 // 1M sheet takes 24 rounds over 380 entries and tests 73 candidates: 0.59 ->
-// 0.33 ms (100k: 163 -> 77 us, 2400: 125 -> 57 us).
+// 0.33 ms (100k: 163 -> 72 us, 2400: 125 -> 27 us).
 //
 // The targets are consecutive slots, in Morton order whatever order the walk
 // takes: a pair is recorded from its lower slot, so subtrees that lie before
@@ -35,6 +35,16 @@ constexpr int kImgBatch = 32;                // images whose items share the fro
 constexpr int kStack = 384;
 constexpr int kReserve = 160;                // depth-first room: 7 siblings on each of 22 levels
 
+// Targets of a tile.  Tiles of 32 leave the GPU idle with few particles (2,400:
+// 75 warps), and a tile's time is its own chain of rounds and candidates: fewer
+// targets have fewer of both, at the price of more rounds in all.  Search of the
+// sheet with 32, 8 and 4 targets a tile: 47, 29 and 27 us at 2,400 particles, 60,
+// 39 and 35 at 10k, 51, 43 and 52 at 20k, 58, 50 and 61 at 30k, 63, 72 and 90 at
+// 60k; of a periodic cube: 61, 33 and 31 us at 10k, 86, 45 and 54 at 30k, 63, 63
+// and 76 at 60k.
+constexpr int kWidth4Max = 10000;
+constexpr int kWidth8Max = 40000;
+
 struct CollArgs {
     const double *x, *y, *z, *r;
     const int32_t *id, *box;
@@ -50,6 +60,7 @@ struct CollArgs {
     int32_t* tq;            // tile queues (emptied by the image-table launch)
     int nq;
     float rmaxf;            // largest radius, rounded up
+    int width;              // targets of a tile (at most 32)
 };
 
 struct SearchSmem {
@@ -167,8 +178,7 @@ __device__ __forceinline__ void record_pairs(const CollArgs& A, const SearchSmem
 // once, from its lower slot (the other particle reaches it through the
 // opposite image).  Found pairs are queued and recorded 32 at a time: their
 // ids and the pair counter are round trips to L2, which one by one, in the
-// loop, took most of the search (57 us against 74 at 2400 particles, 327 against 526
-// at 1M).
+// loop, took most of the search (327 us against 526 at 1M).
 __device__ __forceinline__ void test_candidates(const CollArgs& A, SearchSmem& S, int nc, bool in,
                                                 const Target& T, const ImgTab* itab, int& nh) {
     const unsigned lt = (1u << (threadIdx.x & 31)) - 1u;
@@ -332,7 +342,7 @@ template <bool kCount>
 __device__ __forceinline__ void collide(const CollArgs& A, SearchSmem& S, int wbase, int n,
                                         unsigned long long& visits, unsigned long long& iters) {
     const int lane = threadIdx.x & 31;
-    const bool valid = wbase + lane < n;
+    const bool valid = lane < A.width && wbase + lane < n;
     const int i = valid ? wbase + lane : n - 1;
     const int box = A.box[i];
     const int root = A.box_root[box];   // -1: a removed particle, searches nothing
@@ -391,10 +401,10 @@ template <bool kCount>
 __global__ void __launch_bounds__(kMaxWalkBlock, 4) k_collide(CollArgs A) {
     __shared__ SearchSmem sm[kMaxWalkBlock / 32];
     const int n = min(A.ctl->n_live, A.ncap);
-    const int ntile = (n + 31) >> 5, q = sm_queue(A.nq);
+    const int ntile = (n + A.width - 1) / A.width, q = sm_queue(A.nq);
     unsigned long long visits = 0, iters = 0;
     for (int t = next_tile(A.tq, A.nq, q, ntile); t >= 0; t = next_tile(A.tq, A.nq, q, ntile))
-        collide<kCount>(A, sm[threadIdx.x >> 5], t << 5, n, visits, iters);
+        collide<kCount>(A, sm[threadIdx.x >> 5], t * A.width, n, visits, iters);
     if (kCount && (threadIdx.x & 31) == 0) {
         atomicAdd(&A.ctl->n_visit, visits);
         atomicAdd(&A.ctl->n_siter, iters);
@@ -425,8 +435,9 @@ void collision_search(const Tree& T, const PSet& P, Ctl* ctl, const BoxP* boxes,
     A.tq = T.tq;
     A.nq = T.nq;
     A.nimg = build_image_table(boxes, ctl, C, half_step_offset, T.img, s, T.tq, T.nq);
+    A.width = T.cap_n <= kWidth4Max ? 4 : T.cap_n <= kWidth8Max ? 8 : 32;
     const int grid = walk_grid(count ? (const void*)k_collide<true> : (const void*)k_collide<false>, block,
-                               ceil_div(T.cap_n, 32));
+                               ceil_div(T.cap_n, A.width));
     if (count) k_collide<true><<<grid, block, 0, s>>>(A);
     else k_collide<false><<<grid, block, 0, s>>>(A);
 }

@@ -1,6 +1,8 @@
 """The tree search's shared candidate lists against brute force, bit for bit:
 runs of targets that are cut at gaps, lists that fill up, leaf groups of
-coincident particles, unequal radii, and more images than one batch of 32."""
+coincident particles, unequal radii, and more images than one batch of 32.
+Each with 4, 8 and 32 targets a warp, which the particle capacity decides: a
+simulation that once held more particles keeps the wider runs."""
 import numpy as np
 import pytest
 
@@ -19,12 +21,18 @@ def rb():
 def _compare(rb, orc, pos, r, L, boundary, ng, z_periodic=0):
     n = len(r)
     zero = np.zeros(n)
-    sim = rb.Sim(box=(L, L, L), boundary=boundary, nghost=ng, z_periodic=z_periodic, gravity=0, collisions=1, dt=1e-3)
-    sim.set_particles((*np.ascontiguousarray(pos.T), zero, zero, zero, np.ones(n), r))
     p = orc.Params(L=(L, L, L), boundary=boundary, nghost=ng, z_periodic=z_periodic, gravity=0, collisions=1, dt=1e-3)
     ref = orc.collide_brute(p, 0.0, *np.ascontiguousarray(pos.T), r, np.arange(n))
-    got = rb.pair_keys(*sim.pairs())
-    assert np.array_equal(got, ref)
+    for held in (0, 10_001, 40_001):
+        sim = rb.Sim(box=(L, L, L), boundary=boundary, nghost=ng, z_periodic=z_periodic, gravity=0, collisions=1,
+                     dt=1e-3)
+        if held:
+            z = np.zeros(held)
+            many = np.random.default_rng(held).uniform(-0.5 * L, 0.5 * L, (3, held))
+            sim.set_particles((*many, z, z, z, np.ones(held), np.full(held, 1e-3)))
+            sim.pairs()
+        sim.set_particles((*np.ascontiguousarray(pos.T), zero, zero, zero, np.ones(n), r))
+        assert np.array_equal(rb.pair_keys(*sim.pairs()), ref)
     return len(ref)
 
 
