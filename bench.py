@@ -39,13 +39,15 @@ L_SHEET = 2050.0
 SEED = 5
 FP32_LANES_PER_SM = 128
 # algorithmic bytes per particle of one tree build (sort + gather, topology,
-# moments): each 8-bit radix pass reads and writes an 8-byte key and a 4-byte
-# value; the gather reads and writes the 64-byte FP64 state plus id and box
+# moments): each 8-bit radix pass (five, over the top 40 key bits) reads and
+# writes an 8-byte key and a 4-byte value; the check for runs of keys that agree
+# there reads each key once; the gather reads and writes the 64-byte FP64 state plus id and box
 # (8 B) and writes the slot of each id (4 B); the topology reads each key
 # once; each tree cell writes ~160 B of FP64 and FP32 records
-BUILD_PASSES = 8
+BUILD_PASSES = 5
 BYTES_PASS, BYTES_GATHER, BYTES_KEYS, BYTES_CELL = 24, 148, 8, 160
 BYTES_DIGITS = 8   # one read of the keys counts the digits of every pass
+BYTES_RUNS = 8     # and one finds the runs
 # algorithmic FP32 flops per interaction (FMA = 2, add/mul = 1, rsqrt = 0)
 FLOP_CELL, FLOP_LEAF, FLOP_MAC = 60, 20, 10
 FLOP_MLP = 2 * (12 * 64 + 2 * 64 * 64 + 64 * 3)
@@ -180,9 +182,9 @@ def max_over_ranks(t_ms: float, dist, device) -> float:
 
 
 def search_rate(visits, iters, ms, ms_counted):
-    """Tree collision search: tree entries tested by the targets (nodes
-    visited, all images) per launch, counted by the search's counting
-    variant in one step after the timed ones, over the event-timed search
+    """Tree collision search: tree entries that a warp tests for its targets,
+    times the targets it tests them for (nodes visited, all images), per launch,
+    counted by the search's counting variant in one step after the timed ones, over the event-timed search
     stage of the timed steps (which run the plain variant).  The search is
     bound by L1/L2 latency, so it is reported as a rate, with no roofline."""
     if not (visits > 0 and ms > 0):
@@ -374,7 +376,8 @@ def run_ours(args):
     return line
 
 
-WALK_SOURCES = ("paper_1110_4876_gb300/csrc/rb_walk.cu", "paper_1110_4876_gb300/csrc/rb_internal.cuh")
+WALK_SOURCES = ("paper_1110_4876_gb300/csrc/rb_walk.cu", "paper_1110_4876_gb300/csrc/rb_walk.cuh",
+                "paper_1110_4876_gb300/csrc/rb_internal.cuh")
 BUILD_SOURCES = ("paper_1110_4876_gb300/csrc/rb_sort.cu", "paper_1110_4876_gb300/csrc/rb_step.cu",
                  "paper_1110_4876_gb300/csrc/rb_tree.cu", "paper_1110_4876_gb300/csrc/rb_internal.cuh")
 
@@ -419,7 +422,7 @@ def build_roofline(stage_sum, steps, cells, peaks, tile_order=0):
     time."""
     n = N_SHEET
     ncells = statistics.mean(cells) if cells else 0.0
-    per_particle = BYTES_DIGITS + BUILD_PASSES * BYTES_PASS + BYTES_GATHER + BYTES_KEYS
+    per_particle = BYTES_DIGITS + BUILD_PASSES * BYTES_PASS + BYTES_RUNS + BYTES_GATHER + BYTES_KEYS
     if tile_order:
         # Hilbert tile keys: read the Morton key (8 B), write key and slot
         # (12 B), then the digit counts and 3 radix passes of 24 B
@@ -429,13 +432,14 @@ def build_roofline(stage_sum, steps, cells, peaks, tile_order=0):
     hbm = float(peaks.get("hbm_gbs", 6800.0))
     achieved = nbytes / (ms / 1e3) / 1e9 if ms > 0 else None
     traffic, note = profiled_traffic("tree_build_sheet1m.md", BUILD_SOURCES, "dram_bytes_per_build")
-    return {"bound": "hbm", "kernels": "k_rs_hist + k_rs_pass (8 passes), k_permute, topology, "
-                                       "tile order (k_tile_keys, k_rs_hist + 3 passes), k_moments_level (per depth)",
+    return {"bound": "hbm", "kernels": "k_rs_hist + k_rs_pass (5 passes) + k_rs_runs + k_rs_long, k_permute, "
+                                       "topology, tile order (k_tile_keys, k_rs_hist + 3 passes), "
+                                       "k_moments_range + k_moments_own + k_moments_span",
             "achieved": achieved, "peak": hbm, "unit": "GB/s",
             "frac": achieved / hbm if achieved else None, "traffic": traffic, "traffic_source": note,
             "bytes_per_step": nbytes, "ms_per_step": ms, "cells_per_particle": ncells / n,
             "bytes_model": f"digit counts {BYTES_DIGITS} B + {BUILD_PASSES} radix passes x {BYTES_PASS} B + "
-                           f"gather {BYTES_GATHER} B + keys {BYTES_KEYS} B per particle + {BYTES_CELL} B per cell"
+                           f"runs {BYTES_RUNS} B + gather {BYTES_GATHER} B + keys {BYTES_KEYS} B per particle + {BYTES_CELL} B per cell"
                            + (" + tile order 100 B per particle" if tile_order else ""),
             "peak_source": "MEASURED_PEAKS.json hbm_gbs (measured copy bandwidth)"}
 

@@ -113,7 +113,7 @@ typedef struct rb_stats_t {
     int64_t corrections;      /* learned walk: band cells corrected by the network in the last walk */
     int64_t warp_iterations;  /* FP32 walk: warp iterations of the last walk (union walk: entries
                                  processed, 32 targets each, or with few particles rounds of up
-                                 to 32 entries of one target; group walk: frontier rounds, list
+                                 to 32 entries of one target or two; group walk: frontier rounds, list
                                  entries and mixed-subtree iterations) */
     int64_t walk_group;       /* FP32 walk shape: 0 union walk, 4 group walk (4-lane subgroups
                                  for the mixed subtrees) */
@@ -351,8 +351,7 @@ int rb_energy_sums_noalloc(int64_t n, const double* m, const double* x, const do
                            double* out, void* cuda_stream);
 /* The sort that puts particles in Morton order before every tree build (it
  * replaces the tree reconstruction of Sect. 4.2), the collision queue in
- * canonical pair order (Sect. 5) and the pair ends of the resolution, run on
- * host arrays: a stable LSD radix sort of (key, value) pairs by key bits
+ * canonical pair order (Sect. 5), run on host arrays: a stable LSD radix sort of (key, value) pairs by key bits
  * [0, key_bits), 8-bit digits.  keys / vals: host arrays of n entries, sorted
  * in place (vals may be NULL).  cap >= n sizes the device buffers while the
  * count n is read on the device, as the step's sorts of pairs run; cap < 2^30.

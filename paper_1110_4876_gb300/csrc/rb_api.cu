@@ -3,8 +3,9 @@
 //
 // One step (Sect. 3, drift-kick-drift) is captured once into a CUDA graph:
 //   drift dt/2 + boundaries + Morton keys -> sort -> gather -> tree ->
-//   moments -> gravity walk -> kick + drift dt/2 + boundaries + keys ->
-//   sort -> gather -> tree -> collision search -> pair sort -> resolution.
+//   moments -> gravity walk -> kick + drift dt/2 + boundaries -> collision
+//   boxes on that tree -> collision search -> pair sort -> resolution
+// (without gravity: both drift halves, then one sort and tree for the search).
 // Each gather moves the particles into the other SoA set, so two graphs are
 // captured (one per starting set) and replayed alternately.
 #include <algorithm>

@@ -289,10 +289,11 @@ struct WalkLearn {
 int build_image_table(const BoxP* boxes, const Ctl* ctl, const SimC& C, int half_step_offset, ImgTab* tab,
                       cudaStream_t s, int32_t* tq = nullptr, int nq = 0);
 // Walk and search kernels take their block size (64, 128 or 256 threads)
-// at run time; the autotuner picks it.  They run persistent blocks (as many
-// as fit on the GPU at once) that take tiles of 32 consecutive targets from
-// per-SM queues: queue q holds the q-th contiguous part of the Morton order,
-// so the warps resident on one SM walk neighbouring targets and share the
+// at run time; the autotuner picks it.  They run persistent blocks (the same
+// number on every SM, as many as fit at once) that take tiles of consecutive
+// targets (32; up to 8 for the walks with one or two targets per warp; 4, 8 or 32
+// for the search) from per-SM queues: queue q holds the q-th contiguous part of
+// the targets' order, so the warps resident on one SM walk neighbouring targets and share the
 // tree records they read in that SM's L1.  An empty queue's warps take
 // tiles from the following queues.
 constexpr int kMaxWalkBlock = 256;
@@ -302,7 +303,7 @@ constexpr int kMaxTileQueues = 512;
 // stream capture); returns the number of SMs.
 int walk_prepare();
 // group (plain FP32 walk only): 0 runs the union walk over the warp's 32
-// targets; 4 runs the group walk, whose mixed subtrees are walked by
+// targets, or with fewer targets the walks of rb_twalk.cu; 4 runs the group walk, whose mixed subtrees are walked by
 // subgroups of 4 lanes.  Accepted sets do not depend on block or group.
 void gravity_walk(const Tree& T, const PSet& P, Ctl* ctl, const BoxP* boxes, const SimC& C,
                   int walk_mode, int half_step_offset, const WalkOut& out, bool potential,

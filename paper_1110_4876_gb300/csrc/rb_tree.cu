@@ -857,9 +857,9 @@ struct CollRecArgs {
 // down, upper corner rounded up to FP32), so the search stays exact without a
 // second sort and build.  A cell's record also holds the largest particle
 // slot below it (ra.w), so a search from slot i skips subtrees whose pairs
-// with i are examined from the other particle.  Leaves as in
-// k_coll_records; a removed particle's leaf sits at +infinity and is never
-// close.
+// with i are examined from the other particle.  A leaf's
+// record holds its position (hi/lo), radius and slot; a removed particle's sits
+// at +infinity and is never close.
 // Boxes from particle ranges: a cell of the gravity tree holds the
 // consecutive slots [first, first + count), so its box is the union of its
 // particles' boxes, taken here from the fewest aligned runs that tile the
@@ -929,10 +929,10 @@ __device__ __forceinline__ void cell_put(const CollRecArgs& A, int k, const BoxA
 // down, upper corner rounded up to FP32), so the search stays exact without a
 // second sort and build.  A cell's record also holds the largest particle
 // slot below it (ra.w), so a search from slot i skips subtrees whose pairs
-// with i are examined from the other particle.  Leaves as in
-// k_coll_records; a removed particle's leaf sits at +infinity and is never
-// close.  This launch also writes the box items of every slot and of the
-// runs of 32 and 256 slots (kRunB threads per block).
+// with i are examined from the other particle.  A leaf's
+// record holds its position (hi/lo), radius and slot; a removed particle's sits
+// at +infinity and is never close.  This launch also writes the box items of
+// every slot and of the runs of 32 and 256 slots (kRunB threads per block).
 __global__ void __launch_bounds__(kRunB) k_aabb_leaves(CollRecArgs A) {
     __shared__ BoxAcc wbox[kRunsInB];
     const int n = min(A.ctl->n_live, A.ncap);
