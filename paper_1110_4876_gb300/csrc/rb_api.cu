@@ -96,6 +96,8 @@ struct rb_sim {
     double theta_fb = 0.5;
     std::vector<void*> mlp_allocs;
     // launch shapes (threads per block) of the gravity walk and the search
+    int key_low = 0;          // Morton bits left to the runs, by the boxes' shapes (upload)
+    bool long_runs = false;   // the particles lie too close together for that: every bit is sorted by passes
     int walk_block = 128, search_block = 128;
     int walk_group = 0;   // FP32 walk: 0 union walk; 4 group walk (4-lane subgroups for mixed subtrees)
     int tile_order = kTileMorton;   // order in which walks and search take targets (kTile*)
@@ -167,6 +169,7 @@ void make_constants(rb_sim* s) {
     C.has_test = s->n_active >= 0;
     C.eps_law = s->eps_law;
     C.hold_pair = s->hold_pair;
+    C.key_low = s->long_runs ? 0 : s->key_low;
     C.eps_vc = s->eps_vc;
     C.eps_p = s->eps_p;
     C.G = c.G;
@@ -234,6 +237,34 @@ int alloc_pairs(rb_sim* s, int cap) {
 }
 
 // Allocate for capacity n and upload the staged boxes.
+// Morton key bits that the particle sort's passes leave to the runs (24: five
+// passes to depth 13, 16: six to depth 15, 0: all eight): as many as leave the
+// particles four cells each, in the plane of a thin sheet, at that depth.  In a
+// ring segment of 1M particles, 10^4 times as long as wide, depth 13 holds 122
+// particles a cell, and putting runs of that length in order took 1.0 ms where
+// three passes take 0.05.
+int key_low_bits(const rb_sim* s) {
+    auto room = [&](int depth) {
+        for (int b = 0; b < s->nbox; b++) {
+            const double c = (double)(1 << depth), w = std::max(1.0, c * s->hb[b].L[1] / s->hb[b].L[0]);
+            const double n = s->nbox == 1 ? (double)s->ncap : (double)s->hb[b].n;
+            if (c * w < 4.0 * n) return false;
+        }
+        return true;
+    };
+    return room(13) ? 24 : room(15) ? 16 : 0;
+}
+
+// After a sort: particles that crowd together below the passes' depth (a clump
+// far smaller than its box) make long runs, which one block each puts in order;
+// from then on the passes take every bit.
+void check_runs(rb_sim* s) {
+    if (s->C.key_low == 0 || s->hctl.long_keys <= (unsigned long long)s->ntot / 8 + 4096) return;
+    s->long_runs = true;
+    make_constants(s);
+    drop_graphs(s);
+}
+
 int upload(rb_sim* s) {
     int64_t tot = 0;
     s->base.assign(s->nbox, 0);
@@ -378,6 +409,12 @@ int upload(rb_sim* s) {
         while ((1 << s->box_bits) <= s->nbox) s->box_bits++;
     }
     s->SW.box_bits = s->box_bits;
+    const int low = key_low_bits(s);
+    if (low != s->key_low) {
+        drop_graphs(s);
+        s->long_runs = false;
+    }
+    s->key_low = low;
     make_constants(s);
     if (box_params(s) != RB_OK) return RB_ERR_CUDA;
     s->dirty = false;
@@ -630,6 +667,7 @@ int gravity_now(rb_sim* s, bool potential) {
     s->q32 = !fp64;
     RB_CUDA(s, cudaGetLastError());
     if (int rc = read_ctl(s)) return rc;
+    check_runs(s);
     if (s->hctl.err & kErrWalk)
         return fail(s, RB_ERR_STATE, "gravity walk: an entry index outside the tree (malformed tree)");
     if (s->hctl.err & kErrSortStall)
@@ -932,6 +970,7 @@ int rb_step(rb_sim* s, int64_t nsteps) {
         RB_CUDA(s, cudaEventRecord(s->ev1, s->stream));
         if ((rc = read_ctl(s))) return rc;
         cudaEventElapsedTime(&s->last_ms, s->ev0, s->ev1);
+        check_runs(s);
         if (s->profiling)
             for (int q = 0; q < 12; q++)
                 cudaEventElapsedTime(&s->stage_ms[q], s->ev_stage[q], s->ev_stage[q + 1]);

@@ -45,6 +45,7 @@ struct SimC {
     int has_test;        // some particles are test particles (source mass 0)
     int eps_law;         // 0: constant eps; 1: eps = min(1, (|v_n| / eps_vc)^(-eps_p))
     int hold_pair;       // test hook: the queue's first pair never becomes ready
+    int key_low;         // Morton key bits below those that the particle sort's passes take
     double eps_vc, eps_p;
     // SEI drift coefficients for tau = dt / 2 (x, vx, vy) -> (x, y, vx, vy), and z
     double axx, axu, axv, ayx, ayu, ayv, aux, auu, auv, avx, avu, avv;
@@ -80,6 +81,7 @@ struct Ctl {
     unsigned long long n_siter;       // warp iterations of the last collision search
     // (end of what clear_step clears)
     unsigned long long sweep_wbits;   // plane sweep: largest half extent (double bits)
+    unsigned long long long_keys;     // last particle sort: keys in runs that blocks put in order
 };
 constexpr int kErrNonFinite = 1;
 constexpr int kErrPairOverflow = 2;
@@ -236,8 +238,9 @@ int radix_sort_passes(int key_bits, bool box_pass, int box_bits);
 // grows the buffer and searches again on the unchanged state).
 int radix_sort(uint64_t* k0, uint32_t* v0, uint64_t* k1, uint32_t* v1, int ncap, const int* d_n,
                int key_bits, const int32_t* box_digits, int box_bits, uint32_t* hist, int* err,
-               cudaStream_t s, int low_bit = 0, Ctl* pairs = nullptr);
+               cudaStream_t s, int low_bit = 0, Ctl* pairs = nullptr, unsigned long long* long_keys = nullptr);
 size_t radix_hist_words(int ncap);
+size_t radix_digit_words();   // the digit totals among them
 // rb_tree.cu
 size_t entry_scan_words(int ncap);
 void build_topology(const Tree& T, const PSet& P, Ctl* ctl, const BoxP* boxes, const SimC& C,

@@ -72,7 +72,7 @@ __global__ void __launch_bounds__(kThreads) k_rs_hist(const uint64_t* __restrict
                                                       int passes_key, int passes_box,
                                                       uint32_t* __restrict__ hist,
                                                       uint32_t* __restrict__ status, int tiles_cap,
-                                                      Ctl* pairs) {
+                                                      Ctl* pairs, unsigned long long* long_keys) {
     __shared__ uint32_t h[kMaxPasses][kBins];
     const int P = passes_key + passes_box;
     for (int i = threadIdx.x; i < P * kBins; i += kThreads) (&h[0][0])[i] = 0;
@@ -88,7 +88,10 @@ __global__ void __launch_bounds__(kThreads) k_rs_hist(const uint64_t* __restrict
     } else {
         n = read_n(d_n, ncap);
     }
-    if (low_bit > 0 && blockIdx.x == 0 && threadIdx.x == 0) hist[kLongCount] = 0u;
+    if (low_bit > 0 && blockIdx.x == 0 && threadIdx.x == 0) {
+        hist[kLongCount] = 0u;
+        if (long_keys) *long_keys = 0;
+    }
     const int nt = (n + kTile - 1) / kTile;
     const size_t rows = (size_t)nt * kBins;
     const size_t stride = (size_t)gridDim.x * kThreads;
@@ -327,6 +330,7 @@ __global__ void __launch_bounds__(kThreads, 4) k_rs_pass(const uint64_t* __restr
 // at 1M (with the gather) and 64 -> 48 us at 20k, pairs by the lower id alone
 // 125 -> 76 and 52 -> 28 us.
 constexpr int kShortRun = 16;   // runs up to this length: by one thread, in place
+constexpr int kSlowRun = 2048;  // runs above this length take a block longer than the passes they save
 
 // Do neighbours a, b (a = b - 1) belong to one run?
 __device__ __forceinline__ bool same_run(const uint64_t* key, const uint32_t* val, const int32_t* box, int low_bit,
@@ -376,7 +380,8 @@ __global__ void __launch_bounds__(kThreads) k_rs_long(uint64_t* __restrict__ k0,
                                                       uint64_t* __restrict__ k1, uint32_t* __restrict__ v1,
                                                       const int32_t* __restrict__ box, const int* d_n, int ncap,
                                                       int low_bit, const uint32_t* __restrict__ nlong,
-                                                      const uint32_t* __restrict__ list) {
+                                                      const uint32_t* __restrict__ list,
+                                                      unsigned long long* long_keys) {
     __shared__ uint32_t wcnt[kThreads / 32][kBins], base[kBins], wsum[kThreads / 32];
     __shared__ int end_s;
     const int n = read_n(d_n, ncap), tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -404,6 +409,8 @@ __global__ void __launch_bounds__(kThreads) k_rs_long(uint64_t* __restrict__ k0,
                 if (in(mid)) good = mid; else bad = mid;
             }
             end_s = bad;
+            // what the run costs: its keys, and as much as all keys if one block is long at it
+            if (long_keys) atomicAdd(long_keys, (unsigned long long)(bad - i0 > kSlowRun ? n : bad - i0));
         }
         __syncthreads();
         const int i1 = end_s;
@@ -484,13 +491,15 @@ size_t radix_hist_words(int ncap) {
            2 * (size_t)kBins * (size_t)ceil_div(ncap > 0 ? ncap : 1, kTile);
 }
 
+size_t radix_digit_words() { return (size_t)kMaxPasses * kBins; }
+
 int radix_sort_passes(int key_bits, bool box_pass, int box_bits) {
     return ceil_div(key_bits, 8) + (box_pass ? ceil_div(box_bits, 8) : 0);
 }
 
 int radix_sort(uint64_t* k0, uint32_t* v0, uint64_t* k1, uint32_t* v1, int ncap, const int* d_n,
                int key_bits, const int32_t* box_digits, int box_bits, uint32_t* hist, int* err,
-               cudaStream_t s, int low_bit, Ctl* pairs) {
+               cudaStream_t s, int low_bit, Ctl* pairs, unsigned long long* long_keys) {
     if (ncap <= 0) return 0;
     const int tiles_cap = ceil_div(ncap, kTile);
     uint32_t* status = hist + kMaxPasses * kBins;
@@ -502,10 +511,11 @@ int radix_sort(uint64_t* k0, uint32_t* v0, uint64_t* k1, uint32_t* v1, int ncap,
     const int hgrid = std::max(1, std::min(ceil_div(ncap, 8 * kThreads), 1024));
     if (box_digits)
         k_rs_hist<true><<<hgrid, kThreads, 0, s>>>(k0, v0, box_digits, d_n, ncap, low_bit,
-                                                   passes_key, passes_box, hist, status, tiles_cap, pairs);
+                                                   passes_key, passes_box, hist, status, tiles_cap, pairs,
+                                                   long_keys);
     else
         k_rs_hist<false><<<hgrid, kThreads, 0, s>>>(k0, v0, nullptr, d_n, ncap, low_bit, passes_key, 0, hist,
-                                                    status, tiles_cap, pairs);
+                                                    status, tiles_cap, pairs, long_keys);
     int cur = 0;
     uint64_t* K[2] = {k0, k1};
     uint32_t* V[2] = {v0, v1};
@@ -528,7 +538,7 @@ int radix_sort(uint64_t* k0, uint32_t* v0, uint64_t* k1, uint32_t* v1, int ncap,
         const uint32_t* nlong = hist + kLongCount;
         k_rs_runs<<<ceil_div(ncap, 256), 256, 0, s>>>(K[cur], V[cur], box_digits, d_n, ncap, low_bit, hist, status);
         k_rs_long<<<std::min(ceil_div(ncap, kShortRun), 152), kThreads, 0, s>>>(
-            K[cur], V[cur], K[cur ^ 1], V[cur ^ 1], box_digits, d_n, ncap, low_bit, nlong, status);
+            K[cur], V[cur], K[cur ^ 1], V[cur ^ 1], box_digits, d_n, ncap, low_bit, nlong, status, long_keys);
     }
     return cur;
 }

@@ -536,16 +536,15 @@ void drift_keys(const PSet& P, const Tree& T, Ctl* ctl, const BoxP* boxes, const
     else launch(bool_constant<false>{}, bool_constant<false>{});
 }
 
-// Morton bits below those that the passes sort.
-constexpr int kMortonLowBits = 24;
-
 void sort_and_permute(const PSet& src, const PSet& dst, Tree& T, Pairs& PR, Ctl* ctl,
                       const SimC& C, int ncap, int box_bits, cudaStream_t s) {
     if (ncap <= 0) return;
-    // five passes over the top 40 bits (depth 13), the rest within the short
-    // runs that agree there
+    // passes over the top bits, the rest within the short runs that agree there
     const int which = radix_sort(T.key, T.idx, T.key_alt, T.idx_alt, ncap, nullptr, 64,
-                                 C.nbox > 1 ? T.sbox : nullptr, box_bits, T.hist, &ctl->err, s, kMortonLowBits);
+                                 C.nbox > 1 ? T.sbox : nullptr, box_bits, T.hist, &ctl->err, s, C.key_low, nullptr,
+                                 &ctl->long_keys);
+    // a sort by the top bits counts on zero digit totals, and leaves them
+    if (C.key_low == 0) cudaMemsetAsync(T.hist, 0, sizeof(uint32_t) * radix_digit_words(), s);
     if (which == 1) {
         // keep the sorted keys in T.key for the topology kernels
         uint64_t* k = T.key; T.key = T.key_alt; T.key_alt = k;

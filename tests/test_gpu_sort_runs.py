@@ -54,3 +54,37 @@ def test_forces_of_clumps(rb, orc, n, scale):
             # neighbours, lie scale / 50 away: 3 x 2^-54 x 50 / scale of such a
             # term, below 1e-14 / scale
             assert np.max(np.linalg.norm(a - ref, axis=1) / den) <= 1e-12 + 1e-14 / scale
+
+
+# passes to depth 13, 15 and 21, by the width of a long box and the number of
+# particles that share its cells there
+@pytest.mark.parametrize("n,width", [(1500, 1e-4), (3000, 1e-4), (8200, 1e-5)])
+def test_long_boxes(rb, orc, n, width):
+    g = np.random.default_rng(n)
+    L = (1.0, width, 1.0)
+    pos = (g.random((n, 3)) - 0.5) * (1.0, width, 1e-6)
+    r = g.uniform(0.05, 0.4, n) * width
+    zero = np.zeros(n)
+    cfg = dict(boundary=1, nghost=(1, 1, 0), gravity=0, collisions=1, dt=1e-3)
+    sim = rb.Sim(box=L, **cfg)
+    sim.set_particles((*np.ascontiguousarray(pos.T), zero, zero, zero, np.ones(n), r))
+    ref = orc.collide_brute(orc.Params(L=L, **cfg), 0.0, *np.ascontiguousarray(pos.T), r, np.arange(n))
+    assert len(ref)
+    for _ in range(2):
+        assert np.array_equal(rb.pair_keys(*sim.pairs()), ref)
+
+
+def test_a_clump_of_one_long_run(rb, orc):
+    """5,000 particles within one cell of depth 13 (and one outside): a run too
+    long for one block, after which every key bit is sorted by passes."""
+    P = I.random_cube(5000, 3)
+    for f in ("x", "y", "z"):
+        getattr(P, f)[:-1] = 0.3 + 2e-5 * getattr(P, f)[:-1]
+    p = orc.Params(G=1.0, L=(1.0,) * 3, theta=0.5, soft=1e-9, gravity=1)
+    ref = orc.tree_gravity(p, 0.0, P.x, P.y, P.z, P.m)
+    den = np.maximum(np.linalg.norm(ref, axis=1), 1e-3 * np.sqrt(np.mean((ref ** 2).sum(1))))
+    sim = rb.Sim(G=1.0, box=(1.0,) * 3, theta=0.5, softening=1e-9, gravity=1, walk=rb.RB_WALK_FP64)
+    for _ in range(3):   # by runs, by passes, by passes on the same buffers
+        sim.set_particles(P)
+        # as for the clumps above, scale 2e-5
+        assert np.max(np.linalg.norm(sim.gravity() - ref, axis=1) / den) <= 1e-12 + 1e-14 / 2e-5
