@@ -11,8 +11,9 @@
 // of Eq. 3's that still holds every overlap.
 // Against a walk of each target's own (lane per target, the warp stepping
 // through the union of 32 walks, about 260 dependent entries), a tile of the
-// 1M sheet takes 24 rounds over 380 entries and tests 73 candidates: 0.59 ->
-// 0.33 ms (100k: 163 -> 72 us, 2400: 125 -> 27 us).
+// 1M sheet tests 380 entries and 73 candidates: 0.59 -> 0.28 ms (100k: 163 -> 60
+// us, 2400: 125 -> 22 us).  Bound by instruction issue with many particles, by a
+// tile's chain of rounds with few.
 //
 // The targets are consecutive slots, in Morton order whatever order the walk
 // takes: a pair is recorded from its lower slot, so subtrees that lie before
@@ -20,7 +21,10 @@
 // jumps between octants, and a target may have left the others since the tree
 // was built (a wrap across a periodic face, a close encounter): a box around
 // such a run would hold much of the tree, so it is cut at its widest gaps into
-// compact parts that are searched in turn.
+// compact parts.  Up to four of them are searched together, their items on one
+// frontier and tagged with their part: in turn, a tile's 380 entries took 24
+// rounds, half of whose lanes were idle (1M: 324 -> 283 us, 100k: 70 -> 60, 20k:
+// 43 -> 37, 2400: 27 -> 22).
 #include <algorithm>
 #include <cfloat>
 
@@ -32,16 +36,19 @@ namespace {
 constexpr int kEntBits = 25;                 // entries < 2 (2^24 - 1) < 2^25
 constexpr int kEntMask = (1 << kEntBits) - 1;
 constexpr int kImgBatch = 32;                // images whose items share the frontier
-constexpr int kStack = 384;
+constexpr int kImgShift = kEntBits, kSegShift = 30;
+constexpr unsigned kImgMask = 31u;
+constexpr int kSegs = 4;                     // parts of a tile searched together
+constexpr int kStack = 448;
 constexpr int kReserve = 160;                // depth-first room: 7 siblings on each of 22 levels
 
 // Targets of a tile.  Tiles of 32 leave the GPU idle with few particles (2,400:
 // 75 warps), and a tile's time is its own chain of rounds and candidates: fewer
 // targets have fewer of both, at the price of more rounds in all.  Search of the
-// sheet with 32, 8 and 4 targets a tile: 47, 29 and 27 us at 2,400 particles, 60,
-// 39 and 35 at 10k, 51, 43 and 52 at 20k, 58, 50 and 61 at 30k, 63, 72 and 90 at
-// 60k; of a periodic cube: 61, 33 and 31 us at 10k, 86, 45 and 54 at 30k, 63, 63
-// and 76 at 60k.
+// sheet with 32, 8 and 4 targets a tile (parts searched in turn): 47, 29 and 27 us
+// at 2,400 particles, 60, 39 and 35 at 10k, 51, 43 and 52 at 20k, 58, 50 and 61 at
+// 30k, 63, 72 and 90 at 60k; of a periodic cube: 61, 33 and 31 us at 10k, 86, 45 and
+// 54 at 30k, 63, 63 and 76 at 60k.
 constexpr int kWidth4Max = 10000;
 constexpr int kWidth8Max = 40000;
 
@@ -63,12 +70,21 @@ struct CollArgs {
     int width;              // targets of a tile (at most 32)
 };
 
+// A compact part of a tile's targets.
+struct Segment {
+    float lx, hx, ly, hy, lz, hz;   // bounding box
+    float reach, size;              // widening; largest absolute values that enter its distances
+    int min_slot;                   // lowest slot of its targets
+    int count;                      // its targets
+};
+
 struct SearchSmem {
+    Segment seg[kSegs];
     float4 ca[64], cb[64];        // candidates: image position hi and radius; lo and slot
     float4 ohi[kImgBatch];        // image offset (hi); w: sum of its absolute values
     float4 olo[kImgBatch];
-    int stack[kStack];            // (image of the batch << kEntBits) | entry
-    int cimg[64];                 // the candidates' images
+    unsigned stack[kStack];       // (segment << 30) | (image of the batch << 25) | entry
+    int cimg[64];                 // the candidates' images, (segment << 16) | image
     int hi[64], hj[64], hg[64];   // pairs found: slots, 2 * image + (1: clear of the threshold)
 };
 
@@ -173,13 +189,13 @@ __device__ __forceinline__ void record_pairs(const CollArgs& A, const SearchSmem
     }
 }
 
-// Every lane of the segment against candidates [0, nc), in FP32 on hi/lo
+// Every lane against the candidates [0, nc) of its segment, in FP32 on hi/lo
 // positions (distance good to ~1e-7 relative).  Each unordered pair is found
 // once, from its lower slot (the other particle reaches it through the
 // opposite image).  Found pairs are queued and recorded 32 at a time: their
 // ids and the pair counter are round trips to L2, which one by one, in the
-// loop, took most of the search (327 us against 526 at 1M).
-__device__ __forceinline__ void test_candidates(const CollArgs& A, SearchSmem& S, int nc, bool in,
+// loop, took two fifths of the search at 1M.
+__device__ __forceinline__ void test_candidates(const CollArgs& A, SearchSmem& S, int nc, int seg,
                                                 const Target& T, const ImgTab* itab, int& nh) {
     const unsigned lt = (1u << (threadIdx.x & 31)) - 1u;
     for (int c = 0; c < nc; c++) {
@@ -191,14 +207,15 @@ __device__ __forceinline__ void test_candidates(const CollArgs& A, SearchSmem& S
         const float sr = T.r + a.w;
         const float s2 = sr * sr;
         const int j = __float_as_int(b.w);
-        const bool near = in && j > T.slot && d2 < s2 * 1.0001f;
+        const int ci = S.cimg[c];
+        const bool near = seg == ci >> 16 && j > T.slot && d2 < s2 * 1.0001f;
         const unsigned m = __ballot_sync(kFull, near);
         if (!m) continue;
         if (near) {
             const int at = nh + __popc(m & lt);
             S.hi[at] = T.slot;
             S.hj[at] = j;
-            S.hg[at] = (S.cimg[c] << 1) | (d2 < s2 * 0.9999f ? 1 : 0);
+            S.hg[at] = ((ci & 0xffff) << 1) | (d2 < s2 * 0.9999f ? 1 : 0);
         }
         nh += __popc(m);
         if (nh >= 32) {
@@ -210,19 +227,15 @@ __device__ __forceinline__ void test_candidates(const CollArgs& A, SearchSmem& S
     }
 }
 
-// Targets in one box (the lanes with in) against that box's tree: all images.
-// min_slot: the lowest of their slots (a subtree whose particles all sit at
-// slots <= it holds no pair that is recorded from here).
+// The targets of nseg segments in one box against that box's tree: all images.
+// seg: the lane's segment (-1: none).  A subtree whose particles all sit at
+// slots up to a segment's lowest holds no pair that is recorded from there.
 template <bool kCount>
-__device__ __forceinline__ void search_segment(const CollArgs& A, SearchSmem& S, bool in, const Target& T,
-                                               const Box3& B, float reach, int min_slot, int root,
-                                               const ImgTab* itab, unsigned long long& tested) {
+__device__ __forceinline__ void search_segments(const CollArgs& A, SearchSmem& S, int nseg, int seg, const Target& T,
+                                                int root, const ImgTab* itab, unsigned long long& visits,
+                                                unsigned long long& tested) {
     const int lane = threadIdx.x & 31;
     const unsigned lt = (1u << lane) - 1u;
-    // float boxes and offsets: each subtraction below is good to 2e-7 of the
-    // absolute values that enter it
-    const float size = fmaxf(fabsf(B.lx), fabsf(B.hx)) + fmaxf(fabsf(B.ly), fabsf(B.hy)) +
-                       fmaxf(fabsf(B.lz), fabsf(B.hz));
     int nh = 0;   // pairs found and not yet recorded (warp-uniform, < 32)
     for (int g0 = 0; g0 < A.nimg; g0 += kImgBatch) {
         const int nb = min(kImgBatch, A.nimg - g0);
@@ -231,15 +244,20 @@ __device__ __forceinline__ void search_segment(const CollArgs& A, SearchSmem& S,
             const float4 h = itab[g0 + lane].hi;
             S.ohi[lane] = make_float4(h.x, h.y, h.z, fabsf(h.x) + fabsf(h.y) + fabsf(h.z));
             S.olo[lane] = itab[g0 + lane].lo;
-            S.stack[lane] = (lane << kEntBits) | root;
+            for (int q = 0; q < nseg; q++)
+                S.stack[q * nb + lane] =
+                    ((unsigned)q << kSegShift) | ((unsigned)lane << kImgShift) | (unsigned)root;
         }
-        int fc = nb, nc = 0;   // items on the stack, candidates (warp-uniform)
+        int fc = nb * nseg, nc = 0;   // items on the stack, candidates (warp-uniform)
         while (fc > 0) {
             // 32 items while their children fit above the depth-first reserve,
             // fewer near it: one item at a time adds at most 7 per level
             const int k = min(min(32, fc), max(1, (kStack - kReserve - fc) / 7));
             __syncwarp();
-            const int item = lane < k ? S.stack[fc - k + lane] : -1;
+            const bool have = lane < k;
+            const unsigned item = have ? S.stack[fc - k + lane] : 0u;
+            const int e = (int)(item & kEntMask), img = (int)((item >> kImgShift) & kImgMask);
+            const int sg = (int)(item >> kSegShift);
             fc -= k;
             __syncwarp();
             if (kCount) tested += (unsigned)k;
@@ -247,11 +265,14 @@ __device__ __forceinline__ void search_segment(const CollArgs& A, SearchSmem& S,
             uint32_t cm = 0;
             int4 clo = make_int4(0, 0, 0, 0), chi = clo;
             float4 ra, rb, o;
-            if (item >= 0) {
-                const int e = item & kEntMask;
+            if (have) {
+                const Segment& B = S.seg[sg];
+                if (kCount) visits += (unsigned)B.count;
                 ld_pair(A.ra, e, ra, rb);
-                o = S.ohi[item >> kEntBits];
-                const float lim = reach + 4e-7f * (size + o.w);
+                o = S.ohi[img];
+                // float boxes and offsets: each subtraction below is good to
+                // 2e-7 of the absolute values that enter it
+                const float lim = B.reach + 4e-7f * (B.size + o.w);
                 const bool leaf = __float_as_int(ra.w) < 0;
                 const int top = leaf ? ~__float_as_int(ra.w) : __float_as_int(ra.w);
                 // leaf: its position hi as a box of no extent (lo is below 6e-8 of it)
@@ -260,7 +281,7 @@ __device__ __forceinline__ void search_segment(const CollArgs& A, SearchSmem& S,
                 const float ey = fmaxf(fmaxf(ra.y + (o.y - B.hy), (B.ly - o.y) - uy), 0.f);
                 const float ez = fmaxf(fmaxf(ra.z + (o.z - B.hz), (B.lz - o.z) - uz), 0.f);
                 const float d2 = fmaf(ez, ez, fmaf(ey, ey, ex * ex));
-                const bool close = top > min_slot && d2 < lim * lim;
+                const bool close = top > B.min_slot && d2 < lim * lim;
                 cand = close && leaf;
                 open = close && !leaf;
                 if (open) {
@@ -273,32 +294,33 @@ __device__ __forceinline__ void search_segment(const CollArgs& A, SearchSmem& S,
             }
             // candidates: position of the image, x + o as a hi/lo pair
             const unsigned mc = __ballot_sync(kFull, cand);
-            auto put = [&](int at, int img, const float4& pa, const float4& pb, int slot) {
-                const float4 h = S.ohi[img], l = S.olo[img];
+            auto put = [&](int at, int im, int q, const float4& pa, const float4& pb, int slot) {
+                const float4 h = S.ohi[im], l = S.olo[im];
                 float hx, lx, hy, ly, hz, lz;
                 sub_hilo(pa.x, pb.x, -h.x, -l.x, hx, lx);
                 sub_hilo(pa.y, pb.y, -h.y, -l.y, hy, ly);
                 sub_hilo(pa.z, pb.z, -h.z, -l.z, hz, lz);
                 S.ca[at] = make_float4(hx, hy, hz, pb.w);
                 S.cb[at] = make_float4(lx, ly, lz, __int_as_float(slot));
-                S.cimg[at] = g0 + img;
+                S.cimg[at] = (q << 16) | (g0 + im);
             };
             // room for 32 more
             auto make_room = [&]() {
                 if (nc < 32) return;
                 __syncwarp();
-                test_candidates(A, S, nc, in, T, itab, nh);
+                test_candidates(A, S, nc, seg, T, itab, nh);
                 __syncwarp();
                 nc = 0;
             };
             make_room();
-            if (cand) put(nc + __popc(mc & lt), item >> kEntBits, ra, rb, ~__float_as_int(ra.w));
+            if (cand) put(nc + __popc(mc & lt), img, sg, ra, rb, ~__float_as_int(ra.w));
             nc += __popc(mc);
             // an opened depth-21 group has no child table: its members are the
             // leaves up to its skip entry (any number: 32 at a time)
             for (unsigned m = __ballot_sync(kFull, open && cm == 0); m; m &= m - 1) {
-                const int gi = __shfl_sync(kFull, item, __ffs(m) - 1);
-                const int ge = gi & kEntMask, end = A.e_skip[ge];
+                const unsigned gi = __shfl_sync(kFull, item, __ffs(m) - 1);
+                const int ge = (int)(gi & kEntMask), end = A.e_skip[ge];
+                const int gm = (int)((gi >> kImgShift) & kImgMask), gs = (int)(gi >> kSegShift);
                 for (int c0 = ge + 1; c0 < end; c0 += 32) {
                     const int c = c0 + lane;
                     if (kCount) tested += (unsigned)min(32, end - c0);
@@ -306,7 +328,8 @@ __device__ __forceinline__ void search_segment(const CollArgs& A, SearchSmem& S,
                     if (c < end) {
                         float4 pa, pb;
                         ld_pair(A.ra, c, pa, pb);
-                        put(nc + lane, gi >> kEntBits, pa, pb, ~__float_as_int(pa.w));
+                        put(nc + lane, gm, gs, pa, pb, ~__float_as_int(pa.w));
+                        if (kCount) visits += (unsigned)S.seg[gs].count;
                     }
                     nc += min(32, end - c0);
                 }
@@ -318,20 +341,20 @@ __device__ __forceinline__ void search_segment(const CollArgs& A, SearchSmem& S,
             const unsigned b2 = __ballot_sync(kFull, nch & 4u), b3 = __ballot_sync(kFull, nch & 8u);
             if (nch) {
                 int pos = fc + __popc(b0 & lt) + 2 * __popc(b1 & lt) + 4 * __popc(b2 & lt) + 8 * __popc(b3 & lt);
-                const int gb = item & ~kEntMask;
-                if (cm & 1u) S.stack[pos++] = gb | clo.x;
-                if (cm & 2u) S.stack[pos++] = gb | clo.y;
-                if (cm & 4u) S.stack[pos++] = gb | clo.z;
-                if (cm & 8u) S.stack[pos++] = gb | clo.w;
-                if (cm & 16u) S.stack[pos++] = gb | chi.x;
-                if (cm & 32u) S.stack[pos++] = gb | chi.y;
-                if (cm & 64u) S.stack[pos++] = gb | chi.z;
-                if (cm & 128u) S.stack[pos++] = gb | chi.w;
+                const unsigned gb = item & ~(unsigned)kEntMask;
+                if (cm & 1u) S.stack[pos++] = gb | (unsigned)clo.x;
+                if (cm & 2u) S.stack[pos++] = gb | (unsigned)clo.y;
+                if (cm & 4u) S.stack[pos++] = gb | (unsigned)clo.z;
+                if (cm & 8u) S.stack[pos++] = gb | (unsigned)clo.w;
+                if (cm & 16u) S.stack[pos++] = gb | (unsigned)chi.x;
+                if (cm & 32u) S.stack[pos++] = gb | (unsigned)chi.y;
+                if (cm & 64u) S.stack[pos++] = gb | (unsigned)chi.z;
+                if (cm & 128u) S.stack[pos++] = gb | (unsigned)chi.w;
             }
             fc += __popc(b0) + 2 * __popc(b1) + 4 * __popc(b2) + 8 * __popc(b3);
         }
         __syncwarp();
-        test_candidates(A, S, nc, in, T, itab, nh);
+        test_candidates(A, S, nc, seg, T, itab, nh);
         __syncwarp();
     }
     record_pairs(A, S, 0, nh, itab);
@@ -354,46 +377,52 @@ __device__ __forceinline__ void collide(const CollArgs& A, SearchSmem& S, int wb
     T.r = (float)A.r[i];
     unsigned todo = __ballot_sync(kFull, valid && root >= 0);
     while (todo) {
-        // the next run of targets in one box
-        const int first = __ffs(todo) - 1;
-        const int b = __shfl_sync(kFull, box, first);
-        unsigned seg = __ballot_sync(kFull, box == b) & todo;
-        bool in = (seg >> lane) & 1u;
-        const float reach = (redux_max(in ? T.r : 0.f) + A.rmaxf) * 1.0001f;
-        Box3 B = warp_box(in, T.hx, T.hy, T.hz);
-        // cut it at the widest gap along its widest side while that leaves
-        // less to search; the other part stays in todo
-        while (seg & (seg - 1)) {
-            const float wx = B.hx - B.lx, wy = B.hy - B.ly, wz = B.hz - B.lz, w = fmaxf(wx, fmaxf(wy, wz));
-            if (!(w > 4.f * reach)) break;
-            const float c = w == wx ? T.hx : w == wy ? T.hy : T.hz;
-            float next = __int_as_float(0x7f800000);   // the nearest target further along, if any
-            for (unsigned m = seg; m; m &= m - 1) {
-                const float o = __shfl_sync(kFull, c, __ffs(m) - 1);
-                if (o > c) next = fminf(next, o);
+        // up to kSegs compact parts of the targets left, all in one box
+        int nseg = 0, mine = -1;
+        const int lead = __ffs(todo) - 1, b = __shfl_sync(kFull, box, lead), r = __shfl_sync(kFull, root, lead);
+        const unsigned here = __ballot_sync(kFull, box == b);
+        __syncwarp();   // the last search has read its segments
+        for (; (todo & here) && nseg < kSegs; nseg++) {
+            unsigned seg = here & todo;
+            const int first = __ffs(seg) - 1;
+            bool in = (seg >> lane) & 1u;
+            const float reach = (redux_max(in ? T.r : 0.f) + A.rmaxf) * 1.0001f;
+            Box3 B = warp_box(in, T.hx, T.hy, T.hz);
+            // cut it at the widest gap along its widest side while that leaves
+            // less to search; the other part stays in todo
+            while (seg & (seg - 1)) {
+                const float wx = B.hx - B.lx, wy = B.hy - B.ly, wz = B.hz - B.lz, w = fmaxf(wx, fmaxf(wy, wz));
+                if (!(w > 4.f * reach)) break;
+                const float c = w == wx ? T.hx : w == wy ? T.hy : T.hz;
+                float next = __int_as_float(0x7f800000);   // the nearest target further along, if any
+                for (unsigned m = seg; m; m &= m - 1) {
+                    const float o = __shfl_sync(kFull, c, __ffs(m) - 1);
+                    if (o > c) next = fminf(next, o);
+                }
+                const float gap = in && next < __int_as_float(0x7f800000) ? next - c : 0.f;
+                const float widest = redux_max(gap);
+                if (!(widest > 2.f * reach)) break;
+                const float cut = redux_min(gap == widest ? c : __int_as_float(0x7f800000));
+                const bool lo = in && c <= cut;
+                const Box3 B1 = warp_box(lo, T.hx, T.hy, T.hz), B2 = warp_box(in && !lo, T.hx, T.hy, T.hz);
+                if (!(searched(B1, reach) + searched(B2, reach) < 0.75f * searched(B, reach))) break;
+                const unsigned part = __ballot_sync(kFull, lo);
+                const bool up = (part >> first & 1u) == 0u;   // go on with the first target's part
+                seg &= up ? ~part : part;
+                in = (seg >> lane) & 1u;
+                B = up ? B2 : B1;
             }
-            const float gap = in && next < __int_as_float(0x7f800000) ? next - c : 0.f;
-            const float widest = redux_max(gap);
-            if (!(widest > 2.f * reach)) break;
-            const float cut = redux_min(gap == widest ? c : __int_as_float(0x7f800000));
-            const bool lo = in && c <= cut;
-            const Box3 B1 = warp_box(lo, T.hx, T.hy, T.hz), B2 = warp_box(in && !lo, T.hx, T.hy, T.hz);
-            if (!(searched(B1, reach) + searched(B2, reach) < 0.75f * searched(B, reach))) break;
-            const unsigned part = __ballot_sync(kFull, lo);
-            const bool up = (part >> first & 1u) == 0u;   // go on with the first target's part
-            seg &= up ? ~part : part;
-            in = (seg >> lane) & 1u;
-            B = up ? B2 : B1;
+            todo &= ~seg;
+            if (in) mine = nseg;
+            const int min_slot = (int)__reduce_min_sync(kFull, in ? (unsigned)i : 0x7fffffffu);
+            if (lane == 0) {
+                const float size = fmaxf(fabsf(B.lx), fabsf(B.hx)) + fmaxf(fabsf(B.ly), fabsf(B.hy)) +
+                                   fmaxf(fabsf(B.lz), fabsf(B.hz));
+                S.seg[nseg] = Segment{B.lx, B.hx, B.ly, B.hy, B.lz, B.hz, reach, size, min_slot, __popc(seg)};
+            }
         }
-        todo &= ~seg;
-        const int min_slot = (int)__reduce_min_sync(kFull, in ? (unsigned)i : 0x7fffffffu);
-        const int r = __shfl_sync(kFull, root, first);
-        unsigned long long tested = 0;
-        search_segment<kCount>(A, S, in, T, B, reach, min_slot, r, A.img + (size_t)b * A.nimg, tested);
-        if (kCount) {
-            iters += tested;
-            visits += tested * (unsigned)__popc(seg);
-        }
+        __syncwarp();
+        search_segments<kCount>(A, S, nseg, mine, T, r, A.img + (size_t)b * A.nimg, visits, iters);
     }
 }
 
@@ -405,9 +434,13 @@ __global__ void __launch_bounds__(kMaxWalkBlock, 4) k_collide(CollArgs A) {
     unsigned long long visits = 0, iters = 0;
     for (int t = next_tile(A.tq, A.nq, q, ntile); t >= 0; t = next_tile(A.tq, A.nq, q, ntile))
         collide<kCount>(A, sm[threadIdx.x >> 5], t * A.width, n, visits, iters);
-    if (kCount && (threadIdx.x & 31) == 0) {
-        atomicAdd(&A.ctl->n_visit, visits);
-        atomicAdd(&A.ctl->n_siter, iters);
+    if (kCount) {   // visits: per lane
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) visits += __shfl_down_sync(kFull, visits, o);
+        if ((threadIdx.x & 31) == 0) {
+            atomicAdd(&A.ctl->n_visit, visits);
+            atomicAdd(&A.ctl->n_siter, iters);
+        }
     }
 }
 
