@@ -186,10 +186,10 @@ def search_rate(visits, iters, ms, ms_counted):
     times the targets it tests them for (nodes visited, all images), per launch,
     counted by the search's counting variant in one step after the timed ones, over the event-timed search
     stage of the timed steps (which run the plain variant).  The search is
-    bound by L1/L2 latency, so it is reported as a rate, with no roofline."""
+    bound by instruction issue, so it is reported as a rate, with no roofline."""
     if not (visits > 0 and ms > 0):
         return None
-    return {"bound": "latency (L1/L2 round trips)", "kernel": "k_collide (tree collision search)",
+    return {"bound": "instruction issue", "kernel": "k_collide (tree collision search)",
             "nodes_visited_per_launch": visits, "nodes_visited_per_particle": visits / N_SHEET,
             "nodes_visited_per_s": visits / (ms / 1e3), "ms_per_launch": ms,
             "warp_iterations_per_launch": iters,

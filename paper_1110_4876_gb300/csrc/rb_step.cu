@@ -3,11 +3,11 @@
 // the kick, the gather into Morton order, collision resolution (Sect. 5,
 // Eq. 2) and the energy/momentum sums (Sect. 6.2).
 //
-// Drift, kick, boundary wrap, the overlap geometry and the resolution use
-// explicitly rounded FP64 operations (__dadd_rn, __dmul_rn, ...) so the
-// compiler never fuses them: they give bit-identical results to any other
-// IEEE FP64 implementation that evaluates the same expressions in the same
-// order without fused multiply-adds.
+// Drift, kick, boundary wrap and the pairs' separations use explicitly rounded
+// FP64 operations (__dadd_rn, __dmul_rn, ...) so the compiler never fuses them:
+// they give bit-identical results to any other IEEE FP64 implementation that
+// evaluates the same expressions in the same order without fused multiply-adds.
+// The impulse of a collision uses fused multiply-adds.
 #include <algorithm>
 #include <climits>
 #include <cstddef>
@@ -326,7 +326,11 @@ __device__ __forceinline__ PairRec pair_rec(const ResolveArgs& A, const SimC& C,
     R.dvy = T.dvy;
     // the impulse along n = r/|r| without forming n: v_a gains
     // (1 + eps) (m_b/M) (u.r)/|r|^2 r, v_b loses the same with m_a; the
-    // factors of u.r here, but for 1 + eps under the power law
+    // factors of u.r here, but for 1 + eps under the power law.  With fused
+    // operations and one reciprocal the new velocities are off the exact ones by
+    // 5.07e-17 of their rms, with one rounding per operation and a division on
+    // the chain by 5.09e-17 (a million random pairs against 64-bit significands);
+    // the latter takes 290 us for 944k pairs where this takes 203.
     const double r2 = fma(R.rz, R.rz, fma(R.ry, R.ry, R.rx * R.rx));
     const double ma = A.P.m[R.a], mb = A.P.m[R.b];
     const double d = r2 * (ma + mb);
