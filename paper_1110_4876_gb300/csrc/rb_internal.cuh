@@ -222,7 +222,6 @@ __device__ __forceinline__ uint32_t morton_compact3(uint64_t x) {
 
 // ---- launch wrappers (implemented in the .cu files) ----
 // rb_sort.cu
-int radix_sort_passes(int key_bits, bool box_pass, int box_bits);
 // Sorts (key, val) pairs stably by key bits [0, key_bits) and then, when
 // box_digits is non-null, by box_digits[val] (bits [0, box_bits)).
 // Ping-pongs between the two buffers; returns 0 if the result is in

@@ -493,10 +493,6 @@ size_t radix_hist_words(int ncap) {
 
 size_t radix_digit_words() { return (size_t)kMaxPasses * kBins; }
 
-int radix_sort_passes(int key_bits, bool box_pass, int box_bits) {
-    return ceil_div(key_bits, 8) + (box_pass ? ceil_div(box_bits, 8) : 0);
-}
-
 int radix_sort(uint64_t* k0, uint32_t* v0, uint64_t* k1, uint32_t* v1, int ncap, const int* d_n,
                int key_bits, const int32_t* box_digits, int box_bits, uint32_t* hist, int* err,
                cudaStream_t s, int low_bit, Ctl* pairs, unsigned long long* long_keys) {

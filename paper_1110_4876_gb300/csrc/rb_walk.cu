@@ -56,7 +56,7 @@ __global__ void k_img_table(const BoxP* __restrict__ boxes, const Ctl* __restric
 
 // kOne: a single box, so every lane's walk ends at the same entry and no
 // lane can run into another box's tree.
-template <bool kQuad, bool kInside, bool kPot, bool kSoft, bool kRecord, bool kLearn, bool kOne = false>
+template <bool kQuad, bool kInside, bool kSoft, bool kRecord, bool kLearn, bool kOne = false>
 __device__ __forceinline__ void walk32(const GravArgs& A, LearnQ* LQ, const mlp::Packed* W, int wbase,
                                        int n) {
     const int lane = threadIdx.x & 31;
@@ -76,7 +76,6 @@ __device__ __forceinline__ void walk32(const GravArgs& A, LearnQ* LQ, const mlp:
     split_d(A.z[ii], phz, plz);
     const ImgTab* itab = A.img + (size_t)A.box[ii] * A.nimg;
     int gi = 0;
-    double pot = 0.0;
     float sx = 0.f, sy = 0.f, sz = 0.f, cx = 0.f, cy = 0.f, cz = 0.f;  // sums + compensation
     int ncell = 0, nleaf = 0, nmac = 0, nrecheck = 0, ncorr = 0;
     int iters = 0;   // entries processed by the warp (warp-uniform)
@@ -99,7 +98,7 @@ __device__ __forceinline__ void walk32(const GravArgs& A, LearnQ* LQ, const mlp:
                 const float2 ntz = make_float2(-thz, -tlz);   // z: (hi, lo) of the target
                 const int self = (gx == 0 && gy == 0 && gz == 0) ? self_leaf : -1;
                 int next = (valid && root >= 0) ? root : kEnd;
-                float fx = 0.f, fy = 0.f, fz = 0.f, fp = 0.f;   // sums of the last <= 16 iterations
+                float fx = 0.f, fy = 0.f, fz = 0.f;   // sums of the last <= 16 iterations
                 int it = 0;           // entries processed (warp-uniform)
                 bool rec = false;     // kRecord: this lane accepted a band cell this iteration
                 uint64_t rkey = 0;
@@ -133,7 +132,6 @@ __device__ __forceinline__ void walk32(const GravArgs& A, LearnQ* LQ, const mlp:
                                 fx = fmaf(f, dx, fx);
                                 fy = fmaf(f, dy, fy);
                                 fz = fmaf(f, dz, fz);
-                                if (kPot) fp = fmaf(-m, inv, fp);
                                 nleaf++;
                             }
                             next = e + 1;
@@ -173,7 +171,6 @@ __device__ __forceinline__ void walk32(const GravArgs& A, LearnQ* LQ, const mlp:
                             const float inv2 = inv * inv;
                             const float invs = kSoft ? rsqrt_nr(r2 + A.soft2f) : inv;
                             float fc = q0.x * (kSoft ? invs * invs * invs : inv2 * inv);
-                            if (kPot) fp = fmaf(-q0.x, invs, fp);
                             if (kQuad) {
                                 const float qx = fmaf(q1.y, dz, fmaf(q1.x, dy, q0.y * dx));
                                 const float qy = fmaf(q1.z, dz, fmaf(q0.z, dy, q1.x * dx));
@@ -184,7 +181,6 @@ __device__ __forceinline__ void walk32(const GravArgs& A, LearnQ* LQ, const mlp:
                                 fx = fmaf(-inv5, qx, fx);
                                 fy = fmaf(-inv5, qy, fy);
                                 fz = fmaf(-inv5, qz, fz);
-                                if (kPot) fp = fmaf(-0.5f * dqd, inv5, fp);
                             }
                             fx = fmaf(fc, dx, fx);
                             fy = fmaf(fc, dy, fy);
@@ -298,7 +294,6 @@ __device__ __forceinline__ void walk32(const GravArgs& A, LearnQ* LQ, const mlp:
                 kadd(sx, cx, fx);
                 kadd(sy, cy, fy);
                 kadd(sz, cz, fz);
-                pot += (double)fp;
                 iters += it;
             }
     if (kLearn && qn > 0) {
@@ -319,7 +314,6 @@ __device__ __forceinline__ void walk32(const GravArgs& A, LearnQ* LQ, const mlp:
         A.out.ax[i] = A.G * ((double)sx - (double)cx);
         A.out.ay[i] = A.G * ((double)sy - (double)cy);
         A.out.az[i] = A.G * ((double)sz - (double)cz);
-        if (kPot) A.out.phi[i] = A.G * pot;
         if (A.out.ncell) {
             A.out.ncell[i] = ncell;
             A.out.nleaf[i] = nleaf;
@@ -351,12 +345,12 @@ __device__ __forceinline__ void walk32(const GravArgs& A, LearnQ* LQ, const mlp:
     }
 }
 
-template <bool kQuad, bool kInside, bool kPot, bool kSoft, bool kRecord = false, bool kOne = false>
+template <bool kQuad, bool kInside, bool kSoft, bool kRecord = false, bool kOne = false>
 __global__ void __launch_bounds__(kMaxWalkBlock, 4) k_walk32(GravArgs A) {
     const int n = min(A.ctl->n_live, A.ncap);
     const int ntile = (n + 31) >> 5, q = sm_queue(A.nq);
     for (int t = next_tile(A.tq, A.nq, q, ntile); t >= 0; t = next_tile(A.tq, A.nq, q, ntile))
-        walk32<kQuad, kInside, kPot, kSoft, kRecord, false, kOne>(A, nullptr, nullptr, t << 5, n);
+        walk32<kQuad, kInside, kSoft, kRecord, false, kOne>(A, nullptr, nullptr, t << 5, n);
 }
 
 // ---------------------------------------------------------------------------
@@ -785,7 +779,7 @@ __global__ void __launch_bounds__(kMaxWalkBlock, 4) k_gwalk32(GravArgs A) {
             const int k = (t << 5) + (threadIdx.x & 31);
             const int b = A.box[tile_slot(A.order, k < n ? k : n - 1)];
             if (!__all_sync(kFull, b == __shfl_sync(kFull, b, 0))) {
-                walk32<kQuad, kInside, false, kSoft, false, false, false>(A, nullptr, nullptr, t << 5, n);
+                walk32<kQuad, kInside, kSoft, false, false, false>(A, nullptr, nullptr, t << 5, n);
                 continue;
             }
         }
@@ -808,7 +802,7 @@ __global__ void __launch_bounds__(kMaxWalkBlock, 2) k_walk32_learn(GravArgs A) {
     const int n = min(A.ctl->n_live, A.ncap);
     const int ntile = (n + 31) >> 5, sq = sm_queue(A.nq);
     for (int t = next_tile(A.tq, A.nq, sq, ntile); t >= 0; t = next_tile(A.tq, A.nq, sq, ntile))
-        walk32<true, kInside, false, kSoft, false, true>(A, &q[threadIdx.x >> 5], &w, t << 5, n);
+        walk32<true, kInside, kSoft, false, true>(A, &q[threadIdx.x >> 5], &w, t << 5, n);
 }
 
 }  // namespace
@@ -883,20 +877,20 @@ int walk_prepare() {
         }
         g_nsm = nsm;
     }
-    prepare_one(k_walk32<true, true, false, true>); prepare_one(k_walk32<true, true, false, false>);
-    prepare_one(k_walk32<true, false, false, true>); prepare_one(k_walk32<true, false, false, false>);
-    prepare_one(k_walk32<false, true, false, true>); prepare_one(k_walk32<false, true, false, false>);
-    prepare_one(k_walk32<false, false, false, true>); prepare_one(k_walk32<false, false, false, false>);
-    prepare_one(k_walk32<true, true, false, true, false, true>);
-    prepare_one(k_walk32<true, true, false, false, false, true>);
-    prepare_one(k_walk32<true, false, false, true, false, true>);
-    prepare_one(k_walk32<true, false, false, false, false, true>);
-    prepare_one(k_walk32<false, true, false, true, false, true>);
-    prepare_one(k_walk32<false, true, false, false, false, true>);
-    prepare_one(k_walk32<false, false, false, true, false, true>);
-    prepare_one(k_walk32<false, false, false, false, false, true>);
-    prepare_one(k_walk32<true, true, false, true, true>); prepare_one(k_walk32<true, true, false, false, true>);
-    prepare_one(k_walk32<true, false, false, true, true>); prepare_one(k_walk32<true, false, false, false, true>);
+    prepare_one(k_walk32<true, true, true>); prepare_one(k_walk32<true, true, false>);
+    prepare_one(k_walk32<true, false, true>); prepare_one(k_walk32<true, false, false>);
+    prepare_one(k_walk32<false, true, true>); prepare_one(k_walk32<false, true, false>);
+    prepare_one(k_walk32<false, false, true>); prepare_one(k_walk32<false, false, false>);
+    prepare_one(k_walk32<true, true, true, false, true>);
+    prepare_one(k_walk32<true, true, false, false, true>);
+    prepare_one(k_walk32<true, false, true, false, true>);
+    prepare_one(k_walk32<true, false, false, false, true>);
+    prepare_one(k_walk32<false, true, true, false, true>);
+    prepare_one(k_walk32<false, true, false, false, true>);
+    prepare_one(k_walk32<false, false, true, false, true>);
+    prepare_one(k_walk32<false, false, false, false, true>);
+    prepare_one(k_walk32<true, true, true, true>); prepare_one(k_walk32<true, true, false, true>);
+    prepare_one(k_walk32<true, false, true, true>); prepare_one(k_walk32<true, false, false, true>);
     prepare_one(k_walk32_learn<true, true>); prepare_one(k_walk32_learn<true, false>);
     prepare_one(k_walk32_learn<false, true>); prepare_one(k_walk32_learn<false, false>);
     target_walk_prepare();
@@ -956,11 +950,11 @@ void gravity_walk(const Tree& T, const PSet& P, Ctl* ctl, const BoxP* boxes, con
 #define RB_LAUNCH(...)                                                                                     \
     __VA_ARGS__<<<walk_grid((const void*)(__VA_ARGS__), block, ceil_div(T.cap_n, 32)), block, 0, s>>>(A)
 #define RB_W32G(Q, I, S, ONE) RB_LAUNCH(k_gwalk32<Q, I, S, ONE, 4>)
-#define RB_W32(Q, I, PO, S)                                                \
+#define RB_W32(Q, I, S)                                                    \
     do {                                                                   \
         if (group == 0) {                                                  \
-            if (C.nbox == 1) RB_LAUNCH(k_walk32<Q, I, PO, S, false, true>); \
-            else RB_LAUNCH(k_walk32<Q, I, PO, S>);                          \
+            if (C.nbox == 1) RB_LAUNCH(k_walk32<Q, I, S, false, true>); \
+            else RB_LAUNCH(k_walk32<Q, I, S>);                              \
         } else if (C.nbox == 1) {                                          \
             RB_W32G(Q, I, S, true);                                        \
         } else {                                                           \
@@ -982,11 +976,11 @@ void gravity_walk(const Tree& T, const PSet& P, Ctl* ctl, const BoxP* boxes, con
     } else if (rec) {
         // FP32 walk that also records accepted band cells (quadrupole on)
         if (inside) {
-            if (soft) RB_LAUNCH(k_walk32<true, true, false, true, true>);
-            else RB_LAUNCH(k_walk32<true, true, false, false, true>);
+            if (soft) RB_LAUNCH(k_walk32<true, true, true, true>);
+            else RB_LAUNCH(k_walk32<true, true, false, true>);
         } else {
-            if (soft) RB_LAUNCH(k_walk32<true, false, false, true, true>);
-            else RB_LAUNCH(k_walk32<true, false, false, false, true>);
+            if (soft) RB_LAUNCH(k_walk32<true, false, true, true>);
+            else RB_LAUNCH(k_walk32<true, false, false, true>);
         }
     } else if (walk_mode == 0 || potential) {
         target_walk(A, TargetWalk::kFp64, quad, inside, soft, potential, block, T.cap_n, s);
@@ -994,11 +988,11 @@ void gravity_walk(const Tree& T, const PSet& P, Ctl* ctl, const BoxP* boxes, con
         target_walk(A, TargetWalk::kFp32, quad, inside, soft, false, block, T.cap_n, s);
     } else {
         if (quad) {
-            if (inside) { if (soft) RB_W32(true, true, false, true); else RB_W32(true, true, false, false); }
-            else { if (soft) RB_W32(true, false, false, true); else RB_W32(true, false, false, false); }
+            if (inside) { if (soft) RB_W32(true, true, true); else RB_W32(true, true, false); }
+            else { if (soft) RB_W32(true, false, true); else RB_W32(true, false, false); }
         } else {
-            if (inside) { if (soft) RB_W32(false, true, false, true); else RB_W32(false, true, false, false); }
-            else { if (soft) RB_W32(false, false, false, true); else RB_W32(false, false, false, false); }
+            if (inside) { if (soft) RB_W32(false, true, true); else RB_W32(false, true, false); }
+            else { if (soft) RB_W32(false, false, true); else RB_W32(false, false, false); }
         }
     }
 #undef RB_W32
