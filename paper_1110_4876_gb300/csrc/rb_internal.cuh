@@ -255,6 +255,9 @@ void build_tile_order(Tree& T, const PSet& P, Ctl* ctl, int mode, int box_bits, 
 // records only.
 void build_gravity_records(const Tree& T, const PSet& P, Ctl* ctl, const BoxP* boxes,
                            const SimC& C, bool fp64, cudaStream_t s, bool f32q = false);
+// Up to this capacity the leaves get multipole records too (mass, Q = 0), which
+// the FP32 walks with one or two targets per warp read without asking.
+constexpr int kLeafQMax = 130000;
 size_t moment_span_words(int ncap);
 size_t moment_pieces(int ncap);   // records kept behind the tree's entries
 // Collision records on the tree of the last build at the current positions

@@ -282,6 +282,7 @@ struct GravRecArgs {
     const Ctl* ctl;
     int ncap;
     double crit_scale;  // 1 / theta^2
+    bool leafq;         // leaves get FP32 multipole records (mass, Q = 0)
     bool q32, inside;   // q32: FP32 quadrupole records are read too (not by the FP64 walk)
 };
 
@@ -297,6 +298,10 @@ __device__ __forceinline__ void leaf_record(const GravRecArgs& A, int p) {
     split_hilo(z, hz, lz);
     A.ra[e] = make_float4(hx, hy, hz, lz);
     A.rb[e] = make_float4(lx, ly, -(float)m, __int_as_float(e + 1));
+    if (A.leafq) {
+        A.rq0[e] = make_float4((float)m, 0.f, 0.f, 0.f);
+        A.rq1[e] = make_float4(0.f, 0.f, 0.f, 0.f);
+    }
 }
 
 // A cell's moments come from its children (cells done before it, or particle
@@ -1216,6 +1221,7 @@ void build_gravity_records(const Tree& T, const PSet& P, Ctl* ctl, const BoxP* b
     A.ncap = n;
     A.crit_scale = C.crit_scale;
     A.q32 = !fp64;
+    A.leafq = !fp64 && n <= kLeafQMax;
     A.inside = C.theta2 > (1.0 / 3.0);
     const bool q32 = f32q && !fp64;
     const int slots = moment_slots(n);

@@ -35,7 +35,8 @@
 // of the slots) and the L1 wavefronts of its gathers (70%); pairs by the latency
 // of the gathers with 24 warps per SM.  30,011 targets of the sheet: 215 -> 160
 // us, 50,000: 345 -> 250, 5,000: 69 -> 49.  Loading the children before the
-// terms are formed is 5% of that; 16 warps per SM (no spills) take 20% longer,
+// terms are formed is 5% of that, and leaves with multipole records of their own,
+// which spare the selection, took it to 154, 242 and 47; 16 warps per SM (no spills) take 20% longer,
 // 32 warps 8%.
 #include <algorithm>
 #include <type_traits>
@@ -328,7 +329,7 @@ __device__ __forceinline__ void walk_target(const GravArgs& A, TSmem<k64>& S, Le
                 e = item & kEntMask;
                 const int g = item >> kEntBits;
                 ld_pair(A.ra, e, ra, rb);
-                if (!k64) ld_pair(A.rq0, e, q0, q1);   // of no meaning for a leaf
+                if (!k64) ld_pair(A.rq0, e, q0, q1);   // of a leaf: its mass, Q = 0
                 const float4 t = S.txy[g];
                 const float2 tz = S.tz[g];
                 rec_diff(ra, rb, make_float2(t.x, t.y), make_float2(t.z, t.w), tz, dx, dy, dz, r2);
@@ -368,10 +369,6 @@ __device__ __forceinline__ void walk_target(const GravArgs& A, TSmem<k64>& S, Le
                     L.ncell += acc;
                 }
                 if (!k64 && acc) {
-                    if (leaf) {
-                        q0 = make_float4(-crit, 0.f, 0.f, 0.f);
-                        q1 = make_float4(0.f, 0.f, 0.f, 0.f);
-                    }
                     // a leaf is the cell with Q = 0; its distance may be zero when softened
                     inv = rsqrt_nr(kSoft && leaf ? r2 + A.soft2f : r2);
                     const float inv2 = inv * inv;
@@ -739,12 +736,7 @@ __device__ __forceinline__ void walk_pair(const GravArgs& A, PSmem& S, int i0, i
                     // both targets' terms at once; a leaf is the cell with Q = 0, whose
                     // distance may be zero when softened
                     float4 q0, q1;
-                    if (leaf) {
-                        q0 = make_float4(-crit, 0.f, 0.f, 0.f);
-                        q1 = make_float4(0.f, 0.f, 0.f, 0.f);
-                    } else {
-                        ld_pair(A.rq0, e, q0, q1);
-                    }
+                    ld_pair(A.rq0, e, q0, q1);
                     const float2 rs = kSoft ? __fadd2_rn(r2, two(A.soft2f)) : r2;
                     const float2 inv = rsqrt2_nr(kSoft && leaf ? rs : r2);
                     const float2 inv2 = __fmul2_rn(inv, inv);

@@ -70,6 +70,8 @@ int walk_grid(const void* fn, int block, long long warps);
 constexpr int kTargetWalkMax = 75000;           // targets in a Hilbert order
 constexpr int kTargetWalkMaxMorton = 125000;
 constexpr int kTargetWalkMaxLearned = 130000;
+static_assert(kTargetWalkMax <= kLeafQMax && kTargetWalkMaxMorton <= kLeafQMax && kTargetWalkMaxLearned <= kLeafQMax,
+              "these walks read the leaves' multipole records");
 enum class TargetWalk { kFp32, kFp64, kLearned };
 void target_walk(const GravArgs& A, TargetWalk mode, bool quad, bool inside, bool soft, bool pot, int block,
                  int cap_n, cudaStream_t s);
