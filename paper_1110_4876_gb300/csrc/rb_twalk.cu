@@ -379,7 +379,8 @@ __device__ __forceinline__ void walk_target(const GravArgs& A, TSmem<k64>& S, Le
                         const float qy = fmaf(q1.z, dz, fmaf(q0.z, dy, q1.x * dx));
                         const float qz = fmaf(q0.w, dz, fmaf(q1.z, dy, q1.y * dx));
                         const float dqd = fmaf(dz, qz, fmaf(dy, qy, dx * qx));
-                        const float inv5 = inv2 * inv2 * inv;
+                        // none for a leaf: r^-5 and r^-7 overflow at distances where its term does not
+                        const float inv5 = leaf ? 0.f : inv2 * inv2 * inv;
                         f = fmaf(2.5f, dqd * (inv5 * inv2), f);
                         L.fx = fmaf(-inv5, qx, L.fx);
                         L.fy = fmaf(-inv5, qy, L.fy);
@@ -750,7 +751,8 @@ __device__ __forceinline__ void walk_pair(const GravArgs& A, PSmem& S, int i0, i
                         const float2 qz =
                             __ffma2_rn(two(q0.w), dz, __ffma2_rn(two(q1.z), dy, __fmul2_rn(two(q1.y), dx)));
                         const float2 dqd = __ffma2_rn(dz, qz, __ffma2_rn(dy, qy, __fmul2_rn(dx, qx)));
-                        const float2 inv5 = __fmul2_rn(__fmul2_rn(inv2, inv2), inv);
+                        // none for a leaf, as above
+                        const float2 inv5 = leaf ? two(0.f) : __fmul2_rn(__fmul2_rn(inv2, inv2), inv);
                         f = __ffma2_rn(two(2.5f), __fmul2_rn(dqd, __fmul2_rn(inv5, inv2)), f);
                         const float2 n5 = make_float2(a0 ? -inv5.x : 0.f, a1 ? -inv5.y : 0.f);
                         L.fx = __ffma2_rn(n5, qx, L.fx);
