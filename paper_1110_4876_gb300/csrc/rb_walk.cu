@@ -463,7 +463,7 @@ __device__ __forceinline__ void eval_list(const GravArgs& A, const float4 (*rec)
                 L.nleaf++;
             }
         } else {
-            cell_term<kQuad, kSoft>(dx, dy, dz, r2, rec[j][2], rec[j][3], A.soft2f, L.fx, L.fy, L.fz);
+            cell_term<kQuad, kSoft>(dx, dy, dz, r2, rec[j][2], rec[j][3], false, A.soft2f, L.fx, L.fy, L.fz);
         }
         glane_count(L);
     }
@@ -568,7 +568,7 @@ __device__ __forceinline__ void mixed_walks(const GravArgs& A, const int2* mix, 
                     q0 = __ldg(&A.rq0[e]);
                     q1 = __ldg(&A.rq1[e]);
                 }
-                cell_term<kQuad, kSoft>(dx, dy, dz, r2, q0, q1, A.soft2f, L.fx, L.fy, L.fz);
+                cell_term<kQuad, kSoft>(dx, dy, dz, r2, q0, q1, leaf, A.soft2f, L.fx, L.fy, L.fz);
             }
         }
         L.iters++;

@@ -207,12 +207,14 @@ __device__ __forceinline__ bool inside64(const double4_32a& c, double tx, double
 }
 
 // Monopole + quadrupole term of an accepted cell (reading R3), the same
-// arithmetic as the union walk's; a particle leaf is the cell with Q = 0.
+// arithmetic as the union walk's.  A particle leaf is the cell with Q = 0, but
+// for its distance, which may be zero when softened, and for r^-5 and r^-7,
+// which overflow at distances where its term does not.
 template <bool kQuad, bool kSoft>
 __device__ __forceinline__ void cell_term(float dx, float dy, float dz, float r2, const float4& q0,
-                                          const float4& q1, float soft2f, float& fx, float& fy,
+                                          const float4& q1, bool leaf, float soft2f, float& fx, float& fy,
                                           float& fz) {
-    const float inv = rsqrt_nr(r2);
+    const float inv = rsqrt_nr(kSoft && leaf ? r2 + soft2f : r2);
     const float inv2 = inv * inv;
     const float invs = kSoft ? rsqrt_nr(r2 + soft2f) : inv;
     float fc = q0.x * (kSoft ? invs * invs * invs : inv2 * inv);
@@ -221,7 +223,7 @@ __device__ __forceinline__ void cell_term(float dx, float dy, float dz, float r2
         const float qy = fmaf(q1.z, dz, fmaf(q0.z, dy, q1.x * dx));
         const float qz = fmaf(q0.w, dz, fmaf(q1.z, dy, q1.y * dx));
         const float dqd = fmaf(dz, qz, fmaf(dy, qy, dx * qx));
-        const float inv5 = inv2 * inv2 * inv;
+        const float inv5 = leaf ? 0.f : inv2 * inv2 * inv;
         fc = fmaf(2.5f, dqd * (inv5 * inv2), fc);
         fx = fmaf(-inv5, qx, fx);
         fy = fmaf(-inv5, qy, fy);

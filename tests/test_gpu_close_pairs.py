@@ -11,7 +11,7 @@ pytestmark = pytest.mark.gpu
 
 # the form that runs depends on the particle capacity: one target per warp,
 # two from 3,000, 32 above 130,000; walk group 4 at any size
-FORMS = {"one": (None, 0), "two": (3_003, 0), "union": (130_001, 0)}
+FORMS = {"one": (None, 0), "two": (3_003, 0), "union": (130_001, 0), "group": (None, 4)}
 
 
 @pytest.fixture(scope="module")
@@ -47,9 +47,8 @@ def _check(a, cnt, P, ref, ref_cnt):
         assert np.max(np.linalg.norm((a - ref)[sel], axis=1) / den) <= 1e-5
 
 
-@pytest.mark.parametrize("soft", [0.0, 1e-9])
-@pytest.mark.parametrize("gap", [1e-6, 1e-8])
-@pytest.mark.parametrize("form", ["one", "two", "union"])
+@pytest.mark.parametrize("gap,soft", [(1e-6, 0.0), (1e-8, 0.0), (1e-6, 1e-9), (1e-8, 1e-9), (0.0, 1e-9)])
+@pytest.mark.parametrize("form", FORMS)
 def test_forces_of_close_pairs(rb, orc, form, gap, soft):
     capacity, group = FORMS[form]
     P = _pairs(gap)
