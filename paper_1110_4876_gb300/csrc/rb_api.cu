@@ -168,6 +168,7 @@ void make_constants(rb_sim* s) {
     C.nimg = (2 * C.ngx + 1) * (2 * C.ngy + 1) * (2 * C.ngz + 1);
     C.has_test = s->n_active >= 0;
     C.eps_law = s->eps_law;
+    C.learned = c.walk == RB_WALK_FP32_LEARNED;
     C.hold_pair = s->hold_pair;
     C.key_low = s->long_runs ? 0 : s->key_low;
     C.eps_vc = s->eps_vc;

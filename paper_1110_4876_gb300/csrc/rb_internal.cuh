@@ -44,6 +44,7 @@ struct SimC {
     double crit_scale;   // 1 / theta^2 (FP32 criterion (w / theta)^2)
     int has_test;        // some particles are test particles (source mass 0)
     int eps_law;         // 0: constant eps; 1: eps = min(1, (|v_n| / eps_vc)^(-eps_p))
+    int learned;         // the walk runs the network, which reads the cells' corners at every theta
     int hold_pair;       // test hook: the queue's first pair never becomes ready
     int key_low;         // Morton key bits below those that the particle sort's passes take
     double eps_vc, eps_p;

@@ -283,7 +283,8 @@ struct GravRecArgs {
     int ncap;
     double crit_scale;  // 1 / theta^2
     bool leafq;         // leaves get FP32 multipole records (mass, Q = 0)
-    bool q32, inside;   // q32: FP32 quadrupole records are read too (not by the FP64 walk)
+    bool q32;           // FP32 quadrupole records are read too (not by the FP64 walk)
+    bool corners;       // cell corners are read (inside test, network inputs)
 };
 
 // Leaf record (FP64 and FP32) of particle p.
@@ -458,7 +459,7 @@ __device__ __forceinline__ void mom_finish(const GravRecArgs& A, int k, int dept
     const double w = scale_down(L, v);
     const double lo = -0.5 * L;
     double ix = 0.0, iy = 0.0, iz = 0.0;
-    if (A.inside || !(S.M > 0.0)) cell_index(A.key[first], v, ix, iy, iz);
+    if (A.corners || !(S.M > 0.0)) cell_index(A.key[first], v, ix, iy, iz);
     double cx, cy, cz, ux, uy, uz;   // centre of mass and its offset from o
     if (S.M > 0.0) {
         const double iM = rcp64(S.M);
@@ -480,7 +481,7 @@ __device__ __forceinline__ void mom_finish(const GravRecArgs& A, int k, int dept
         A.d_q1[k] = make_double4_32a(S.q[3], S.q[4], S.q[5], w);
     }
     double c0x = 0.0, c0y = 0.0, c0z = 0.0;
-    if (A.inside) {
+    if (A.corners) {
         // cell corner lo + i w, rounded as two separate operations
         c0x = __dadd_rn(lo, __dmul_rn(ix, w));
         c0y = __dadd_rn(lo, __dmul_rn(iy, w));
@@ -503,7 +504,7 @@ __device__ __forceinline__ void mom_finish(const GravRecArgs& A, int k, int dept
             A.rq1[k] = make_float4((float)S.q[3], (float)S.q[4], (float)S.q[5], 0.f);
         }
     }
-    if (A.inside) {
+    if (A.corners) {
         split_hilo(c0x, hx, lx);
         split_hilo(c0y, hy, ly);
         split_hilo(c0z, hz, lz);
@@ -1222,7 +1223,7 @@ void build_gravity_records(const Tree& T, const PSet& P, Ctl* ctl, const BoxP* b
     A.crit_scale = C.crit_scale;
     A.q32 = !fp64;
     A.leafq = !fp64 && n <= kLeafQMax;
-    A.inside = C.theta2 > (1.0 / 3.0);
+    A.corners = C.theta2 > (1.0 / 3.0) || C.learned;
     const bool q32 = f32q && !fp64;
     const int slots = moment_slots(n);
     const int nr = ceil_div(n, slots);

@@ -204,6 +204,36 @@ def test_correction_equals_oracle_sum_over_band_cells(rb, orc):
         assert np.linalg.norm(got - expect) <= 2e-2 * np.linalg.norm(expect) + 1e-3 * np.linalg.norm(a0[i])
 
 
+@pytest.mark.parametrize("capacity", [None, 130_001])   # one target per warp, 32 targets per warp
+def test_correction_at_an_opening_angle_without_the_inside_rule(rb, orc, capacity):
+    """theta = 0.55 < 1/sqrt(3): no cell's corner takes part in the opening test,
+    but the network's inputs 4 and 6 to 8 (the cell's width, the centre of mass
+    in the cell) are read from the corner records all the same."""
+    L, N = 100.0, 2400
+    P = I.sheet(L, N, 1)
+    w = omlp.init(5) * 0.3
+    acc = []
+    for walk in (rb.RB_WALK_FP32, rb.RB_WALK_FP32_LEARNED):
+        sim = rb.Sim(**sheet_cfg(rb, L, walk, 0.55))
+        if walk == rb.RB_WALK_FP32_LEARNED:
+            rb.rb_load_mlp(sim.h, w, 0.4)
+        if capacity:
+            sim.set_particles(I.sheet(L, capacity, 2))
+            sim.gravity()
+        sim.set_particles(P)
+        acc.append(sim.gravity())
+    targets = list(range(7, N, 300))
+    ref = _oracle_band_samples(orc, P, L, targets, 0.55, 0.4)
+    wb = _bf16(w)
+    for i in targets:
+        rows = [v for k, v in ref.items() if k[0] == i]
+        Yp, _ = omlp.forward(wb, _bf16(np.array([r[0] for r in rows])))
+        expect = (np.array([r[3] for r in rows]) * I.G_SI) @ Yp
+        got = acc[1][i] - acc[0][i]
+        # as in the test above
+        assert np.linalg.norm(got - expect) <= 2e-2 * np.linalg.norm(expect) + 1e-3 * np.linalg.norm(acc[0][i])
+
+
 def test_zero_network_is_the_plain_walk(rb):
     """With every weight zero the network outputs zero, so the learned walk
     (band cells queued through the network inside the walk) gives the plain
