@@ -13,6 +13,7 @@
 #include <cstddef>
 #include <type_traits>
 
+#include "rb_fp64.cuh"
 #include "rb_internal.cuh"
 
 namespace rb {
@@ -271,18 +272,6 @@ __global__ void __launch_bounds__(256) k_pair_link(ResolveArgs A) {
         A.link[k] = atomicExch(&A.head[key_b(A.key[k])], k);
         A.done[k] = 0;
     }
-}
-
-// 1/x from the hardware's coarse FP64 estimate and one step of the cubically
-// convergent iteration y (1 + h + h^2), h = 1 - x y; x outside the range
-// where the estimate is safe takes the division.
-__device__ __forceinline__ double rcp64(double x) {
-    const int e = (int)((__double_as_longlong(x) >> 52) & 0x7ff);
-    if (e < 64 || e > 1982) return __ddiv_rn(1.0, x);
-    double y;
-    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
-    const double h = fma(-x, y, 1.0);
-    return fma(y, fma(h, h, h), y);
 }
 
 // The last pair before k in particle p's list (pairs in which p is the higher

@@ -20,6 +20,7 @@
 #include <algorithm>
 #include <cfloat>
 
+#include "rb_fp64.cuh"
 #include "rb_internal.cuh"
 
 namespace rb {
@@ -403,19 +404,6 @@ __device__ __forceinline__ bool group_has_chain(const GravRecArgs& A, int first,
     if (first > 0 && A.box[first - 1] == b) d = max(d, common_levels(A.key[first - 1], kf));
     if (last + 1 < n && A.box[last + 1] == b) d = max(d, common_levels(kf, A.key[last + 1]));
     return d < kMaxDepth - 1;
-}
-
-// 1/x from the hardware's coarse FP64 estimate and one step of the cubically
-// convergent iteration y (1 + h + h^2), h = 1 - x y (four FP64 operations; a
-// division takes three times as many); x outside the range where the estimate
-// is safe takes the division.
-__device__ __forceinline__ double rcp64(double x) {
-    const int e = (int)((__double_as_longlong(x) >> 52) & 0x7ff);
-    if (e < 64 || e > 1982) return 1.0 / x;
-    double y;
-    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
-    const double h = fma(-x, y, 1.0);
-    return fma(y, fma(h, h, h), y);
 }
 
 // x 2^-v for x with exponent well inside the normal range (v <= 21).

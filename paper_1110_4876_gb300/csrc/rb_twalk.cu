@@ -41,6 +41,7 @@
 #include <algorithm>
 #include <type_traits>
 
+#include "rb_fp64.cuh"
 #include "rb_walk.cuh"
 
 namespace rb {
@@ -93,16 +94,6 @@ __device__ __forceinline__ void tsum_flush(TSum& L) {
     kadd(L.sy, L.cy, L.fy);
     kadd(L.sz, L.cz, L.fz);
     L.fx = L.fy = L.fz = 0.f;
-}
-
-// 1/sqrt(x) in FP64 from the hardware's coarse FP64 estimate and one step of
-// the cubically convergent iteration y (1 + h/2 + 3 h^2/8), h = 1 - x y^2
-// (the series of (1 - h)^(-1/2)): five FP64 operations.
-__device__ __forceinline__ double rsqrt64(double x) {
-    double y;
-    asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
-    const double h = fma(-x * y, y, 1.0);
-    return fma(y * h, fma(h, 0.375, 0.5), y);
 }
 
 // The child entries of a cell's octants (slots of empty octants hold any value).
