@@ -162,8 +162,9 @@ int rb_set_particles(rb_sim* sim, int box, int64_t n, const double* x, const dou
  * RB_ERR_NONFINITE (a position became non-finite or left the box by more
  * than 4096 box lengths in one drift half), RB_ERR_STATE (a malformed tree
  * met by a walk; the learned walk without weights), RB_ERR_TIMEOUT (a
- * bounded device wait gave up: the resolution queue's or a radix pass's
- * look-back), RB_ERR_CUDA. */
+ * bounded device wait gave up: the resolution's for an earlier pair, or that of
+ * a sort for its earlier tiles; what a sort left incomplete is not used further,
+ * and the particles have to be set again), RB_ERR_CUDA. */
 int rb_step(rb_sim* sim, int64_t nsteps);
 
 /* Copy the live particles of box `box`, in ascending id order, into host
@@ -225,6 +226,11 @@ int rb_set_pair_capacity(rb_sim* sim, int64_t cap);
  * step returns RB_ERR_TIMEOUT with the device context intact (velocities then
  * hold a partial resolution).  0 restores normal resolution. */
 int rb_debug_hold_pair(rb_sim* sim, int on);
+/* Test hook: the first tile of the sorts in `mask` (1 particles, 2 the scan of
+ * tree entries, 4 target order, 8 pairs, 16 plane-sweep items; 0 none) never
+ * publishes its counts: later tiles wait at most half a second, and the call
+ * returns RB_ERR_TIMEOUT with the device context intact. */
+int rb_debug_hold_sort(rb_sim* sim, int mask);
 /* Set / read the simulation time (restarts the step counter at t). */
 int rb_set_time(rb_sim* sim, double t);
 int rb_get_time(rb_sim* sim, double* t);

@@ -76,6 +76,7 @@ struct rb_sim {
     int64_t n_active = -1;                 // test particles: ids >= n_active per box
     int eps_law = 0;                       // restitution law (RB_EPS_*)
     int hold_pair = 0;                     // test hook (rb_debug_hold_pair)
+    int hold_sort = 0;                     // test hook (rb_debug_hold_sort)
     double eps_vc = 1.0, eps_p = 0.0;
     std::string err;
     cudaEvent_t ev0 = nullptr, ev1 = nullptr;
@@ -170,6 +171,7 @@ void make_constants(rb_sim* s) {
     C.eps_law = s->eps_law;
     C.learned = c.walk == RB_WALK_FP32_LEARNED;
     C.hold_pair = s->hold_pair;
+    C.hold_sort = s->hold_sort;
     C.key_low = s->long_runs ? 0 : s->key_low;
     C.eps_vc = s->eps_vc;
     C.eps_p = s->eps_p;
@@ -353,6 +355,10 @@ int upload(rb_sim* s) {
         }
         if (rc) return RB_ERR_CUDA;
         RB_CUDA(s, cudaMemsetAsync(T.hist, 0, sizeof(uint32_t) * radix_hist_words(cap), s->stream));
+        // slots that a pass which gave up has not written hold the last sort's
+        // values, or these: indices either way
+        for (uint32_t* v : {T.idx, T.idx_alt})
+            RB_CUDA(s, cudaMemsetAsync(v, 0, sizeof(uint32_t) * cap, s->stream));
         RB_CUDA(s, cudaMemsetAsync(s->ctl, 0, sizeof(Ctl), s->stream));
         s->ncap = cap;
         // a freshly drawn dense sheet overlaps about one pair per particle
@@ -474,7 +480,7 @@ int record_step(rb_sim* s, int p) {
         // arrays: it runs on the side stream while the moments run here
         cudaEventRecord(s->ev_fork, st);
         cudaStreamWaitEvent(s->side, s->ev_fork, 0);
-        build_tile_order(s->T, s->P[c], s->ctl, s->tile_order, s->box_bits, s->side);
+        build_tile_order(s->T, s->P[c], s->ctl, s->C, s->tile_order, s->box_bits, s->side);
         cudaEventRecord(s->ev_join, s->side);
         mark(s, 3);
         build_gravity_records(s->T, s->P[c], s->ctl, s->d_boxes, s->C, s->cfg.walk == RB_WALK_FP64, st, true);
@@ -504,7 +510,7 @@ int record_step(rb_sim* s, int p) {
         for (int k = 7; k <= 9; k++) mark(s, k);
         sweep_search(s->P[c], s->ctl, s->d_boxes, s->C, s->SW, s->PR, 2, s->ncap, st);
         mark(s, 10);
-        sort_pairs(s->PR, s->ctl, st, pair_key_bits(s));
+        sort_pairs(s->PR, s->ctl, s->C, st, pair_key_bits(s));
         mark(s, 11);
         resolve_pairs(s->P[c], s->ctl, s->d_boxes, s->C, s->PR, 2, s->T.img, false, true, st);
     } else if (s->cfg.collisions && s->cfg.gravity) {
@@ -517,7 +523,7 @@ int record_step(rb_sim* s, int p) {
         collision_search(s->T, s->P[c], s->ctl, s->d_boxes, s->C, s->PR, 2, st, s->search_block, s->rmax,
                          s->profiling == 2);
         mark(s, 10);
-        sort_pairs(s->PR, s->ctl, st, pair_key_bits(s));
+        sort_pairs(s->PR, s->ctl, s->C, st, pair_key_bits(s));
         mark(s, 11);
         resolve_pairs(s->P[c], s->ctl, s->d_boxes, s->C, s->PR, 2, s->T.img, true, true, st);
     } else if (s->cfg.collisions) {
@@ -531,7 +537,7 @@ int record_step(rb_sim* s, int p) {
         collision_search(s->T, s->P[c], s->ctl, s->d_boxes, s->C, s->PR, 2, st, s->search_block, s->rmax,
                          s->profiling == 2);
         mark(s, 10);
-        sort_pairs(s->PR, s->ctl, st, pair_key_bits(s));
+        sort_pairs(s->PR, s->ctl, s->C, st, pair_key_bits(s));
         mark(s, 11);
         resolve_pairs(s->P[c], s->ctl, s->d_boxes, s->C, s->PR, 2, s->T.img, true, true, st);
     } else {
@@ -584,30 +590,31 @@ int read_ctl(rb_sim* s) {
     return RB_OK;
 }
 
-int clear_err(rb_sim* s) {
-    RB_CUDA(s, cudaMemsetAsync(&s->ctl->err, 0, sizeof(int), s->stream));
-    return RB_OK;
+// A sort or scan of the last launches gave up a wait.
+int check_sorts(rb_sim* s) {
+    if (!(s->hctl.err & kErrSortStall)) return RB_OK;
+    s->acc_set = -1;   // no tree and no forces came of it
+    return fail(s, RB_ERR_TIMEOUT, "sort: a bounded wait for the earlier tiles gave up; set the particles again");
 }
 
 // Collision search + pair sort on set c at half-step offset hs; grows the
-// pair buffer and searches again if it overflowed.  Resolves when asked.
+// pair buffer and searches again if it overflowed.  Resolves when asked.  The
+// error word holds what the build before found.
 int collide_with_retry(rb_sim* s, int c, int hs, bool resolve) {
     for (int attempt = 0; attempt < 2; attempt++) {
         RB_CUDA(s, cudaMemsetAsync(&s->ctl->pair_count, 0, sizeof(int), s->stream));
         clear_search_stats(s->ctl, s->stream);
-        if (clear_err(s)) return RB_ERR_CUDA;
         if (s->cfg.collisions == RB_COLL_SWEEP)
             sweep_search(s->P[c], s->ctl, s->d_boxes, s->C, s->SW, s->PR, hs, s->ncap, s->stream);
         else
             collision_search(s->T, s->P[c], s->ctl, s->d_boxes, s->C, s->PR, hs, s->stream,
                              s->search_block, s->rmax, s->profiling == 2);
-        sort_pairs(s->PR, s->ctl, s->stream, pair_key_bits(s));
+        sort_pairs(s->PR, s->ctl, s->C, s->stream, pair_key_bits(s));
         if (read_ctl(s)) return RB_ERR_CUDA;
         if (s->hctl.err & kErrSweepLong)
             return fail(s, RB_ERR_CAPACITY, "plane sweep: a trajectory overlaps more than 65536 others in x "
                                             "(use the tree detector)");
-        if (s->hctl.err & kErrSortStall)
-            return fail(s, RB_ERR_TIMEOUT, "radix sort: a bounded look-back wait gave up");
+        if (int rc = check_sorts(s)) return rc;
         if (s->hctl.pair_count <= s->PR.cap) {
             if (resolve) {
                 resolve_pairs(s->P[c], s->ctl, s->d_boxes, s->C, s->PR, hs, s->T.img,
@@ -635,27 +642,27 @@ int ensure_ready(rb_sim* s) {
     return RB_OK;
 }
 
-// Keys of the current positions (no drift), sort, gather, topology.
-int rebuild_now(rb_sim* s) {
+// Keys of the current positions (no drift), sort, gather, topology; walk: for a
+// gravity walk, whose counters are cleared too.
+int rebuild_now(rb_sim* s, bool walk) {
     const int c = s->cur;
+    clear_build(s->ctl, walk, s->stream);
     drift_keys(s->P[c], s->T, s->ctl, s->d_boxes, s->C, s->ncap, 0, 0, nullptr, nullptr, nullptr,
                false, true, s->stream);
     sort_and_permute(s->P[c], s->P[1 - c], s->T, s->PR, s->ctl, s->C, s->ncap, s->box_bits, s->stream);
     s->cur = 1 - c;
     build_topology(s->T, s->P[s->cur], s->ctl, s->d_boxes, s->C, s->stream);
-    build_tile_order(s->T, s->P[s->cur], s->ctl, s->tile_order, s->box_bits, s->stream);
+    build_tile_order(s->T, s->P[s->cur], s->ctl, s->C, s->tile_order, s->box_bits, s->stream);
     return RB_OK;
 }
 
 int gravity_now(rb_sim* s, bool potential) {
     const bool learned = !potential && s->cfg.walk == RB_WALK_FP32_LEARNED;
     if (learned && !s->mlp_loaded) return fail(s, RB_ERR_STATE, "the learned walk needs rb_load_mlp first");
-    rebuild_now(s);
+    rebuild_now(s, true);
     const bool fp64 = potential || s->cfg.walk == RB_WALK_FP64;
     build_gravity_records(s->T, s->P[s->cur], s->ctl, s->d_boxes, s->C, fp64, s->stream, true);
-    clear_walk_stats(s->ctl, s->stream);
     if (learned) {
-        cudaMemsetAsync(&s->ctl->req_count, 0, sizeof(int), s->stream);
         const WalkLearn L = learn_args(s);
         gravity_walk(s->T, s->P[s->cur], s->ctl, s->d_boxes, s->C, RB_WALK_FP32, 0, walk_out(s), false,
                      true, s->stream, nullptr, s->walk_block, &L);
@@ -671,9 +678,7 @@ int gravity_now(rb_sim* s, bool potential) {
     check_runs(s);
     if (s->hctl.err & kErrWalk)
         return fail(s, RB_ERR_STATE, "gravity walk: an entry index outside the tree (malformed tree)");
-    if (s->hctl.err & kErrSortStall)
-        return fail(s, RB_ERR_TIMEOUT, "radix sort: a bounded look-back wait gave up");
-    return RB_OK;
+    return check_sorts(s);
 }
 
 template <typename T>
@@ -978,6 +983,7 @@ int rb_step(rb_sim* s, int64_t nsteps) {
         s->cur = s->gafter[p];
         s->acc_set = s->cfg.gravity ? s->cur : -1;   // the walk's particle set (no second sort)
         s->q32 = s->cfg.walk != RB_WALK_FP64;
+        if ((rc = check_sorts(s))) return rc;
         if (s->hctl.err & kErrNonFinite)
             return fail(s, RB_ERR_NONFINITE, "a position became non-finite (or left the box by more than "
                                              "4096 box lengths in one drift half)");
@@ -988,10 +994,9 @@ int rb_step(rb_sim* s, int64_t nsteps) {
                                             "(use the tree detector)");
         if (s->hctl.err & kErrResolveStall)
             return fail(s, RB_ERR_TIMEOUT, "collision resolution: a bounded wait for the ready queue gave up");
-        if (s->hctl.err & kErrSortStall)
-            return fail(s, RB_ERR_TIMEOUT, "radix sort: a bounded look-back wait gave up");
         if (s->cfg.collisions && s->hctl.pair_count > s->PR.cap) {
             // the step ended before resolution: search again with a larger buffer
+            clear_build(s->ctl, false, s->stream);
             if ((rc = collide_with_retry(s, s->cur, 0, true))) return rc;
         }
     }
@@ -1085,7 +1090,7 @@ int rb_detect_collisions(rb_sim* s) {
     int rc = ensure_ready(s);
     if (rc) return rc;
     if (s->ntot == 0) return RB_OK;
-    rebuild_now(s);
+    rebuild_now(s, false);
     if (s->cfg.collisions != RB_COLL_SWEEP)
         build_collision_aabb(s->T, s->P[s->cur], s->ctl, s->C, s->stream);
     return collide_with_retry(s, s->cur, 0, false);
@@ -1160,6 +1165,14 @@ int rb_set_pair_capacity(rb_sim* s, int64_t cap) {
 int rb_debug_hold_pair(rb_sim* s, int on) {
     if (!s) return fail(s, RB_ERR_ARG, "null simulation");
     s->hold_pair = on ? 1 : 0;
+    make_constants(s);
+    drop_graphs(s);
+    return RB_OK;
+}
+
+int rb_debug_hold_sort(rb_sim* s, int mask) {
+    if (!s || mask < 0 || mask > 31) return fail(s, RB_ERR_ARG, "null simulation, or mask outside 0..31");
+    s->hold_sort = mask;
     make_constants(s);
     drop_graphs(s);
     return RB_OK;
@@ -1297,15 +1310,22 @@ int rb_autotune(rb_sim* s, int use_cache) {
     // the sort that builds it; the smallest sum wins
     const int ocand[3] = {kTileMorton, kTileHilbertXY, kTileHilbertXYZ};
     float best_total = 1e30f;
+    const int order0 = s->tile_order;
+    auto stalled = [&]() {   // a failed run leaves the order as it was
+        int e = read_ctl(s);
+        if (!e) e = check_sorts(s);
+        if (e) s->tile_order = order0;
+        return e;
+    };
     for (int t : ocand) {
         s->tile_order = t;
         int wb_t = wb, sb_t = sb, wg_t = wg;
         float total = 0.f;
         if (s->cfg.gravity) {
-            rebuild_now(s);
+            rebuild_now(s, true);
             if (t != kTileMorton)
                 total += time_best(s, [&] {
-                    build_tile_order(s->T, s->P[s->cur], s->ctl, t, s->box_bits, s->stream);
+                    build_tile_order(s->T, s->P[s->cur], s->ctl, s->C, t, s->box_bits, s->stream);
                 });
             build_gravity_records(s->T, s->P[s->cur], s->ctl, s->d_boxes, s->C, fp64, s->stream, true);
             float best = 1e30f;
@@ -1321,9 +1341,10 @@ int rb_autotune(rb_sim* s, int use_cache) {
                 }
             total += best;
             s->acc_set = -1;   // the tuning walks left no consistent acceleration record
+            if ((rc = stalled())) return rc;
         }
         if (s->cfg.collisions == RB_COLL_TREE) {
-            rebuild_now(s);
+            rebuild_now(s, false);
             build_collision_aabb(s->T, s->P[s->cur], s->ctl, s->C, s->stream);
             float best = 1e30f;
             for (int b : cand) {
@@ -1336,6 +1357,7 @@ int rb_autotune(rb_sim* s, int use_cache) {
             }
             total += best;
             cudaMemsetAsync(&s->ctl->pair_n, 0, sizeof(int), s->stream);
+            if ((rc = stalled())) return rc;
         }
         if (total < best_total) {
             best_total = total;
@@ -1467,7 +1489,7 @@ int rb_mlp_samples(rb_sim* s, double theta_hi, double theta_lo, double prob, uin
     if (!s->cfg.gravity) return fail(s, RB_ERR_STATE, "gravity is off");
     *n_out = 0;
     if (s->ntot == 0) return RB_OK;
-    rebuild_now(s);
+    rebuild_now(s, true);
     SimC C2 = s->C;
     C2.theta = theta_hi;
     C2.theta2 = theta_hi * theta_hi;
@@ -1482,19 +1504,17 @@ int rb_mlp_samples(rb_sim* s, double theta_hi, double theta_lo, double prob, uin
         free_list(s, tmp);
         return RB_ERR_CUDA;
     }
-    cudaMemsetAsync(&s->ctl->req_count, 0, sizeof(int), s->stream);
     const uint32_t thresh = prob >= 1.0 ? 0xffffffffu : (uint32_t)(prob * 4294967296.0);
     const WalkRecord rec{req, &s->ctl->req_count, (int)cap,
                          (float)((theta_lo / theta_hi) * (theta_lo / theta_hi)), thresh,
                          (uint32_t)(seed ^ (seed >> 32))};
-    clear_walk_stats(s->ctl, s->stream);
     gravity_walk(s->T, s->P[s->cur], s->ctl, s->d_boxes, C2, RB_WALK_FP32, 0, walk_out(s), false, true,
                  s->stream, &rec);
     s->acc_set = s->cur;
     s->q32 = false;
     mlp::label_async(req_args(s, s->cur, 0, req, (int)cap), dX, dY, dmeta, (int)cap, s->stream);
-    rc = read_ctl(s);
-    const int64_t n = std::min<int64_t>(s->hctl.req_count, cap);
+    if (!(rc = read_ctl(s))) rc = check_sorts(s);
+    const int64_t n = rc ? 0 : std::min<int64_t>(s->hctl.req_count, cap);
     if (!rc && n > 0) {
         if (X) cudaMemcpyAsync(X, dX, sizeof(float) * 12 * n, cudaMemcpyDeviceToHost, s->stream);
         if (Y) cudaMemcpyAsync(Y, dY, sizeof(float) * 3 * n, cudaMemcpyDeviceToHost, s->stream);

@@ -429,7 +429,7 @@ __device__ __forceinline__ void collide(const CollArgs& A, SearchSmem& S, int wb
 template <bool kCount>
 __global__ void __launch_bounds__(kMaxWalkBlock, 4) k_collide(CollArgs A) {
     __shared__ SearchSmem sm[kMaxWalkBlock / 32];
-    const int n = min(A.ctl->n_live, A.ncap);
+    const int n = sorted_n(A.ctl, A.ncap);
     const int ntile = (n + A.width - 1) / A.width, q = sm_queue(A.nq);
     unsigned long long visits = 0, iters = 0;
     for (int t = next_tile(A.tq, A.nq, q, ntile); t >= 0; t = next_tile(A.tq, A.nq, q, ntile))

@@ -13,6 +13,7 @@
 //    keep ~1e-7 relative accuracy), 32-byte double4 records for the FP64
 //    walk, and the FP64 moments (M, centre of mass, traceless quadrupole).
 #pragma once
+#include <cstddef>
 #include <cstdint>
 #include <string>
 
@@ -46,6 +47,7 @@ struct SimC {
     int eps_law;         // 0: constant eps; 1: eps = min(1, (|v_n| / eps_vc)^(-eps_p))
     int learned;         // the walk runs the network, which reads the cells' corners at every theta
     int hold_pair;       // test hook: the queue's first pair never becomes ready
+    int hold_sort;       // test hook: sorts whose first tile never publishes (kHold*)
     int key_low;         // Morton key bits below those that the particle sort's passes take
     double eps_vc, eps_p;
     // SEI drift coefficients for tau = dt / 2 (x, vx, vy) -> (x, y, vx, vy), and z
@@ -63,19 +65,19 @@ struct PSet {
 // Device control block (scalars written by kernels).
 struct Ctl {
     long long step;            // steps since the last set_particles / set_time
-    int n_live;                // live particles after the last sort
     int n_live_next;           // live particles counted by the keys kernel
     int n_entries;             // tree entries (cells + leaves) of the last build
-    int pair_n;                // pairs to resolve (0 when the search overflowed)
     int resolved;              // pairs that were approaching and were resolved
-    int sweep_items;           // plane sweep: trajectory extents of the last search
     int out_live;              // host exchange: live particles of the box read out
-    int pad_;
+    int pad_[2];
+    // the counts and the error word that gates them, in one aligned load (sorted_n)
+    int pair_n;                // pairs to resolve (0 when the search overflowed)
+    int sweep_items;           // plane sweep: trajectory extents of the last search
+    int n_live;                // live particles after the last sort
     // cleared at the start of every step (clear_step)
-    int pair_count;            // pairs found by the last search (may exceed capacity)
     int err;                   // error bits (kErr*)
+    int pair_count;            // pairs found by the last search (may exceed capacity)
     int req_count;             // learned walk: cells corrected by the last walk
-    int pad2_;
     unsigned long long n_cell, n_leaf, n_mac, n_recheck;
     unsigned long long n_iter;        // warp iterations of the last FP32 walk (entries visited)
     unsigned long long n_visit;       // tree entries tested by the targets of the last collision search
@@ -84,6 +86,7 @@ struct Ctl {
     unsigned long long sweep_wbits;   // plane sweep: largest half extent (double bits)
     unsigned long long long_keys;     // last particle sort: keys in runs that blocks put in order
 };
+static_assert(offsetof(Ctl, pair_n) % 16 == 0 && offsetof(Ctl, err) == offsetof(Ctl, pair_n) + 12, "one int4");
 constexpr int kErrNonFinite = 1;
 constexpr int kErrPairOverflow = 2;
 constexpr int kErrSweepLong = 4;    // a plane-sweep item met more than kMaxSweepScan extents
@@ -91,6 +94,7 @@ constexpr int kErrResolveStall = 8; // the resolution queue stopped filling (bou
 constexpr int kErrWalk = 16;        // a walk met an entry index outside the tree (malformed tree)
 constexpr int kErrSortStall = 32;   // a radix pass's look-back stopped advancing (bounded wait gave up)
 constexpr int kMaxSweepScan = 1 << 16;
+constexpr int kHoldParticles = 1, kHoldScan = 2, kHoldTiles = 4, kHoldPairs = 8, kHoldSweep = 16;
 
 // One ghost image of one box at the time of a walk or search (Sect. 2.3):
 // the offset in FP64 and as hi/lo floats, and the image's y velocity offset.
@@ -190,6 +194,17 @@ __device__ __forceinline__ double source_mass(const BoxP& bp, int id, double m) 
     return id - bp.base_id < bp.n_active ? m : 0.0;
 }
 
+// Particles of the current tree, items of the sweep and pairs; none when a wait
+// of a sort or of the entry scan gave up: what it would have put in order is
+// incomplete, and nothing may be indexed by it.  One load: a second one behind
+// the error word's test cost every launch an L2 round trip (two steps of 20k
+// particles: 1,008 against 996 us a pass).
+__device__ __forceinline__ int4 sorted_counts(const Ctl* ctl) {   // pairs, items, particles
+    const int4 c = *reinterpret_cast<const int4*>(&ctl->pair_n);
+    return (c.w & kErrSortStall) ? make_int4(0, 0, 0, c.w) : c;
+}
+__device__ __forceinline__ int sorted_n(const Ctl* ctl, int ncap) { return min(sorted_counts(ctl).z, ncap); }
+
 // Time after 2 * step + hs drift halves: t0 + h * (dt / 2).
 __device__ __forceinline__ double time_of(const Ctl* ctl, double t0, double half_dt, int hs) {
     const double h = (double)(2 * ctl->step + hs);
@@ -236,9 +251,11 @@ __device__ __forceinline__ uint32_t morton_compact3(uint64_t x) {
 // pairs: the sort of the collision pairs also sets their number, pair_n, from
 // pair_count (0 when the search overflowed: it resolves nothing, and the host
 // grows the buffer and searches again on the unchanged state).
+// hold (test hook): the first tile of every pass never publishes its counts.
 int radix_sort(uint64_t* k0, uint32_t* v0, uint64_t* k1, uint32_t* v1, int ncap, const int* d_n,
                int key_bits, const int32_t* box_digits, int box_bits, uint32_t* hist, int* err,
-               cudaStream_t s, int low_bit = 0, Ctl* pairs = nullptr, unsigned long long* long_keys = nullptr);
+               cudaStream_t s, int low_bit = 0, Ctl* pairs = nullptr, unsigned long long* long_keys = nullptr,
+               bool hold = false);
 size_t radix_hist_words(int ncap);
 size_t radix_digit_words();   // the digit totals among them
 // rb_tree.cu
@@ -249,7 +266,7 @@ void build_topology(const Tree& T, const PSet& P, Ctl* ctl, const BoxP* boxes, c
 // kTileMorton leaves T.order null; kTileHilbertXY sorts the slots by a
 // 10-level 2D Hilbert key of (x, y) (thin sheets), kTileHilbertXYZ by a
 // 7-level 3D Hilbert key, the box id above either; ties keep Morton order.
-void build_tile_order(Tree& T, const PSet& P, Ctl* ctl, int mode, int box_bits, cudaStream_t s);
+void build_tile_order(Tree& T, const PSet& P, Ctl* ctl, const SimC& C, int mode, int box_bits, cudaStream_t s);
 // Moments and walk records.  fp64 (FP64 walk, potential): FP64 records and
 // the FP32 records of the opening test; otherwise all FP64 and FP32 records,
 // and with f32q the quadrupole is summed in FP32 and written to the FP32
@@ -340,7 +357,7 @@ void resolve_pairs(const PSet& P, Ctl* ctl, const BoxP* boxes, const SimC& C, Pa
 // stream capture).
 void resolve_prepare(int nsm);
 // key_bits: bits of the largest pair key, 36 + the bits of the largest id
-void sort_pairs(Pairs& PR, Ctl* ctl, cudaStream_t s, int key_bits = 60);
+void sort_pairs(Pairs& PR, Ctl* ctl, const SimC& C, cudaStream_t s, int key_bits = 60);
 void energy_terms(const PSet& P, Ctl* ctl, const SimC& C, const double* phi, int box,
                   double* partials, int nparts, double* out7, cudaStream_t s);
 void step_advance(Ctl* ctl, cudaStream_t s);
@@ -404,7 +421,8 @@ cudaError_t grad_f32_async(const float* w, const float* X, const float* Y, int n
 void label_async(const ReqArgs& A, float* X, float* Y, int64_t* meta, int max_req, cudaStream_t s);
 }  // namespace mlp
 void clear_step(Ctl* ctl, cudaStream_t s);
-void clear_walk_stats(Ctl* ctl, cudaStream_t s);
+// Before a build outside a step: the error word; for a walk all that a step clears.
+void clear_build(Ctl* ctl, bool walk, cudaStream_t s);
 void clear_search_stats(Ctl* ctl, cudaStream_t s);
 
 }  // namespace rb

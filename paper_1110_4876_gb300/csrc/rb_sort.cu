@@ -157,7 +157,7 @@ __global__ void __launch_bounds__(kThreads, 4) k_rs_pass(const uint64_t* __restr
                                                       const int* d_n, int ncap, int shift, int pass,
                                                       const uint32_t* __restrict__ hist,
                                                       uint32_t* __restrict__ status, int tiles_cap,
-                                                      int* __restrict__ err) {
+                                                      int* __restrict__ err, bool hold) {
     __shared__ uint32_t wcnt[kThreads / 32][kBins];
     __shared__ uint32_t gstart[kBins];   // where digit d of this tile starts in the output
     __shared__ uint32_t lstart[kBins];   // where digit d starts inside the tile
@@ -243,7 +243,7 @@ __global__ void __launch_bounds__(kThreads, 4) k_rs_pass(const uint64_t* __restr
             cnt += x;
         }
         volatile uint32_t* row = mine + (size_t)tile * kBins;
-        row[d] = (tile == 0 ? kFlagPre : kFlagAgg) | cnt;
+        if (!hold || tile > 0) row[d] = (tile == 0 ? kFlagPre : kFlagAgg) | cnt;
         {
             // where digit d starts inside the tile (block scan of the counts)
             uint32_t x = cnt;
@@ -340,12 +340,15 @@ __device__ __forceinline__ bool same_run(const uint64_t* key, const uint32_t* va
 
 // Insertion sort (stable) of every run of up to kShortRun keys by the thread
 // of its first key; the first keys of longer runs are listed.  Keys of all
-// ones (removed particles) are equal and stay as they are.
+// ones (removed particles) are equal and stay as they are, and so do all keys
+// after a pass whose look-back gave up: there the runs are not together, and
+// blocks at parts of one would write over each other's.
 __global__ void __launch_bounds__(256) k_rs_runs(uint64_t* __restrict__ key, uint32_t* __restrict__ val,
                                                  const int32_t* __restrict__ box, const int* d_n, int ncap,
                                                  int low_bit, uint32_t* __restrict__ hist,
-                                                 uint32_t* __restrict__ list) {
-    const int n = read_n(d_n, ncap);
+                                                 uint32_t* __restrict__ list, const int* __restrict__ err) {
+    const int gave_up = *err & kErrSortStall, keys = read_n(d_n, ncap);
+    const int n = gave_up ? 0 : keys;
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     // the digit totals are done with: zero for the next sort
     for (int k = i; k < kLongCount; k += gridDim.x * blockDim.x) hist[k] = 0u;
@@ -495,7 +498,7 @@ size_t radix_digit_words() { return (size_t)kMaxPasses * kBins; }
 
 int radix_sort(uint64_t* k0, uint32_t* v0, uint64_t* k1, uint32_t* v1, int ncap, const int* d_n,
                int key_bits, const int32_t* box_digits, int box_bits, uint32_t* hist, int* err,
-               cudaStream_t s, int low_bit, Ctl* pairs, unsigned long long* long_keys) {
+               cudaStream_t s, int low_bit, Ctl* pairs, unsigned long long* long_keys, bool hold) {
     if (ncap <= 0) return 0;
     const int tiles_cap = ceil_div(ncap, kTile);
     uint32_t* status = hist + kMaxPasses * kBins;
@@ -521,18 +524,19 @@ int radix_sort(uint64_t* k0, uint32_t* v0, uint64_t* k1, uint32_t* v1, int ncap,
         if (boxp)
             k_rs_pass<true><<<tiles_cap, kThreads, 0, s>>>(K[cur], V[cur], K[cur ^ 1], V[cur ^ 1],
                                                            box_digits, d_n, ncap, sh, p, hist,
-                                                           status, tiles_cap, err);
+                                                           status, tiles_cap, err, hold);
         else
             k_rs_pass<false><<<tiles_cap, kThreads, 0, s>>>(K[cur], V[cur], K[cur ^ 1], V[cur ^ 1],
                                                             nullptr, d_n, ncap, sh, p, hist, status,
-                                                            tiles_cap, err);
+                                                            tiles_cap, err, hold);
         cur ^= 1;
     }
     if (low_bit > 0) {
         // the list of long runs takes the status words, which the passes are
         // done with (at most one run per kShortRun + 1 keys)
         const uint32_t* nlong = hist + kLongCount;
-        k_rs_runs<<<ceil_div(ncap, 256), 256, 0, s>>>(K[cur], V[cur], box_digits, d_n, ncap, low_bit, hist, status);
+        k_rs_runs<<<ceil_div(ncap, 256), 256, 0, s>>>(K[cur], V[cur], box_digits, d_n, ncap, low_bit, hist, status,
+                                                        err);
         k_rs_long<<<std::min(ceil_div(ncap, kShortRun), 152), kThreads, 0, s>>>(
             K[cur], V[cur], K[cur ^ 1], V[cur ^ 1], box_digits, d_n, ncap, low_bit, nlong, status, long_keys);
     }

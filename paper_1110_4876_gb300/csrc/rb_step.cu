@@ -266,7 +266,7 @@ __device__ __forceinline__ int key_b(uint64_t k) { return (int)((k >> 12) & 0xFF
 // Every pair joins the list of its higher particle id; head is -1 for every
 // particle on entry.
 __global__ void __launch_bounds__(256) k_pair_link(ResolveArgs A) {
-    const int n = A.ctl->pair_n;
+    const int n = sorted_counts(A.ctl).x;
     if (blockIdx.x == 0 && threadIdx.x == 0) *A.claim = 0;
     for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < n; k += gridDim.x * blockDim.x) {
         A.link[k] = atomicExch(&A.head[key_b(A.key[k])], k);
@@ -371,7 +371,7 @@ __device__ __forceinline__ int ld_flag(const int32_t* p) {
 template <bool kPower>
 __global__ void __launch_bounds__(256) k_resolve(ResolveArgs A, SimC C) {
     if (A.advance && blockIdx.x == 0 && threadIdx.x == 0) A.ctl->step += 1;   // nothing here reads the time
-    const int n = A.ctl->pair_n;
+    const int n = sorted_counts(A.ctl).x;
     const int lane = threadIdx.x & 31;
     int nres = 0;
     for (;;) {
@@ -535,7 +535,7 @@ void sort_and_permute(const PSet& src, const PSet& dst, Tree& T, Pairs& PR, Ctl*
     // passes over the top bits, the rest within the short runs that agree there
     const int which = radix_sort(T.key, T.idx, T.key_alt, T.idx_alt, ncap, nullptr, 64,
                                  C.nbox > 1 ? T.sbox : nullptr, box_bits, T.hist, &ctl->err, s, C.key_low, nullptr,
-                                 &ctl->long_keys);
+                                 &ctl->long_keys, (C.hold_sort & kHoldParticles) != 0);
     // a sort by the top bits counts on zero digit totals, and leaves them
     if (C.key_low == 0) cudaMemsetAsync(T.hist, 0, sizeof(uint32_t) * radix_digit_words(), s);
     if (which == 1) {
@@ -648,12 +648,13 @@ void reset_slots(const PSet& P, int32_t* slot_of_id, int n, int ncap, int nbox, 
     if (ncap > 0) k_reset_slots<<<ceil_div(ncap, 256), 256, 0, s>>>(P, slot_of_id, n, ncap, nbox);
 }
 
-void sort_pairs(Pairs& PR, Ctl* ctl, cudaStream_t s, int key_bits) {
+void sort_pairs(Pairs& PR, Ctl* ctl, const SimC& C, cudaStream_t s, int key_bits) {
     // passes over the lower id's bits, then each id's pairs among themselves;
     // an odd number of passes leaves the keys in key_alt; the buffers are
     // not swapped, so every captured graph finds them in the same place
     PR.sorted_alt = radix_sort(PR.key, PR.val, PR.key_alt, PR.val_alt, PR.cap, &ctl->pair_n,
-                               key_bits, nullptr, 0, PR.hist, &ctl->err, s, 36, ctl) == 1;
+                               key_bits, nullptr, 0, PR.hist, &ctl->err, s, 36, ctl, nullptr,
+                               (C.hold_sort & kHoldPairs) != 0) == 1;
 }
 
 void resolve_pairs(const PSet& P, Ctl* ctl, const BoxP* boxes, const SimC& C, Pairs& PR,
@@ -682,14 +683,16 @@ void energy_terms(const PSet& P, Ctl* ctl, const SimC& C, const double* phi, int
 
 void step_advance(Ctl* ctl, cudaStream_t s) { k_step_advance<<<1, 1, 0, s>>>(ctl); }
 
-// What a step starts from zero: the pair count, the error word, and the
-// counters of the walk (n_cell .. n_iter) and of the search (n_visit, n_siter).
+// What a step starts from zero: the error word, the pair count, and the
+// counters of the walk (req_count, n_cell .. n_iter) and of the search (n_visit,
+// n_siter).
 void clear_step(Ctl* ctl, cudaStream_t s) {
-    cudaMemsetAsync(&ctl->pair_count, 0, offsetof(Ctl, sweep_wbits) - offsetof(Ctl, pair_count), s);
+    cudaMemsetAsync(&ctl->err, 0, offsetof(Ctl, sweep_wbits) - offsetof(Ctl, err), s);
 }
 
-void clear_walk_stats(Ctl* ctl, cudaStream_t s) {
-    cudaMemsetAsync(&ctl->n_cell, 0, 7 * sizeof(unsigned long long), s);
+void clear_build(Ctl* ctl, bool walk, cudaStream_t s) {
+    if (walk) clear_step(ctl, s);
+    else cudaMemsetAsync(&ctl->err, 0, sizeof(int), s);
 }
 
 void clear_search_stats(Ctl* ctl, cudaStream_t s) {

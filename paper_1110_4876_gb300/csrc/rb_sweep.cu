@@ -139,7 +139,7 @@ __device__ __forceinline__ void split_hl(double v, float& hi, float& lo) {
 __global__ void __launch_bounds__(256) k_sweep_gather(SweepArgs A, const uint32_t* __restrict__ val,
                                                       SweepRec* __restrict__ rec) {
     const int k = blockIdx.x * blockDim.x + threadIdx.x;
-    const int nitem = min(A.ctl->sweep_items, A.item_cap);
+    const int nitem = min(sorted_counts(A.ctl).y, A.item_cap);
     if (k >= nitem) return;
     const uint32_t v = val[k];
     const int i = (int)(v >> 3);
@@ -242,7 +242,7 @@ __global__ void __launch_bounds__(128) k_sweep_pairs(SweepArgs A, const SweepRec
     SweepQueue& Q = queue[threadIdx.x >> 5];
     const int k = blockIdx.x * blockDim.x + threadIdx.x, lane = threadIdx.x & 31;
     const unsigned lt = (1u << lane) - 1u;
-    const int nitem = min(A.ctl->sweep_items, A.item_cap);
+    const int nitem = min(sorted_counts(A.ctl).y, A.item_cap);
     if (k - lane >= nitem) return;   // the whole warp
     bool scan = k < nitem;
     const SweepRec P = rec[scan ? k : nitem - 1];
@@ -373,7 +373,7 @@ void sweep_search(const PSet& P, Ctl* ctl, const BoxP* boxes, const SimC& C, Swe
     k_sweep_items<<<ceil_div(ncap, 256), 256, 0, s>>>(A);
     const int key_bits = 32 + S.box_bits;
     const int which = radix_sort(S.key, S.val, S.key_alt, S.val_alt, S.cap, &ctl->sweep_items, key_bits,
-                                 nullptr, 0, S.hist, &ctl->err, s);
+                                 nullptr, 0, S.hist, &ctl->err, s, 0, nullptr, nullptr, (C.hold_sort & kHoldSweep) != 0);
     if (which == 1) {
         A.key = S.key_alt;
         A.val = S.val_alt;

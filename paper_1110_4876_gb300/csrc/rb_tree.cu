@@ -45,7 +45,7 @@ __global__ void __launch_bounds__(256) k_nodes(const uint64_t* __restrict__ key,
                                                int32_t* __restrict__ node_b,
                                                int8_t* __restrict__ node_v,
                                                uint32_t* __restrict__ mask) {
-    const int n = min(ctl->n_live, ncap);
+    const int n = sorted_n(ctl, ncap);
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i == 0) ctl->n_live_next = 0;   // committed by the gather
     if (i >= n - 1) return;
@@ -101,9 +101,9 @@ constexpr int kScanTile = 2048;
 constexpr uint32_t kScanAgg = 1u << 30, kScanPre = 2u << 30, kScanMask = (1u << 30) - 1u;
 
 __global__ void __launch_bounds__(256) k_entry_scan(const uint32_t* __restrict__ mask, Ctl* ctl, int ncap,
-                                                    int32_t* __restrict__ start, uint32_t* stat) {
+                                                    int32_t* __restrict__ start, uint32_t* stat, bool hold) {
     __shared__ uint32_t ws[8], before_s;
-    const int n = min(ctl->n_live, ncap);
+    const int n = sorted_n(ctl, ncap);
     const int b = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int base = b * kScanTile;
     if (base >= n) {
@@ -135,7 +135,7 @@ __global__ void __launch_bounds__(256) k_entry_scan(const uint32_t* __restrict__
         total += ws[w];
     }
     volatile uint32_t* st = stat;
-    if (tid == 0) st[b] = (b == 0 ? kScanPre : kScanAgg) | total;
+    if (tid == 0 && (!hold || b > 0)) st[b] = (b == 0 ? kScanPre : kScanAgg) | total;
     if (warp == 0) {
         uint32_t excl = 0;
         unsigned long long since = 0;
@@ -196,7 +196,7 @@ __global__ void __launch_bounds__(256) k_emit(const uint32_t* __restrict__ mask,
                                               uint32_t* __restrict__ e_cmask,
                                               const int32_t* __restrict__ box,
                                               int32_t* __restrict__ box_root) {
-    const int n = min(ctl->n_live, ncap);
+    const int n = sorted_n(ctl, ncap);
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
     // the root of a box starts at its first particle; the others stay -1
@@ -397,7 +397,7 @@ __device__ __forceinline__ int common_levels(uint64_t a, uint64_t b) {
 // record carries that cell's width and corner.  Without such a cell the group
 // is never accepted.
 __device__ __forceinline__ bool group_has_chain(const GravRecArgs& A, int first, int last) {
-    const int n = min(A.ctl->n_live, A.ncap);
+    const int n = sorted_n(A.ctl, A.ncap);
     const uint64_t kf = A.key[first];
     const int b = A.box[first];
     int d = -1;   // depth of the group's parent cell
@@ -611,7 +611,7 @@ template <bool kF32Q>
 __global__ void __launch_bounds__(256, 4) k_moments_range(GravRecArgs A, int slots, int32_t* __restrict__ span) {
     __shared__ int cnt[kBuckets], off[kBuckets], over[kDepths];
     __shared__ uint16_t list[2 * kMomSlots];   // the range's cells by bucket, as entry - e0
-    const int n = min(A.ctl->n_live, A.ncap);
+    const int n = sorted_n(A.ctl, A.ncap);
     const int p0 = blockIdx.x * slots, tid = threadIdx.x;
     if (p0 >= n) {
         if (tid < kDepths) span[blockIdx.x * kDepths + tid] = -1;
@@ -929,7 +929,7 @@ __device__ __forceinline__ void cell_put(const CollRecArgs& A, int k, const BoxA
 // every slot and of the runs of 32 and 256 slots (kRunB threads per block).
 __global__ void __launch_bounds__(kRunB) k_aabb_leaves(CollRecArgs A) {
     __shared__ BoxAcc wbox[kRunsInB];
-    const int n = min(A.ctl->n_live, A.ncap);
+    const int n = sorted_n(A.ctl, A.ncap);
     const int p = blockIdx.x * blockDim.x + threadIdx.x;
     BoxAcc B = box_empty();
     if (p < n) {
@@ -992,7 +992,7 @@ __device__ __forceinline__ Split split_runs(int lo, int hi, int ratio) {
 // Box items of the runs of 8192 slots, from their 32 runs of 256 (a warp per
 // run).
 __global__ void __launch_bounds__(256) k_aabb_runs(CollRecArgs A) {
-    const int n = min(A.ctl->n_live, A.ncap);
+    const int n = sorted_n(A.ctl, A.ncap);
     const long long nA = (A.ncap + kRunA - 1) / kRunA, nB = (A.ncap + kRunB - 1) / kRunB;
     const int lane = threadIdx.x & 31;
     const int w = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, nw = (gridDim.x * blockDim.x) >> 5;
@@ -1036,7 +1036,8 @@ __device__ __forceinline__ void range_fold(const CollRecArgs& A, int a, int e, i
 // A lane takes a cell of at most eight slots alone; larger cells are taken
 // afterwards by the whole warp, one at a time.
 __global__ void __launch_bounds__(256) k_aabb_cells(CollRecArgs A) {
-    const int E = min(A.ctl->n_entries, A.ecap);
+    const int entries = min(A.ctl->n_entries, A.ecap);
+    const int E = sorted_n(A.ctl, 1) ? entries : 0;
     const int lane = threadIdx.x & 31;
     const int w = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, nw = (gridDim.x * blockDim.x) >> 5;
     for (int e0 = 32 * w; e0 < E; e0 += 32 * nw) {
@@ -1082,7 +1083,8 @@ void build_topology(const Tree& T, const PSet& P, Ctl* ctl, const BoxP* boxes, c
     else
         k_nodes<false><<<nb, 256, 0, s>>>(T.key, P.box, ctl, n, T.node_a, T.node_b, T.node_v,
                                           T.mask);
-    k_entry_scan<<<ceil_div(n, kScanTile), 256, 0, s>>>(T.mask, ctl, n, T.start, T.scan_stat);
+    k_entry_scan<<<ceil_div(n, kScanTile), 256, 0, s>>>(T.mask, ctl, n, T.start, T.scan_stat,
+                                                        (C.hold_sort & kHoldScan) != 0);
     k_emit<<<nb, 256, 0, s>>>(T.mask, T.start, T.node_a, T.node_b, T.node_v, ctl, n, T.e_first,
                               T.e_count, T.e_skip, T.e_level, T.leaf_of, T.key, T.e_child, T.e_cmask, P.box,
                               T.box_root);
@@ -1149,7 +1151,7 @@ __global__ void __launch_bounds__(256) k_tile_keys(const uint64_t* __restrict__ 
                                                    const int32_t* __restrict__ box,
                                                    const Ctl* __restrict__ ctl, int ncap, int mode,
                                                    uint64_t* __restrict__ tkey, uint32_t* __restrict__ tval) {
-    const int n = min(ctl->n_live, ncap);
+    const int n = sorted_n(ctl, ncap);
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
     const uint64_t k = key[i];
@@ -1162,14 +1164,15 @@ __global__ void __launch_bounds__(256) k_tile_keys(const uint64_t* __restrict__ 
 
 }  // namespace
 
-void build_tile_order(Tree& T, const PSet& P, Ctl* ctl, int mode, int box_bits, cudaStream_t s) {
+void build_tile_order(Tree& T, const PSet& P, Ctl* ctl, const SimC& C, int mode, int box_bits, cudaStream_t s) {
     if (mode == kTileMorton || T.cap_n <= 0) {
         T.order = nullptr;
         return;
     }
     k_tile_keys<<<ceil_div(T.cap_n, 256), 256, 0, s>>>(T.key, P.box, ctl, T.cap_n, mode, T.tkey, T.tval);
     const int which = radix_sort(T.tkey, T.tval, T.tkey_alt, T.tval_alt, T.cap_n, &ctl->n_live,
-                                 21 + box_bits, nullptr, 0, T.thist, &ctl->err, s);
+                                 21 + box_bits, nullptr, 0, T.thist, &ctl->err, s, 0, nullptr, nullptr,
+                                 (C.hold_sort & kHoldTiles) != 0);
     T.order = which ? T.tval_alt : T.tval;
 }
 

@@ -509,7 +509,7 @@ template <bool kQuad, bool kInside, bool kSoft, bool kPot, bool k64, bool kLearn
 __device__ __forceinline__ void target_units(const GravArgs& A, int per, TSmem<k64>& S, LearnQ* LQ,
                                              const mlp::Packed* W) {
     const int lane = threadIdx.x & 31;
-    const int n = min(A.ctl->n_live, A.ncap);
+    const int n = sorted_n(A.ctl, A.ncap);
     const int nunit = (n + per - 1) / per, q = sm_queue(A.nq);
     TTotal N;
     for (int u = next_tile(A.tq, A.nq, q, nunit); u >= 0; u = next_tile(A.tq, A.nq, q, nunit)) {
@@ -811,7 +811,7 @@ __device__ __forceinline__ void walk_pair(const GravArgs& A, PSmem& S, int i0, i
 template <bool kQuad, bool kInside, bool kSoft>
 __device__ __forceinline__ void pair_units(const GravArgs& A, int per, PSmem& S) {
     const int lane = threadIdx.x & 31;
-    const int n = min(A.ctl->n_live, A.ncap);
+    const int n = sorted_n(A.ctl, A.ncap);
     const int nunit = (n + per - 1) / per, q = sm_queue(A.nq);
     TTotal N;
     for (int u = next_tile(A.tq, A.nq, q, nunit); u >= 0; u = next_tile(A.tq, A.nq, q, nunit)) {

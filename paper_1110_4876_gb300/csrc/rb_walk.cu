@@ -347,7 +347,7 @@ __device__ __forceinline__ void walk32(const GravArgs& A, LearnQ* LQ, const mlp:
 
 template <bool kQuad, bool kInside, bool kSoft, bool kRecord = false, bool kOne = false>
 __global__ void __launch_bounds__(kMaxWalkBlock, 4) k_walk32(GravArgs A) {
-    const int n = min(A.ctl->n_live, A.ncap);
+    const int n = sorted_n(A.ctl, A.ncap);
     const int ntile = (n + 31) >> 5, q = sm_queue(A.nq);
     for (int t = next_tile(A.tq, A.nq, q, ntile); t >= 0; t = next_tile(A.tq, A.nq, q, ntile))
         walk32<kQuad, kInside, kSoft, kRecord, false, kOne>(A, nullptr, nullptr, t << 5, n);
@@ -772,7 +772,7 @@ template <bool kQuad, bool kInside, bool kSoft, bool kOne, int kS>
 __global__ void __launch_bounds__(kMaxWalkBlock, 4) k_gwalk32(GravArgs A) {
     __shared__ GroupSmem gs[kMaxWalkBlock / 32];
     GroupSmem& G = gs[threadIdx.x >> 5];
-    const int n = min(A.ctl->n_live, A.ncap);
+    const int n = sorted_n(A.ctl, A.ncap);
     const int ntile = (n + 31) >> 5, q = sm_queue(A.nq);
     for (int t = next_tile(A.tq, A.nq, q, ntile); t >= 0; t = next_tile(A.tq, A.nq, q, ntile)) {
         if (!kOne) {
@@ -799,7 +799,7 @@ __global__ void __launch_bounds__(kMaxWalkBlock, 2) k_walk32_learn(GravArgs A) {
         for (int k = threadIdx.x; k < (int)(sizeof(mlp::Packed) / 16); k += blockDim.x) dst[k] = src[k];
     }
     __syncthreads();
-    const int n = min(A.ctl->n_live, A.ncap);
+    const int n = sorted_n(A.ctl, A.ncap);
     const int ntile = (n + 31) >> 5, sq = sm_queue(A.nq);
     for (int t = next_tile(A.tq, A.nq, sq, ntile); t >= 0; t = next_tile(A.tq, A.nq, sq, ntile))
         walk32<true, kInside, kSoft, false, true>(A, &q[threadIdx.x >> 5], &w, t << 5, n);

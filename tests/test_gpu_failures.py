@@ -105,3 +105,43 @@ def test_resolution_wait_is_bounded(rb):
     a, b = s.particles(), ref.particles()
     for k in ("x", "y", "z", "vx", "vy", "vz"):
         assert np.array_equal(a[k], b[k]), k
+
+
+# sort held back (rb_debug_hold_sort), options, and the calls that meet it
+@pytest.mark.parametrize("mask,nbox,cfg", [
+    (1, 1, {}), (1, 3, {}), (1, 1, dict(gravity=0)), (2, 1, {}), (4, 1, {}), (8, 1, {}), (8, 1, dict(gravity=0)),
+    (16, 1, dict(collisions=2))])
+def test_sort_waits_are_bounded_and_nothing_is_built_on_their_output(rb, mask, nbox, cfg):
+    """A sort whose first tile never publishes (test hook) makes the other
+    tiles' waits run out: each call reports RB_ERR_TIMEOUT, also the first one
+    on buffers that no sort has filled, and the context stays usable (fresh
+    particles step as in an untouched simulation)."""
+    L, N = 160.0, 6000   # three tiles of 2048 keys, and more than 2048 pairs
+
+    def fresh():
+        s = rb.Sim(nbox=nbox, **sheet(rb, L, **cfg))
+        rb.rb_set_launch_shape(s.h, 128, 128, 0, rb.RB_TILE_HILBERT_XY)
+        for b in range(nbox):
+            s.set_particles(I.sheet(L, N, 7 + b), b)
+        return s
+
+    s = fresh()
+    calls = [lambda: s.step(1), lambda: s.pairs()]
+    if mask in (1, 2, 4) and s.cfg.gravity:
+        calls += [lambda: s.gravity(), lambda: s.energy(), lambda: rb.rb_autotune(s.h, use_cache=False),
+                  lambda: rb.rb_mlp_samples(s.h, 0.8, 0.5, 0.01, 1, 1000)]
+    rb.rb_debug_hold_sort(s.h, mask)
+    for call in calls:
+        with pytest.raises(rb.RbError) as e:
+            call()
+        assert e.value.code == rb.RB_ERR_TIMEOUT
+    rb.rb_debug_hold_sort(s.h, 0)
+    ref = fresh()
+    for b in range(nbox):
+        s.set_particles(I.sheet(L, N, 7 + b), b)
+    s.step(2)
+    ref.step(2)
+    for b in range(nbox):
+        x, y = s.particles(b), ref.particles(b)
+        for k in ("x", "y", "z", "vx", "vy", "vz"):
+            assert np.array_equal(x[k], y[k]), k
