@@ -590,8 +590,10 @@ int read_ctl(rb_sim* s) {
     return RB_OK;
 }
 
-// A sort or scan of the last launches gave up a wait.
+// After a build, with the control block read: whether the next sorts leave bits
+// to the runs, and whether a sort or scan gave up a wait.
 int check_sorts(rb_sim* s) {
+    check_runs(s);
     if (!(s->hctl.err & kErrSortStall)) return RB_OK;
     s->acc_set = -1;   // no tree and no forces came of it
     return fail(s, RB_ERR_TIMEOUT, "sort: a bounded wait for the earlier tiles gave up; set the particles again");
@@ -675,10 +677,10 @@ int gravity_now(rb_sim* s, bool potential) {
     s->q32 = !fp64;
     RB_CUDA(s, cudaGetLastError());
     if (int rc = read_ctl(s)) return rc;
-    check_runs(s);
+    if (int rc = check_sorts(s)) return rc;
     if (s->hctl.err & kErrWalk)
         return fail(s, RB_ERR_STATE, "gravity walk: an entry index outside the tree (malformed tree)");
-    return check_sorts(s);
+    return RB_OK;
 }
 
 template <typename T>
@@ -976,7 +978,6 @@ int rb_step(rb_sim* s, int64_t nsteps) {
         RB_CUDA(s, cudaEventRecord(s->ev1, s->stream));
         if ((rc = read_ctl(s))) return rc;
         cudaEventElapsedTime(&s->last_ms, s->ev0, s->ev1);
-        check_runs(s);
         if (s->profiling)
             for (int q = 0; q < 12; q++)
                 cudaEventElapsedTime(&s->stage_ms[q], s->ev_stage[q], s->ev_stage[q + 1]);

@@ -88,3 +88,35 @@ def test_a_clump_of_one_long_run(rb, orc):
         sim.set_particles(P)
         # as for the clumps above, scale 2e-5
         assert np.max(np.linalg.norm(sim.gravity() - ref, axis=1) / den) <= 1e-12 + 1e-14 / 2e-5
+
+
+def _clump():
+    """5,000 particles within one cell of depth 13: a run that one block puts in
+    order, longer than the passes over its bits would take."""
+    P = I.random_cube(5000, 3)
+    for f in ("x", "y", "z"):
+        getattr(P, f)[:] = 0.3 + 2e-5 * getattr(P, f)
+    P.r[:] = 1e-9
+    return P
+
+
+def _sim(rb):
+    return rb.Sim(box=(1.0,) * 3, gravity=0, collisions=1, dt=1e-9)
+
+
+def _kernels(rb, sim):
+    sim.step(1)
+    return sim.stats()["kernels_per_step"]
+
+
+def test_detecting_pairs_finds_long_runs(rb):
+    """Every call that sorts notices the long run: after rb_detect_collisions the
+    first step already sorts all bits by passes, as a simulation that only steps
+    does from its second step on."""
+    stepped, detected = _sim(rb), _sim(rb)
+    for s in (stepped, detected):
+        s.set_particles(_clump())
+    runs, passes = _kernels(rb, stepped), _kernels(rb, stepped)
+    assert runs != passes
+    detected.pairs()
+    assert _kernels(rb, detected) == passes
