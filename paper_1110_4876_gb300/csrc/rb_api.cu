@@ -99,6 +99,7 @@ struct rb_sim {
     // launch shapes (threads per block) of the gravity walk and the search
     int key_low = 0;          // Morton bits left to the runs, by the boxes' shapes (upload)
     bool long_runs = false;   // the particles lie too close together for that: every bit is sorted by passes
+    int long_seen = 0;        // times that was found since key_low was chosen
     int walk_block = 128, search_block = 128;
     int walk_group = 0;   // FP32 walk: 0 union walk; 4 group walk (4-lane subgroups for mixed subtrees)
     int tile_order = kTileMorton;   // order in which walks and search take targets (kTile*)
@@ -264,6 +265,17 @@ int key_low_bits(const rb_sim* s) {
 void check_runs(rb_sim* s) {
     if (s->C.key_low == 0 || s->hctl.long_keys <= (unsigned long long)s->ntot / 8 + 4096) return;
     s->long_runs = true;
+    s->long_seen++;
+    make_constants(s);
+    drop_graphs(s);
+}
+
+// New particles may lie apart again.  A program that sets clumped ones time
+// after time would have its graphs captured twice for each set: after the
+// second clump every bit stays with the passes.
+void forget_runs(rb_sim* s) {
+    if (!s->long_runs || s->long_seen > 1) return;
+    s->long_runs = false;
     make_constants(s);
     drop_graphs(s);
 }
@@ -420,8 +432,10 @@ int upload(rb_sim* s) {
     if (low != s->key_low) {
         drop_graphs(s);
         s->long_runs = false;
+        s->long_seen = 0;
     }
     s->key_low = low;
+    forget_runs(s);
     make_constants(s);
     if (box_params(s) != RB_OK) return RB_ERR_CUDA;
     s->dirty = false;
@@ -932,6 +946,7 @@ int rb_set_particles(rb_sim* s, int box, int64_t n, const double* x, const doubl
         RB_CUDA(s, cudaGetLastError());
         if (rm != s->rmax) drop_graphs(s);   // R_max is a launch argument of the graphs
         s->rmax = rm;
+        forget_runs(s);
         s->cur = c;
         s->acc_set = -1;
         s->ntot = (int)n;

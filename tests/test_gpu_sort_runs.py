@@ -120,3 +120,24 @@ def test_detecting_pairs_finds_long_runs(rb):
     assert runs != passes
     detected.pairs()
     assert _kernels(rb, detected) == passes
+
+
+def test_new_particles_may_lie_apart_again(rb):
+    """A set of spread-out particles after a clump is sorted by runs again; after
+    a second clump the passes keep every bit."""
+    spread = I.random_cube(5000, 3)
+    spread.r[:] = 1e-9
+    sim = _sim(rb)
+    sim.set_particles(spread)
+    runs = _kernels(rb, sim)
+    sim.set_particles(_clump())
+    sim.step(1)
+    passes = _kernels(rb, sim)
+    assert runs != passes
+    sim.set_particles(spread)
+    assert _kernels(rb, sim) == runs
+    sim.set_particles(_clump())
+    sim.step(1)
+    assert _kernels(rb, sim) == passes
+    sim.set_particles(spread)
+    assert _kernels(rb, sim) == passes
