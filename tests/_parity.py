@@ -10,6 +10,22 @@ resolution must agree to 1e-12 of each particle's speed (floored at 1e-3 of
 the rms speed)."""
 import numpy as np
 
+from paper_1110_4876_gb300 import inputs as I
+
+LARGE = 130_001   # particle capacity above which every FP32 walk runs over 32 targets per warp
+
+
+def give_capacity(sim, n, L):
+    """The launch rules go by the particle capacity, the most particles a
+    simulation has held; fewer set afterwards keep it."""
+    if n:
+        P = I.random_cube(n, 1)
+        for f in ("x", "y", "z"):
+            getattr(P, f)[:] *= L
+        sim.set_particles(P)
+        sim.particles()   # uploads them
+
+
 FIELDS = ("x", "y", "z", "vx", "vy", "vz")
 
 

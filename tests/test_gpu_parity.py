@@ -13,7 +13,7 @@ import math
 import numpy as np
 import pytest
 
-from _parity import arrays, state_arrays, stepwise, vel_rel_err
+from _parity import LARGE, arrays, give_capacity, state_arrays, stepwise, vel_rel_err
 from paper_1110_4876_gb300 import inputs as I
 
 pytestmark = pytest.mark.gpu
@@ -87,14 +87,17 @@ def test_fp64_walk_matches_oracle_tree(rb, orc, theta):
 
 @pytest.mark.parametrize("group,order", [(0, 0), (4, 0), (0, 1), (4, 2)])
 @pytest.mark.parametrize("theta,quad", [(0.5, 1), (0.5, 0), (0.3, 1)])
-def test_fp32_walk_matches_oracle_tree(rb, orc, theta, quad, group, order):
-    """Both warp shapes of the FP32 walk (the union walk and the group walk:
-    group decisions, staged interaction list, 4-lane mixed subtrees) and the
-    tile orders of the targets (Morton, 2D and 3D Hilbert)."""
+@pytest.mark.parametrize("capacity", [None, LARGE])
+def test_fp32_walk_matches_oracle_tree(rb, orc, theta, quad, group, order, capacity):
+    """Every warp shape of the FP32 walk (group 0: two targets per warp, or the
+    union walk at a large capacity; the group walk: group decisions, staged
+    interaction list, 4-lane mixed subtrees) and the tile orders of the targets
+    (Morton, 2D and 3D Hilbert)."""
     L, N = 160.0, 6000
     P = I.sheet(L, N, 7)
     sim = rb.Sim(**sheet_cfg(rb, L, rb.RB_WALK_FP32, theta=theta, quadrupole=quad))
     rb.rb_set_launch_shape(sim.h, 128, 128, group, order)
+    give_capacity(sim, capacity, L)
     sim.set_particles(P)
     a, (nc, nl, nm) = sim.gravity(counts=True)
     p = sheet_params(orc, L, theta, quadrupole=quad)
@@ -110,8 +113,10 @@ def test_fp32_walk_matches_oracle_tree(rb, orc, theta, quad, group, order):
     assert sim.stats()["fp64_rechecks"] > 0
 
 
-@pytest.mark.parametrize("walk,group,order", [(0, 0, 0), (1, 0, 0), (1, 4, 0), (1, 0, 2), (0, 0, 2)])
-def test_plummer_open_inside_rule(rb, orc, walk, group, order):
+@pytest.mark.parametrize("walk,group,order,capacity", [
+    (0, 0, 0, None), (1, 0, 0, None), (1, 4, 0, None), (1, 0, 2, None), (0, 0, 2, None), (1, 0, 0, LARGE),
+    (1, 0, 2, LARGE)])
+def test_plummer_open_inside_rule(rb, orc, walk, group, order, capacity):
     """theta = 0.7 > 1/sqrt(3): the target-inside-cell rule is active (the
     group walk must also keep its group decisions clear of the cell cube)."""
     N = 5000
@@ -120,6 +125,7 @@ def test_plummer_open_inside_rule(rb, orc, walk, group, order):
                theta=0.7, softening=1e-3, dt=1e-3, gravity=1, collisions=0, walk=walk)
     sim = rb.Sim(**cfg)
     rb.rb_set_launch_shape(sim.h, 128, 128, group, order)
+    give_capacity(sim, capacity, 128.0)
     sim.set_particles(P)
     a, (nc, nl, nm) = sim.gravity(counts=True)
     p = orc.Params(G=1.0, L=(128.0,) * 3, theta=0.7, soft=1e-3, dt=1e-3, gravity=1)
@@ -287,8 +293,8 @@ def test_step_pairs_on_the_gravity_tree(rb, orc, walk):
         assert np.array_equal(keys, ref), k
 
 
-@pytest.mark.parametrize("walk", [0, 1])
-def test_coincident_particles_leaf_groups(rb, orc, walk):
+@pytest.mark.parametrize("walk,capacity", [(0, None), (1, None), (1, LARGE)])
+def test_coincident_particles_leaf_groups(rb, orc, walk, capacity):
     """Particles that share a Morton key (exactly coincident, or one ulp
     apart) end in depth-21 leaf groups whose members are interacted one by
     one, softened, as in the oracle's insertion tree (Sect. 4.2): the cells,
@@ -305,6 +311,7 @@ def test_coincident_particles_leaf_groups(rb, orc, walk):
     zero = np.zeros(n)
     sim = rb.Sim(G=1.0, box=(L, L, L), boundary=rb.RB_BC_OPEN, integrator=rb.RB_INT_LEAPFROG, theta=0.5,
                  softening=0.01, dt=1e-3, gravity=1, collisions=0, walk=walk)
+    give_capacity(sim, capacity, L)
     sim.set_particles((x, y, z, zero, zero, zero, m, zero))
     a, (nc, nl, nm) = sim.gravity(counts=True)
     p = orc.Params(G=1.0, L=(L,) * 3, theta=0.5, soft=0.01, quadrupole=1)
@@ -345,9 +352,9 @@ def test_ensemble_with_empty_and_tiny_boxes(rb, orc, walk):
         assert np.max(np.abs(arrays(ge) - arrays(go))) <= tol * L
 
 
-@pytest.mark.parametrize("walk", [0, 1])
+@pytest.mark.parametrize("walk,capacity", [(0, None), (1, None), (1, LARGE)])
 @pytest.mark.parametrize("theta,quad", [(0.9, 1), (1.2, 1), (0.9, 0), (0.5, 0)])
-def test_wide_opening_angles_and_monopole(rb, orc, walk, theta, quad):
+def test_wide_opening_angles_and_monopole(rb, orc, walk, capacity, theta, quad):
     """Wide opening angles (most cells accepted, the inside rule deciding
     many of them) and the monopole-only walk, on a Plummer sphere and on a
     sheet with its ghost images: forces and per-target counts equal the
@@ -356,6 +363,7 @@ def test_wide_opening_angles_and_monopole(rb, orc, walk, theta, quad):
     P = I.plummer(N, 5)
     sim = rb.Sim(G=1.0, box=(128.0,) * 3, boundary=rb.RB_BC_OPEN, integrator=rb.RB_INT_LEAPFROG,
                  theta=theta, quadrupole=quad, softening=1e-3, dt=1e-3, gravity=1, collisions=0, walk=walk)
+    give_capacity(sim, capacity, 128.0)
     sim.set_particles(P)
     a, (nc, nl, nm) = sim.gravity(counts=True)
     p = orc.Params(G=1.0, L=(128.0,) * 3, theta=theta, quadrupole=quad, soft=1e-3, dt=1e-3, gravity=1)
@@ -367,6 +375,7 @@ def test_wide_opening_angles_and_monopole(rb, orc, walk, theta, quad):
     L = 100.0
     S = I.sheet(L, 2400, 9)
     sim = rb.Sim(**sheet_cfg(rb, L, walk, theta=theta, quadrupole=quad))
+    give_capacity(sim, capacity, L)
     sim.set_particles(S)
     a, (nc, nl, nm) = sim.gravity(counts=True)
     a_ref, (rc, rl, rm) = orc.tree_gravity(sheet_params(orc, L, theta, quadrupole=quad), 0.0, S.x, S.y,
@@ -412,9 +421,9 @@ def test_sei_with_a_distinct_vertical_frequency(rb, orc):
     assert stepwise(rb, orc, sim, p, 5) > 50
 
 
-@pytest.mark.parametrize("walk", [0, 1])
+@pytest.mark.parametrize("walk,capacity", [(0, None), (1, None), (1, LARGE)])
 @pytest.mark.parametrize("nghost,zper", [((2, 2, 0), 0), ((1, 1, 1), 1)])
-def test_more_ghost_images(rb, orc, walk, nghost, zper):
+def test_more_ghost_images(rb, orc, walk, capacity, nghost, zper):
     """Two rings of ghost boxes in x and y (25 images), and one ring with a
     periodic z (27 images), Sect. 2.3: forces and per-target counts equal the
     oracle's tree over the same images."""
@@ -423,6 +432,7 @@ def test_more_ghost_images(rb, orc, walk, nghost, zper):
     cfg = sheet_cfg(rb, L, walk, nghost=nghost, z_periodic=zper)
     p = sheet_params(orc, L, nghost=nghost, z_periodic=zper)
     sim = rb.Sim(**cfg)
+    give_capacity(sim, capacity, L)
     sim.set_particles(P)
     a, (nc, nl, nm) = sim.gravity(counts=True)
     a_ref, (rc, rl, rm) = orc.tree_gravity(p, 0.0, P.x, P.y, P.z, P.m, counts=True)

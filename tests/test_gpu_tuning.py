@@ -9,6 +9,7 @@ within 1e-5 of the FP64 tree (the parity tests), so two shapes are within
 import numpy as np
 import pytest
 
+from _parity import LARGE, give_capacity
 from paper_1110_4876_gb300 import inputs as I
 
 pytestmark = pytest.mark.gpu
@@ -51,9 +52,13 @@ def test_autotune_keeps_results():
 
 
 @pytest.mark.parametrize("theta", [0.5, 0.7])
-def test_every_launch_shape_gives_the_same_forces_and_pairs(theta):
+@pytest.mark.parametrize("capacity", [LARGE, None])
+def test_every_launch_shape_gives_the_same_forces_and_pairs(theta, capacity):
     """Every block size of the walk and of the search, every warp shape of
-    the FP32 walk (theta = 0.7 also exercises the inside rule)."""
+    the FP32 walk (theta = 0.7 also exercises the inside rule): the union and
+    the group walk at a large capacity; at that of the 6,000 particles the walk
+    with two targets per warp, which takes one block size whatever is set, and
+    the group walk."""
     from paper_1110_4876_gb300 import build, rb
 
     build.build()
@@ -62,6 +67,7 @@ def test_every_launch_shape_gives_the_same_forces_and_pairs(theta):
     cfg = dict(G=I.G_SI, omega=I.OMEGA, box=(L, L, L), nghost=(1, 1, 0), boundary=rb.RB_BC_SHEAR,
                integrator=rb.RB_INT_SEI, theta=theta, eps=0.5, dt=I.DT_SHEET, gravity=1, collisions=1)
     sim = rb.Sim(**cfg)
+    give_capacity(sim, capacity, L)
     sim.set_particles(P)
     rb.rb_set_profiling(sim.h, 2)   # the counting search
     ref_a, ref_c, ref_p, ref_v = None, None, None, None
