@@ -221,8 +221,7 @@ int rb_get_pairs(rb_sim* sim, int box, int64_t cap, int64_t* n, int64_t* id_a, i
  * depend on cap. */
 int rb_set_pair_capacity(rb_sim* sim, int64_t cap);
 /* Test hook: with `on` nonzero the first pair of every sorted collision queue
- * waits for one predecessor too many, so it never becomes ready; the
- * resolution's threads wait for its queue slot at most half a second and the
+ * waits for itself; it and the pairs behind it wait at most half a second and the
  * step returns RB_ERR_TIMEOUT with the device context intact (velocities then
  * hold a partial resolution).  0 restores normal resolution. */
 int rb_debug_hold_pair(rb_sim* sim, int on);

@@ -240,7 +240,6 @@ int alloc_pairs(rb_sim* s, int cap) {
     return RB_OK;
 }
 
-// Allocate for capacity n and upload the staged boxes.
 // Morton key bits that the particle sort's passes leave to the runs (24: five
 // passes to depth 13, 16: six to depth 15, 0: all eight): as many as leave the
 // particles four cells each, in the plane of a thin sheet, at that depth.  In a
@@ -280,6 +279,7 @@ void forget_runs(rb_sim* s) {
     drop_graphs(s);
 }
 
+// Allocate for the staged boxes' particles and upload them.
 int upload(rb_sim* s) {
     int64_t tot = 0;
     s->base.assign(s->nbox, 0);
@@ -638,7 +638,7 @@ int collide_with_retry(rb_sim* s, int c, int hs, bool resolve) {
                 if (read_ctl(s)) return RB_ERR_CUDA;
                 if (s->hctl.err & kErrResolveStall)
                     return fail(s, RB_ERR_TIMEOUT,
-                                "collision resolution: a bounded wait for the ready queue gave up");
+                                "collision resolution: a bounded wait for an earlier pair gave up");
             }
             return RB_OK;
         }
@@ -1009,7 +1009,7 @@ int rb_step(rb_sim* s, int64_t nsteps) {
             return fail(s, RB_ERR_CAPACITY, "plane sweep: a trajectory overlaps more than 65536 others in x "
                                             "(use the tree detector)");
         if (s->hctl.err & kErrResolveStall)
-            return fail(s, RB_ERR_TIMEOUT, "collision resolution: a bounded wait for the ready queue gave up");
+            return fail(s, RB_ERR_TIMEOUT, "collision resolution: a bounded wait for an earlier pair gave up");
         if (s->cfg.collisions && s->hctl.pair_count > s->PR.cap) {
             // the step ended before resolution: search again with a larger buffer
             clear_build(s->ctl, false, s->stream);

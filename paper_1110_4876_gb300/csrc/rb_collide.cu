@@ -11,7 +11,7 @@
 // of Eq. 3's that still holds every overlap.
 // Against a walk of each target's own (lane per target, the warp stepping
 // through the union of 32 walks, about 260 dependent entries), a tile of the
-// 1M sheet tests 380 entries and 73 candidates: 0.59 -> 0.28 ms (100k: 163 -> 60
+// 1M sheet tests 370 entries and 73 candidates: 0.59 -> 0.28 ms (100k: 163 -> 60
 // us, 2400: 125 -> 22 us).  Bound by instruction issue with many particles, by a
 // tile's chain of rounds with few.
 //
@@ -22,7 +22,7 @@
 // was built (a wrap across a periodic face, a close encounter): a box around
 // such a run would hold much of the tree, so it is cut at its widest gaps into
 // compact parts.  Up to four of them are searched together, their items on one
-// frontier and tagged with their part: in turn, a tile's 380 entries took 24
+// frontier and tagged with their part: in turn, a tile's 370 entries took 24
 // rounds, half of whose lanes were idle (1M: 324 -> 283 us, 100k: 70 -> 60, 20k:
 // 43 -> 37, 2400: 27 -> 22).
 #include <algorithm>

@@ -46,7 +46,7 @@ struct SimC {
     int has_test;        // some particles are test particles (source mass 0)
     int eps_law;         // 0: constant eps; 1: eps = min(1, (|v_n| / eps_vc)^(-eps_p))
     int learned;         // the walk runs the network, which reads the cells' corners at every theta
-    int hold_pair;       // test hook: the queue's first pair never becomes ready
+    int hold_pair;       // test hook: the first pair waits for itself
     int hold_sort;       // test hook: sorts whose first tile never publishes (kHold*)
     int key_low;         // Morton key bits below those that the particle sort's passes take
     double eps_vc, eps_p;
@@ -90,9 +90,9 @@ static_assert(offsetof(Ctl, pair_n) % 16 == 0 && offsetof(Ctl, err) == offsetof(
 constexpr int kErrNonFinite = 1;
 constexpr int kErrPairOverflow = 2;
 constexpr int kErrSweepLong = 4;    // a plane-sweep item met more than kMaxSweepScan extents
-constexpr int kErrResolveStall = 8; // the resolution queue stopped filling (bounded wait gave up)
+constexpr int kErrResolveStall = 8; // a pair's bounded wait for an earlier one gave up
 constexpr int kErrWalk = 16;        // a walk met an entry index outside the tree (malformed tree)
-constexpr int kErrSortStall = 32;   // a radix pass's look-back stopped advancing (bounded wait gave up)
+constexpr int kErrSortStall = 32;   // a bounded look-back of a radix pass or of the entry scan gave up
 constexpr int kMaxSweepScan = 1 << 16;
 constexpr int kHoldParticles = 1, kHoldScan = 2, kHoldTiles = 4, kHoldPairs = 8, kHoldSweep = 16;
 
@@ -353,7 +353,7 @@ void sort_and_permute(const PSet& src, const PSet& dst, Tree& T, Pairs& PR, Ctl*
                       const SimC& C, int ncap, int box_bits, cudaStream_t s);
 void resolve_pairs(const PSet& P, Ctl* ctl, const BoxP* boxes, const SimC& C, Pairs& PR,
                    int half_step_offset, ImgTab* img, bool have_img, bool advance, cudaStream_t s);
-// Queries the resident blocks of the resolution queue once (outside any
+// Queries the resident blocks of the resolution once (outside any
 // stream capture).
 void resolve_prepare(int nsm);
 // key_bits: bits of the largest pair key, 36 + the bits of the largest id

@@ -8,8 +8,8 @@
 // a stack of (ghost image, entry) items, which starts with the root of every
 // image.  Each round the lanes pop up to 32 items, test each with the target's
 // own opening test, evaluate the accepted cells and leaves, and push the
-// children of the opened cells: about 25 rounds of independent loads instead
-// of the chain.  Each target tests exactly the entries its own walk visits, so
+// children of the opened cells: 16 rounds of independent loads (2400
+// particles) instead of the chain.  Each target tests exactly the entries its own walk visits, so
 // accepted sets and counts are those of the other walks.
 //
 // FP64: the opening test is decided in FP32 on the hi/lo records wherever that
@@ -30,8 +30,8 @@
 // in its two upper bits; its records are read once for both, whose terms are one
 // packed FP32 operation each, and its children are pushed for the targets that
 // opened it, so each target still tests exactly the entries of its own walk.
-// Neighbours' walks have most entries in common (the rounds of a pair are 1.06
-// times those of one).  One target per warp is bound by instruction issue (64%
+// Neighbours' walks have most entries in common (the rounds of a pair, 22 at
+// 20,000 and 24 at 60,000 targets, are 1.06 times those of one).  One target per warp is bound by instruction issue (64%
 // of the slots) and the L1 wavefronts of its gathers (70%); pairs by the latency
 // of the gathers with 24 warps per SM.  30,011 targets of the sheet: 215 -> 160
 // us, 50,000: 345 -> 250, 5,000: 69 -> 49.  Loading the children before the

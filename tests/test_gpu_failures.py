@@ -1,7 +1,7 @@
 """Error handling through the C ABI without any GPU fault: the pair buffer
 overflow is repaired inside the step, bad inputs and states return their
 codes, a position that overflows to infinity is reported, and the bounded
-wait of the resolution queue gives up with RB_ERR_TIMEOUT."""
+waits of the resolution and of the sorts give up with RB_ERR_TIMEOUT."""
 import numpy as np
 import pytest
 
@@ -80,10 +80,10 @@ def test_overflowing_position_is_reported(rb):
 
 
 def test_resolution_wait_is_bounded(rb):
-    """A pair held back from the resolution's ready queue (test hook) makes
-    the threads' bounded wait for its slot run out: the step reports
-    RB_ERR_TIMEOUT after about half a second, and the context stays usable
-    (a fresh upload steps normally, equal to an untouched simulation)."""
+    """A pair that waits for itself (test hook) makes its bounded wait, and those
+    of the pairs behind it, run out: the step reports RB_ERR_TIMEOUT after about
+    half a second, and the context stays usable (a fresh upload steps normally,
+    equal to an untouched simulation)."""
     import time
 
     L, N = 100.0, 2400
