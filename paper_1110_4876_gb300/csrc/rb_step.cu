@@ -396,7 +396,7 @@ __global__ void __launch_bounds__(256) k_resolve(ResolveArgs A, SimC C) {
                     const double vxb = __ldcg(xb), vyb = __ldcg(yb), vzb = __ldcg(zb);
                     const double ux = vxb - vxa, uy = (vyb + R.dvy) - vya, uz = vzb - vza;
                     const double rv = fma(R.rz, uz, fma(R.ry, uy, R.rx * ux));
-                    if (rv < 0.0) {
+                    if (!(rv >= 0.0)) {   // approaching, or not a number: it spreads to both
                         double g = rv;
                         if (kPower) {
                             // velocity-dependent restitution: min(1, (|v_n| / v_c)^(-p)),

@@ -40,3 +40,22 @@ def test_one_body_with_many_contacts(rb, orc, n, at):
     # n of them against the oracle's form of Eq. 2 stay below 2e-12
     found = stepwise(rb, orc, sim, p, 2, vtol=2e-12)
     assert found >= n // 2
+
+
+def test_a_speed_that_is_not_a_number_spreads(rb, orc):
+    """Two massless bodies in contact leave Eq. 2 with 0/0; the next pair of
+    either carries it on to its other body, as in the oracle, and a pair apart
+    from them stays as it is."""
+    x = np.array([0.0, 1.0, 2.0, 3.0, 10.0, 11.0])
+    zero = np.zeros(6)
+    vx = np.array([1.0, 0.0, -1.0, -2.0, 1.0, -1.0])
+    m, r = np.array([0.0, 0.0, 1.0, 1.0, 1.0, 1.0]), np.full(6, 0.6)
+    cfg = dict(eps=0.5, dt=1e-4, gravity=0, collisions=1)
+    sim = rb.Sim(box=(64.0,) * 3, boundary=rb.RB_BC_OPEN, **cfg)
+    sim.set_particles((x, zero, zero, vx, zero, zero, m, r))
+    sim.step(1)
+    st = orc.State(orc.Params(L=(64.0,) * 3, boundary=0, integrator=0, **cfg), x, zero, zero, vx, zero, zero, m, r)
+    st.step(1)
+    got = sim.particles()["vx"]
+    assert np.isnan(st.vx[:4]).all() and not np.isnan(st.vx[4:]).any()
+    np.testing.assert_allclose(got, st.vx, rtol=1e-15)
