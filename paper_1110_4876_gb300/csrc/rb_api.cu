@@ -679,6 +679,7 @@ int gravity_now(rb_sim* s, bool potential) {
     const bool fp64 = potential || s->cfg.walk == RB_WALK_FP64;
     build_gravity_records(s->T, s->P[s->cur], s->ctl, s->d_boxes, s->C, fp64, s->stream, true);
     if (learned) {
+        cudaMemsetAsync(&s->ctl->req_count, 0, sizeof(int), s->stream);
         const WalkLearn L = learn_args(s);
         gravity_walk(s->T, s->P[s->cur], s->ctl, s->d_boxes, s->C, RB_WALK_FP32, 0, walk_out(s), false,
                      true, s->stream, nullptr, s->walk_block, &L);
@@ -1338,7 +1339,7 @@ int rb_autotune(rb_sim* s, int use_cache) {
         int wb_t = wb, sb_t = sb, wg_t = wg;
         float total = 0.f;
         if (s->cfg.gravity) {
-            rebuild_now(s, true);
+            rebuild_now(s, false);
             if (t != kTileMorton)
                 total += time_best(s, [&] {
                     build_tile_order(s->T, s->P[s->cur], s->ctl, s->C, t, s->box_bits, s->stream);
@@ -1520,6 +1521,7 @@ int rb_mlp_samples(rb_sim* s, double theta_hi, double theta_lo, double prob, uin
         free_list(s, tmp);
         return RB_ERR_CUDA;
     }
+    cudaMemsetAsync(&s->ctl->req_count, 0, sizeof(int), s->stream);
     const uint32_t thresh = prob >= 1.0 ? 0xffffffffu : (uint32_t)(prob * 4294967296.0);
     const WalkRecord rec{req, &s->ctl->req_count, (int)cap,
                          (float)((theta_lo / theta_hi) * (theta_lo / theta_hi)), thresh,

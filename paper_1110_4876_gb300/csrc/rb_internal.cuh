@@ -74,14 +74,15 @@ struct Ctl {
     int pair_n;                // pairs to resolve (0 when the search overflowed)
     int sweep_items;           // plane sweep: trajectory extents of the last search
     int n_live;                // live particles after the last sort
-    // cleared at the start of every step (clear_step)
+    // cleared at the start of every step (clear_step), down to n_siter before
+    // every other walk (clear_build)
     int err;                   // error bits (kErr*)
-    int pair_count;            // pairs found by the last search (may exceed capacity)
-    int req_count;             // learned walk: cells corrected by the last walk
     unsigned long long n_cell, n_leaf, n_mac, n_recheck;
     unsigned long long n_iter;        // warp iterations of the last FP32 walk (entries visited)
     unsigned long long n_visit;       // tree entries tested by the targets of the last collision search
     unsigned long long n_siter;       // warp iterations of the last collision search
+    int pair_count;            // pairs found by the last search (may exceed capacity)
+    int req_count;             // learned walk: cells corrected by the last walk
     // (end of what clear_step clears)
     unsigned long long sweep_wbits;   // plane sweep: largest half extent (double bits)
     unsigned long long long_keys;     // last particle sort: keys in runs that blocks put in order
@@ -421,7 +422,7 @@ cudaError_t grad_f32_async(const float* w, const float* X, const float* Y, int n
 void label_async(const ReqArgs& A, float* X, float* Y, int64_t* meta, int max_req, cudaStream_t s);
 }  // namespace mlp
 void clear_step(Ctl* ctl, cudaStream_t s);
-// Before a build outside a step: the error word; for a walk all that a step clears.
+// Before a build outside a step: the error word, for a walk its counters too.
 void clear_build(Ctl* ctl, bool walk, cudaStream_t s);
 void clear_search_stats(Ctl* ctl, cudaStream_t s);
 

@@ -681,16 +681,14 @@ void energy_terms(const PSet& P, Ctl* ctl, const SimC& C, const double* phi, int
 
 void step_advance(Ctl* ctl, cudaStream_t s) { k_step_advance<<<1, 1, 0, s>>>(ctl); }
 
-// What a step starts from zero: the error word, the pair count, and the
-// counters of the walk (req_count, n_cell .. n_iter) and of the search (n_visit,
-// n_siter).
+// What a step starts from zero: the error word, the counters of the walk and of
+// the search, and the counts of pairs and of corrected cells.
 void clear_step(Ctl* ctl, cudaStream_t s) {
     cudaMemsetAsync(&ctl->err, 0, offsetof(Ctl, sweep_wbits) - offsetof(Ctl, err), s);
 }
 
 void clear_build(Ctl* ctl, bool walk, cudaStream_t s) {
-    if (walk) clear_step(ctl, s);
-    else cudaMemsetAsync(&ctl->err, 0, sizeof(int), s);
+    cudaMemsetAsync(&ctl->err, 0, walk ? offsetof(Ctl, pair_count) - offsetof(Ctl, err) : sizeof(int), s);
 }
 
 void clear_search_stats(Ctl* ctl, cudaStream_t s) {

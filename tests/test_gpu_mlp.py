@@ -307,3 +307,16 @@ def test_learned_walk_beats_plain_wide_walk(rb, orc, trained):
         err[name] = orc.e_sum(a[sel], a_dir)
     print(err)
     assert err["learned 0.8"] < err["plain 0.8"]
+
+
+def test_the_count_of_corrections_is_that_of_the_last_learned_walk(rb):
+    """The FP64 potential walk of the energy corrects no cells and leaves the count."""
+    L, N = 100.0, 2400
+    sim = rb.Sim(**sheet_cfg(rb, L, rb.RB_WALK_FP32_LEARNED, 0.8))
+    rb.rb_load_mlp(sim.h, omlp.init(5) * 0.3, 0.5)
+    sim.set_particles(I.sheet(L, N, 1))
+    sim.gravity()
+    n = sim.stats()["corrections"]
+    assert n > 0
+    sim.energy()
+    assert sim.stats()["corrections"] == n
